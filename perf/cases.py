@@ -150,21 +150,29 @@ def _seed(seed, *at):
     return seed
 
 
-def _weights(session, model, layer, seed, fp8):
-    """Installs one layer's surrogate; returns the fp32 matrices that its scores are computed from."""
+def _make_weights(model, seed, fp8):
+    """One layer's surrogate: what the binding is given, and the fp32 matrices that its scores are computed from."""
     d_model, hidden = MODELS[model]
     if hidden:
         w = synth.mlp_weights(d_model, hidden, H, seed, "cuda", bias_sigma=0.02)
     else:
         w = synth.linear_weights(d_model, H, seed, "cuda", bias_sigma=0.02)
-    W1 = w[0].float()
+    W1, rest = w[0].float(), (w[1],) + tuple(x.float() for x in w[2:])
     if fp8:
         codes, scale = synth.quantize_e4m3(w[0])
-        binding.kvzap_set_weights_fp8(session.handle, layer, codes, scale, w[1], *(w[2:] if hidden else (None, None)))
         W1 = codes.view(torch.float8_e4m3fn).float() * scale[:, None]
+        w = (codes, scale, w[1]) + (tuple(w[2:]) if hidden else (None, None))
+    return w, (W1,) + rest
+
+
+def _weights(session, model, layer, seed, fp8):
+    """Installs one layer's surrogate; returns the fp32 matrices."""
+    w, matrices = _make_weights(model, seed, fp8)
+    if fp8:
+        binding.kvzap_set_weights_fp8(session.handle, layer, *w)
     else:
         session.ctx.set_weights(layer, *w)
-    return (W1, w[1]) + (tuple(x.float() for x in w[2:]) if hidden else ())
+    return matrices
 
 
 def _scores(x, w):
@@ -342,10 +350,7 @@ def _prepare_decode(case, seed):
     ws = [_weights(s, case["model"], l, _seed(seed, l, 3), fp8) for l in range(L)]
 
     def inputs(k):
-        x = [_hidden(B, case["model"], ws[l], _seed(seed, l, k, 4), fp8) for l in range(L)]
-        X = torch.stack([t[0] for t in x] if fp8 else x)
-        scale = torch.stack([t[1] for t in x]) if fp8 else None
-        return X, scale, _rows((L, B, H), _seed(seed, k, 5), fp8), _rows((L, B, H), _seed(seed, k, 6), fp8)
+        return _decode_inputs(case, seed, ws, k)
 
     def step(at, b, e, scores):
         X, scale, K, V = at
@@ -367,6 +372,15 @@ def _prepare_decode(case, seed):
         calls += [step(now, b, e, scores[b:e]), attend(s.handle, s.cache, b, e, Q[b:e], 1.0 / math.sqrt(D), O[b:e])]
     torch.cuda.synchronize()
     return {"kind": "calls", "session": s, "calls": calls, "outs": [(scores, O)], "pools": (K_pool, V_pool)}
+
+
+def _decode_inputs(case, seed, ws, k):
+    """The k-th step's hidden states (with scales if 8-bit) and new K and V rows, all layers."""
+    B, L, fp8 = case["seqs"], case["layers"], case["fp8"]
+    x = [_hidden(B, case["model"], ws[l], _seed(seed, l, k, 4), fp8) for l in range(L)]
+    X = torch.stack([t[0] for t in x] if fp8 else x)
+    scale = torch.stack([t[1] for t in x]) if fp8 else None
+    return X, scale, _rows((L, B, H), _seed(seed, k, 5), fp8), _rows((L, B, H), _seed(seed, k, 6), fp8)
 
 
 def _prefixes(case, seed):
@@ -446,3 +460,103 @@ def tolerance(case):
     if case["kind"] == "prefill":
         return {"rel": 2.5e-5}                      # scores: fp32 sums of exact products (6e-6 seen at K = 5120); rows are copied
     return {"rel": 1e-2}                            # attention: probabilities and results rounded to bf16 (2.4e-3 seen)
+
+
+def exact(case, seed):
+    """What the first run() on a state of this seed returns, in 64 bits; None for rows that are copied and for counts."""
+    if case["kind"] == "prune":
+        return None
+    return {"prefill": _exact_prefill, "append": _exact_append, "decode": _exact_decode}[case["kind"]](case, seed)
+
+
+def _exact_scores(x, w, scale=None):
+    """Scores [n, H] in fp64 of hidden states x (bf16, or E4M3 codes with a scale per token)."""
+    w = [m.double() for m in w]
+    out = []
+    for a in range(0, x.shape[0], 16384):
+        part = x[a:a + 16384]
+        part = part.double() if scale is None else \
+            part.view(torch.float8_e4m3fn).float().double() * scale[a:a + 16384, None].double()
+        out.append(_scores(part, w))
+    return torch.cat(out)
+
+
+def _exact_rows(rows):
+    """K or V rows in fp64: bf16 [..., 128], or 8-bit rows with their scale [..., 72]."""
+    if rows.shape[-1] == D:
+        return rows.double()
+    raw = rows.contiguous().view(torch.uint8)
+    scale = raw[..., D:D + 4].contiguous().view(torch.float32).double()
+    return raw[..., :D].contiguous().view(torch.float8_e4m3fn).float().double() * scale
+
+
+def _exact_attention(q, k, v, log_count=None):
+    """q [G, D] over rows k, v [n, D]; log_count [n]: a row that a list holds several times."""
+    logits = q @ k.t() / math.sqrt(D)
+    if log_count is not None:
+        logits = logits + log_count
+    return torch.softmax(logits, dim=1) @ v
+
+
+def _exact_prefill(case, seed):
+    outs = []
+    for l in range(case["layers"]):
+        _, w = _make_weights(case["model"], _seed(seed, l, 1), case["fp8"])
+        X = _hidden(case["tokens"], case["model"], w, _seed(seed, l, 2), case["fp8"], case["sigma"])
+        scores = _exact_scores(*((X[0], w, X[1]) if case["fp8"] else (X, w)))
+        outs.append((None,) * (5 if case["paged"] else 3) + (scores,))
+    return outs
+
+
+def _exact_append(case, seed):
+    N, m, C, L = case["prompts"], case["chunk"], case["chunks"], case["layers"]
+    lens = [_lengths(N * m, N, seed + c) for c in range(C)]
+    Q = _rows((L, 2 * N, H_Q), _seed(seed, 5)).double()
+    O = torch.zeros_like(Q)
+    scores = [[None] * L for _ in range(C)]
+    for l in range(L):
+        _, w = _make_weights(case["model"], _seed(seed, l, 1), False)
+        K, V = [], []
+        for c in range(C):
+            scores[c][l] = _exact_scores(_hidden(N * m, case["model"], w, _seed(seed, l, c, 2)), w)
+            K.append(_rows((H, N * m), _seed(seed, l, c, 3)).double())
+            V.append(_rows((H, N * m), _seed(seed, l, c, 4)).double())
+        for i in range(N):
+            at = [slice(sum(x[:i]), sum(x[:i + 1])) for x in lens]
+            keep = torch.cat([scores[c][l][at[c]] for c in range(C)]) >= TAU
+            keep[-WINDOW:] = True
+            k, v = (torch.cat([x[c][:, at[c]] for c in range(C)], dim=1) for x in (K, V))
+            for h in range(H):
+                g = slice(h * H_Q // H, (h + 1) * H_Q // H)
+                O[l, 2 * i + 1, g] = _exact_attention(Q[l, 2 * i + 1, g], k[h][keep[:, h]], v[h][keep[:, h]])
+    return [x for per_layer in scores for x in per_layer] + [None, O]
+
+
+def _exact_decode(case, seed):
+    B, L, fp8 = case["seqs"], case["layers"], case["fp8"]
+    prefix = _prefixes(case, seed)
+    pages = (prefix + PAGE - 1) // PAGE
+    first = np.concatenate([[0], np.cumsum(pages)[:-1]])
+    pools = [_rows((int(pages.sum()) + 16 * prefix.size, PAGE), _seed(seed, i), fp8) for i in (1, 2)]
+    pools = [x.view(-1, x.shape[-1]) for x in pools]
+    ws = [_make_weights(case["model"], _seed(seed, l, 3), fp8)[1] for l in range(L)]
+    at = [_decode_inputs(case, seed, ws, k) for k in range(4)]
+    scores = [[_exact_scores(*((at[k][0][l], ws[l], at[k][1][l]) if fp8 else (at[k][0][l], ws[l]))) for l in range(L)]
+              for k in (0, 3)]
+    kept = (torch.stack(scores[0]) >= TAU).cpu()                  # the window's oldest token leaves with this step
+    new = [torch.stack([_exact_rows(at[k][i]) for k in range(4)]) for i in (2, 3)]          # [4, L, B, H, D]
+    often = [sum(i % 3 == k for i in range(1, WINDOW)) for k in range(3)] + [1]
+    Q = _rows((L, B, H_Q), _seed(seed, 7)).double()
+    O = torch.zeros_like(Q)
+    counts = [torch.tensor([often[0] + e] + often[1:], dtype=torch.float64, device="cuda").log() for e in (0, 1)]
+    for b in range(B):
+        for l in range(L):
+            for h in range(H):
+                li = (b * L + l) * H + h
+                n = int(prefix[li])
+                k, v = (torch.cat([_exact_rows(pool[int(first[li]) * PAGE:int(first[li]) * PAGE + n]), x[:, l, b, h]])
+                        for pool, x in zip(pools, new))
+                log_count = torch.cat([torch.zeros(n, dtype=torch.float64, device="cuda"), counts[int(kept[l, b, h])]])
+                g = slice(h * H_Q // H, (h + 1) * H_Q // H)
+                O[l, b, g] = _exact_attention(Q[l, b, g], k, v, log_count)
+    return [(torch.stack(scores[1]), O)]
