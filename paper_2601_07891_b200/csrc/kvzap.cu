@@ -51,18 +51,23 @@ struct kvzap_ctx {
         CUtensorMap tmap_w;          // box = the W1 rows one CTA stages per MMA chunk
     } sched[2];
     int pair_clusters = 0;           // CTA pairs that can be resident at once; 0 = pairs unavailable
-    // few-token scoring (decode): clusters of split_n CTAs share a tile, each takes hidden / split_n units
-    int split_n = 0, split_k = 1, split_stages = 0, split_tmem_cols = 0;   // cluster = split_n * split_k CTAs
-    uint32_t split_smem = 0;
-    CUtensorMap split_tmap_w;
-    CUtensorMap split_tmap_w8;           // the 8-bit copy of the weights, same slices (set by kvzap_set_weights_fp8)
-    bool split8_ok = false;
-    // the same kernel with eight CTAs per tile (4 slices x 2 halves of K) for launches of even fewer tiles
-    // (a short prompt or a chunk of one): set when the shape allows it
-    int wide_n = 0, wide_k = 1, wide_stages = 0, wide_tmem_cols = 0;
-    uint32_t wide_smem = 0;
-    CUtensorMap wide_tmap_w;
-    uint32_t *wide_arrive = nullptr;     // its own arrival counts (the count per tile is taken modulo the slices)
+    // few-token scoring (decode, short prompts, chunks): n * k CTAs share a 128-token tile, n slices of the hidden
+    // units times k parts of the K range (a cluster of k CTAs).  [0] is the layout for the largest launches this
+    // kernel serves; the others, widest first, are taken by launches of fewer tiles (split_layout()).
+    struct SplitLayout {
+        int n = 0, k = 1, stages = 0, tmem_cols = 0;
+        int max_clusters = 0;            // clusters of this layout that the device holds at once
+        uint32_t smem = 0;
+        CUtensorMap tmap_w;
+        CUtensorMap tmap_w8;             // the 8-bit copy of the weights, same slices (set by kvzap_set_weights_fp8)
+        bool ok8 = false;
+        uint32_t *arrive = nullptr;      // [sm_count] arrivals per tile over all launches (taken modulo the slices)
+    };
+    static constexpr int kMaxLayouts = 4;
+    SplitLayout layouts[kMaxLayouts];
+    int n_layouts = 0;
+    int split_smem_limit = 0;            // dynamic shared memory the few-token kernel may use
+    uint64_t weights_seq = 0;            // op_seq of the last call that set weights
     // weights of all layers, stacked so that one tensor map / one base pointer serves any layer range
     void *w1_all = nullptr;          // bf16 [L * w1_rows, d_model]
     float *b1_all = nullptr;         // [L][w1_rows]
@@ -85,8 +90,7 @@ struct kvzap_ctx {
     float *select_tau = nullptr;         //                         [max_seqs][H] cut values when the caller wants none
     float *plan_scores = nullptr;        // kvzap_prefill_plan without scores_out: [max_tokens][H] (allocated on first use)
     int64_t *batch_map = nullptr;        // kvzap_prefill_to_cache_batch: first list of each sequence of the call [max_seqs]
-    float *split_part = nullptr;         // few-token kernel: [sm_count tiles][4 slices][128][8] partial scores
-    uint32_t *split_arrive = nullptr;    //                   [sm_count] arrival counts per tile
+    float *split_part = nullptr;         // few-token kernel: [tile][slice][128][8] partial scores, tiles * slices <= sm_count
     uint64_t score_turn = 0;
     bool last_score_early = false;       // the last scoring launch was allowed to start early
     const void *last_scores = nullptr;   // scores buffer of the previous scoring launch, and its size
@@ -124,6 +128,7 @@ struct kvzap_ctx {
     // kernel ahead of it has finished only when that kernel is the fused step of the call just before, on
     // the same cache: those two order their cache accesses through the step counters, nothing else does.
     uint64_t op_seq = 0, fused_seq = 0;
+    int fused_layout = -1;                          // ... in this layout of the few-token kernel
     const kvzap_cache *fused_cache = nullptr;
     std::vector<kvzap_cache *> caches;              // caches created on this context (their step counters are
                                                     // cleared when a timeout has been polled)
@@ -399,8 +404,7 @@ static void free_all(kvzap_ctx *ctx)
     cudaFree(ctx->batch_map);
     cudaFree(ctx->select_hist);
     cudaFree(ctx->select_tau);
-    cudaFree(ctx->split_arrive);
-    cudaFree(ctx->wide_arrive);
+    for (auto &l : ctx->layouts) cudaFree(l.arrive);
     cudaFree(ctx->list_page0);
     cudaFree(ctx->list_base);
     cudaFree(ctx->op_mask); cudaFree(ctx->op_counts); cudaFree(ctx->op_len_acc);
@@ -498,16 +502,32 @@ struct CompactArgs {
     bool tok_major;
 };
 
+// The layout in which a launch of n_tiles tiles runs on the few-token kernel: the widest whose CTAs find an SM each
+// and whose clusters the device holds at once; -1 when there are too many tiles even for the first one.  Measured
+// at 4096 -> 512 -> 8, one launch: a decode step of one tile 27.5 us with 2 x 2 CTAs, 15.0 us with 4 x 8; the scoring of
+// 7 tiles 20.3 us with 4 x 2, 13.5 us with 4 x 4.  What bounds a launch is one CTA's load, (128 + hidden / n) * d_model / k
+// elements at about 55 bytes per clock, on top of some 8 us for its serial parts.
+static int split_layout(const kvzap_ctx *ctx, int64_t n_tiles, bool fp8)
+{
+    for (int i = 1; i < ctx->n_layouts; ++i) {
+        const kvzap_ctx::SplitLayout &l = ctx->layouts[i];
+        if ((!fp8 || l.ok8) && n_tiles * l.n * l.k <= ctx->sm_count && n_tiles * l.n <= l.max_clusters) return i;
+    }
+    if (ctx->n_layouts > 0 && (!fp8 || ctx->layouts[0].ok8) &&
+        n_tiles * ctx->layouts[0].n * ctx->layouts[0].k <= ctx->sm_count) return 0;
+    return -1;
+}
+
 // Launches the scoring kernel over layers [layer, layer + n_layers); hidden is [n_layers][n_tokens][d_model],
 // scores [n_layers][n_tokens][H]; maskbits != nullptr fuses the threshold/window test.
 static kvzap_status launch_score(kvzap_ctx *ctx, int32_t layer, int32_t n_layers, const void *hidden, int64_t n_tokens,
                                  float *scores, uint32_t *maskbits, const int32_t *cu_seqlens, int32_t n_seqs,
                                  float tau, int32_t w, cudaStream_t stream, int32_t window_keep = 1,
-                                 const DecodeFuse *fuse = nullptr, bool *fused = nullptr, bool fuse_chain = false,
+                                 const DecodeFuse *fuse = nullptr, int *fused_layout = nullptr, const int *fuse_chain = nullptr,
                                  const CompactArgs *compact = nullptr, bool *compacted = nullptr,
                                  bool fp8 = false, const float *x_scale = nullptr)
 {
-    if (fused) *fused = false;
+    if (fused_layout) *fused_layout = -1;
     if (compacted) *compacted = false;
     // Early start.  When the grid fills the machine (one CTA per SM), this kernel is allowed to start
     // while the kernels ahead of it in the stream -- the previous call's scoring kernel finishing its
@@ -530,15 +550,15 @@ static kvzap_status launch_score(kvzap_ctx *ctx, int32_t layer, int32_t n_layers
     // ... and with the K split left out (two CTAs per tile, each a slice of the hidden units over the whole K
     // range) the same kernel serves launches of up to half as many tiles as there are SMs, where CTA pairs
     // would leave most SMs idle.
-    const bool slices_only = ctx->split_n == 2 && ctx->split_k == 2 && fuse == nullptr && !fp8 &&
-                             blocks_per_layer * n_layers * 4 > ctx->sm_count && blocks_per_layer * n_layers * 2 <= ctx->sm_count;
-    if (fp8 && !(ctx->split8_ok && blocks_per_layer * n_layers * ctx->split_n * ctx->split_k <= ctx->sm_count))
+    const int64_t few_tiles = blocks_per_layer * n_layers;
+    const int layout_i = split_layout(ctx, few_tiles, fp8);
+    const bool slices_only = layout_i < 0 && ctx->n_layouts > 0 && ctx->layouts[0].n == 2 && ctx->layouts[0].k == 2 &&
+                             fuse == nullptr && !fp8 && few_tiles * 2 <= ctx->sm_count;
+    if (fp8 && layout_i < 0)
         return fail(ctx, KVZAP_ERR_UNSUPPORTED, "8-bit few-token scoring: this shape has no four-CTA layout");
-    if (ctx->split_n > 0 && (slices_only || blocks_per_layer * n_layers * ctx->split_n * ctx->split_k <= ctx->sm_count)) {
-        // eight CTAs per tile when even those fit (not for the fused decode step, which is laid out for four)
-        const bool wide = ctx->wide_n > 0 && fuse == nullptr && !fp8 &&
-                          blocks_per_layer * n_layers * ctx->wide_n * ctx->wide_k <= ctx->sm_count;
-        const int split_n = wide ? ctx->wide_n : ctx->split_n, split_k = wide ? ctx->wide_k : (slices_only ? 1 : ctx->split_k);
+    if (layout_i >= 0 || slices_only) {
+        const kvzap_ctx::SplitLayout &layout = ctx->layouts[slices_only ? 0 : layout_i];
+        const int split_n = layout.n, split_k = slices_only ? 1 : layout.k;
         CUtensorMap tmap_x;
         kvzap_status st = fp8 ? make_tmap8(ctx, &tmap_x, hidden, static_cast<uint64_t>(n_tokens), static_cast<uint64_t>(c.d_model),
                                            kTileM, static_cast<uint64_t>(n_layers), false)
@@ -558,9 +578,9 @@ static kvzap_status launch_score(kvzap_ctx *ctx, int32_t layer, int32_t n_layers
         p.d_model = c.d_model;
         p.group_w = p.chunk_n = c.hidden / split_n;
         p.n_groups = p.n_chunks = 1;
-        p.n_stages = wide ? ctx->wide_stages : ctx->split_stages;
+        p.n_stages = layout.stages;
         p.acc_bufs = 1;
-        p.tmem_cols = wide ? ctx->wide_tmem_cols : ctx->split_tmem_cols;
+        p.tmem_cols = layout.tmem_cols;
         p.n_hidden = c.hidden;
         p.n_heads = c.n_kv_heads;
         p.b1 = ctx->b1_all;
@@ -576,7 +596,7 @@ static kvzap_status launch_score(kvzap_ctx *ctx, int32_t layer, int32_t n_layers
         p.tau = tau;
         p.status = ctx->status_dev;
         p.split_part = ctx->split_part;
-        p.split_arrive = wide ? ctx->wide_arrive : ctx->split_arrive;
+        p.split_arrive = layout.arrive;
         // Early start (consecutive decode steps): this kernel reads only hidden states and weights; the one
         // thing it may not do is write a scores buffer that the kernels of the previous call still read.
         const size_t sbytes = scores ? sizeof(float) * static_cast<size_t>(n_layers) * n_tokens * c.n_kv_heads : 0;
@@ -590,34 +610,41 @@ static kvzap_status launch_score(kvzap_ctx *ctx, int32_t layer, int32_t n_layers
         const int n_ctas = split_n * split_k;
         DecodeFuse f;
         memset(&f, 0, sizeof f);
-        const bool fuse_ok = fuse != nullptr && !ctx->profiling && n_ctas == 4;
+        const bool fuse_ok = fuse != nullptr && !ctx->profiling && !slices_only;
         if (fuse_ok) {
             f = *fuse;
             f.enabled = 1;
-            if (fused) *fused = true;
+            // counters of this layout's CTAs: behind those of the layouts before it (kvzap_cache_create)
+            const int64_t cache_tiles = static_cast<int64_t>(c.n_layers) * blocks_per_layer;
+            for (int i = 0; i < layout_i; ++i) {
+                f.done += cache_tiles * ctx->layouts[i].n;
+                f.ticket += cache_tiles * ctx->layouts[i].n * ctx->layouts[i].k;
+            }
+            *fused_layout = layout_i;
         }
-        // The fused decode step touches the cache (counters, page allocator, rows) before it has waited for
-        // the kernel ahead; its clusters order themselves through `done`, which covers earlier fused steps
-        // only.  So it is started early only directly behind the fused step of the previous call on the
-        // same cache (fuse_chain) -- never behind a prompt chunk's page assignment, a release or an export,
-        // whose kernels it would race with -- and with a grid of at least half the SMs and its own scores
-        // buffer.  Without the fused part the kernel reads nothing but hidden states and weights until
-        // every thread has waited, and writes only after: it may always start early.
-        const bool early = !ctx->profiling &&
-                           (fuse_ok ? (fuse_chain && !clash && p.n_tiles * n_ctas * 2 >= ctx->sm_count) : true);
-        p.wait_before_load = ctx->trusted ? 0 : 1;
+        // Early start.  Without the fused part the kernel reads nothing but weights, and hidden states of trusted
+        // producers, until every thread has waited for the kernel ahead, and writes only after.  The fused decode
+        // step touches the cache (counters, page allocator, rows): its clusters order themselves through `done`,
+        // which covers earlier fused steps of the same layout only, so it does that before the wait only directly
+        // behind such a step of the previous call on the same cache (fuse_chain) -- never behind a prompt chunk's
+        // page assignment, a release or an export, whose kernels it would race with -- and with a grid of at least
+        // half the SMs and its own scores buffer; else all it does before the wait is to fetch its first W1 tiles.
+        // Directly behind the call that wrote the weights not even that is allowed.
+        const bool overlap = fuse_ok && fuse_chain != nullptr && *fuse_chain == layout_i && !clash &&
+                             p.n_tiles * n_ctas * 2 >= ctx->sm_count;
+        const bool early = !ctx->profiling && ctx->weights_seq + 1 != ctx->op_seq;
+        p.wait_before_load = ctx->trusted && (!fuse_ok || overlap) ? 0 : 1;
         ctx->last_score_early = early;
         {
             ProfScope prof(ctx, KVZAP_KERNEL_SCORE, stream);
             cudaLaunchConfig_t cfg;
             cudaLaunchAttribute attrs[2];
-            make_launch(&cfg, attrs, dim3(static_cast<unsigned>(p.n_tiles * n_ctas)), dim3(kScoreThreads),
-                        wide ? ctx->wide_smem : ctx->split_smem, stream, early, split_k);
+            make_launch(&cfg, attrs, dim3(static_cast<unsigned>(p.n_tiles * n_ctas)), dim3(kScoreThreads), layout.smem, stream, early,
+                        split_k);
             if (fp8)
-                KVZAP_CUDA(ctx, cudaLaunchKernelEx(&cfg, score_split_kernel<true>, tmap_x, ctx->split_tmap_w8, p, split_n, split_k, f));
+                KVZAP_CUDA(ctx, cudaLaunchKernelEx(&cfg, score_split_kernel<true>, tmap_x, layout.tmap_w8, p, split_n, split_k, f));
             else
-                KVZAP_CUDA(ctx, cudaLaunchKernelEx(&cfg, score_split_kernel<false>, tmap_x, wide ? ctx->wide_tmap_w : ctx->split_tmap_w, p,
-                                                   split_n, split_k, f));
+                KVZAP_CUDA(ctx, cudaLaunchKernelEx(&cfg, score_split_kernel<false>, tmap_x, layout.tmap_w, p, split_n, split_k, f));
         }
         ctx->launches += 1;
         return KVZAP_OK;
@@ -1245,44 +1272,39 @@ kvzap_status kvzap_create(kvzap_ctx **out, const kvzap_config *cfg)
         }
     }
     if (c.hidden > 0) {
-        // few-token schedule: four CTAs per tile.  2 x 2 (two slices of hidden units, two halves of K) when
-        // a slice of hidden / 2 units fits one MMA and the K blocks divide evenly, else four slices.
-        const bool two_by_two = c.hidden / 2 <= 256 && (c.hidden / 4) % 16 == 0 && (c.d_model / kBlockK) % 2 == 0;
-        const int n_split = two_by_two ? 2 : 4, k_split = two_by_two ? 2 : 1, ns = c.hidden / n_split;
-        int stages = kMaxStages;
-        for (; stages >= 2; --stages)
-            if (static_cast<int>(split_smem_layout(ns, stages, 4).total) <= budget - 4096) break;   // 4 KB static
-        if (stages >= 2 && ns % 16 == 0 && ns <= 256) {
-            ctx->split_stages = stages;
-            ctx->split_smem = split_smem_layout(ns, stages, 4).total + 1024;
-            ctx->split_tmem_cols = next_pow2(ns);
-            CREATE_CUDA(cudaFuncSetAttribute(score_split_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                             static_cast<int>(ctx->split_smem)));
-            if (make_tmap_w(ctx, &ctx->split_tmap_w, ctx->w1_all, static_cast<uint64_t>(c.n_layers) * ctx->w1_rows,
-                            static_cast<uint64_t>(c.d_model / kBlockK), static_cast<uint32_t>(ns)) == KVZAP_OK) {
-                ctx->split_n = n_split;
-                ctx->split_k = k_split;
+        ctx->split_smem_limit = budget + 1024 - 4608;       // the kernel has 4112 bytes of static shared memory
+        // the limit is the function's, not the context's: the most that any layout of any context takes
+        CREATE_CUDA(cudaFuncSetAttribute(score_split_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, ctx->split_smem_limit));
+        // Few-token layouts.  The first takes the largest launches: four CTAs per tile, 2 x 2 (two slices of hidden
+        // units, two parts of K) when a slice of hidden / 2 units fits one MMA and the K blocks divide evenly, else
+        // four slices.  The others spread a tile over more CTAs, widest first; of two of the same width the one whose
+        // CTAs load less comes first and the other is left out.
+        const int kb = c.d_model / kBlockK;
+        const bool two_by_two = c.hidden / 2 <= 256 && (c.hidden / 4) % 16 == 0 && kb % 2 == 0;
+        const int shapes[][2] = {{two_by_two ? 2 : 4, two_by_two ? 2 : 1}, {8, 8}, {5, 8}, {4, 8}, {5, 4}, {4, 4}, {4, 2}};
+        for (const auto &sh : shapes) {
+            const int n = sh[0], k = sh[1], ns = c.hidden / n, i = ctx->n_layouts;
+            if (i == kvzap_ctx::kMaxLayouts || c.hidden % (16 * n * k) != 0 || ns > 256 || kb % k != 0) continue;
+            if (i > 1 && n * k > ctx->layouts[i - 1].n * ctx->layouts[i - 1].k / 2) continue;
+            kvzap_ctx::SplitLayout &l = ctx->layouts[i];
+            l.n = n;
+            l.k = k;
+            for (l.stages = kMaxStages; l.stages >= 2; --l.stages)
+                if (split_smem_fits(ns, l.stages, k, ctx->split_smem_limit - 1024)) break;
+            if (l.stages < 2) { if (i == 0) break; else continue; }
+            l.smem = split_smem_layout(ns, l.stages, k).total + 1024;
+            l.tmem_cols = next_pow2(ns);
+            if (make_tmap_w(ctx, &l.tmap_w, ctx->w1_all, static_cast<uint64_t>(c.n_layers) * ctx->w1_rows,
+                            static_cast<uint64_t>(kb), static_cast<uint32_t>(ns)) != KVZAP_OK) {
+                if (i == 0) break; else continue;
             }
-        }
-        // 4 x 2: slices of hidden / 4 units, each CTA finishing hidden / 8 of them
-        const int ns8 = c.hidden / 4;
-        if (ctx->split_n > 0 && c.hidden % 128 == 0 && ns8 <= 256 && (c.d_model / kBlockK) % 2 == 0) {
-            int st8 = kMaxStages;
-            for (; st8 >= 2; --st8)
-                if (static_cast<int>(split_smem_layout(ns8, st8, 8).total) <= budget - 4096) break;
-            if (st8 >= 2) {
-                ctx->wide_stages = st8;
-                ctx->wide_smem = split_smem_layout(ns8, st8, 8).total + 1024;
-                ctx->wide_tmem_cols = next_pow2(ns8);
-                if (ctx->wide_smem > ctx->split_smem)
-                    CREATE_CUDA(cudaFuncSetAttribute(score_split_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                                     static_cast<int>(ctx->wide_smem)));
-                if (make_tmap_w(ctx, &ctx->wide_tmap_w, ctx->w1_all, static_cast<uint64_t>(c.n_layers) * ctx->w1_rows,
-                                static_cast<uint64_t>(c.d_model / kBlockK), static_cast<uint32_t>(ns8)) == KVZAP_OK) {
-                    ctx->wide_n = 4;
-                    ctx->wide_k = 2;
-                }
-            }
+            cudaLaunchConfig_t cfg;
+            cudaLaunchAttribute attrs[2];
+            make_launch(&cfg, attrs, dim3(static_cast<unsigned>(n * k)), dim3(kScoreThreads), l.smem, nullptr, false, k);
+            CREATE_CUDA(cudaOccupancyMaxActiveClusters(&l.max_clusters, score_split_kernel<false>, &cfg));
+            CREATE_CUDA(cudaMalloc(&l.arrive, sizeof(uint32_t) * static_cast<size_t>(ctx->sm_count)));
+            CREATE_CUDA(cudaMemset(l.arrive, 0, sizeof(uint32_t) * static_cast<size_t>(ctx->sm_count)));
+            ctx->n_layouts = i + 1;
         }
     }
     ctx->max_blocks = (c.max_tokens + kBlockTokens - 1) / kBlockTokens;
@@ -1294,13 +1316,8 @@ kvzap_status kvzap_create(kvzap_ctx **out, const kvzap_config *cfg)
     CREATE_CUDA(cudaMemset(ctx->tile_counters, 0, sizeof(int32_t) * kMaskRing));
     CREATE_CUDA(cudaMalloc(&ctx->select_hist, sizeof(uint32_t) * 4 * static_cast<size_t>(c.max_seqs) * c.n_kv_heads * 256));
     CREATE_CUDA(cudaMalloc(&ctx->select_tau, sizeof(float) * static_cast<size_t>(c.max_seqs) * c.n_kv_heads));
-    if (ctx->split_n > 0) {
-        CREATE_CUDA(cudaMalloc(&ctx->split_part, sizeof(float) * static_cast<size_t>(ctx->sm_count) * 4 * kTileM * kMaxHeads));
-        CREATE_CUDA(cudaMalloc(&ctx->split_arrive, sizeof(uint32_t) * static_cast<size_t>(ctx->sm_count)));
-        CREATE_CUDA(cudaMemset(ctx->split_arrive, 0, sizeof(uint32_t) * static_cast<size_t>(ctx->sm_count)));
-        CREATE_CUDA(cudaMalloc(&ctx->wide_arrive, sizeof(uint32_t) * static_cast<size_t>(ctx->sm_count)));
-        CREATE_CUDA(cudaMemset(ctx->wide_arrive, 0, sizeof(uint32_t) * static_cast<size_t>(ctx->sm_count)));
-    }
+    if (ctx->n_layouts > 0)
+        CREATE_CUDA(cudaMalloc(&ctx->split_part, sizeof(float) * static_cast<size_t>(ctx->sm_count) * kTileM * kMaxHeads));
     {
         // one-launch pruning: a grid never larger than what the device holds at once (its CTAs wait for one another)
         // No shared-memory carve-out is asked for: with the largest one (which the compaction that runs beside
@@ -1391,6 +1408,7 @@ kvzap_status kvzap_set_weights(kvzap_ctx *ctx, int32_t layer, const void *W1, co
     }
     ctx->layer_set[layer] = 1;
     ctx->layer_fp8[layer] = 0;
+    ctx->weights_seq = ctx->op_seq;
     return KVZAP_OK;
 }
 
@@ -1421,15 +1439,17 @@ kvzap_status kvzap_set_weights_fp8(kvzap_ctx *ctx, int32_t layer, const void *W1
                                          static_cast<uint64_t>(c.d_model), static_cast<uint32_t>(ctx->sched[mode].chunk_n / (mode + 1)), 0, true);
             if (st != KVZAP_OK) return st;
         }
-        if (c.hidden > 0 && ctx->split_n > 0 && (c.d_model / 128) % ctx->split_k == 0) {
-            // the few-token layout (a decode step): the same slices of hidden units, K blocks of 128 codes
-            if (make_tmap8(ctx, &ctx->split_tmap_w8, ctx->w1_fp8_all, static_cast<uint64_t>(rows_total), static_cast<uint64_t>(c.d_model),
-                           static_cast<uint32_t>(c.hidden / ctx->split_n), 0, true) == KVZAP_OK &&
-                cudaFuncSetAttribute(score_split_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                     static_cast<int>(ctx->split_smem)) == cudaSuccess &&
-                cudaFuncSetAttribute(score_split_kernel<true>, cudaFuncAttributePreferredSharedMemoryCarveout,
-                                     static_cast<int>(cudaSharedmemCarveoutMaxShared)) == cudaSuccess)
-                ctx->split8_ok = true;
+        for (int i = 0; i < ctx->n_layouts; ++i) {
+            // the few-token layouts: the same slices of hidden units, K blocks of 128 codes
+            kvzap_ctx::SplitLayout &l = ctx->layouts[i];
+            if ((c.d_model / 128) % l.k != 0) continue;
+            l.ok8 = make_tmap8(ctx, &l.tmap_w8, ctx->w1_fp8_all, static_cast<uint64_t>(rows_total), static_cast<uint64_t>(c.d_model),
+                               static_cast<uint32_t>(c.hidden / l.n), 0, true) == KVZAP_OK;
+        }
+        if (ctx->n_layouts > 0) {
+            KVZAP_CUDA(ctx, cudaFuncSetAttribute(score_split_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, ctx->split_smem_limit));
+            KVZAP_CUDA(ctx, cudaFuncSetAttribute(score_split_kernel<true>, cudaFuncAttributePreferredSharedMemoryCarveout,
+                                                 static_cast<int>(cudaSharedmemCarveoutMaxShared)));
         }
         if (c.hidden > 0) {
             KVZAP_CUDA(ctx, cudaFuncSetAttribute(score_kernel<true, false, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(ctx->sched[0].smem)));
@@ -1465,6 +1485,7 @@ kvzap_status kvzap_set_weights_fp8(kvzap_ctx *ctx, int32_t layer, const void *W1
         ctx->launches += 1;
     }
     ctx->layer_set[layer] = 0;       // the bf16 entry points refuse this layer from now on
+    ctx->weights_seq = ctx->op_seq;
     ctx->layer_fp8[layer] = 1;
     return KVZAP_OK;
 }
@@ -1632,7 +1653,7 @@ static kvzap_status prefill_fused_impl(kvzap_ctx *ctx, int32_t layer, const void
     const CompactArgs compact{K, V, K_out, V_out, lengths, tok_major};
     bool compacted = false;
     st = launch_score(ctx, layer, 1, hidden, n_tokens, scores_out, mask, cu_seqlens, n_seqs, tau, w, stream, 1, nullptr, nullptr,
-                      false, &compact, &compacted);
+                      nullptr, &compact, &compacted);
     if (st != KVZAP_OK || compacted) return st;
     return launch_compaction(ctx, mask, K, V, cu_seqlens, n_seqs, n_tokens, K_out, V_out, lengths, stream, true, tok_major);
 }
@@ -1702,8 +1723,8 @@ kvzap_status kvzap_poll_status(kvzap_ctx *ctx, void *stream_)
     if (v == 0) return KVZAP_OK;
     // a scoring kernel that gave up may have left its work-tile counter in an unknown state
     cudaMemsetAsync(ctx->tile_counters, 0, sizeof(int32_t) * kMaskRing, stream);
-    if (ctx->split_arrive) cudaMemsetAsync(ctx->split_arrive, 0, sizeof(uint32_t) * static_cast<size_t>(ctx->sm_count), stream);
-    if (ctx->wide_arrive) cudaMemsetAsync(ctx->wide_arrive, 0, sizeof(uint32_t) * static_cast<size_t>(ctx->sm_count), stream);
+    for (int i = 0; i < ctx->n_layouts; ++i)
+        cudaMemsetAsync(ctx->layouts[i].arrive, 0, sizeof(uint32_t) * static_cast<size_t>(ctx->sm_count), stream);
     if (v == KVZAP_ERR_TIMEOUT) {
         reset_step_counters(ctx, stream);
         // a one-launch pruning call that gave up may have left its list-length sums and arrival count behind
@@ -1865,8 +1886,8 @@ struct kvzap_cache {
     int64_t n_lists = 0;
     int step_parity = 0;
     // fused decode steps: per-cluster count of completed steps on the device, and the host's view of it
-    int32_t *done = nullptr;             // [n_layers * ceil(n_seqs / 128)][4]: one per cluster of the fused step
-    int32_t *ticket = nullptr;           // behind `done`: [tiles][4][2] steps started per (slice, rank), see DecodeFuse
+    int32_t *done = nullptr;             // per layout [n_layers * ceil(n_seqs / 128)][n]: one per cluster of the fused step
+    int32_t *ticket = nullptr;           // behind `done`: per layout [tiles][n][k] steps started per (slice, rank), see DecodeFuse
     size_t n_step_counters = 0;          // ints in done + ticket together
     // attention over the cache: tensor maps of the page pools and of the window rings (built on first use)
     CUtensorMap tm_kpool, tm_vpool, tm_kring, tm_vring;
@@ -1881,7 +1902,7 @@ namespace kvzap {
 static void reset_step_counters(kvzap_ctx *ctx, cudaStream_t stream)
 {
     for (kvzap_cache *cache : ctx->caches) {
-        cudaMemsetAsync(cache->done, 0, sizeof(int32_t) * cache->n_step_counters, stream);
+        if (cache->done) cudaMemsetAsync(cache->done, 0, sizeof(int32_t) * cache->n_step_counters, stream);
     }
     ctx->fused_cache = nullptr;
 }
@@ -2102,9 +2123,14 @@ kvzap_status kvzap_cache_create(kvzap_ctx *ctx, kvzap_cache **out, int32_t n_seq
     if (e == cudaSuccess) e = cudaMemset(v.active, 1, static_cast<size_t>(n_seqs));      // every slot takes part until released
     {
         const size_t tiles = static_cast<size_t>(c.n_layers) * ((n_seqs + 127) / 128);
-        cache->n_step_counters = 12 * tiles;          // done [tiles][4], then ticket [tiles][4][2]
-        alloc(reinterpret_cast<void **>(&cache->done), sizeof(int32_t) * cache->n_step_counters, true);
-        cache->ticket = cache->done ? cache->done + 4 * tiles : nullptr;
+        size_t n_done = 0, n_ticket = 0;              // per layout of the step: done [tiles][n]; then ticket [tiles][n][k]
+        for (int i = 0; i < ctx->n_layouts; ++i) {
+            n_done += tiles * ctx->layouts[i].n;
+            n_ticket += tiles * ctx->layouts[i].n * ctx->layouts[i].k;
+        }
+        cache->n_step_counters = n_done + n_ticket;
+        if (n_done > 0) alloc(reinterpret_cast<void **>(&cache->done), sizeof(int32_t) * cache->n_step_counters, true);
+        cache->ticket = cache->done ? cache->done + n_done : nullptr;
     }
     // two halves used by alternate steps when the caller does not ask for the scores
     alloc(reinterpret_cast<void **>(&cache->scores), 2 * sizeof(float) * static_cast<size_t>(c.n_layers) * n_seqs * c.n_kv_heads,
@@ -2130,7 +2156,8 @@ kvzap_status kvzap_cache_debug_skew_steps(kvzap_cache *cache, int32_t delta)
     if (!cache) return KVZAP_ERR_INVALID_ARG;
     DeviceGuard guard(cache->ctx->cfg.device);
     if (cudaDeviceSynchronize() != cudaSuccess) return KVZAP_ERR_CUDA;
-    const int n = static_cast<int>(cache->n_step_counters / 3 * 2);
+    const int n = cache->ticket ? static_cast<int>(cache->done + cache->n_step_counters - cache->ticket) : 0;
+    if (n == 0) return KVZAP_OK;
     add_int_kernel<<<(n + 255) / 256, 256>>>(cache->ticket, n, delta);
     if (cudaDeviceSynchronize() != cudaSuccess) return KVZAP_ERR_CUDA;
     return KVZAP_OK;
@@ -2194,12 +2221,13 @@ static kvzap_status decode_step_impl(kvzap_ctx *ctx, kvzap_cache *cache, int32_t
         fuse.done = cache->done;
         fuse.wait_limit = ctx->wait_limit;
     }
-    bool fused = false;
+    int fused_layout = -1;
     // the call just before this one was a fused step on this cache: the two may overlap
     const bool chain = ctx->fused_cache == cache && ctx->fused_seq + 1 == ctx->op_seq;
+    const int chain_layout = chain ? ctx->fused_layout : -1;
     kvzap_status st = KVZAP_OK;
     const int64_t step_tiles = (static_cast<int64_t>(cache->v.n_seqs) + kTileM - 1) / kTileM * n_layers;
-    if (fp8 && !(c.hidden > 0 && ctx->split8_ok && step_tiles * ctx->split_n * ctx->split_k <= ctx->sm_count)) {
+    if (fp8 && split_layout(ctx, step_tiles, true) < 0) {
         // no few-token layout for this shape: layer after layer through the prefill scoring kernel
         for (int l = 0; l < n_layers && st == KVZAP_OK; ++l)
             st = launch_score_fp8(ctx, layer_begin + l, static_cast<const uint8_t *>(hidden) + static_cast<size_t>(l) * cache->v.n_seqs * c.d_model,
@@ -2207,11 +2235,12 @@ static kvzap_status decode_step_impl(kvzap_ctx *ctx, kvzap_cache *cache, int32_t
                                   scores + static_cast<size_t>(l) * cache->v.n_seqs * c.n_kv_heads, nullptr, nullptr, 1, 0.0f, 0, stream);
     } else {
         st = launch_score(ctx, layer_begin, n_layers, hidden, cache->v.n_seqs, scores, nullptr, nullptr, 1,
-                          0.0f, 0, stream, 1, can_fuse ? &fuse : nullptr, &fused, chain, nullptr, nullptr, fp8, x_scale);
+                          0.0f, 0, stream, 1, can_fuse ? &fuse : nullptr, &fused_layout, &chain_layout, nullptr, nullptr, fp8, x_scale);
     }
     if (st != KVZAP_OK) return st;
-    if (fused) {
+    if (fused_layout >= 0) {
         ctx->fused_cache = cache;
+        ctx->fused_layout = fused_layout;
         ctx->fused_seq = ctx->op_seq;
         return KVZAP_OK;
     }

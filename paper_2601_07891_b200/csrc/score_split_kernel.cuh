@@ -3,19 +3,23 @@
 // most SMs idle and every byte of W1 has to come from HBM.
 //
 // n_split * k_split CTAs share one 128-token tile.  The hidden units are cut into n_split slices of
-// Ns = hidden / n_split; a slice is computed by a cluster of k_split CTAs (1 or 2).  With k_split = 2
-// each CTA of the pair runs half of the K range (so an X tile is read by two CTAs per slice and every
-// byte of W1 exactly once), and the two partial pre-activation tiles are combined before the GELU:
-// each CTA sends the half of its accumulator that its partner owns through distributed shared memory
-// (into the partner's pipeline stages, idle by then) and finishes the columns it owns itself: bias,
-// GELU, its part of the second layer.  The 8 partial sums per token go to the pair's first CTA
-// (distributed shared memory, one cluster barrier).
+// Ns = hidden / n_split; a slice is computed by a cluster of k_split CTAs (1, 2, 4 or 8).  Each CTA of a
+// cluster runs its part of the K range (so every byte of W1 is read once, and an X tile once per slice),
+// and the partial pre-activation tiles are combined before the GELU: a CTA owns Ns / k_split columns of
+// the slice, sends each of the others the columns of its accumulator which that one owns through
+// distributed shared memory (into the receiver's pipeline stages, idle by then) and finishes its own:
+// the parts in rank order, bias, GELU, its part of the second layer.  The 8 partial sums per token go to
+// the cluster's first CTA (distributed shared memory, one cluster barrier).
 //
 // The slices of a tile meet in global memory: the first CTA of every cluster stores its 128 x 8 partial
 // sums and counts itself in; the cluster that arrives last adds the parts in slice order (so the sum
 // does not depend on who was last) plus b2 and writes the scores (and, if asked for, the keep bits).
-// Clusters are kept this small on purpose: 36 layers x 2 slices x 2 CTAs fill the machine at once,
-// whereas clusters of four do not all find four free SMs in one GPC and leave a second wave.
+// How many CTAs share a tile is the host's choice by the number of tiles (see SplitLayout): what a launch
+// of few tiles costs is the time in which one CTA pulls its part of X and W1, so it takes the widest layout
+// whose clusters are all resident at once.  Many tiles (36 layers x 2 slices) keep clusters of two: those
+// fill the machine at once, whereas clusters of four do not all find four free SMs in one GPC and leave a
+// second wave.  W1 is the context's own copy, so its first tiles are fetched before the wait for the work
+// ahead in the stream.
 //
 // Warp roles as in score_kernel: warp 0 TMA producer, warp 1 MMA issuer / TMEM owner, warps 2..9
 // epilogue (TMEM lane quarter = warp % 4; the two warps of a quarter take alternate 16-column chunks).
@@ -28,7 +32,7 @@ namespace kvzap {
 
 // Decode step fused into the scoring launch (enabled != 0): while the MMAs run, the epilogue warps
 // of a cluster do the cache update of the cluster's own lists -- 128 sequences x H heads of one layer,
-// a quarter per CTA -- exactly as decode_update_kernel does (the token that leaves the window is
+// an equal part per CTA -- exactly as decode_update_kernel does (the token that leaves the window is
 // judged by its buffered score, so nothing here needs the new scores); the cluster's first CTA puts
 // the new scores into the score buffer at the very end (the last cluster of the tile to arrive).
 // Consecutive steps may overlap in time (the next launch starts as SMs become free): `done[cluster]`
@@ -39,7 +43,7 @@ namespace kvzap {
 // host knows -- a captured CUDA graph of steps can be replayed.
 struct DecodeFuse {
     int32_t enabled;
-    int32_t *ticket;                // [n_layers * tiles_per_layer][4][2]: steps started, per (slice, rank in the cluster)
+    int32_t *ticket;                // [n_layers * tiles_per_layer][n_split][k_split]: steps started, per (slice, rank in the cluster)
     CacheView c;
     const uint4 *K_new, *V_new;     // [n_layers_call][B][H][D] bf16
     float tau;
@@ -50,7 +54,9 @@ struct DecodeFuse {
 struct SplitSmemLayout {
     uint32_t stage_bytes, stages_end, w2s, b1s, w1s, part, xpart, bars, total;
 };
-__host__ __device__ inline SplitSmemLayout split_smem_layout(int ns, int n_stages, int n_split)
+// The parts received from the other CTAs of the cluster ([k_split - 1][own / 4][128 rows] float4) lie over the
+// stages, idle by then, and behind them the sums that the cluster's CTAs leave with its first one ([k_split][128][8]).
+__host__ __device__ inline SplitSmemLayout split_smem_layout(int ns, int n_stages, int k_split)
 {
     SplitSmemLayout L;
     L.stage_bytes = kATileBytes + static_cast<uint32_t>(ns) * kBlockK * 2;
@@ -59,15 +65,21 @@ __host__ __device__ inline SplitSmemLayout split_smem_layout(int ns, int n_stage
     L.b1s = L.w2s + static_cast<uint32_t>(ns) * kMaxHeads * 4;
     L.w1s = L.b1s + static_cast<uint32_t>(ns) * 4;            // first-layer row scales (8-bit inputs)
     L.part = L.w1s + static_cast<uint32_t>(ns) * 4;
-    L.xpart = L.part + kTileM * kMaxHeads * 4;
-    L.bars = L.xpart + static_cast<uint32_t>(n_split) * kTileM * kMaxHeads * 4;
+    L.xpart = static_cast<uint32_t>(ns / k_split * (k_split - 1)) * kTileM * 4;
+    L.bars = L.part + kTileM * kMaxHeads * 4;
     L.total = L.bars + 256;
     return L;
+}
+__host__ inline bool split_smem_fits(int ns, int n_stages, int k_split, int budget)
+{
+    const SplitSmemLayout L = split_smem_layout(ns, n_stages, k_split);
+    return static_cast<int>(L.total) <= budget &&
+           L.xpart + static_cast<uint32_t>(k_split) * kTileM * kMaxHeads * 4 <= L.stages_end;
 }
 
 // p.group_w = p.chunk_n = Ns (the MMA's N); p.n_chunks = 1; p.acc_bufs = 1; p.n_tiles = 128-token tiles
 // over all layers of the call; cluster dimension k_split, gridDim.x = n_split * k_split * p.n_tiles.
-// A CTA ends up owning Ns / k_split hidden units: xpart and the W2 / b1 slices are sized for those.
+// A CTA ends up owning Ns / k_split hidden units.
 // kFp8: hidden states and W1 are E4M3 bytes (K blocks of 128 codes, tcgen05.mma kind::f8f6f4); the scales
 // x_scale[token] * w1_scale[hidden unit] multiply the summed pre-activation before the bias.
 template <bool kFp8>
@@ -86,7 +98,7 @@ score_split_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_cons
     const uint32_t smem_base = raw_addr + pad;
     const int ns = p.chunk_n;
     const int n_ctas = n_split * k_split;
-    const SplitSmemLayout L = split_smem_layout(ns, p.n_stages, n_ctas);
+    const SplitSmemLayout L = split_smem_layout(ns, p.n_stages, k_split);
 
     ulonglong2 *w2p = reinterpret_cast<ulonglong2 *>(smem + L.w2s);
     float *w2f = reinterpret_cast<float *>(smem + L.w2s);
@@ -118,13 +130,10 @@ score_split_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_cons
         // the step number, drawn before any thread of this CTA lets the next launch be placed: a CTA of that launch
         // starts only after every CTA of this one has passed the instruction below, hence after this draw
         if (threadIdx.x == 0)
-            fuse_step = atomicAdd(f.ticket + ((layer * p.tiles_per_layer + m_tile) * 4 + nh) * 2 + kh, 1);
+            fuse_step = atomicAdd(f.ticket + ((layer * p.tiles_per_layer + m_tile) * n_split + nh) * k_split + kh, 1);
         __syncthreads();
     }
     griddep_launch_dependents();
-    // unless the caller vouches for the producers of its inputs, nothing of them is read before the work
-    // ahead in the stream has completed (every thread waits: the loads below are issued by several warps)
-    if (p.wait_before_load) griddep_wait();
     const int own_n = ns / k_split;                      // accumulator columns this CTA finishes
     const int own_c0 = kh * own_n;                       // the first of them
     const int j_first = nh * ns + own_c0;                // = first hidden unit of this CTA
@@ -149,16 +158,16 @@ score_split_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_cons
     const int w_row = layer * p.w_rows + nh * ns;
     const int row0 = m_tile * kTileM;
     const int n_pre = k_blocks < p.n_stages ? k_blocks : p.n_stages;
+    // The first loads go out before the CTA-wide barrier below (TMEM allocation, the other warps): the
+    // stages are empty and their barriers were initialised by this warp's lane 0 just above.  W1 is the
+    // context's own copy and is not written by anything that may still be running ahead of this launch.
     if (warp == 0) {
-        // The first loads go out before the CTA-wide barrier below (TMEM allocation, the other warps): the
-        // stages are empty and their barriers were initialised by this warp's lane 0 just above.
         __syncwarp();
         if (elect_one()) {
             for (int kb = 0; kb < n_pre; ++kb) {
                 const uint32_t sa = smem_base + kb * L.stage_bytes;
                 mbar_arrive_expect_tx(bar_full + 8 * kb, L.stage_bytes);
                 tma_load_3d(sa + kATileBytes, &tmap_w, bar_full + 8 * kb, 0, w_row, kb_first + kb, pol_w);
-                tma_load_3d(sa, &tmap_x, bar_full + 8 * kb, (kb_first + kb) * kElems, row0, l_rel, pol_x);
             }
         }
         __syncwarp();
@@ -166,6 +175,16 @@ score_split_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_cons
     if (warp == 1) {
         tmem_alloc(smem_u32(const_cast<uint32_t *>(tmem_slot)), static_cast<uint32_t>(p.tmem_cols));
         tmem_relinquish();
+    }
+    // unless the caller vouches for the producers of its inputs, nothing of them is read before the work
+    // ahead in the stream has completed (every thread waits: the loads below are issued by several warps)
+    if (p.wait_before_load) griddep_wait();
+    if (warp == 0) {
+        __syncwarp();
+        if (elect_one())
+            for (int kb = 0; kb < n_pre; ++kb)
+                tma_load_3d(smem_base + kb * L.stage_bytes, &tmap_x, bar_full + 8 * kb, (kb_first + kb) * kElems, row0, l_rel, pol_x);
+        __syncwarp();
     }
     tc_fence_before_sync();
     __syncthreads();
@@ -266,13 +285,15 @@ score_split_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_cons
             }
             named_barrier_sync(1, 256);
             const bool go = *abort_flag == 0;
-            const int rows_per_cta = kTileM / n_ctas;
+            const int64_t seqs_left = static_cast<int64_t>(c.n_seqs) - static_cast<int64_t>(m_tile) * kTileM;
+            const int tile_seqs = seqs_left < kTileM ? static_cast<int>(seqs_left) : kTileM;
+            const int rows_per_cta = (tile_seqs + n_ctas - 1) / n_ctas;
             // one thread per list: which row leaves, where it goes, which slot the new token takes
             {
                 const int b_loc = pos * rows_per_cta + etid / kMaxHeads, h = etid % kMaxHeads;
                 const int64_t b = static_cast<int64_t>(m_tile) * kTileM + b_loc;
                 int64_t dst = -1, ring = -1;
-                if (go && etid < rows_per_cta * kMaxHeads && b < c.n_seqs && h < c.n_heads && c.active[b] != 0) {
+                if (go && etid < rows_per_cta * kMaxHeads && b_loc < tile_seqs && h < c.n_heads && c.active[b] != 0) {
                     const int64_t li = (b * c.n_layers + layer) * c.n_heads + h;
                     // two round trips to memory instead of four: both counters first, then the score of
                     // the slot's old token and the page the prefix ends in, whether or not it will be needed
@@ -356,35 +377,51 @@ score_split_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_cons
         ok = mbar_wait(bar_tfull, 0, abort_flag);
         tc_fence_after_sync();
     }
-    const int n16 = own_n >> 4;             // 16-column chunks this CTA owns (and as many it sends away)
-    float4 *recv = reinterpret_cast<float4 *>(smem);          // [own_n / 4][128 rows] float4, over the idle stages
-    if (k_split == 2) {
+    const int n16 = own_n >> 4;             // 16-column chunks this CTA owns (and as many it sends to each of the others)
+    // lanes of a warp whose 32 tokens all lie past the input take no part in the exchange and the second layer
+    const bool rows_live = ok && static_cast<int64_t>(row0) + q * 32 < p.n_tokens;
+    float4 *recv = reinterpret_cast<float4 *>(smem);          // [k_split - 1][own_n / 4][128 rows] float4, over the idle stages
+    if (k_split > 1) {
         // every CTA's MMAs are complete once all have passed this barrier: the stages may be overwritten
         tc_fence_before_sync();
         cluster_sync_all();
-        if (epi && ok) {
-            const uint32_t partner = rank ^ 1u;
-            const int send_c0 = (1 - kh) * own_n;               // the columns the partner owns
-            const uint32_t dst0 = map_to_cta(smem_base, partner);
-            for (int c = hsel; c < n16; c += 2) {
+        if (epi && rows_live) {
+            for (int i = hsel; i < (k_split - 1) * n16; i += 2) {
+                const uint32_t c = static_cast<uint32_t>(i % n16);
+                const uint32_t to = (rank + 1u + static_cast<uint32_t>(i / n16)) % static_cast<uint32_t>(k_split);
+                const uint32_t slot = rank < to ? rank : rank - 1u;         // the receiver's parts in rank order, itself left out
+                const uint32_t dst0 = map_to_cta(smem_base, to) + (slot * (static_cast<uint32_t>(own_n) >> 2) + c * 4) * kTileM * 16;
                 uint32_t r[16];
-                tmem_ld_x16(t_row + send_c0 + c * 16, r);
+                tmem_ld_x16(t_row + to * own_n + c * 16, r);
                 tmem_wait_ld();
                 reg_fence16(r);
 #pragma unroll
-                for (int i = 0; i < 4; ++i)
-                    st_shared_cluster_v4(dst0 + (static_cast<uint32_t>(c * 4 + i) * kTileM + row) * 16,
-                                         __uint_as_float(r[4 * i]), __uint_as_float(r[4 * i + 1]),
-                                         __uint_as_float(r[4 * i + 2]), __uint_as_float(r[4 * i + 3]));
+                for (int j = 0; j < 4; ++j)
+                    st_shared_cluster_v4(dst0 + (static_cast<uint32_t>(j) * kTileM + row) * 16,
+                                         __uint_as_float(r[4 * j]), __uint_as_float(r[4 * j + 1]),
+                                         __uint_as_float(r[4 * j + 2]), __uint_as_float(r[4 * j + 3]));
             }
         }
-        cluster_sync_all();                                     // the partner's half has arrived
+        cluster_sync_all();                                     // the others' parts have arrived
     }
+    // adds what the other CTAs of the cluster sent for 16-column chunk c of this CTA's columns
+    auto add_received = [&](uint32_t (&r)[16], int c) {
+        for (int part_i = 0; part_i < k_split - 1; ++part_i) {
+#pragma unroll
+            for (int i = 0; i < 4; ++i) {
+                const float4 o = recv[(part_i * (own_n >> 2) + c * 4 + i) * kTileM + row];
+                r[4 * i] = __float_as_uint(__uint_as_float(r[4 * i]) + o.x);
+                r[4 * i + 1] = __float_as_uint(__uint_as_float(r[4 * i + 1]) + o.y);
+                r[4 * i + 2] = __float_as_uint(__uint_as_float(r[4 * i + 2]) + o.z);
+                r[4 * i + 3] = __float_as_uint(__uint_as_float(r[4 * i + 3]) + o.w);
+            }
+        }
+    };
     if (epi) {
         uint64_t acc[kMaxHeads];
 #pragma unroll
         for (int h = 0; h < kMaxHeads; ++h) acc[h] = 0ull;
-        if (ok) {
+        if (rows_live) {
             // the first warp of a lane quarter takes the 16-column chunks 0, 2, 4, ..., the second the odd ones
             uint32_t ra[16], rb[16];
             uint64_t sx2 = 0ull;                                   // 8-bit inputs: this row's token scale, twice
@@ -400,16 +437,7 @@ score_split_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_cons
                 tmem_wait_ld();
                 reg_fence16(ra);
                 if (c + 2 < n16) tmem_ld_x16(t_row + own_c0 + (c + 2) * 16, rb);
-                if (k_split == 2) {
-#pragma unroll
-                    for (int i = 0; i < 4; ++i) {
-                        const float4 o = recv[(c * 4 + i) * kTileM + row];
-                        ra[4 * i] = __float_as_uint(__uint_as_float(ra[4 * i]) + o.x);
-                        ra[4 * i + 1] = __float_as_uint(__uint_as_float(ra[4 * i + 1]) + o.y);
-                        ra[4 * i + 2] = __float_as_uint(__uint_as_float(ra[4 * i + 2]) + o.z);
-                        ra[4 * i + 3] = __float_as_uint(__uint_as_float(ra[4 * i + 3]) + o.w);
-                    }
-                }
+                add_received(ra, c);
                 if constexpr (kFp8) mlp_columns_scaled<16>(ra, c * 16, b1s, w1s, sx2, w2p, acc);
                 else mlp_columns<16>(ra, c * 16, b1s, w2p, acc);
                 c += 2;
@@ -417,16 +445,7 @@ score_split_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_cons
                     tmem_wait_ld();
                     reg_fence16(rb);
                     if (c + 2 < n16) tmem_ld_x16(t_row + own_c0 + (c + 2) * 16, ra);
-                    if (k_split == 2) {
-#pragma unroll
-                        for (int i = 0; i < 4; ++i) {
-                            const float4 o = recv[(c * 4 + i) * kTileM + row];
-                            rb[4 * i] = __float_as_uint(__uint_as_float(rb[4 * i]) + o.x);
-                            rb[4 * i + 1] = __float_as_uint(__uint_as_float(rb[4 * i + 1]) + o.y);
-                            rb[4 * i + 2] = __float_as_uint(__uint_as_float(rb[4 * i + 2]) + o.z);
-                            rb[4 * i + 3] = __float_as_uint(__uint_as_float(rb[4 * i + 3]) + o.w);
-                        }
-                    }
+                    add_received(rb, c);
                     if constexpr (kFp8) mlp_columns_scaled<16>(rb, c * 16, b1s, w1s, sx2, w2p, acc);
                     else mlp_columns<16>(rb, c * 16, b1s, w2p, acc);
                     c += 2;

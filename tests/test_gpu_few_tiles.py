@@ -1,0 +1,88 @@
+"""GPU parity of the few-token scoring kernel over the layouts it chooses by the number of 128-token tiles: scores at
+the sizes where one layout gives way to the next, and decode steps of one cache that change layout from call to call
+(all layers in one call, then layer by layer), against the CPU oracle."""
+import numpy as np
+import pytest
+import torch
+
+from paper_2601_07891_b200 import binding, synth
+from tests import parity
+
+pytestmark = pytest.mark.gpu
+
+# An fp32 pre-activation is a chain of at most d_model / 16 + 8 additions of partial sums below 6 in magnitude, each off
+# by at most 2^-23 of it; the second layer adds up |w2| of `hidden` of them: 0.8 sqrt(hidden) * 6 * 2^-23 * 72 at
+# d_model = 1024 and hidden = 1024 is 1.3e-3.
+ATOL = 2e-3
+
+
+@pytest.mark.parametrize("hidden", [128, 512, 640, 1024])
+@pytest.mark.parametrize("T", [1, 33, 128, 129, 513, 1153, 2305, 4737])
+def test_scores_of_every_layout(oracle, hidden, T):
+    d_model, H = 1024, 8
+    ctx = binding.Kvzap(d_model, hidden, H, 64, 2, max_tokens=T)
+    X = synth.hidden_states(T, d_model, seed=T + hidden)
+    for layer in range(2):
+        wts = synth.mlp_weights(d_model, hidden, H, 40 + layer, "cpu", 0.3)
+        ctx.set_weights(layer, *[parity.dev(x) for x in wts])      # the call behind this one may not start early
+        scores = torch.full((T, H), 7.0, dtype=torch.float32, device="cuda")
+        ctx.score(layer, parity.dev(X), out=scores)
+        again = torch.full_like(scores, 7.0)
+        ctx.score(layer, parity.dev(X), out=again)
+        torch.cuda.synchronize()
+        assert ctx.poll_status() == 0
+        rows = np.unique(np.concatenate([np.arange(min(T, 160)), np.arange(max(0, T - 160), T)]))
+        _, err = parity.check_scores(oracle, scores, X, wts, rows)
+        assert err <= ATOL
+        assert torch.equal(scores, again)
+    ctx.close()
+
+
+@pytest.mark.parametrize("B,L,trusted", [(5, 20, True), (5, 20, False), (130, 3, True)])
+def test_decode_steps_that_change_layout(oracle, B, L, trusted):
+    d_model, hidden, H, D, w, P, tau, n_steps = 512, 512, 8, 64, 4, 4, 0.1, 12
+    ctx = binding.Kvzap(d_model, hidden, H, D, L, max_tokens=max(B, 128), trusted_producers=trusted)
+    for l in range(L):
+        ctx.set_weights(l, *[parity.dev(x) for x in synth.mlp_weights(d_model, hidden, H, 60 + l, "cpu", 0.3)])
+    n_pool = B * L * H * (n_steps // P + 2)
+    K_pool = torch.zeros(n_pool, P, D, dtype=torch.bfloat16, device="cuda")
+    V_pool = torch.zeros_like(K_pool)
+    cache = binding.kvzap_cache_create(ctx.handle, B, w, P, K_pool, V_pool, n_steps // P + 2)
+    dec = oracle.DecodeOracle(B, L, H, D, w)
+    steps, scores = [], []
+    for step in range(n_steps):
+        X = synth.hidden_states(L * B, d_model, seed=300 + step).view(L, B, d_model)
+        K, V = (t.view(L, B, H, D) for t in synth.keys_values(L * B, H, D, seed=400 + step))
+        steps.append([parity.dev(t) for t in (X, K, V)])
+        scores.append(torch.empty(L, B, H, dtype=torch.float32, device="cuda"))
+    torch.cuda.synchronize()
+    for step, (X, K, V) in enumerate(steps):         # enqueued back to back
+        cuts = [0, L] if step % 3 == 0 else list(range(L + 1)) if step % 3 == 1 else [0, 1, L]
+        for a, b in zip(cuts[:-1], cuts[1:]):
+            binding.kvzap_decode_step(ctx.handle, cache, a, b, X[a:b], K[a:b], V[a:b], tau, scores[step][a:b])
+    torch.cuda.synchronize()
+    assert ctx.poll_status() == 0
+    for (X, K, V), s in zip(steps, scores):
+        s, Kb, Vb = s.cpu().numpy(), synth.bits(K.cpu()), synth.bits(V.cpu())
+        for l in range(L):
+            for b in range(B):
+                dec.append(b, l, s[l, b], Kb[l, b], Vb[l, b], tau)
+    lengths = torch.zeros(B, L, H, dtype=torch.int32, device="cuda")
+    binding.kvzap_cache_lengths(ctx.handle, cache, lengths)
+    ln = lengths.cpu().numpy()
+    out = [torch.zeros(n_steps, D, dtype=torch.bfloat16, device="cuda") for _ in range(2)]
+    n = torch.zeros(1, dtype=torch.int32, device="cuda")
+    for b in range(B):
+        for l in range(L):
+            for h in range(H):
+                assert ln[b, l, h] == dec.length(b, l, h)
+                if b in (0, 3, 4, 127, 128, 129) and l in (0, 1, L - 1):
+                    _, Kd, Vd = dec.logical(b, l, h)
+                    binding.kvzap_cache_export(ctx.handle, cache, b, l, h, *out, n)
+                    torch.cuda.synchronize()
+                    m = int(n.item())
+                    assert m == len(Kd)
+                    np.testing.assert_array_equal(synth.bits(out[0])[:m], Kd)
+                    np.testing.assert_array_equal(synth.bits(out[1])[:m], Vd)
+    binding.kvzap_cache_destroy(cache)
+    ctx.close()
