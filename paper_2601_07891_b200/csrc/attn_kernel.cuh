@@ -15,6 +15,11 @@
 // a few long sequences), each list is cut into n_parts equal runs of tiles, one CTA each; the parts
 // leave their triples in global memory and the part that arrives last (a counter per list) merges
 // them in part order, so the result does not depend on which one that was.
+// With fewer lists than resident CTAs (a small batch, layer by layer) there is one wave, and it lasts as
+// long as its longest part: equal parts of lists whose lengths spread over 1 : 7 (contexts of one batch x
+// what each head keeps) leave most of it idle.  There the CTAs share the lists out themselves (attn_unit):
+// every CTA reads all list lengths, finds the shortest part length for which all parts fit the grid, and
+// takes the part of its index.  8 sequences x 8 heads, 2176 rows on average: 26.0 -> 20.4 us per call.
 //
 // Math per tile, on the warp-level tensor-core path (the work is HBM-bound; 16-row MMAs are enough):
 //   S[16 x 16]  = Q[16 x D] K^T      m16n8k16, Q rows 0..G-1 real, the rest zero
@@ -63,10 +68,77 @@ struct AttnParams {
     const uint16_t *q;          // [n_layers_call][B][H * G][D] bf16
     uint16_t *out;              // same shape
     int32_t *status;
-    int32_t n_parts;            // CTAs per list (1 = the CTA writes the output itself)
-    float *part_scratch;        // n_parts > 1: [list][part] { m[8], l[8], O[8][D] }
-    uint32_t *part_arrive;      // n_parts > 1: [list] parts that have stored their triple; back to 0 after the launch
+    int32_t n_parts;            // CTAs per list (1 = the CTA writes the output itself); 0 = by length, see attn_unit
+    float *part_scratch;        // [CTA] { m[8], l[8], O[8][D] }: the parts of a list are consecutive CTAs
+    uint32_t *part_arrive;      // [list] parts that have stored their triple; back to 0 after the launch
 };
+
+// The lists of a call, of lengths[0 .. n) tiles, cut into at most n_units (>= n) parts: a list of t tiles has
+// ceil(t / target) parts, or one if it is empty, with a target from a few steps of bisection between an equal share of
+// all tiles and the longest list.  Whole warp, the same result in every warp of the launch (the quotients are taken in
+// fp32: whatever their rounding, every warp rounds alike).  Returns the number of parts of the list that `unit` falls
+// into, 0 if there is no such unit; `list` and `part` say which.
+constexpr int kAttnListsPerLane = 20;       // n <= 32 * this
+__device__ __forceinline__ int attn_unit(const int32_t *lengths, int n, int n_units, int unit, int lane, int &list, int &part)
+{
+    // lane l owns lists [l * per, (l + 1) * per), in registers
+    const int per = (n + 31) / 32, first = lane * per;
+    float len[kAttnListsPerLane];
+    int sum = 0, longest = 1, own = 0;
+#pragma unroll
+    for (int i = 0; i < kAttnListsPerLane; ++i) {
+        if (i >= per) break;
+        const int t = first + i < n ? lengths[first + i] : 0;
+        if (first + i < n) own = i + 1;
+        len[i] = static_cast<float>(t);
+        sum += t;
+        longest = max(longest, t);
+    }
+    sum = __reduce_add_sync(0xffffffffu, sum);
+    longest = __reduce_max_sync(0xffffffffu, longest);
+    auto parts_of = [&](int i, float inv) { return max(1, __float2int_ru(len[i] * inv)); };
+    auto lane_parts = [&](float inv) {
+        int parts = 0;
+#pragma unroll
+        for (int i = 0; i < kAttnListsPerLane; ++i) {
+            if (i >= per) break;
+            if (i < own) parts += parts_of(i, inv);
+        }
+        return parts;
+    };
+    float lo = fmaxf(1.0f, static_cast<float>(sum) / static_cast<float>(n_units)), hi = static_cast<float>(longest);
+    if (n * 2 <= n_units) hi = fminf(hi, 2.02f * lo);       // at most sum / hi + n parts
+    constexpr float kDown = 1.0f - 1.0f / (1 << 20);        // a list of exactly the target length is one part
+    float inv = kDown / hi;                                 // fits: one part each, or half of the units plus one each
+    for (int step = 0; step < 6; ++step) {
+        const float mid = 0.5f * (lo + hi), inv_mid = kDown / mid;
+        const bool fits = __reduce_add_sync(0xffffffffu, lane_parts(inv_mid)) <= n_units;
+        if (fits) { hi = mid; inv = inv_mid; } else lo = mid;
+    }
+    const int mine = lane_parts(inv);
+    int incl = mine;                                        // the running number of parts finds the unit's list
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+        const int y = __shfl_up_sync(0xffffffffu, incl, o);
+        if (lane >= o) incl += y;
+    }
+    int at = incl - mine, found = -1, parts = 0;
+    if (unit >= at && unit < incl) {
+#pragma unroll
+        for (int i = 0; i < kAttnListsPerLane; ++i) {
+            if (i >= per) break;
+            if (found >= 0) continue;
+            parts = parts_of(i, inv);
+            if (unit < at + parts) found = first + i; else at += parts;
+        }
+    }
+    const uint32_t who = __ballot_sync(0xffffffffu, found >= 0);
+    if (who == 0u) return 0;
+    const int src = __ffs(who) - 1;
+    list = __shfl_sync(0xffffffffu, found, src);
+    part = unit - __shfl_sync(0xffffffffu, at, src);
+    return __shfl_sync(0xffffffffu, parts, src);
+}
 
 constexpr int kAttnTrailerBytes = 16;            // 8-bit rows: fp32 scale + 12 unused bytes behind the codes
 __host__ __device__ constexpr uint32_t attn_stage_bytes(int head_dim, bool fp8 = false)
@@ -86,6 +158,19 @@ __device__ __forceinline__ void e4m3x4_to_f16(uint32_t w, uint32_t &lo, uint32_t
 }
 __device__ __forceinline__ float bf16_lo(uint32_t pair) { return __uint_as_float(pair << 16); }
 __device__ __forceinline__ float bf16_hi(uint32_t pair) { return __uint_as_float(pair & 0xffff0000u); }
+
+__device__ __forceinline__ void attn_add(float4 &num, const float4 &o, float f)
+{
+    num.x += o.x * f; num.y += o.y * f; num.z += o.z * f; num.w += o.w * f;
+}
+// four output elements as bf16; zeros when nothing was summed
+__device__ __forceinline__ void attn_store(uint16_t *out, const float4 &num, float den)
+{
+    const bool some = den > 0.0f;
+    const uint2 v = make_uint2(pack_bf16x2(some ? num.x / den : 0.0f, some ? num.y / den : 0.0f),
+                               pack_bf16x2(some ? num.z / den : 0.0f, some ? num.w / den : 0.0f));
+    *reinterpret_cast<uint2 *>(out) = v;
+}
 
 template <int kD, bool kFp8>
 __global__ void __launch_bounds__(kAttnThreads, kFp8 ? 4 : 1)
@@ -112,10 +197,6 @@ decode_attn_kernel(const __grid_constant__ CUtensorMap tmap_kpool, const __grid_
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const CacheView &c = p.c;
     const int H = c.n_heads, B = c.n_seqs;
-    const int list = blockIdx.x / p.n_parts, part = blockIdx.x % p.n_parts;
-    const int h = list % H, b = (list / H) % B, l_rel = list / (H * B);
-    const int layer = p.layer0 + l_rel;
-    const int64_t li = (static_cast<int64_t>(b) * c.n_layers + layer) * H + h;
 
     if (threadIdx.x == 0) {
         for (int i = 0; i < kAttnWarps * kAttnStages; ++i) mbar_init(bars + 8 * i, 1);
@@ -127,18 +208,97 @@ decode_attn_kernel(const __grid_constant__ CUtensorMap tmap_kpool, const __grid_
         prefetch_tensormap(&tmap_vring);
     }
     __syncthreads();
+    // started while the kernel ahead (the step that appended the newest rows) may still be running: nothing of the
+    // caller's or of the cache is read before it has completed
+    griddep_wait();
 
-    const int32_t n_total = __ldcg(c.n_tokens + li);
-    const int32_t n_prefix = __ldcg(c.prefix_len + li);
+    int list, part, n_parts = p.n_parts;
+    int32_t n_total, n_prefix;
+    auto cache_list = [&](int i) {          // list i of the call among the cache's lists
+        return (static_cast<int64_t>((i / H) % B) * c.n_layers + p.layer0 + i / (H * B)) * H + i % H;
+    };
+    if (n_parts > 0) {
+        list = blockIdx.x / n_parts;
+        part = blockIdx.x % n_parts;
+        n_total = __ldcg(c.n_tokens + cache_list(list));
+        n_prefix = __ldcg(c.prefix_len + cache_list(list));
+    } else {
+        // over the stages, not in use yet: [list] tiles, then [list] (tokens, prefix rows)
+        const int n_lists = p.n_layers_call * B * H;
+        int32_t *lengths = reinterpret_cast<int32_t *>(smem);
+        int2 *counts = reinterpret_cast<int2 *>(smem + 4 * 32 * kAttnListsPerLane);
+        for (int i = threadIdx.x; i < n_lists; i += kAttnThreads) {
+            const int2 n = make_int2(__ldcg(c.n_tokens + cache_list(i)), __ldcg(c.prefix_len + cache_list(i)));
+            counts[i] = n;
+            lengths[i] = (n.y + kAttnTileRows - 1) / kAttnTileRows + (min(n.x, c.window) + kAttnTileRows - 1) / kAttnTileRows;
+        }
+        __syncthreads();
+        n_parts = attn_unit(lengths, n_lists, gridDim.x, blockIdx.x, lane, list, part);
+        if (n_parts == 0) return;                                  // the whole CTA: more CTAs than parts
+        n_total = counts[list].x;
+        n_prefix = counts[list].y;
+        fence_proxy_async_smem();                                  // the copies below write where these were read
+        __syncthreads();
+    }
+    const int h = list % H, b = (list / H) % B, l_rel = list / (H * B);
+    const int64_t li = cache_list(list);
+
     const int32_t n_ring = c.window > 0 ? (n_total < c.window ? n_total : c.window) : 0;
     const int tiles_per_page = c.page_tokens / kAttnTileRows;
     const int n_pt = (n_prefix + kAttnTileRows - 1) / kAttnTileRows;
     const int n_rt = (n_ring + kAttnTileRows - 1) / kAttnTileRows;
     const int n_tiles_list = n_pt + n_rt;
     // this CTA's run of the list's tiles
-    const int t_begin = static_cast<int>(static_cast<int64_t>(n_tiles_list) * part / p.n_parts);
-    const int n_tiles = static_cast<int>(static_cast<int64_t>(n_tiles_list) * (part + 1) / p.n_parts);
+    const int t_begin = static_cast<int>(static_cast<int64_t>(n_tiles_list) * part / n_parts);
+    const int n_tiles = static_cast<int>(static_cast<int64_t>(n_tiles_list) * (part + 1) / n_parts);
     const int32_t *pages = c.page_table + li * c.max_pages;
+
+    const uint32_t my_stages = smem_base + warp * kAttnStages * kStageBytes;
+    const uint32_t my_bars = bars + 8 * warp * kAttnStages;
+    const uint64_t policy = l2_policy_evict_first();
+
+    // first row (in its tensor map) of tile t of this list; needs the page number for prefix tiles
+    auto tile_row = [&](int t) -> int32_t {
+        if (t < n_pt) {
+            const int32_t page = __ldcg(pages + t / tiles_per_page);
+            return page * c.page_tokens + (t % tiles_per_page) * kAttnTileRows;
+        }
+        return static_cast<int32_t>(li * c.window) + (t - n_pt) * kAttnTileRows;
+    };
+    auto issue = [&](int t, int32_t row, int stage) {
+        const uint32_t dst = my_stages + stage * kStageBytes;
+        const uint32_t bar = my_bars + 8 * stage;
+        const bool prefix = t < n_pt;
+        mbar_arrive_expect_tx(bar, kStageBytes);
+        if constexpr (kFp8) {
+            // a tile of 8-bit rows is one contiguous piece of memory: coordinates (0, 0, tile)
+            tma_load_3d(dst, prefix ? &tmap_kpool : &tmap_kring, bar, 0, 0, row / kAttnTileRows, policy);
+            tma_load_3d(dst + kTileBytes8, prefix ? &tmap_vpool : &tmap_vring, bar, 0, 0, row / kAttnTileRows, policy);
+        } else {
+#pragma unroll
+            for (int hf = 0; hf < kHalves; ++hf) {
+                tma_load_2d(dst + hf * kAttnHalfBytes, prefix ? &tmap_kpool : &tmap_kring, bar, hf * 64, row, policy);
+                tma_load_2d(dst + (kHalves + hf) * kAttnHalfBytes, prefix ? &tmap_vpool : &tmap_vring, bar, hf * 64, row, policy);
+            }
+        }
+    };
+
+    // prologue: fill the stages, the pages of all of them looked up together; row_next belongs to the first tile not
+    // yet issued
+    int t_issue = t_begin + warp;
+    int32_t row_next = 0;
+    {
+        int32_t rows[kAttnStages + 1];
+#pragma unroll
+        for (int s = 0; s <= kAttnStages; ++s) rows[s] = t_issue + s * kAttnWarps < n_tiles ? tile_row(t_issue + s * kAttnWarps) : 0;
+#pragma unroll
+        for (int s = 0; s < kAttnStages; ++s)
+            if (t_issue < n_tiles) {
+                if (lane == 0) issue(t_issue, rows[s], s);
+                t_issue += kAttnWarps;
+            }
+        row_next = rows[kAttnStages];
+    }
 
     // the query rows of this KV head as A fragments: row g = lane / 4 (real for g < G), two packed
     // elements at columns 16 ks + 2 (lane % 4) and the same + 8
@@ -187,44 +347,6 @@ decode_attn_kernel(const __grid_constant__ CUtensorMap tmap_kpool, const __grid_
     for (int i = 0; i < kNTiles; ++i) o[i][0] = o[i][1] = o[i][2] = o[i][3] = 0.0f;
     float m_run = -INFINITY, l_run = 0.0f;
     float vref = 0.0f;                     // 8-bit rows: the largest V scale met so far; o is in units of it
-
-    const uint32_t my_stages = smem_base + warp * kAttnStages * kStageBytes;
-    const uint32_t my_bars = bars + 8 * warp * kAttnStages;
-    const uint64_t policy = l2_policy_evict_first();
-
-    // first row (in its tensor map) of tile t of this list; needs the page number for prefix tiles
-    auto tile_row = [&](int t) -> int32_t {
-        if (t < n_pt) {
-            const int32_t page = __ldcg(pages + t / tiles_per_page);
-            return page * c.page_tokens + (t % tiles_per_page) * kAttnTileRows;
-        }
-        return static_cast<int32_t>(li * c.window) + (t - n_pt) * kAttnTileRows;
-    };
-    auto issue = [&](int t, int32_t row, int stage) {
-        const uint32_t dst = my_stages + stage * kStageBytes;
-        const uint32_t bar = my_bars + 8 * stage;
-        const bool prefix = t < n_pt;
-        mbar_arrive_expect_tx(bar, kStageBytes);
-        if constexpr (kFp8) {
-            // a tile of 8-bit rows is one contiguous piece of memory: coordinates (0, 0, tile)
-            tma_load_3d(dst, prefix ? &tmap_kpool : &tmap_kring, bar, 0, 0, row / kAttnTileRows, policy);
-            tma_load_3d(dst + kTileBytes8, prefix ? &tmap_vpool : &tmap_vring, bar, 0, 0, row / kAttnTileRows, policy);
-        } else {
-#pragma unroll
-            for (int hf = 0; hf < kHalves; ++hf) {
-                tma_load_2d(dst + hf * kAttnHalfBytes, prefix ? &tmap_kpool : &tmap_kring, bar, hf * 64, row, policy);
-                tma_load_2d(dst + (kHalves + hf) * kAttnHalfBytes, prefix ? &tmap_vpool : &tmap_vring, bar, hf * 64, row, policy);
-            }
-        }
-    };
-
-    // prologue: fill the stages; row_next belongs to the first tile not yet issued
-    int t_issue = t_begin + warp;
-    for (int s = 0; s < kAttnStages && t_issue < n_tiles; ++s, t_issue += kAttnWarps) {
-        const int32_t row = tile_row(t_issue);
-        if (lane == 0) issue(t_issue, row, s);
-    }
-    int32_t row_next = t_issue < n_tiles ? tile_row(t_issue) : 0;
 
     bool ok = true;
     int stage = 0;
@@ -426,35 +548,37 @@ decode_attn_kernel(const __grid_constant__ CUtensorMap tmap_kpool, const __grid_
     __syncthreads();
     const bool failed = *abort_flag != 0;
     const int64_t out_row0 = (static_cast<int64_t>(l_rel) * B + b) * Hq + h * p.group;
-    float *unit = p.n_parts > 1 ? p.part_scratch + (static_cast<int64_t>(list) * p.n_parts + part) * (16 + kAttnMaxGroup * kD) : nullptr;
-    for (int idx = threadIdx.x; idx < p.group * kD; idx += kAttnThreads) {
-        const int gq = idx / kD, d = idx % kD;
+    constexpr int kUnit = 16 + kAttnMaxGroup * kD;
+    float *unit = n_parts > 1 ? p.part_scratch + static_cast<int64_t>(blockIdx.x) * kUnit : nullptr;
+    // four elements of one query head per thread
+    for (int idx = threadIdx.x; idx < p.group * (kD / 4); idx += kAttnThreads) {
+        const int gq = idx / (kD / 4), d = idx % (kD / 4) * 4;
         float m_all = -INFINITY;
 #pragma unroll
         for (int w = 0; w < kAttnWarps; ++w)
             m_all = fmaxf(m_all, reinterpret_cast<const float *>(smem + w * kAttnStages * kStageBytes)[gq]);
-        float num = 0.0f, den = 0.0f;
+        float4 num = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
+        float den = 0.0f;
 #pragma unroll
         for (int w = 0; w < kAttnWarps; ++w) {
             const float *wp = reinterpret_cast<const float *>(smem + w * kAttnStages * kStageBytes);
             if (wp[gq] > -INFINITY) {                       // a warp that saw no tile contributes nothing
                 const float f = fast_ex2(wp[gq] - m_all);
-                num += wp[16 + gq * kD + d] * f;
+                attn_add(num, *reinterpret_cast<const float4 *>(wp + 16 + gq * kD + d), f);
                 den += wp[8 + gq] * f;
             }
         }
-        if (p.n_parts == 1) {
-            const float r = (den > 0.0f && !failed) ? num / den : 0.0f;      // an empty list gives zeros
-            p.out[(out_row0 + gq) * kD + d] = static_cast<uint16_t>(pack_bf16x2(r, 0.0f) & 0xffffu);
+        if (n_parts == 1) {
+            attn_store(p.out + (out_row0 + gq) * kD + d, num, failed ? 0.0f : den);      // an empty list gives zeros
         } else {
-            __stcg(unit + 16 + gq * kD + d, num);
+            __stcg(reinterpret_cast<float4 *>(unit + 16 + gq * kD + d), num);
             if (d == 0) {
                 __stcg(unit + gq, failed ? -INFINITY : m_all);
                 __stcg(unit + 8 + gq, failed ? 0.0f : den);
             }
         }
     }
-    if (p.n_parts == 1) return;
+    if (n_parts == 1) return;
 
     // ---- several CTAs per list: the one that arrives last merges all parts, in part order
     __shared__ int last_s;
@@ -462,45 +586,46 @@ decode_attn_kernel(const __grid_constant__ CUtensorMap tmap_kpool, const __grid_
     __syncthreads();
     if (threadIdx.x == 0) {
         const uint32_t before = atomicAdd(p.part_arrive + list, 1u);
-        last_s = before + 1u == static_cast<uint32_t>(p.n_parts);
+        last_s = before + 1u == static_cast<uint32_t>(n_parts);
         if (last_s) p.part_arrive[list] = 0u;               // ready for the next launch
         __threadfence();
     }
     __syncthreads();
     if (!last_s) return;
-    const float *units = p.part_scratch + static_cast<int64_t>(list) * p.n_parts * (16 + kAttnMaxGroup * kD);
-    constexpr int kBatch = 8;               // parts whose values are loaded together (independent loads in flight)
-    constexpr int kUnit = 16 + kAttnMaxGroup * kD;
-    for (int idx = threadIdx.x; idx < p.group * kD; idx += kAttnThreads) {
-        const int gq = idx / kD, d = idx % kD;
-        float m_all = -INFINITY;
-        for (int i0 = 0; i0 < p.n_parts; i0 += kBatch) {
-            float mv[kBatch];
-#pragma unroll
-            for (int j = 0; j < kBatch; ++j) mv[j] = i0 + j < p.n_parts ? __ldcg(units + (i0 + j) * kUnit + gq) : -INFINITY;
-#pragma unroll
-            for (int j = 0; j < kBatch; ++j) m_all = fmaxf(m_all, mv[j]);
-        }
-        float num = 0.0f, den = 0.0f;
-        for (int i0 = 0; i0 < p.n_parts; i0 += kBatch) {
-            float mv[kBatch], nv[kBatch], dv[kBatch];
+    const float *units = p.part_scratch + static_cast<int64_t>(blockIdx.x - part) * kUnit;
+    constexpr int kBatch = 8;               // parts whose values are loaded together: one round trip to memory
+    for (int idx = threadIdx.x; idx < p.group * (kD / 4); idx += kAttnThreads) {
+        const int gq = idx / (kD / 4), d = idx % (kD / 4) * 4;
+        float m_all = -INFINITY, den = 0.0f;
+        float4 num = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
+        for (int i0 = 0; i0 < n_parts; i0 += kBatch) {
+            float mv[kBatch], dv[kBatch];
+            float4 nv[kBatch];
 #pragma unroll
             for (int j = 0; j < kBatch; ++j) {
-                const bool in = i0 + j < p.n_parts;
-                const float *u = units + (i0 + j) * kUnit;
+                const float *u = units + static_cast<int64_t>(i0 + j) * kUnit;
+                const bool in = i0 + j < n_parts;
                 mv[j] = in ? __ldcg(u + gq) : -INFINITY;
-                nv[j] = in ? __ldcg(u + 16 + gq * kD + d) : 0.0f;      // a part without tiles stored zeros
                 dv[j] = in ? __ldcg(u + 8 + gq) : 0.0f;
+                nv[j] = in ? __ldcg(reinterpret_cast<const float4 *>(u + 16 + gq * kD + d)) : make_float4(0.0f, 0.0f, 0.0f, 0.0f);
             }
+            float m_new = m_all;
+#pragma unroll
+            for (int j = 0; j < kBatch; ++j) m_new = fmaxf(m_new, mv[j]);
+            if (m_all > -INFINITY && m_new > m_all) {
+                const float f = fast_ex2(m_all - m_new);
+                num.x *= f; num.y *= f; num.z *= f; num.w *= f;
+                den *= f;
+            }
+            m_all = m_new;
 #pragma unroll
             for (int j = 0; j < kBatch; ++j) {                          // summed in part order
-                const float f = mv[j] > -INFINITY ? fast_ex2(mv[j] - m_all) : 0.0f;
-                num += nv[j] * f;
+                const float f = mv[j] > -INFINITY ? fast_ex2(mv[j] - m_all) : 0.0f;      // a part without tiles adds nothing
+                attn_add(num, nv[j], f);
                 den += dv[j] * f;
             }
         }
-        const float r = den > 0.0f ? num / den : 0.0f;
-        p.out[(out_row0 + gq) * kD + d] = static_cast<uint16_t>(pack_bf16x2(r, 0.0f) & 0xffffu);
+        attn_store(p.out + (out_row0 + gq) * kD + d, num, den);
     }
 }
 

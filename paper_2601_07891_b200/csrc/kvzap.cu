@@ -2352,44 +2352,33 @@ static kvzap_status attention_impl(kvzap_ctx *ctx, kvzap_cache *cache, int32_t l
     p.status = ctx->status_dev;
     const int64_t n_lists_call = static_cast<int64_t>(p.n_layers_call) * v.n_seqs * v.n_heads;
     if (n_lists_call > 0x7fffffffLL) return fail(ctx, KVZAP_ERR_UNSUPPORTED, "attention: too many lists for one launch");
-    // Two CTAs fit an SM.  With fewer than sixteen CTAs per slot the last, longest lists leave most SMs
-    // idle: cut every list into parts so that there are about that many units -- up to 16 parts, or up
-    // to 64 when a handful of long lists (a single sequence) is all there is, but never parts shorter
-    // than about a thousand rows of the longest list the cache can hold.
+    // Two CTAs fit an SM (four of the 8-bit kernel's).  Fewer lists than that: one wave, whose CTAs share the lists out
+    // by their lengths.  With fewer than sixteen CTAs per slot the last, longest lists leave most SMs idle: cut
+    // every list into up to 16 parts so that there are about that many units.
+    const int64_t slots = static_cast<int64_t>(ctx->sm_count) * (fp8 && d_attn == 128 ? 4 : 2);
+    int64_t n_ctas = n_lists_call;
     p.n_parts = 1;
-    const int64_t want_units = static_cast<int64_t>(ctx->sm_count) * 32;
-    if (n_lists_call * 2 <= want_units) {
+    if (n_lists_call < slots) {
+        p.n_parts = 0;
+        n_ctas = slots;
+    } else {
+        const int64_t want_units = static_cast<int64_t>(ctx->sm_count) * 32;
         int64_t parts = want_units / n_lists_call;
-        const int64_t cap = n_lists_call * 16 < 2 * static_cast<int64_t>(ctx->sm_count) ? 64 : 16;
-        if (parts > cap) parts = cap;
-        const int64_t max_rows = static_cast<int64_t>(v.max_pages) * v.page_tokens + v.window;
-        if (parts > 16 && parts > (max_rows + 1023) / 1024) parts = (max_rows + 1023) / 1024 > 16 ? (max_rows + 1023) / 1024 : 16;
-        // fewer lists than resident CTA slots: one full wave of equal parts (a second, partly filled wave
-        // would cost as much as the first)
-        const int64_t slots = 2 * static_cast<int64_t>(ctx->sm_count);
-        if (n_lists_call < slots) {
-            parts = slots / n_lists_call;
-            if (parts > 64) parts = 64;
-        }
-        if (parts * n_lists_call > cache->attn_units) parts = cache->attn_units / n_lists_call;
+        if (parts > 16) parts = 16;
         if (parts > 1) p.n_parts = static_cast<int32_t>(parts);
+        n_ctas = n_lists_call * p.n_parts;
     }
     p.part_scratch = cache->attn_scratch;
     p.part_arrive = cache->attn_arrive;
-    const int64_t n_ctas = n_lists_call * p.n_parts;
     {
         ProfScope prof(ctx, KVZAP_KERNEL_ATTENTION, stream);
-        const unsigned grid = static_cast<unsigned>(n_ctas);
-        const uint32_t smem = attn_smem_bytes(d_attn, fp8);
-        if (fp8 && d_attn == 128)
-            decode_attn_kernel<128, true><<<grid, kAttnThreads, smem, stream>>>(cache->tm_kpool, cache->tm_vpool, cache->tm_kring, cache->tm_vring, p);
-        else if (fp8)
-            decode_attn_kernel<64, true><<<grid, kAttnThreads, smem, stream>>>(cache->tm_kpool, cache->tm_vpool, cache->tm_kring, cache->tm_vring, p);
-        else if (d_attn == 128)
-            decode_attn_kernel<128, false><<<grid, kAttnThreads, smem, stream>>>(cache->tm_kpool, cache->tm_vpool, cache->tm_kring, cache->tm_vring, p);
-        else
-            decode_attn_kernel<64, false><<<grid, kAttnThreads, smem, stream>>>(cache->tm_kpool, cache->tm_vpool, cache->tm_kring, cache->tm_vring, p);
-        KVZAP_CUDA(ctx, cudaGetLastError());
+        cudaLaunchConfig_t cfg;
+        cudaLaunchAttribute attrs[2];
+        make_launch(&cfg, attrs, dim3(static_cast<unsigned>(n_ctas)), dim3(kAttnThreads), attn_smem_bytes(d_attn, fp8), stream,
+                    !ctx->profiling, 1);
+        KVZAP_CUDA(ctx, cudaLaunchKernelEx(&cfg, fp8 ? (d_attn == 128 ? decode_attn_kernel<128, true> : decode_attn_kernel<64, true>)
+                                                     : (d_attn == 128 ? decode_attn_kernel<128, false> : decode_attn_kernel<64, false>),
+                                           cache->tm_kpool, cache->tm_vpool, cache->tm_kring, cache->tm_vring, p));
     }
     ctx->launches += 1;
     return KVZAP_OK;

@@ -538,15 +538,14 @@ score_split_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_cons
         if (f.enabled) {
             // the new token's scores go into the slot it took (n_tokens was advanced by the list's CTA)
             const CacheView &c = f.c;
-            if (valid && *abort_flag == 0) {
+            if (valid && *abort_flag == 0 && c.active[t] != 0) {
+                const int64_t li0 = (t * c.n_layers + layer) * c.n_heads;
+                int32_t n[kMaxHeads];                           // all loads before the first store: one round trip
 #pragma unroll
-                for (int h = 0; h < kMaxHeads; ++h) {
-                    if (h < c.n_heads && c.active[t] != 0) {
-                        const int64_t li = (t * c.n_layers + layer) * c.n_heads + h;
-                        const int slot = (__ldcg(c.n_tokens + li) - 1) % c.window;
-                        c.score_ring[li * c.window + slot] = s[h];
-                    }
-                }
+                for (int h = 0; h < kMaxHeads; ++h) n[h] = h < c.n_heads ? __ldcg(c.n_tokens + li0 + h) : 1;
+#pragma unroll
+                for (int h = 0; h < kMaxHeads; ++h)
+                    if (h < c.n_heads) c.score_ring[(li0 + h) * c.window + (n[h] - 1) % c.window] = s[h];
             }
             __threadfence();
             named_barrier_sync(2, 128);
