@@ -926,38 +926,66 @@ static kvzap_status launch_score_fp8(kvzap_ctx *ctx, int32_t layer, const void *
     return KVZAP_OK;
 }
 
+// The launch of the compaction kernel over n_blocks blocks of every head.
+struct CompactShape {
+    int blocks_per_cta, threads;
+    dim3 grid;
+    bool alone;
+};
+static CompactShape compact_shape(const kvzap_ctx *ctx, int64_t n_blocks, bool paged, bool append)
+{
+    const kvzap_config &c = ctx->cfg;
+    const int64_t H = c.n_kv_heads;
+    CompactShape s;
+    s.alone = !ctx->trusted || append;
+    // Beside the next layer's scoring: resident all at once next to its CTAs (the MLP scoring kernel leaves registers
+    // for two CTAs of 128 threads per SM, the Linear one for several).  Alone, CTAs of 256 threads and many of them, four
+    // to an SM at a time: the serial part of a CTA (words, ranks) then runs under the row moves of the others, and a
+    // short input spreads the rows of a block over several CTAs.  32k tokens x 8 heads, 65 MB, from the end of the scoring
+    // launch to the end of this one: 40 us with the shape that fits beside a scoring kernel, 26.4 / 25.1 / 23.6 us with
+    // 4 / 8 / 16 CTAs per SM; 777 tokens 8 -> 4 us.
+    int64_t max_ctas = static_cast<int64_t>(ctx->sm_count) * (s.alone ? 16 : c.hidden > 0 ? 2 : 6);
+    int64_t chunks = max_ctas / H;
+    if (chunks < 1) chunks = 1;
+    if (chunks > n_blocks) chunks = n_blocks;
+    s.blocks_per_cta = static_cast<int>((n_blocks + chunks - 1) / chunks);
+    chunks = (n_blocks + s.blocks_per_cta - 1) / s.blocks_per_cta;
+    // a short input (one block per CTA, a grid that is resident at once anyway): CTAs of 256 threads
+    const bool short_input = s.blocks_per_cta == 1 && chunks * H <= 4 * static_cast<int64_t>(ctx->sm_count);
+    s.threads = s.alone || (short_input && !paged) ? kDenseThreadsShort : kDenseThreads;
+    unsigned nz = 1;
+    if (s.alone)
+        while (nz < 4 && 2 * nz * chunks * H <= 4 * static_cast<int64_t>(ctx->sm_count) && s.blocks_per_cta == 1) nz *= 2;
+    s.grid = dim3(static_cast<unsigned>(chunks), static_cast<unsigned>(H), nz);
+    return s;
+}
+
+template <typename... Args>
+static cudaError_t launch_compact_kernel(const CompactShape &s, cudaStream_t stream, bool early, Args... args)
+{
+    cudaLaunchConfig_t cfg;
+    cudaLaunchAttribute attrs[2];
+    make_launch(&cfg, attrs, s.grid, dim3(static_cast<unsigned>(s.threads)), 0, stream, early, 1);
+    if (s.alone) return cudaLaunchKernelEx(&cfg, compact_dense_kernel<kDenseThreadsShort, true>, args...);
+    if (s.threads == kDenseThreadsShort) return cudaLaunchKernelEx(&cfg, compact_dense_kernel<kDenseThreadsShort, false>, args...);
+    return cudaLaunchKernelEx(&cfg, compact_dense_kernel<kDenseThreads, false>, args...);
+}
+
 // Dense-ragged compaction over the mask words in `mask` (one kernel, no scan pass).
 static kvzap_status launch_compaction(kvzap_ctx *ctx, const uint32_t *mask, const void *K, const void *V,
                                       const int32_t *cu_seqlens, int32_t n_seqs, int64_t n_tokens, void *K_out,
-                                      void *V_out, int32_t *lengths, cudaStream_t stream, bool beside_scoring = true,
-                                      bool tok_major = false)
+                                      void *V_out, int32_t *lengths, cudaStream_t stream, bool tok_major = false)
 {
     const kvzap_config &c = ctx->cfg;
     const int64_t n_blocks = (n_tokens + kBlockTokens - 1) / kBlockTokens;
     const int64_t n_words = n_blocks * 4;
-    // A grid that is resident all at once, next to the scoring kernel's CTAs: the MLP scoring kernel
-    // leaves registers for two of these CTAs per SM, the Linear one for several.
-    // On its own (kvzap_prune_prefill) the kernel fills every SM instead: eight CTAs each.
-    const int per_sm = !beside_scoring ? 8 : (c.hidden > 0 ? 2 : 6);
-    const int64_t max_ctas = static_cast<int64_t>(ctx->sm_count) * per_sm;
-    int64_t chunks = max_ctas / c.n_kv_heads;
-    if (chunks < 1) chunks = 1;
-    if (chunks > n_blocks) chunks = n_blocks;
-    const int blocks_per_cta = static_cast<int>((n_blocks + chunks - 1) / chunks);
-    chunks = (n_blocks + blocks_per_cta - 1) / blocks_per_cta;
+    const CompactShape shape = compact_shape(ctx, n_blocks, false, false);
     {
         ProfScope prof(ctx, KVZAP_KERNEL_COMPACT, stream);
-        cudaLaunchConfig_t cfg;
-        cudaLaunchAttribute attrs[2];
-        // a short input (one block per CTA, a grid that is resident at once anyway): CTAs of 256 threads
-        const bool short_input = blocks_per_cta == 1 && chunks * c.n_kv_heads <= 4 * static_cast<int64_t>(ctx->sm_count);
-        make_launch(&cfg, attrs, dim3(static_cast<unsigned>(chunks), static_cast<unsigned>(c.n_kv_heads)),
-                    dim3(short_input ? kDenseThreadsShort : kDenseThreads), 0, stream, !ctx->profiling, 1);
-        KVZAP_CUDA(ctx, cudaLaunchKernelEx(&cfg, short_input ? compact_dense_kernel<kDenseThreadsShort> : compact_dense_kernel<kDenseThreads>,
-                                           static_cast<const uint4 *>(K),
+        KVZAP_CUDA(ctx, launch_compact_kernel(shape, stream, !ctx->profiling, static_cast<const uint4 *>(K),
                                            static_cast<const uint4 *>(V), static_cast<uint4 *>(K_out),
-                                           static_cast<uint4 *>(V_out), mask, n_words, n_blocks, blocks_per_cta,
-                                           cu_seqlens, n_seqs, n_tokens, c.n_kv_heads, c.head_dim / 8, lengths, 0,
+                                           static_cast<uint4 *>(V_out), mask, n_words, n_blocks, shape.blocks_per_cta,
+                                           cu_seqlens, static_cast<int>(n_seqs), n_tokens, static_cast<int>(c.n_kv_heads), static_cast<int>(c.head_dim / 8), lengths, 0,
                                            static_cast<const int32_t *>(nullptr),
                                            tok_major ? int64_t{1} : n_tokens,
                                            tok_major ? static_cast<int64_t>(c.n_kv_heads) : int64_t{1},
@@ -1221,9 +1249,9 @@ kvzap_status kvzap_create(kvzap_ctx **out, const kvzap_config *cfg)
 
     // Kernels share an SM only if they ask for the same split of the L1 / shared-memory array; the
     // scoring kernels need the largest shared-memory split, so the compaction asks for it too.
-    CREATE_CUDA(cudaFuncSetAttribute(compact_dense_kernel<kDenseThreads>, cudaFuncAttributePreferredSharedMemoryCarveout,
+    CREATE_CUDA(cudaFuncSetAttribute(compact_dense_kernel<kDenseThreads, false>, cudaFuncAttributePreferredSharedMemoryCarveout,
                                      static_cast<int>(cudaSharedmemCarveoutMaxShared)));
-    CREATE_CUDA(cudaFuncSetAttribute(compact_dense_kernel<kDenseThreadsShort>, cudaFuncAttributePreferredSharedMemoryCarveout,
+    CREATE_CUDA(cudaFuncSetAttribute(compact_dense_kernel<kDenseThreadsShort, false>, cudaFuncAttributePreferredSharedMemoryCarveout,
                                      static_cast<int>(cudaSharedmemCarveoutMaxShared)));
     CREATE_CUDA(cudaFuncSetAttribute(decode_update_kernel, cudaFuncAttributePreferredSharedMemoryCarveout,
                                      static_cast<int>(cudaSharedmemCarveoutMaxShared)));
@@ -1533,7 +1561,7 @@ kvzap_status kvzap_prefill_fused_fp8(kvzap_ctx *ctx, int32_t layer, const void *
     uint32_t *mask = next_mask_slice(ctx);
     st = launch_score_fp8(ctx, layer, hidden_e4m3, x_scale, n_tokens, scores_out, mask, cu_seqlens, n_seqs, tau, w, stream);
     if (st != KVZAP_OK) return st;
-    return launch_compaction(ctx, mask, K, V, cu_seqlens, n_seqs, n_tokens, K_out, V_out, lengths, stream, true, false);
+    return launch_compaction(ctx, mask, K, V, cu_seqlens, n_seqs, n_tokens, K_out, V_out, lengths, stream);
 }
 
 kvzap_status kvzap_score(kvzap_ctx *ctx, int32_t layer, const void *hidden, int64_t n_tokens, float *scores,
@@ -1655,7 +1683,7 @@ static kvzap_status prefill_fused_impl(kvzap_ctx *ctx, int32_t layer, const void
     st = launch_score(ctx, layer, 1, hidden, n_tokens, scores_out, mask, cu_seqlens, n_seqs, tau, w, stream, 1, nullptr, nullptr,
                       nullptr, &compact, &compacted);
     if (st != KVZAP_OK || compacted) return st;
-    return launch_compaction(ctx, mask, K, V, cu_seqlens, n_seqs, n_tokens, K_out, V_out, lengths, stream, true, tok_major);
+    return launch_compaction(ctx, mask, K, V, cu_seqlens, n_seqs, n_tokens, K_out, V_out, lengths, stream, tok_major);
 }
 
 kvzap_status kvzap_prefill_fused(kvzap_ctx *ctx, int32_t layer, const void *hidden, const void *K, const void *V,
@@ -1914,7 +1942,7 @@ static kvzap_status launch_compaction_paged(kvzap_ctx *ctx, const uint32_t *mask
                                             int32_t *page_table, int32_t max_pages, int32_t *lengths,
                                             int32_t *n_pages_used, cudaStream_t stream,
                                             int32_t *page_cursor = nullptr, bool tok_major = false, bool append = false,
-                                            bool beside_scoring = true, const int32_t *free_stack = nullptr,
+                                            const int32_t *free_stack = nullptr,
                                             int32_t *free_top = nullptr, const int64_t *list_map = nullptr)
 {
     const kvzap_config &c = ctx->cfg;
@@ -1933,20 +1961,12 @@ static kvzap_status launch_compaction_paged(kvzap_ctx *ctx, const uint32_t *mask
                                            static_cast<int>(max_pages), ctx->list_page0, page_table, n_pages_used,
                                            page_cursor, ctx->status_dev, append ? 1 : 0, ctx->list_base, free_stack, free_top, list_map));
     }
-    // the same resident-at-once grid as the dense-ragged output (see launch_compaction)
-    const int64_t max_ctas = static_cast<int64_t>(ctx->sm_count) * (!beside_scoring ? 8 : (c.hidden > 0 ? 2 : 6));
-    int64_t chunks = max_ctas / c.n_kv_heads;
-    if (chunks < 1) chunks = 1;
-    if (chunks > n_blocks) chunks = n_blocks;
-    const int blocks_per_cta = static_cast<int>((n_blocks + chunks - 1) / chunks);
-    chunks = (n_blocks + blocks_per_cta - 1) / blocks_per_cta;
+    const CompactShape shape = compact_shape(ctx, n_blocks, true, append);
     {
         ProfScope prof(ctx, KVZAP_KERNEL_COMPACT, stream);
-        make_launch(&cfg, attrs, dim3(static_cast<unsigned>(chunks), static_cast<unsigned>(c.n_kv_heads)),
-                    dim3(kDenseThreads), 0, stream, !ctx->profiling, 1);
-        KVZAP_CUDA(ctx, cudaLaunchKernelEx(&cfg, compact_dense_kernel<kDenseThreads>, static_cast<const uint4 *>(K),
+        KVZAP_CUDA(ctx, launch_compact_kernel(shape, stream, !ctx->profiling, static_cast<const uint4 *>(K),
                                            static_cast<const uint4 *>(V), static_cast<uint4 *>(K_pool),
-                                           static_cast<uint4 *>(V_pool), mask, n_words, n_blocks, blocks_per_cta,
+                                           static_cast<uint4 *>(V_pool), mask, n_words, n_blocks, shape.blocks_per_cta,
                                            cu_seqlens, static_cast<int>(n_seqs), n_tokens, static_cast<int>(c.n_kv_heads),
                                            static_cast<int>(c.head_dim / 8), lengths, static_cast<int>(page_tokens),
                                            static_cast<const int32_t *>(ctx->list_page0),
@@ -2514,7 +2534,7 @@ kvzap_status kvzap_prefill_to_cache(kvzap_ctx *ctx, kvzap_cache *cache, int32_t 
     ctx->launches += 1;
     return launch_compaction_paged(ctx, mask, K, V, nullptr, 1, n_tokens, v.k_pool, v.v_pool, v.n_pages_pool, v.page_tokens, 0,
                                    v.page_table + li0 * v.max_pages, v.max_pages, v.prefix_len + li0, nullptr, stream,
-                                   v.page_cursor, false, true, true, v.free_stack, v.free_top);
+                                   v.page_cursor, false, true, v.free_stack, v.free_top);
 }
 
 kvzap_status kvzap_prefill_to_cache_batch(kvzap_ctx *ctx, kvzap_cache *cache, int32_t layer, const int32_t *seq_ids,
@@ -2568,7 +2588,7 @@ kvzap_status kvzap_prefill_to_cache_batch(kvzap_ctx *ctx, kvzap_cache *cache, in
     ctx->launches += 1;
     return launch_compaction_paged(ctx, mask, K, V, cu_seqlens, n_seqs, n_tokens, v.k_pool, v.v_pool, v.n_pages_pool,
                                    v.page_tokens, 0, v.page_table, v.max_pages, v.prefix_len, nullptr, stream, v.page_cursor,
-                                   false, true, true, v.free_stack, v.free_top, ctx->batch_map);
+                                   false, true, v.free_stack, v.free_top, ctx->batch_map);
 }
 
 }  // extern "C"

@@ -481,7 +481,9 @@ __device__ __forceinline__ int popc_below(uint32_t w0, uint32_t w1, uint32_t w2,
 // register-file quarters that the MLP scoring kernel's ten warps leave free, so the compaction of layer
 // l runs beside the scoring of layer l + 1 at full width; at 72 registers only one fits and the layer
 // period of the fused path grows by ~10 us.
-template <int kThreads>
+// kAlone: the launch that runs beside nothing (a context that does not trust its producers: the scoring behind it waits
+// for it); see launch_compaction.  gridDim.z CTAs share the kept rows of a block.
+template <int kThreads, bool kAlone>
 __global__ void __launch_bounds__(kThreads, 1024 / kThreads)
 compact_dense_kernel(const uint4 *__restrict__ K, const uint4 *__restrict__ V, uint4 *__restrict__ K_out,
                      uint4 *__restrict__ V_out, const uint32_t *__restrict__ maskbits, int64_t n_words,
@@ -515,7 +517,8 @@ compact_dense_kernel(const uint4 *__restrict__ K, const uint4 *__restrict__ V, u
     griddep_launch_dependents();
     griddep_wait();
 
-    if (blockIdx.x == 0 && cu_seqlens != nullptr && !paged)   // empty sequences have no last token to write for them
+    const int z = blockIdx.z, nz = gridDim.z;
+    if (blockIdx.x == 0 && z == 0 && cu_seqlens != nullptr && !paged)   // empty sequences have no last token to write for them
         for (int b = tid; b < n_seqs; b += kThreads)
             if (cu_seqlens[b + 1] == cu_seqlens[b]) lengths[b * n_heads + h] = 0;
     if (blk0 >= n_blocks) return;
@@ -591,7 +594,7 @@ compact_dense_kernel(const uint4 *__restrict__ K, const uint4 *__restrict__ V, u
                         dst_row[r] = static_cast<int64_t>(h) * n_tokens + s + n;
                     }
                 }
-                if (t + 1 == e && !paged) lengths[b * n_heads + h] = running + r + (keep ? 1 : 0) - base;
+                if (t + 1 == e && !paged && z == 0) lengths[b * n_heads + h] = running + r + (keep ? 1 : 0) - base;
                 if (tid == kBlockTokens - 1 || t + 1 == n_tokens) {
                     // base of the sequence in progress at the next block's first token
                     int32_t nb = base;
@@ -602,12 +605,12 @@ compact_dense_kernel(const uint4 *__restrict__ K, const uint4 *__restrict__ V, u
         }
         __syncthreads();
         const int64_t head_row0 = static_cast<int64_t>(h) * in_stride_h + blk_start * in_stride_t;
-        for (int i0 = group; i0 < cnt; i0 += kGroups * kRowsInFlight) {
+        for (int i0 = group + z * kGroups; i0 < cnt; i0 += nz * kGroups * kRowsInFlight) {
             for (int u0 = gl; u0 < row_units; u0 += 16) {
                 uint4 kv[kRowsInFlight], vv[kRowsInFlight];
 #pragma unroll
                 for (int j = 0; j < kRowsInFlight; ++j) {
-                    const int i = i0 + j * kGroups;
+                    const int i = i0 + j * nz * kGroups;
                     if (i < cnt) {
                         const int64_t src = (head_row0 + src_tok[i] * in_stride_t) * row_units + u0;
                         kv[j] = __ldg(K + src);
@@ -616,7 +619,7 @@ compact_dense_kernel(const uint4 *__restrict__ K, const uint4 *__restrict__ V, u
                 }
 #pragma unroll
                 for (int j = 0; j < kRowsInFlight; ++j) {
-                    const int i = i0 + j * kGroups;
+                    const int i = i0 + j * nz * kGroups;
                     if (i < cnt && dst_row[i] >= 0) {
                         const int64_t d = dst_row[i] * row_units + u0;
                         K_out[d] = kv[j];
