@@ -54,6 +54,29 @@ __device__ __forceinline__ int32_t cache_take_page(const CacheView &c, int32_t *
     return got;
 }
 
+// The same for n pages at once (n <= 128), by a whole warp: one page at a time costs two round trips to memory each.
+// The pages go to pages[0 .. n), in lane-strided order; returns how many there were (the status word says if not all).
+__device__ __forceinline__ int cache_take_pages(const CacheView &c, int32_t *status, int n, int32_t *pages, int lane)
+{
+    int32_t top = 0, got = 0, cur = 0;
+    if (lane == 0 && n > 0) {
+        if (__ldcg(c.free_top) > 0) {
+            top = atomicSub(c.free_top, n);
+            got = top <= 0 ? 0 : top < n ? top : n;
+            if (got < n) atomicAdd(c.free_top, n - got);      // the stack did not hold as many
+        }
+        if (got < n) cur = atomicAdd(c.page_cursor, n - got);
+    }
+    top = __shfl_sync(0xffffffffu, top, 0);
+    got = __shfl_sync(0xffffffffu, got, 0);
+    cur = __shfl_sync(0xffffffffu, cur, 0);
+    const int64_t left = c.n_pages_pool - cur;
+    const int fresh = got == n || left <= 0 ? 0 : left < n - got ? static_cast<int>(left) : n - got;
+    if (got + fresh < n && lane == 0) atomicCAS(status, 0, 4 /* KVZAP_ERR_OOM_PAGES */);
+    for (int i = lane; i < got + fresh; i += 32) pages[i] = i < got ? __ldcg(c.free_stack + top - 1 - i) : cur + (i - got);
+    return got + fresh;
+}
+
 constexpr int kDecodeThreads = 256;
 constexpr int kDecodeLanes = 8;        // lanes that share one list (a 256-byte row = two 16-byte units per lane)
 
@@ -179,162 +202,14 @@ decode_update_kernel(const CacheView c, int layer0, int n_layers_call, const flo
     }
 }
 
-// Chunked prefill, the window side of one chunk of m prompt tokens appended to lists li0 .. li0+H-1
-// (one CTA per list), after the chunk has been scored:
-//   1. the tokens of the present window that the chunk pushes out (positions below n_old + m - w) are
-//      decided by their buffered scores, oldest first, and the kept ones appended to the list's paged
-//      prefix (pages from the cache's cursor) -- what m decode steps would have done;
-//   2. the chunk's last min(m, w) tokens (rows of K, V [H][m][D], scores [m][H]) take the ring slots of
-//      their absolute positions n_old + chunk index;
-//   3. n_tokens advances by m.
-// The chunk's own tokens before its last w are appended to the prefix afterwards by the compaction.
-// A batch of prompts in one launch (grid (H, n_seqs)): sequence b's chunk is tokens cu_seqlens[b] .. cu_seqlens[b+1]
-// of the packed buffers (K, V [H][n_total][D], scores [n_total][H]) and its lists start at list_map[b];
-// list_map == nullptr: one sequence, lists li0 .. li0+H-1, m = n_total tokens.
-__global__ void __launch_bounds__(256)
-chunk_ring_kernel(const CacheView c, int64_t li0, const float *__restrict__ scores, const uint4 *__restrict__ K,
-                  const uint4 *__restrict__ V, int64_t n_total, float tau, int32_t *__restrict__ status,
-                  const int64_t *__restrict__ list_map, const int32_t *__restrict__ cu_seqlens)
-{
-    __shared__ int64_t exit_src[128];       // ring row of an exiting token
-    __shared__ int64_t exit_dst[128];       // its pool row, -1 = dropped
-    __shared__ int64_t len_s;
-    __shared__ int ok_s;
-    const int h = blockIdx.x;
-    const int64_t li = (list_map != nullptr ? list_map[blockIdx.y] : li0) + h;
-    const int64_t tok0 = list_map != nullptr ? static_cast<int64_t>(cu_seqlens[blockIdx.y]) : 0;
-    const int64_t m = list_map != nullptr ? static_cast<int64_t>(cu_seqlens[blockIdx.y + 1]) - tok0 : n_total;
-    if (m <= 0) return;                     // an empty chunk leaves its lists as they are
-    K += tok0 * c.row_units;                // row (h, i) of the chunk is row h * n_total + tok0 + i of the buffers
-    V += tok0 * c.row_units;
-    scores += tok0 * c.n_heads;
-    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-    const int64_t n_old = c.n_tokens[li];
-    const int64_t in_ring = n_old < c.window ? n_old : c.window;
-    const int64_t first = n_old - in_ring;                         // oldest position still in the window
-    int64_t exit_end = n_old + m - c.window;                       // positions below it leave the window
-    if (exit_end > n_old) exit_end = n_old;
-    const int64_t n_exit = exit_end > first ? exit_end - first : 0;
-    int32_t *table = c.page_table + li * c.max_pages;
-    if (tid == 0) { len_s = c.prefix_len[li]; ok_s = 1; }
-    __syncthreads();
-    for (int64_t base = 0; base < n_exit && ok_s; base += 128) {
-        if (warp == 0) {
-            int64_t len = len_s;
-            for (int i = lane; i < 128; i += 32) exit_dst[i] = -1;     // nothing is copied unless it is decided below
-            float sc4[4];                                              // the buffered scores of the batch, loaded together
-#pragma unroll
-            for (int j = 0; j < 4; ++j) {
-                const int64_t pos = first + base + 32 * j + lane;
-                sc4[j] = base + 32 * j + lane < n_exit ? c.score_ring[li * c.window + pos % c.window] : 0.0f;
-            }
-            __syncwarp();
-#pragma unroll
-            for (int sub = 0; sub < 128; sub += 32) {
-                if (base + sub >= n_exit) break;
-                const int64_t pos = first + base + sub + lane;
-                const bool valid = base + sub + lane < n_exit;
-                const int64_t slot = li * c.window + pos % c.window;
-                const bool keep = valid && sc4[sub >> 5] >= tau;
-                const uint32_t kept = __ballot_sync(0xffffffffu, keep);
-                const int cnt = __popc(kept);
-                const int64_t have = (len + c.page_tokens - 1) / c.page_tokens;
-                const int64_t want = (len + cnt + c.page_tokens - 1) / c.page_tokens;
-                int ok = 1;
-                if (lane == 0 && want > have) {
-                    if (want > c.max_pages) {
-                        ok = 0;
-                        atomicCAS(status, 0, 4 /* KVZAP_ERR_OOM_PAGES */);
-                    } else {
-                        for (int64_t i = have; i < want && ok; ++i) {
-                            const int32_t page = cache_take_page(c, status);
-                            if (page < 0) ok = 0;
-                            else table[i] = page;
-                        }
-                    }
-                }
-                ok = __shfl_sync(0xffffffffu, ok, 0);
-                __syncwarp();
-                if (valid) {
-                    int64_t dst = -1;
-                    if (keep && ok) {
-                        const int64_t nn = len + __popc(kept & ((1u << lane) - 1u));
-                        const int64_t page = *(volatile int32_t *)(table + nn / c.page_tokens);
-                        dst = page * c.page_tokens + nn % c.page_tokens;
-                    }
-                    exit_src[sub + lane] = slot;
-                    exit_dst[sub + lane] = dst;
-                }
-                if (!ok) { if (lane == 0) ok_s = 0; break; }       // what was appended so far stays valid
-                len += cnt;
-            }
-            if (lane == 0) len_s = len;
-        }
-        __syncthreads();
-        // rows of this batch of exits: 16 lanes per row
-        const int64_t n_batch = n_exit - base < 128 ? n_exit - base : 128;
-        for (int64_t i0 = tid >> 4; i0 < n_batch; i0 += 64) {     // four rows per lane group in flight
-            for (int u = tid & 15; u < c.row_units; u += 16) {
-                uint4 kr[4], vr[4];
-#pragma unroll
-                for (int j = 0; j < 4; ++j) {
-                    const int64_t i = i0 + 16 * j;
-                    if (i < n_batch && exit_dst[i] >= 0) {
-                        kr[j] = c.k_ring[exit_src[i] * c.row_units + u];
-                        vr[j] = c.v_ring[exit_src[i] * c.row_units + u];
-                    }
-                }
-#pragma unroll
-                for (int j = 0; j < 4; ++j) {
-                    const int64_t i = i0 + 16 * j;
-                    if (i < n_batch && exit_dst[i] >= 0) {
-                        c.k_pool[exit_dst[i] * c.row_units + u] = kr[j];
-                        c.v_pool[exit_dst[i] * c.row_units + u] = vr[j];
-                    }
-                }
-            }
-        }
-        __syncthreads();
-    }
-    // the chunk's last min(m, w) tokens into the ring (the slots they take were read above)
-    const int64_t n_win = m < c.window ? m : c.window;
-    for (int64_t i0 = tid; i0 < n_win * c.row_units; i0 += 4 * 256) {     // four units per thread in flight
-        uint4 kr[4], vr[4];
-#pragma unroll
-        for (int j = 0; j < 4; ++j) {
-            const int64_t i = i0 + 256 * j;
-            if (i < n_win * c.row_units) {
-                const int64_t src = (static_cast<int64_t>(h) * n_total + m - n_win + i / c.row_units) * c.row_units + i % c.row_units;
-                kr[j] = __ldg(K + src);
-                vr[j] = __ldg(V + src);
-            }
-        }
-#pragma unroll
-        for (int j = 0; j < 4; ++j) {
-            const int64_t i = i0 + 256 * j;
-            if (i < n_win * c.row_units) {
-                const int64_t ci = m - n_win + i / c.row_units;        // index inside the chunk
-                const int u = static_cast<int>(i % c.row_units);
-                const int64_t slot = li * c.window + (n_old + ci) % c.window;
-                c.k_ring[slot * c.row_units + u] = kr[j];
-                c.v_ring[slot * c.row_units + u] = vr[j];
-                if (u == 0) c.score_ring[slot] = scores[ci * c.n_heads + h];
-            }
-        }
-    }
-    if (tid == 0) {
-        c.prefix_len[li] = static_cast<int32_t>(len_s);
-        c.n_tokens[li] = static_cast<int32_t>(n_old + m);
-        if (h == 0) c.active[li / (static_cast<int64_t>(c.n_layers) * c.n_heads)] = 1;     // the slot holds a sequence again
-    }
-}
-
 // A sequence has ended: the pages of all its lists (L x H of them, one warp each) go onto the stack of
 // released pages and the lists become empty.  Runs alone on the stream (it is the one kernel that adds
 // to the stack).
 __global__ void __launch_bounds__(32)
 release_seq_kernel(const CacheView c, int32_t seq)
 {
+    griddep_wait();              // every kernel that touches the cache waits for the one ahead before it does
+    griddep_launch_dependents();
     const int64_t li = static_cast<int64_t>(seq) * c.n_layers * c.n_heads + blockIdx.x;
     const int lane = threadIdx.x;
     const int32_t n_pages = (c.prefix_len[li] + c.page_tokens - 1) / c.page_tokens;
@@ -348,19 +223,6 @@ release_seq_kernel(const CacheView c, int32_t seq)
         c.n_tokens[li] = 0;
         if (blockIdx.x == 0) c.active[seq] = 0;
     }
-}
-
-// no window: only the token count advances
-__global__ void tokens_add_kernel(const CacheView c, int64_t li0, int64_t m, const int64_t *__restrict__ list_map,
-                                  const int32_t *__restrict__ cu_seqlens)
-{
-    if (list_map != nullptr) {              // one block per sequence of a batch
-        li0 = list_map[blockIdx.x];
-        m = cu_seqlens[blockIdx.x + 1] - cu_seqlens[blockIdx.x];
-        if (m <= 0) return;
-    }
-    if (threadIdx.x < c.n_heads) c.n_tokens[li0 + threadIdx.x] += static_cast<int32_t>(m);
-    if (threadIdx.x == 0) c.active[li0 / (static_cast<int64_t>(c.n_layers) * c.n_heads)] = 1;
 }
 
 // lengths[li] = prefix_len + min(n_tokens, w)

@@ -19,6 +19,7 @@
 #include "prune_kernels.cuh"
 #include "prune_onepass_kernel.cuh"
 #include "score_kernel.cuh"
+#include "chunk_kernel.cuh"
 #include "score_linear_split_kernel.cuh"
 #include "score_split_kernel.cuh"
 #include "select_kernels.cuh"
@@ -89,7 +90,8 @@ struct kvzap_ctx {
     uint32_t *select_hist = nullptr;     // fixed-budget selection: [4 passes][max_seqs][H][256] histograms
     float *select_tau = nullptr;         //                         [max_seqs][H] cut values when the caller wants none
     float *plan_scores = nullptr;        // kvzap_prefill_plan without scores_out: [max_tokens][H] (allocated on first use)
-    int64_t *batch_map = nullptr;        // kvzap_prefill_to_cache_batch: first list of each sequence of the call [max_seqs]
+    int64_t *batch_map = nullptr;        // chunks into a cache: first list of each sequence of the call [max_seqs]
+    uint32_t *chunk_arrive = nullptr;    //                      lists that are done, zero between launches
     float *split_part = nullptr;         // few-token kernel: [tile][slice][128][8] partial scores, tiles * slices <= sm_count
     uint64_t score_turn = 0;
     bool last_score_early = false;       // the last scoring launch was allowed to start early
@@ -402,6 +404,7 @@ static void free_all(kvzap_ctx *ctx)
     cudaFree(ctx->split_part);
     cudaFree(ctx->plan_scores);
     cudaFree(ctx->batch_map);
+    cudaFree(ctx->chunk_arrive);
     cudaFree(ctx->select_hist);
     cudaFree(ctx->select_tau);
     for (auto &l : ctx->layouts) cudaFree(l.arrive);
@@ -1340,6 +1343,9 @@ kvzap_status kvzap_create(kvzap_ctx **out, const kvzap_config *cfg)
     CREATE_CUDA(cudaMalloc(&ctx->maskbits, sizeof(uint32_t) * kMaskRing * ctx->max_words * c.n_kv_heads));
     CREATE_CUDA(cudaMalloc(&ctx->list_page0, sizeof(int32_t) * static_cast<int64_t>(c.max_seqs) * c.n_kv_heads));
     CREATE_CUDA(cudaMalloc(&ctx->list_base, sizeof(int32_t) * static_cast<int64_t>(c.max_seqs) * c.n_kv_heads));
+    CREATE_CUDA(cudaMalloc(&ctx->batch_map, sizeof(int64_t) * static_cast<size_t>(c.max_seqs)));
+    CREATE_CUDA(cudaMalloc(&ctx->chunk_arrive, sizeof(uint32_t)));
+    CREATE_CUDA(cudaMemset(ctx->chunk_arrive, 0, sizeof(uint32_t)));
     CREATE_CUDA(cudaMalloc(&ctx->tile_counters, sizeof(int32_t) * kMaskRing));
     CREATE_CUDA(cudaMemset(ctx->tile_counters, 0, sizeof(int32_t) * kMaskRing));
     CREATE_CUDA(cudaMalloc(&ctx->select_hist, sizeof(uint32_t) * 4 * static_cast<size_t>(c.max_seqs) * c.n_kv_heads * 256));
@@ -1943,14 +1949,15 @@ static kvzap_status launch_compaction_paged(kvzap_ctx *ctx, const uint32_t *mask
                                             int32_t *n_pages_used, cudaStream_t stream,
                                             int32_t *page_cursor = nullptr, bool tok_major = false, bool append = false,
                                             const int32_t *free_stack = nullptr,
-                                            int32_t *free_top = nullptr, const int64_t *list_map = nullptr)
+                                            int32_t *free_top = nullptr, const int64_t *list_map = nullptr,
+                                            bool pages_assigned = false)
 {
     const kvzap_config &c = ctx->cfg;
     const int64_t n_blocks = (n_tokens + kBlockTokens - 1) / kBlockTokens;
     const int64_t n_words = n_blocks * 4;
-    cudaLaunchConfig_t cfg;
-    cudaLaunchAttribute attrs[2];
-    {
+    if (!pages_assigned) {
+        cudaLaunchConfig_t cfg;
+        cudaLaunchAttribute attrs[2];
         // lengths and the first page of every list (the only step that needs all lists at once)
         ProfScope prof(ctx, KVZAP_KERNEL_SCAN, stream);
         make_launch(&cfg, attrs, dim3(1), dim3(1024), 0, stream, !ctx->profiling, 1);
@@ -1960,6 +1967,7 @@ static kvzap_status launch_compaction_paged(kvzap_ctx *ctx, const uint32_t *mask
                                            lengths, static_cast<int>(page_tokens), first_page, n_pages_pool,
                                            static_cast<int>(max_pages), ctx->list_page0, page_table, n_pages_used,
                                            page_cursor, ctx->status_dev, append ? 1 : 0, ctx->list_base, free_stack, free_top, list_map));
+        ctx->launches += 1;
     }
     const CompactShape shape = compact_shape(ctx, n_blocks, true, append);
     {
@@ -1975,7 +1983,7 @@ static kvzap_status launch_compaction_paged(kvzap_ctx *ctx, const uint32_t *mask
                                            static_cast<const int32_t *>(append ? ctx->list_base : nullptr),
                                            static_cast<const int32_t *>(page_table), static_cast<int>(max_pages), list_map));
     }
-    ctx->launches += 2;
+    ctx->launches += 1;
     return KVZAP_OK;
 }
 
@@ -2423,9 +2431,11 @@ kvzap_status kvzap_cache_release_seq(kvzap_cache *cache, int32_t seq, void *stre
     begin_op(ctx);
     if (seq < 0 || seq >= cache->v.n_seqs) return fail(ctx, KVZAP_ERR_INVALID_ARG, "release: seq %d out of range", seq);
     DeviceGuard guard(ctx->cfg.device);
-    release_seq_kernel<<<static_cast<unsigned>(cache->v.n_layers * cache->v.n_heads), 32, 0,
-                         static_cast<cudaStream_t>(stream_)>>>(cache->v, seq);
-    KVZAP_CUDA(ctx, cudaGetLastError());
+    cudaLaunchConfig_t cfg;
+    cudaLaunchAttribute attrs[2];
+    make_launch(&cfg, attrs, dim3(static_cast<unsigned>(cache->v.n_layers * cache->v.n_heads)), dim3(32), 0,
+                static_cast<cudaStream_t>(stream_), !ctx->profiling, 1);
+    KVZAP_CUDA(ctx, cudaLaunchKernelEx(&cfg, release_seq_kernel, cache->v, seq));
     ctx->launches += 1;
     return KVZAP_OK;
 }
@@ -2496,6 +2506,43 @@ kvzap_status kvzap_cache_snapshot(kvzap_cache *cache, int32_t *prefix_len, int32
     return KVZAP_OK;
 }
 
+// The window side of a scored chunk (or of a chunk of each of several prompts, cu_seqlens) and the appending of its kept
+// rows; `seqs` names the sequence slots.
+static kvzap_status append_chunk(kvzap_ctx *ctx, kvzap_cache *cache, int32_t layer, const int32_t *seqs, int32_t n_seqs,
+                                 const int32_t *cu_seqlens, const uint32_t *mask, const float *scores, const void *K, const void *V,
+                                 int64_t n_tokens, float tau, cudaStream_t stream)
+{
+    const kvzap_config &c = ctx->cfg;
+    const CacheView &v = cache->v;
+    ChunkSeqs by_value;
+    by_value.n = n_seqs <= kMaxChunkSeqs ? n_seqs : 0;
+    for (int i = 0; i < by_value.n; ++i) by_value.slot[i] = seqs[i];
+    if (by_value.n == 0) {
+        // from pageable host memory: staged by the driver before the call returns; ordered on the stream behind the
+        // kernels of an earlier call that still read the previous map
+        std::vector<int64_t> map(static_cast<size_t>(n_seqs));
+        for (int i = 0; i < n_seqs; ++i) map[i] = (static_cast<int64_t>(seqs[i]) * v.n_layers + layer) * v.n_heads;
+        KVZAP_CUDA(ctx, cudaMemcpyAsync(ctx->batch_map, map.data(), sizeof(int64_t) * map.size(), cudaMemcpyHostToDevice, stream));
+    }
+    const int64_t n_words = (n_tokens + kBlockTokens - 1) / kBlockTokens * 4;
+    if (v.window > 0) {
+        cudaLaunchConfig_t cfg;
+        cudaLaunchAttribute attrs[2];
+        make_launch(&cfg, attrs, dim3(static_cast<unsigned>(v.n_heads), static_cast<unsigned>(n_seqs)), dim3(kChunkThreads), 0, stream,
+                    !ctx->profiling, 1);
+        KVZAP_CUDA(ctx, cudaLaunchKernelEx(&cfg, chunk_ring_kernel, v, by_value, static_cast<int>(layer), ctx->batch_map, scores,
+                                           static_cast<const uint4 *>(K), static_cast<const uint4 *>(V), n_tokens, tau, cu_seqlens, mask,
+                                           n_words, ctx->list_base, ctx->list_page0, ctx->chunk_arrive, ctx->status_dev));
+    } else {
+        tokens_add_kernel<<<static_cast<unsigned>(n_seqs), 32, 0, stream>>>(v, by_value, layer, ctx->batch_map, n_tokens, cu_seqlens);
+        KVZAP_CUDA(ctx, cudaGetLastError());
+    }
+    ctx->launches += 1;
+    return launch_compaction_paged(ctx, mask, K, V, cu_seqlens, n_seqs, n_tokens, v.k_pool, v.v_pool, v.n_pages_pool,
+                                   v.page_tokens, 0, v.page_table, v.max_pages, v.prefix_len, nullptr, stream, v.page_cursor,
+                                   false, true, v.free_stack, v.free_top, ctx->batch_map, v.window > 0);
+}
+
 kvzap_status kvzap_prefill_to_cache(kvzap_ctx *ctx, kvzap_cache *cache, int32_t layer, int32_t seq, const void *hidden,
                                     const void *K, const void *V, int64_t n_tokens, float tau, float *scores_out,
                                     void *stream_)
@@ -2515,7 +2562,6 @@ kvzap_status kvzap_prefill_to_cache(kvzap_ctx *ctx, kvzap_cache *cache, int32_t 
     if (!hidden || !K || !V || !scores_out || !aligned16(hidden) || !aligned16(K) || !aligned16(V))
         return fail(ctx, KVZAP_ERR_INVALID_ARG, "prefill_to_cache: hidden, K, V, scores_out must be non-NULL, aligned");
     DeviceGuard guard(c.device);
-    const int64_t li0 = (static_cast<int64_t>(seq) * v.n_layers + layer) * v.n_heads;
     // The lists may already hold earlier chunks of the prompt.  Scoring first (mask = threshold only, the
     // chunk's last `window` tokens left out: they go to the ring); then the window side -- the tokens the
     // chunk pushes out of the present window are decided by their buffered scores and appended to the
@@ -2524,17 +2570,7 @@ kvzap_status kvzap_prefill_to_cache(kvzap_ctx *ctx, kvzap_cache *cache, int32_t 
     uint32_t *mask = next_mask_slice(ctx);
     st = launch_score(ctx, layer, 1, hidden, n_tokens, scores_out, mask, nullptr, 1, tau, v.window, stream, 0);
     if (st != KVZAP_OK) return st;
-    if (v.window > 0)
-        chunk_ring_kernel<<<static_cast<unsigned>(v.n_heads), 256, 0, stream>>>(
-            v, li0, scores_out, static_cast<const uint4 *>(K), static_cast<const uint4 *>(V), n_tokens, tau, ctx->status_dev,
-            nullptr, nullptr);
-    else
-        tokens_add_kernel<<<1, 32, 0, stream>>>(v, li0, n_tokens, nullptr, nullptr);
-    KVZAP_CUDA(ctx, cudaGetLastError());
-    ctx->launches += 1;
-    return launch_compaction_paged(ctx, mask, K, V, nullptr, 1, n_tokens, v.k_pool, v.v_pool, v.n_pages_pool, v.page_tokens, 0,
-                                   v.page_table + li0 * v.max_pages, v.max_pages, v.prefix_len + li0, nullptr, stream,
-                                   v.page_cursor, false, true, v.free_stack, v.free_top);
+    return append_chunk(ctx, cache, layer, &seq, 1, nullptr, mask, scores_out, K, V, n_tokens, tau, stream);
 }
 
 kvzap_status kvzap_prefill_to_cache_batch(kvzap_ctx *ctx, kvzap_cache *cache, int32_t layer, const int32_t *seq_ids,
@@ -2555,7 +2591,6 @@ kvzap_status kvzap_prefill_to_cache_batch(kvzap_ctx *ctx, kvzap_cache *cache, in
     if (!ctx->layer_set[layer]) return fail(ctx, KVZAP_ERR_STATE, "layer %d has no weights", layer);
     // the lists of head 0 of every sequence; slots must be in range and distinct (two chunks for one list in
     // one launch would race)
-    std::vector<int64_t> map(static_cast<size_t>(n_seqs));
     {
         std::vector<int32_t> sorted(seq_ids, seq_ids + n_seqs);
         std::sort(sorted.begin(), sorted.end());
@@ -2564,31 +2599,16 @@ kvzap_status kvzap_prefill_to_cache_batch(kvzap_ctx *ctx, kvzap_cache *cache, in
                 return fail(ctx, KVZAP_ERR_INVALID_ARG, "prefill_to_cache_batch: sequence slot %d out of range", sorted[i]);
             if (i > 0 && sorted[i] == sorted[i - 1])
                 return fail(ctx, KVZAP_ERR_INVALID_ARG, "prefill_to_cache_batch: sequence slot %d given twice", sorted[i]);
-            map[i] = (static_cast<int64_t>(seq_ids[i]) * v.n_layers + layer) * v.n_heads;
         }
     }
     if (n_tokens == 0) return KVZAP_OK;
     if (!hidden || !K || !V || !scores_out || !aligned16(hidden) || !aligned16(K) || !aligned16(V))
         return fail(ctx, KVZAP_ERR_INVALID_ARG, "prefill_to_cache_batch: hidden, K, V, scores_out must be non-NULL, aligned");
     DeviceGuard guard(c.device);
-    if (!ctx->batch_map) KVZAP_CUDA(ctx, cudaMalloc(&ctx->batch_map, sizeof(int64_t) * static_cast<size_t>(c.max_seqs)));
-    // from pageable host memory: staged by the driver before the call returns; ordered on the stream behind the
-    // kernels of an earlier batch that still read the previous map
-    KVZAP_CUDA(ctx, cudaMemcpyAsync(ctx->batch_map, map.data(), sizeof(int64_t) * map.size(), cudaMemcpyHostToDevice, stream));
     uint32_t *mask = next_mask_slice(ctx);
     st = launch_score(ctx, layer, 1, hidden, n_tokens, scores_out, mask, cu_seqlens, n_seqs, tau, v.window, stream, 0);
     if (st != KVZAP_OK) return st;
-    if (v.window > 0)
-        chunk_ring_kernel<<<dim3(static_cast<unsigned>(v.n_heads), static_cast<unsigned>(n_seqs)), 256, 0, stream>>>(
-            v, 0, scores_out, static_cast<const uint4 *>(K), static_cast<const uint4 *>(V), n_tokens, tau, ctx->status_dev,
-            ctx->batch_map, cu_seqlens);
-    else
-        tokens_add_kernel<<<static_cast<unsigned>(n_seqs), 32, 0, stream>>>(v, 0, 0, ctx->batch_map, cu_seqlens);
-    KVZAP_CUDA(ctx, cudaGetLastError());
-    ctx->launches += 1;
-    return launch_compaction_paged(ctx, mask, K, V, cu_seqlens, n_seqs, n_tokens, v.k_pool, v.v_pool, v.n_pages_pool,
-                                   v.page_tokens, 0, v.page_table, v.max_pages, v.prefix_len, nullptr, stream, v.page_cursor,
-                                   false, true, v.free_stack, v.free_top, ctx->batch_map);
+    return append_chunk(ctx, cache, layer, seq_ids, n_seqs, cu_seqlens, mask, scores_out, K, V, n_tokens, tau, stream);
 }
 
 }  // extern "C"

@@ -102,7 +102,7 @@ __device__ __forceinline__ int32_t kept_before(const uint32_t *__restrict__ mask
 // at list_map[b] + h, list_map [n_seqs] naming the list of head 0 of each of the call's sequences.
 __device__ __forceinline__ int64_t list_at(const int64_t *__restrict__ list_map, int idx, int n_heads)
 {
-    return list_map != nullptr ? list_map[idx / n_heads] + idx % n_heads : static_cast<int64_t>(idx);
+    return list_map != nullptr ? __ldcg(list_map + idx / n_heads) + idx % n_heads : static_cast<int64_t>(idx);
 }
 
 // ---------------------------------------------------------------------------
@@ -156,9 +156,9 @@ assign_pages(int n_heads, int n_seqs, int32_t *__restrict__ lengths, int page_to
         const int idx = base + tid;
         int32_t need = 0;
         if (idx < n_lists) {
-            need = (lengths[list_at(list_map, idx, n_heads)] + page_tokens - 1) / page_tokens;
+            need = (__ldcg(lengths + list_at(list_map, idx, n_heads)) + page_tokens - 1) / page_tokens;
             if (need > max_pages) fail_s = 1;
-            if (append) need -= (list_base[idx] + page_tokens - 1) / page_tokens;     // pages the list already owns
+            if (append) need -= (__ldcg(list_base + idx) + page_tokens - 1) / page_tokens;     // pages the list already owns
         }
         int32_t total;
         const int32_t incl = block_scan(need, total);
@@ -171,7 +171,7 @@ assign_pages(int n_heads, int n_seqs, int32_t *__restrict__ lengths, int page_to
     const int32_t used = carry_s;
     int32_t n_free = 0;
     if (page_cursor != nullptr && free_top != nullptr) {
-        n_free = *free_top;
+        n_free = __ldcg(free_top);
         if (n_free < 0) n_free = 0;
     }
     const int32_t from_stack = used < n_free ? used : n_free;
@@ -179,7 +179,7 @@ assign_pages(int n_heads, int n_seqs, int32_t *__restrict__ lengths, int page_to
     if (fail) {
         for (int idx = tid; idx < n_lists; idx += NT) {
             list_page0[idx] = -1;
-            if (append) lengths[list_at(list_map, idx, n_heads)] = list_base[idx];
+            if (append) lengths[list_at(list_map, idx, n_heads)] = __ldcg(list_base + idx);
         }
         if (tid == 0) {
             atomicCAS(status, 0, 4 /* KVZAP_ERR_OOM_PAGES */);
@@ -197,13 +197,13 @@ assign_pages(int n_heads, int n_seqs, int32_t *__restrict__ lengths, int page_to
     if (!fill_table) return;
     for (int idx = warp; idx < n_lists; idx += NT / 32) {            // a warp per list
         const int32_t p0 = list_page0[idx];
-        const int32_t have = append ? (list_base[idx] + page_tokens - 1) / page_tokens : 0;
+        const int32_t have = append ? (__ldcg(list_base + idx) + page_tokens - 1) / page_tokens : 0;
         const int64_t li = list_at(list_map, idx, n_heads);
-        const int32_t need = (lengths[li] + page_tokens - 1) / page_tokens - have;
+        const int32_t need = (__ldcg(lengths + li) + page_tokens - 1) / page_tokens - have;
         for (int32_t i = lane; i < need; i += 32) {
             const int32_t j = p0 - first_page + i;            // ordinal among the pages assigned by this call
             page_table[li * max_pages + have + i] =
-                j < from_stack ? free_stack[n_free - 1 - j] : first_page + (j - from_stack);
+                j < from_stack ? __ldcg(free_stack + n_free - 1 - j) : first_page + (j - from_stack);
         }
     }
 }
@@ -577,15 +577,15 @@ compact_dense_kernel(const uint4 *__restrict__ K, const uint4 *__restrict__ V, u
                     src_tok[r] = tid;
                     const int64_t n = running + r - base;                  // rank inside list (b,h)
                     if (paged) {
-                        const int32_t p0 = list_page0[b * n_heads + h];
+                        const int32_t p0 = __ldcg(list_page0 + b * n_heads + h);
                         if (list_base == nullptr) {
                             dst_row[r] = p0 < 0 ? -1 : (static_cast<int64_t>(p0) + n / page_tokens) * page_tokens + n % page_tokens;
                         } else {
-                            const int64_t nn = list_base[b * n_heads + h] + n;
+                            const int64_t nn = __ldcg(list_base + b * n_heads + h) + n;
                             if (p0 < 0) {
                                 dst_row[r] = -1;
                             } else {
-                                const int64_t trow = list_map != nullptr ? list_map[b] + h : static_cast<int64_t>(b * n_heads + h);
+                                const int64_t trow = list_map != nullptr ? __ldcg(list_map + b) + h : static_cast<int64_t>(b * n_heads + h);
                                 const int64_t page = __ldcg(page_table + trow * max_pages + nn / page_tokens);
                                 dst_row[r] = page * page_tokens + nn % page_tokens;
                             }
