@@ -14,7 +14,7 @@ struct ChunkSeqs {
     int32_t slot[kMaxChunkSeqs];
 };
 
-constexpr int kChunkThreads = 1024;     // one round of row moves for a window of 128: the rows are 64 KB per list and side
+constexpr int kChunkThreads = 256;
 
 // For every list (sequence of the call, head) of one layer, one CTA each (grid (H, n_seqs)), after the chunk has been
 // scored and its tokens outside the window have been thresholded into mask words:
@@ -28,28 +28,30 @@ constexpr int kChunkThreads = 1024;     // one round of row moves for a window o
 // and the CTA that is done last assigns pages for all lists' new rows (assign_pages, all or nothing), which the
 // compaction reads.  Sequence b's chunk is tokens cu_seqlens[b] .. cu_seqlens[b+1] of the packed buffers (cu_seqlens ==
 // nullptr: all of them).
-// What bounds it is a chain of round trips to memory (counts, scores, pages, rows).  One launch for this and the page
-// assignment, pages taken a batch at a time, all rows of a window in flight at once: 4 prompts x 8 heads, a window of 128
-// pushed out, 17.5 + 7 us (page by page with 256 threads, then a launch of its own) -> 16 us.
-__global__ void __launch_bounds__(kChunkThreads)
+// What bounds it is a chain of round trips to memory (counts, scores, pages, rows, arrival, assignment).  Most of it
+// depends on nothing that the scoring computes: with `beside` != 0 the launch ahead is a scoring kernel that lets this one
+// start once everything ahead of IT has completed, and 1 and the rows of 2 run beside it; the CTAs are small enough to
+// share an SM with its CTAs.  Only the counting of the chunk's kept rows, its scores and the page assignment are left for
+// the time after it.  4 prompts x 8 heads, a window of 128 pushed out, from the end of the scoring launch: 24.5 us page by
+// page with a launch of its own for the assignment, 16 us as one launch of 1024 threads per list behind the scoring,
+// 7.7 us beside it.
+__global__ void __launch_bounds__(kChunkThreads, 4)      // 64 registers: see compact_dense_kernel
 chunk_ring_kernel(const CacheView c, const __grid_constant__ ChunkSeqs seqs, int layer, int64_t *__restrict__ list_map,
                   const float *__restrict__ scores, const uint4 *__restrict__ K, const uint4 *__restrict__ V, int64_t n_total, float tau,
                   const int32_t *__restrict__ cu_seqlens, const uint32_t *__restrict__ maskbits, int64_t n_words,
                   int32_t *__restrict__ list_base, int32_t *__restrict__ list_page0, uint32_t *__restrict__ arrive,
-                  int32_t *__restrict__ status)
+                  int32_t *__restrict__ status, int beside)
 {
     __shared__ int64_t exit_src[128];       // ring row of an exiting token
     __shared__ int64_t exit_dst[128];       // its pool row, -1 = dropped
     __shared__ int32_t new_pages[128];
     __shared__ int64_t len_s;
-    __shared__ int ok_s, kept_s, last_s;
-    griddep_wait();
-    griddep_launch_dependents();
+    __shared__ int ok_s, kept_s, last_s, cursor_s;
+    if (!beside) griddep_wait();
     const int h = blockIdx.x, b = blockIdx.y, H = c.n_heads;
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const int64_t list0 = seqs.n > 0 ? (static_cast<int64_t>(seqs.slot[b]) * c.n_layers + layer) * H : __ldcg(list_map + b);
     const int64_t li = list0 + h;
-    if (seqs.n > 0 && h == 0 && tid == 0) list_map[b] = list0;      // for the compaction
     const int64_t tok0 = cu_seqlens != nullptr ? static_cast<int64_t>(cu_seqlens[b]) : 0;
     const int64_t m = cu_seqlens != nullptr ? static_cast<int64_t>(cu_seqlens[b + 1]) - tok0 : n_total;
     K += tok0 * c.row_units;                // row (h, i) of the chunk is row h * n_total + tok0 + i of the buffers
@@ -58,19 +60,6 @@ chunk_ring_kernel(const CacheView c, const __grid_constant__ ChunkSeqs seqs, int
     const int64_t n_old = __ldcg(c.n_tokens + li);
     if (tid == 0) { len_s = __ldcg(c.prefix_len + li); ok_s = 1; kept_s = 0; }
     __syncthreads();
-    // the chunk's own kept rows
-    {
-        const uint32_t *words = maskbits + static_cast<int64_t>(h) * n_words;
-        int cnt = 0;
-        for (int64_t wi = tok0 / 32 + tid; wi * 32 < tok0 + m; wi += kChunkThreads) {
-            uint32_t w = __ldcg(words + wi);
-            if (wi * 32 < tok0) w &= ~0u << static_cast<int>(tok0 - wi * 32);                    // bits below the chunk
-            if (wi * 32 + 32 > tok0 + m) w &= (1u << static_cast<int>(tok0 + m - wi * 32)) - 1u; // bits above it
-            cnt += __popc(w);
-        }
-        cnt = __reduce_add_sync(0xffffffffu, cnt);
-        if (lane == 0 && cnt) atomicAdd(&kept_s, cnt);
-    }
     const int64_t in_ring = n_old < c.window ? n_old : c.window;
     const int64_t first = n_old - in_ring;                         // oldest position still in the window
     int64_t exit_end = n_old + m - c.window;                       // positions below it leave the window
@@ -78,7 +67,7 @@ chunk_ring_kernel(const CacheView c, const __grid_constant__ ChunkSeqs seqs, int
     const int64_t n_exit = m > 0 && exit_end > first ? exit_end - first : 0;      // an empty chunk leaves its list as it is
     int32_t *table = c.page_table + li * c.max_pages;
     const int group = tid >> 4, gl = tid & 15;
-    constexpr int kGroups = kChunkThreads / 16;
+    constexpr int kGroups = kChunkThreads / 16, kRows = 2;         // 16 lanes per row, two rows per lane group in flight
     for (int64_t base = 0; base < n_exit && ok_s; base += 128) {
         if (warp == 0) {
             const int64_t len = len_s;
@@ -133,24 +122,25 @@ chunk_ring_kernel(const CacheView c, const __grid_constant__ ChunkSeqs seqs, int
             }
         }
         __syncthreads();
-        // rows of this batch of exits: 16 lanes per row, two rows per lane group in flight
         const int n_batch = n_exit - base < 128 ? static_cast<int>(n_exit - base) : 128;
-        for (int u = gl; u < c.row_units; u += 16) {
-            uint4 kr[128 / kGroups], vr[128 / kGroups];
+        for (int i0 = group; i0 < n_batch; i0 += kRows * kGroups) {
+            for (int u = gl; u < c.row_units; u += 16) {
+                uint4 kr[kRows], vr[kRows];
 #pragma unroll
-            for (int j = 0; j < 128 / kGroups; ++j) {
-                const int i = group + kGroups * j;
-                if (i < n_batch && exit_dst[i] >= 0) {
-                    kr[j] = __ldcg(c.k_ring + exit_src[i] * c.row_units + u);
-                    vr[j] = __ldcg(c.v_ring + exit_src[i] * c.row_units + u);
+                for (int j = 0; j < kRows; ++j) {
+                    const int i = i0 + kGroups * j;
+                    if (i < n_batch && exit_dst[i] >= 0) {
+                        kr[j] = __ldcg(c.k_ring + exit_src[i] * c.row_units + u);
+                        vr[j] = __ldcg(c.v_ring + exit_src[i] * c.row_units + u);
+                    }
                 }
-            }
 #pragma unroll
-            for (int j = 0; j < 128 / kGroups; ++j) {
-                const int i = group + kGroups * j;
-                if (i < n_batch && exit_dst[i] >= 0) {
-                    c.k_pool[exit_dst[i] * c.row_units + u] = kr[j];
-                    c.v_pool[exit_dst[i] * c.row_units + u] = vr[j];
+                for (int j = 0; j < kRows; ++j) {
+                    const int i = i0 + kGroups * j;
+                    if (i < n_batch && exit_dst[i] >= 0) {
+                        c.k_pool[exit_dst[i] * c.row_units + u] = kr[j];
+                        c.v_pool[exit_dst[i] * c.row_units + u] = vr[j];
+                    }
                 }
             }
         }
@@ -158,11 +148,11 @@ chunk_ring_kernel(const CacheView c, const __grid_constant__ ChunkSeqs seqs, int
     }
     // the chunk's last min(m, w) tokens into the ring (the slots they take were read above)
     const int64_t n_win = m < c.window ? m : c.window;
-    for (int64_t i0 = group; i0 < n_win; i0 += 2 * kGroups) {
+    for (int64_t i0 = group; i0 < n_win; i0 += kRows * kGroups) {
         for (int u = gl; u < c.row_units; u += 16) {
-            uint4 kr[2], vr[2];
+            uint4 kr[kRows], vr[kRows];
 #pragma unroll
-            for (int j = 0; j < 2; ++j) {
+            for (int j = 0; j < kRows; ++j) {
                 const int64_t i = i0 + kGroups * j;
                 if (i < n_win) {
                     const int64_t src = (static_cast<int64_t>(h) * n_total + m - n_win + i) * c.row_units + u;
@@ -171,20 +161,39 @@ chunk_ring_kernel(const CacheView c, const __grid_constant__ ChunkSeqs seqs, int
                 }
             }
 #pragma unroll
-            for (int j = 0; j < 2; ++j) {
+            for (int j = 0; j < kRows; ++j) {
                 const int64_t i = i0 + kGroups * j;
                 if (i < n_win) {
-                    const int64_t ci = m - n_win + i;              // index inside the chunk
-                    const int64_t slot = li * c.window + (n_old + ci) % c.window;
+                    const int64_t slot = li * c.window + (n_old + m - n_win + i) % c.window;
                     c.k_ring[slot * c.row_units + u] = kr[j];
                     c.v_ring[slot * c.row_units + u] = vr[j];
-                    if (u == 0) c.score_ring[slot] = __ldcg(scores + ci * H + h);
                 }
             }
         }
     }
+    if (beside) griddep_wait();
+    griddep_launch_dependents();
+    // the chunk's own kept rows; the scores of those in the ring
+    {
+        const uint32_t *words = maskbits + static_cast<int64_t>(h) * n_words;
+        int cnt = 0;
+        for (int64_t wi = tok0 / 32 + tid; wi * 32 < tok0 + m; wi += kChunkThreads) {
+            uint32_t w = __ldcg(words + wi);
+            if (wi * 32 < tok0) w &= ~0u << static_cast<int>(tok0 - wi * 32);                    // bits below the chunk
+            if (wi * 32 + 32 > tok0 + m) w &= (1u << static_cast<int>(tok0 + m - wi * 32)) - 1u; // bits above it
+            cnt += __popc(w);
+        }
+        cnt = __reduce_add_sync(0xffffffffu, cnt);
+        if (lane == 0 && cnt) atomicAdd(&kept_s, cnt);
+    }
+    for (int64_t i = tid; i < n_win; i += kChunkThreads) {
+        const int64_t ci = m - n_win + i;                          // index inside the chunk
+        c.score_ring[li * c.window + (n_old + ci) % c.window] = __ldcg(scores + ci * H + h);
+    }
+    __syncthreads();
     if (tid == 0) {
         const int32_t len = static_cast<int32_t>(len_s);
+        if (seqs.n > 0 && h == 0) list_map[b] = list0;             // for the page assignment and the compaction
         list_base[b * H + h] = len;
         c.prefix_len[li] = len + kept_s;
         c.n_tokens[li] = static_cast<int32_t>(n_old + m);
@@ -193,10 +202,11 @@ chunk_ring_kernel(const CacheView c, const __grid_constant__ ChunkSeqs seqs, int
         last_s = atomicAdd(arrive, 1u) + 1u == gridDim.x * gridDim.y;
         if (last_s) *arrive = 0u;                                  // ready for the next launch
         __threadfence();
+        cursor_s = __ldcg(c.page_cursor);
     }
     __syncthreads();
     if (!last_s) return;
-    assign_pages<kChunkThreads>(H, gridDim.y, c.prefix_len, c.page_tokens, __ldcg(c.page_cursor), c.n_pages_pool, c.max_pages, list_page0,
+    assign_pages<kChunkThreads>(H, gridDim.y, c.prefix_len, c.page_tokens, cursor_s, c.n_pages_pool, c.max_pages, list_page0,
                                 c.page_table, nullptr, c.page_cursor, status, 1, list_base, c.free_stack, c.free_top, 1, list_map);
 }
 

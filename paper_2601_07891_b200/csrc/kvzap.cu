@@ -95,6 +95,7 @@ struct kvzap_ctx {
     float *split_part = nullptr;         // few-token kernel: [tile][slice][128][8] partial scores, tiles * slices <= sm_count
     uint64_t score_turn = 0;
     bool last_score_early = false;       // the last scoring launch was allowed to start early
+    bool last_score_late = false;        // ... lets the launch behind it start only when all work ahead of it has completed
     const void *last_scores = nullptr;   // scores buffer of the previous scoring launch, and its size
     size_t last_scores_bytes = 0;
     int32_t *list_page0 = nullptr;   // [max_seqs * H] first page of each list (paged output)
@@ -528,8 +529,9 @@ static kvzap_status launch_score(kvzap_ctx *ctx, int32_t layer, int32_t n_layers
                                  float tau, int32_t w, cudaStream_t stream, int32_t window_keep = 1,
                                  const DecodeFuse *fuse = nullptr, int *fused_layout = nullptr, const int *fuse_chain = nullptr,
                                  const CompactArgs *compact = nullptr, bool *compacted = nullptr,
-                                 bool fp8 = false, const float *x_scale = nullptr)
+                                 bool fp8 = false, const float *x_scale = nullptr, bool late_trigger = false)
 {
+    ctx->last_score_late = false;
     if (fused_layout) *fused_layout = -1;
     if (compacted) *compacted = false;
     // Early start.  When the grid fills the machine (one CTA per SM), this kernel is allowed to start
@@ -637,6 +639,8 @@ static kvzap_status launch_score(kvzap_ctx *ctx, int32_t layer, int32_t n_layers
                              p.n_tiles * n_ctas * 2 >= ctx->sm_count;
         const bool early = !ctx->profiling && ctx->weights_seq + 1 != ctx->op_seq;
         p.wait_before_load = ctx->trusted && (!fuse_ok || overlap) ? 0 : 1;
+        p.late_trigger = late_trigger && p.wait_before_load;
+        ctx->last_score_late = p.late_trigger != 0;
         ctx->last_score_early = early;
         {
             ProfScope prof(ctx, KVZAP_KERNEL_SCORE, stream);
@@ -1255,6 +1259,8 @@ kvzap_status kvzap_create(kvzap_ctx **out, const kvzap_config *cfg)
     CREATE_CUDA(cudaFuncSetAttribute(compact_dense_kernel<kDenseThreads, false>, cudaFuncAttributePreferredSharedMemoryCarveout,
                                      static_cast<int>(cudaSharedmemCarveoutMaxShared)));
     CREATE_CUDA(cudaFuncSetAttribute(compact_dense_kernel<kDenseThreadsShort, false>, cudaFuncAttributePreferredSharedMemoryCarveout,
+                                     static_cast<int>(cudaSharedmemCarveoutMaxShared)));
+    CREATE_CUDA(cudaFuncSetAttribute(chunk_ring_kernel, cudaFuncAttributePreferredSharedMemoryCarveout,
                                      static_cast<int>(cudaSharedmemCarveoutMaxShared)));
     CREATE_CUDA(cudaFuncSetAttribute(decode_update_kernel, cudaFuncAttributePreferredSharedMemoryCarveout,
                                      static_cast<int>(cudaSharedmemCarveoutMaxShared)));
@@ -2525,6 +2531,8 @@ static kvzap_status append_chunk(kvzap_ctx *ctx, kvzap_cache *cache, int32_t lay
         KVZAP_CUDA(ctx, cudaMemcpyAsync(ctx->batch_map, map.data(), sizeof(int64_t) * map.size(), cudaMemcpyHostToDevice, stream));
     }
     const int64_t n_words = (n_tokens + kBlockTokens - 1) / kBlockTokens * 4;
+    // directly behind a scoring launch that lets it start when all work ahead of that launch has completed
+    const bool beside = ctx->last_score_late && by_value.n > 0;
     if (v.window > 0) {
         cudaLaunchConfig_t cfg;
         cudaLaunchAttribute attrs[2];
@@ -2532,7 +2540,8 @@ static kvzap_status append_chunk(kvzap_ctx *ctx, kvzap_cache *cache, int32_t lay
                     !ctx->profiling, 1);
         KVZAP_CUDA(ctx, cudaLaunchKernelEx(&cfg, chunk_ring_kernel, v, by_value, static_cast<int>(layer), ctx->batch_map, scores,
                                            static_cast<const uint4 *>(K), static_cast<const uint4 *>(V), n_tokens, tau, cu_seqlens, mask,
-                                           n_words, ctx->list_base, ctx->list_page0, ctx->chunk_arrive, ctx->status_dev));
+                                           n_words, ctx->list_base, ctx->list_page0, ctx->chunk_arrive, ctx->status_dev,
+                                           beside ? 1 : 0));
     } else {
         tokens_add_kernel<<<static_cast<unsigned>(n_seqs), 32, 0, stream>>>(v, by_value, layer, ctx->batch_map, n_tokens, cu_seqlens);
         KVZAP_CUDA(ctx, cudaGetLastError());
@@ -2568,7 +2577,8 @@ kvzap_status kvzap_prefill_to_cache(kvzap_ctx *ctx, kvzap_cache *cache, int32_t 
     // prefix, the chunk's last tokens take their ring slots; then the chunk's kept tokens are appended
     // behind what the lists hold by then.
     uint32_t *mask = next_mask_slice(ctx);
-    st = launch_score(ctx, layer, 1, hidden, n_tokens, scores_out, mask, nullptr, 1, tau, v.window, stream, 0);
+    st = launch_score(ctx, layer, 1, hidden, n_tokens, scores_out, mask, nullptr, 1, tau, v.window, stream, 0, nullptr, nullptr, nullptr,
+                      nullptr, nullptr, false, nullptr, v.window > 0);
     if (st != KVZAP_OK) return st;
     return append_chunk(ctx, cache, layer, &seq, 1, nullptr, mask, scores_out, K, V, n_tokens, tau, stream);
 }
@@ -2606,7 +2616,8 @@ kvzap_status kvzap_prefill_to_cache_batch(kvzap_ctx *ctx, kvzap_cache *cache, in
         return fail(ctx, KVZAP_ERR_INVALID_ARG, "prefill_to_cache_batch: hidden, K, V, scores_out must be non-NULL, aligned");
     DeviceGuard guard(c.device);
     uint32_t *mask = next_mask_slice(ctx);
-    st = launch_score(ctx, layer, 1, hidden, n_tokens, scores_out, mask, cu_seqlens, n_seqs, tau, v.window, stream, 0);
+    st = launch_score(ctx, layer, 1, hidden, n_tokens, scores_out, mask, cu_seqlens, n_seqs, tau, v.window, stream, 0, nullptr, nullptr,
+                      nullptr, nullptr, nullptr, false, nullptr, v.window > 0);
     if (st != KVZAP_OK) return st;
     return append_chunk(ctx, cache, layer, seq_ids, n_seqs, cu_seqlens, mask, scores_out, K, V, n_tokens, tau, stream);
 }

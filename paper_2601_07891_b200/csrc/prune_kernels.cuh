@@ -147,33 +147,46 @@ assign_pages(int n_heads, int n_seqs, int32_t *__restrict__ lengths, int page_to
         total = warp_sums[31];
         return x + (warp > 0 ? warp_sums[warp - 1] : 0);
     };
-    // paged output: exclusive scan of the per-list page counts in (b,h) order
+    // paged output: exclusive scan of the per-list page counts in (b,h) order.  What a list's thread knows of it stays in
+    // shared memory for the table (of the first lists; the others are looked up again).
+    constexpr int kKnown = 128;
+    __shared__ int32_t s_page0[kKnown], s_have[kKnown], s_need[kKnown];
+    __shared__ int64_t s_list[kKnown];
+    int32_t n_free = 0;                                                 // asked for ahead of the scan
+    if (page_cursor != nullptr && free_top != nullptr) n_free = __ldcg(free_top);
     __syncthreads();
     if (tid == 0) { carry_s = 0; fail_s = 0; }
     __syncthreads();
     const int n_lists = n_heads * n_seqs;
     for (int base = 0; base < n_lists; base += NT) {
         const int idx = base + tid;
-        int32_t need = 0;
+        int32_t need = 0, have = 0;
+        int64_t li = 0;
         if (idx < n_lists) {
-            need = (__ldcg(lengths + list_at(list_map, idx, n_heads)) + page_tokens - 1) / page_tokens;
+            li = list_at(list_map, idx, n_heads);
+            need = (__ldcg(lengths + li) + page_tokens - 1) / page_tokens;
             if (need > max_pages) fail_s = 1;
-            if (append) need -= (__ldcg(list_base + idx) + page_tokens - 1) / page_tokens;     // pages the list already owns
+            if (append) have = (__ldcg(list_base + idx) + page_tokens - 1) / page_tokens;     // pages the list already owns
+            need -= have;
         }
         int32_t total;
         const int32_t incl = block_scan(need, total);
         const int32_t carry = carry_s;
-        if (idx < n_lists) list_page0[idx] = first_page + carry + incl - need;
+        if (idx < n_lists) {
+            list_page0[idx] = first_page + carry + incl - need;
+            if (idx < kKnown) {
+                s_page0[idx] = first_page + carry + incl - need;
+                s_have[idx] = have;
+                s_need[idx] = need;
+                s_list[idx] = li;
+            }
+        }
         __syncthreads();
         if (tid == 0) carry_s = carry + total;
         __syncthreads();
     }
     const int32_t used = carry_s;
-    int32_t n_free = 0;
-    if (page_cursor != nullptr && free_top != nullptr) {
-        n_free = __ldcg(free_top);
-        if (n_free < 0) n_free = 0;
-    }
+    if (n_free < 0) n_free = 0;
     const int32_t from_stack = used < n_free ? used : n_free;
     const bool fail = fail_s != 0 || static_cast<int64_t>(first_page) + (used - from_stack) > n_pages_pool;
     if (fail) {
@@ -196,10 +209,19 @@ assign_pages(int n_heads, int n_seqs, int32_t *__restrict__ lengths, int page_to
     __syncthreads();      // list_page0 and lengths of all lists are final
     if (!fill_table) return;
     for (int idx = warp; idx < n_lists; idx += NT / 32) {            // a warp per list
-        const int32_t p0 = list_page0[idx];
-        const int32_t have = append ? (__ldcg(list_base + idx) + page_tokens - 1) / page_tokens : 0;
-        const int64_t li = list_at(list_map, idx, n_heads);
-        const int32_t need = (__ldcg(lengths + li) + page_tokens - 1) / page_tokens - have;
+        int32_t p0, have, need;
+        int64_t li;
+        if (idx < kKnown) {
+            p0 = s_page0[idx];
+            have = s_have[idx];
+            need = s_need[idx];
+            li = s_list[idx];
+        } else {
+            p0 = list_page0[idx];
+            have = append ? (__ldcg(list_base + idx) + page_tokens - 1) / page_tokens : 0;
+            li = list_at(list_map, idx, n_heads);
+            need = (__ldcg(lengths + li) + page_tokens - 1) / page_tokens - have;
+        }
         for (int32_t i = lane; i < need; i += 32) {
             const int32_t j = p0 - first_page + i;            // ordinal among the pages assigned by this call
             page_table[li * max_pages + have + i] =

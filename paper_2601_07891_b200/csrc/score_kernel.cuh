@@ -76,6 +76,7 @@ struct ScoreParams {
     int32_t *status;      // device status word
     int32_t wait_before_write;    // 1: the epilogue waits for the kernel ahead in the stream before its first store
     int32_t wait_before_load;     // 1: every thread waits for the work ahead in the stream before caller data is read
+    int32_t late_trigger;         // few-token kernel: 1: the next launch may start once that wait is over (else at once)
     int32_t *tile_counter;        // work tiles handed out beyond the first one of every CTA (or pair); starts at 0
     int32_t *tile_counter_reset;  // the counter of the launch after next: set to 0 by this launch
     // 8-bit inputs (score_kernel<.., .., true>): hidden states and first-layer weights are E4M3 bytes, a 128-byte

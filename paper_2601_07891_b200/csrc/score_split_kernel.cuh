@@ -133,7 +133,7 @@ score_split_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_cons
             fuse_step = atomicAdd(f.ticket + ((layer * p.tiles_per_layer + m_tile) * n_split + nh) * k_split + kh, 1);
         __syncthreads();
     }
-    griddep_launch_dependents();
+    if (!p.late_trigger) griddep_launch_dependents();
     const int own_n = ns / k_split;                      // accumulator columns this CTA finishes
     const int own_c0 = kh * own_n;                       // the first of them
     const int j_first = nh * ns + own_c0;                // = first hidden unit of this CTA
@@ -179,6 +179,7 @@ score_split_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_cons
     // unless the caller vouches for the producers of its inputs, nothing of them is read before the work
     // ahead in the stream has completed (every thread waits: the loads below are issued by several warps)
     if (p.wait_before_load) griddep_wait();
+    if (p.late_trigger) griddep_launch_dependents();     // whatever starts now finds all work ahead of this launch complete
     if (warp == 0) {
         __syncwarp();
         if (elect_one())
