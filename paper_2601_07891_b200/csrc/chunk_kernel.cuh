@@ -206,7 +206,7 @@ chunk_ring_kernel(const CacheView c, const __grid_constant__ ChunkSeqs seqs, int
     }
     __syncthreads();
     if (!last_s) return;
-    assign_pages<kChunkThreads>(H, gridDim.y, c.prefix_len, c.page_tokens, cursor_s, c.n_pages_pool, c.max_pages, list_page0,
+    assign_pages<kChunkThreads, 128>(H, gridDim.y, c.prefix_len, c.page_tokens, cursor_s, c.n_pages_pool, c.max_pages, list_page0,
                                 c.page_table, nullptr, c.page_cursor, status, 1, list_base, c.free_stack, c.free_top, 1, list_map);
 }
 

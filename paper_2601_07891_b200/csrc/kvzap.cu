@@ -997,7 +997,7 @@ static kvzap_status launch_compaction(kvzap_ctx *ctx, const uint32_t *mask, cons
                                            tok_major ? int64_t{1} : n_tokens,
                                            tok_major ? static_cast<int64_t>(c.n_kv_heads) : int64_t{1},
                                            static_cast<const int32_t *>(nullptr), static_cast<const int32_t *>(nullptr), 0,
-                                           static_cast<const int64_t *>(nullptr)));
+                                           static_cast<const int64_t *>(nullptr), PageAssign{}));
     }
     ctx->launches += 1;
     return KVZAP_OK;
@@ -1961,7 +1961,19 @@ static kvzap_status launch_compaction_paged(kvzap_ctx *ctx, const uint32_t *mask
     const kvzap_config &c = ctx->cfg;
     const int64_t n_blocks = (n_tokens + kBlockTokens - 1) / kBlockTokens;
     const int64_t n_words = n_blocks * 4;
-    if (!pages_assigned) {
+    PageAssign assign;
+    memset(&assign, 0, sizeof assign);
+    if (!append && page_cursor == nullptr && n_words * c.n_kv_heads <= kAssignWords &&
+        static_cast<int64_t>(n_seqs) * c.n_kv_heads <= kAssignLists) {
+        assign.enabled = 1;
+        assign.first_page = first_page;
+        assign.max_pages = max_pages;
+        assign.n_pages_pool = n_pages_pool;
+        assign.page_table = page_table;
+        assign.n_pages_used = n_pages_used;
+        assign.status = ctx->status_dev;
+    }
+    if (!pages_assigned && !assign.enabled) {
         cudaLaunchConfig_t cfg;
         cudaLaunchAttribute attrs[2];
         // lengths and the first page of every list (the only step that needs all lists at once)
@@ -1987,7 +1999,7 @@ static kvzap_status launch_compaction_paged(kvzap_ctx *ctx, const uint32_t *mask
                                            tok_major ? int64_t{1} : n_tokens,
                                            tok_major ? static_cast<int64_t>(c.n_kv_heads) : int64_t{1},
                                            static_cast<const int32_t *>(append ? ctx->list_base : nullptr),
-                                           static_cast<const int32_t *>(page_table), static_cast<int>(max_pages), list_map));
+                                           static_cast<const int32_t *>(page_table), static_cast<int>(max_pages), list_map, assign));
     }
     ctx->launches += 1;
     return KVZAP_OK;

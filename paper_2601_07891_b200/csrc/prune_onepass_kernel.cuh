@@ -288,7 +288,7 @@ prune_onepass_kernel(const PruneParams p)
                 p.len_acc[idx] = 0;
             }
             __syncthreads();
-            assign_pages<kOpThreads>(H, p.n_seqs, p.lengths, p.page_tokens, p.first_page, p.n_pages_pool, p.max_pages,
+            assign_pages<kOpThreads, 0>(H, p.n_seqs, p.lengths, p.page_tokens, p.first_page, p.n_pages_pool, p.max_pages,
                                      p.list_page0, p.page_table, p.n_pages_used, nullptr, p.status, 0, nullptr, nullptr,
                                      nullptr, 0);
             __threadfence();
