@@ -87,7 +87,9 @@ struct kvzap_ctx {
     uint32_t *maskbits = nullptr;    // [kMaskRing][H][max_words]: consecutive calls use different slices
     uint64_t mask_turn = 0;
     int32_t *tile_counters = nullptr;    // [kMaskRing] work-tile counters of the scoring launches, used in rotation
-    uint32_t *select_hist = nullptr;     // fixed-budget selection: [4 passes][max_seqs][H][256] histograms
+    uint32_t *select_hist = nullptr;     // fixed-budget selection: [passes][max_seqs][H][bins] histograms, zero between calls
+    bool select_clean = false;           //                         ... as far as the host knows
+    uint32_t *select_arrive = nullptr;   //                         [max_seqs][H] CTAs that are done, zero between launches
     float *select_tau = nullptr;         //                         [max_seqs][H] cut values when the caller wants none
     float *plan_scores = nullptr;        // kvzap_prefill_plan without scores_out: [max_tokens][H] (allocated on first use)
     int64_t *batch_map = nullptr;        // chunks into a cache: first list of each sequence of the call [max_seqs]
@@ -136,9 +138,9 @@ struct kvzap_ctx {
     std::vector<kvzap_cache *> caches;              // caches created on this context (their step counters are
                                                     // cleared when a timeout has been polled)
     // one-launch pruning (kvzap_prune_prefill and its paged / fixed-budget forms): kOpRing scratch sets in rotation
-    int op_capacity = 0;                 // CTAs of prune_onepass_kernel the device holds at once
+    int op_capacity = 0;                 // half of the CTAs of prune_onepass_kernel that the device holds at once
     uint32_t *op_mask = nullptr;         // [kOpRing][H][max_words]
-    uint64_t *op_counts = nullptr;       // [kOpRing][op_capacity][8]
+    uint64_t *op_counts = nullptr;       // [kOpRing][2 * op_capacity][8]
     int32_t *op_len_acc = nullptr;       // [kOpRing][max_seqs * H], zero between calls
     uint32_t *op_arrive = nullptr;       // [kOpRing]
     int32_t *op_scan_flag = nullptr;     // [kOpRing]
@@ -408,6 +410,7 @@ static void free_all(kvzap_ctx *ctx)
     cudaFree(ctx->chunk_arrive);
     cudaFree(ctx->select_hist);
     cudaFree(ctx->select_tau);
+    cudaFree(ctx->select_arrive);
     for (auto &l : ctx->layouts) cudaFree(l.arrive);
     cudaFree(ctx->list_page0);
     cudaFree(ctx->list_base);
@@ -460,6 +463,11 @@ static kvzap_status hidden_tmap(kvzap_ctx *ctx, CUtensorMap *out, const void *ba
     else { ctx->tmap_cache[ctx->tmap_next] = e; ctx->tmap_next = (ctx->tmap_next + 1) % kEntries; }
     *out = e.map;
     return KVZAP_OK;
+}
+
+static size_t select_hist_bytes(const kvzap_config &c)
+{
+    return sizeof(uint32_t) * kSelectPasses * static_cast<size_t>(c.max_seqs) * c.n_kv_heads * kSelectBins;
 }
 
 static uint32_t *next_mask_slice(kvzap_ctx *ctx)
@@ -1011,27 +1019,12 @@ static kvzap_status launch_prune_onepass(kvzap_ctx *ctx, const float *scores, co
                                          int64_t n_tokens, void *K_out, void *V_out, int32_t *lengths, int32_t page_tokens,
                                          int32_t first_page, int64_t n_pages_pool, int32_t max_pages, int32_t *page_table,
                                          int32_t *n_pages_used, cudaStream_t stream, int32_t *slot_out = nullptr,
-                                         bool scores_just_made = false)
+                                         bool scores_just_made = false, uint32_t *clear = nullptr, int64_t clear_words = 0)
 {
     const kvzap_config &c = ctx->cfg;
     if (page_tokens > 0 && n_pages_pool * page_tokens >= 0xffffffffLL)
         return fail(ctx, KVZAP_ERR_UNSUPPORTED, "paged pruning: the pool must hold fewer than 2^32 - 1 rows");
     const int64_t n_blocks = (n_tokens + kBlockTokens - 1) / kBlockTokens;
-    // Heads per CTA: as many as still leave a CTA a dozen blocks or more.  The one CTA that holds a sequence's window
-    // keeps all rows of a block where the others keep a quarter or a third; with many blocks per CTA that is a small
-    // surplus, with two or three it would make that CTA the last to finish by far.
-    int heads_per_cta = kMaxHeads, groups = 1;
-    int64_t grid = 1, per_cta = n_blocks;
-    for (int hg = kMaxHeads; hg >= 1; hg >>= 1) {
-        heads_per_cta = hg;
-        groups = (c.n_kv_heads + hg - 1) / hg;
-        grid = ctx->op_capacity / groups;
-        if (grid < 1) grid = 1;
-        if (grid > n_blocks) grid = n_blocks;
-        per_cta = (n_blocks + grid - 1) / grid;
-        grid = (n_blocks + per_cta - 1) / per_cta;
-        if (per_cta >= 12) break;
-    }
     const int set = static_cast<int>(ctx->op_turn % kOpRing);
     ctx->op_turn += 1;
     ctx->op_epoch = ctx->op_epoch == 0x7fffffff ? 1 : ctx->op_epoch + 1;
@@ -1066,9 +1059,29 @@ static kvzap_status launch_prune_onepass(kvzap_ctx *ctx, const float *scores, co
         note_range(ctx, page_table, sizeof(int32_t) * n_lists * max_pages, true);
         note_range(ctx, n_pages_used, sizeof(int32_t), true);
     }
+    // A launch that waits for the work ahead takes every slot of the device (32k tokens, a quarter kept: 40 -> 31 us); one
+    // that may run beside the launch ahead (and the one behind it beside this one) half of them, and so does the paged
+    // output, whose CTAs all wait for one another: two such launches on two streams still fit side by side.
+    // Heads per CTA: as many as still leave a CTA a dozen blocks or more.  The one CTA that holds a sequence's window
+    // keeps all rows of a block where the others keep a quarter or a third; with many blocks per CTA that is a small
+    // surplus, with two or three it would make that CTA the last to finish by far.
+    int heads_per_cta = kMaxHeads, groups = 1;
+    int64_t grid = 1, per_cta = n_blocks;
+    for (int hg = kMaxHeads; hg >= 1; hg >>= 1) {
+        heads_per_cta = hg;
+        groups = (c.n_kv_heads + hg - 1) / hg;
+        grid = ctx->op_capacity * (wait_first && page_tokens == 0 ? 2 : 1) / groups;
+        if (grid < 1) grid = 1;
+        if (grid > n_blocks) grid = n_blocks;
+        per_cta = (n_blocks + grid - 1) / grid;
+        grid = (n_blocks + per_cta - 1) / per_cta;
+        if (per_cta >= 12) break;
+    }
     PruneParams p;
     memset(&p, 0, sizeof p);
     p.scores = scores;
+    p.clear = reinterpret_cast<uint4 *>(clear);
+    p.clear_units = clear_words / 4;
     p.tau_list = tau_list;
     p.tau = tau;
     p.window = w;
@@ -1080,6 +1093,7 @@ static kvzap_status launch_prune_onepass(kvzap_ctx *ctx, const float *scores, co
     p.cu_seqlens = cu_seqlens;
     p.blocks_per_cta = static_cast<int32_t>(per_cta);
     p.heads_per_cta = heads_per_cta;
+    p.recount = page_tokens == 0 && heads_per_cta == 1 && n_blocks <= kOpRecountBlocks ? 1 : 0;
     p.K = static_cast<const uint4 *>(K);
     p.V = static_cast<const uint4 *>(V);
     p.K_out = static_cast<uint4 *>(K_out);
@@ -1098,7 +1112,7 @@ static kvzap_status launch_prune_onepass(kvzap_ctx *ctx, const float *scores, co
     p.n_pages_used = n_pages_used;
     p.status = ctx->status_dev;
     p.maskbits = ctx->op_mask + static_cast<size_t>(set) * ctx->max_words * c.n_kv_heads;
-    p.cta_counts = ctx->op_counts + static_cast<size_t>(set) * ctx->op_capacity * kMaxHeads;
+    p.cta_counts = ctx->op_counts + static_cast<size_t>(set) * 2 * ctx->op_capacity * kMaxHeads;
     p.len_acc = ctx->op_len_acc + static_cast<size_t>(set) * c.max_seqs * c.n_kv_heads;
     p.arrive = ctx->op_arrive + set;
     p.scan_flag = ctx->op_scan_flag + set;
@@ -1354,7 +1368,9 @@ kvzap_status kvzap_create(kvzap_ctx **out, const kvzap_config *cfg)
     CREATE_CUDA(cudaMemset(ctx->chunk_arrive, 0, sizeof(uint32_t)));
     CREATE_CUDA(cudaMalloc(&ctx->tile_counters, sizeof(int32_t) * kMaskRing));
     CREATE_CUDA(cudaMemset(ctx->tile_counters, 0, sizeof(int32_t) * kMaskRing));
-    CREATE_CUDA(cudaMalloc(&ctx->select_hist, sizeof(uint32_t) * 4 * static_cast<size_t>(c.max_seqs) * c.n_kv_heads * 256));
+    CREATE_CUDA(cudaMalloc(&ctx->select_hist, select_hist_bytes(c)));
+    CREATE_CUDA(cudaMalloc(&ctx->select_arrive, sizeof(uint32_t) * static_cast<size_t>(c.max_seqs) * c.n_kv_heads));
+    CREATE_CUDA(cudaMemset(ctx->select_arrive, 0, sizeof(uint32_t) * static_cast<size_t>(c.max_seqs) * c.n_kv_heads));
     CREATE_CUDA(cudaMalloc(&ctx->select_tau, sizeof(float) * static_cast<size_t>(c.max_seqs) * c.n_kv_heads));
     if (ctx->n_layouts > 0)
         CREATE_CUDA(cudaMalloc(&ctx->split_part, sizeof(float) * static_cast<size_t>(ctx->sm_count) * kTileM * kMaxHeads));
@@ -1371,7 +1387,7 @@ kvzap_status kvzap_create(kvzap_ctx **out, const kvzap_config *cfg)
         // half of what fits: the next call's kernel then finds room beside this one
         ctx->op_capacity = per_sm * ctx->sm_count / 2;
         if (ctx->op_capacity < 1) ctx->op_capacity = 1;
-        const size_t cap = static_cast<size_t>(ctx->op_capacity);
+        const size_t cap = 2 * static_cast<size_t>(ctx->op_capacity);
         CREATE_CUDA(cudaMalloc(&ctx->op_mask, sizeof(uint32_t) * kOpRing * ctx->max_words * c.n_kv_heads));
         CREATE_CUDA(cudaMalloc(&ctx->op_counts, sizeof(uint64_t) * kOpRing * cap * kMaxHeads));
         CREATE_CUDA(cudaMemset(ctx->op_counts, 0, sizeof(uint64_t) * kOpRing * cap * kMaxHeads));
@@ -1643,26 +1659,25 @@ kvzap_status kvzap_prune_prefill_topk(kvzap_ctx *ctx, const void *K, const void 
     if (st != KVZAP_OK) return st;
     if (!scores) return fail(ctx, KVZAP_ERR_INVALID_ARG, "scores is NULL");
     const int n_sel = per_layer ? 1 : c.n_kv_heads;
-    KVZAP_CUDA(ctx, cudaMemsetAsync(ctx->select_hist, 0, sizeof(uint32_t) * 4 * static_cast<size_t>(n_seqs) * n_sel * 256, stream));
-    const dim3 grid(static_cast<unsigned>((n_tokens + kSelectThreads - 1) / kSelectThreads), static_cast<unsigned>(n_seqs));
-    const bool early = !ctx->profiling;
-    cudaLaunchConfig_t cfg;
-    cudaLaunchAttribute attrs[2];
-    for (int pass = 0; pass < 4; ++pass) {
-        make_launch(&cfg, attrs, grid, dim3(kSelectThreads), 0, stream, early, 1);
-        KVZAP_CUDA(ctx, cudaLaunchKernelEx(&cfg, select_hist_kernel, scores, n_tokens, static_cast<int>(c.n_kv_heads), cu_seqlens,
+    if (!ctx->select_clean) KVZAP_CUDA(ctx, cudaMemsetAsync(ctx->select_hist, 0, select_hist_bytes(c), stream));
+    ctx->select_clean = false;               // until the launch that clears them is in the stream
+    const dim3 grid(static_cast<unsigned>((n_tokens + kSelectTokens - 1) / kSelectTokens), static_cast<unsigned>(c.n_kv_heads),
+                    static_cast<unsigned>(n_seqs));
+    for (int pass = 0; pass < kSelectPasses; ++pass) {
+        cudaLaunchConfig_t cfg;
+        cudaLaunchAttribute attrs[2];
+        make_launch(&cfg, attrs, grid, dim3(kSelectThreads), 0, stream, !ctx->profiling, 1);
+        KVZAP_CUDA(ctx, cudaLaunchKernelEx(&cfg, select_pass_kernel, scores, n_tokens, static_cast<int>(c.n_kv_heads), cu_seqlens,
                                            static_cast<int>(n_seqs), static_cast<int>(w), keep_ratio, per_layer ? 1 : 0, pass,
-                                           ctx->select_hist));
+                                           ctx->select_hist, ctx->select_arrive, tau_list, ctx->status_dev));
+        ctx->launches += 1;
     }
-    make_launch(&cfg, attrs, dim3(static_cast<unsigned>(n_seqs)), dim3(kSelectThreads), 0, stream, early, 1);
-    KVZAP_CUDA(ctx, cudaLaunchKernelEx(&cfg, select_finish_kernel, n_tokens, static_cast<int>(c.n_kv_heads), cu_seqlens,
-                                       static_cast<int>(n_seqs), static_cast<int>(w), keep_ratio, per_layer ? 1 : 0,
-                                       static_cast<const uint32_t *>(ctx->select_hist), tau_list, ctx->status_dev));
-    KVZAP_CUDA(ctx, cudaGetLastError());
-    ctx->launches += 5;
     // the same mask + compaction launch as kvzap_prune_prefill, with the cut values as per-list thresholds
-    return launch_prune_onepass(ctx, scores, tau_list, 0.0f, w, K, V, cu_seqlens, n_seqs, n_tokens, K_out, V_out, lengths, 0,
-                                0, 0, 0, nullptr, nullptr, stream);
+    st = launch_prune_onepass(ctx, scores, tau_list, 0.0f, w, K, V, cu_seqlens, n_seqs, n_tokens, K_out, V_out, lengths, 0,
+                              0, 0, 0, nullptr, nullptr, stream, nullptr, false, ctx->select_hist,
+                              static_cast<int64_t>(kSelectPasses) * n_seqs * n_sel * kSelectBins);
+    ctx->select_clean = st == KVZAP_OK;
+    return st;
 }
 
 // tok_major: K and V are [n_tokens][H][D] (the K/V projection's output) instead of [H][n_tokens][D]
@@ -1770,6 +1785,7 @@ kvzap_status kvzap_poll_status(kvzap_ctx *ctx, void *stream_)
         // a one-launch pruning call that gave up may have left its list-length sums and arrival count behind
         cudaMemsetAsync(ctx->op_len_acc, 0, sizeof(int32_t) * kOpRing * static_cast<size_t>(ctx->cfg.max_seqs) * ctx->cfg.n_kv_heads, stream);
         cudaMemsetAsync(ctx->op_arrive, 0, sizeof(uint32_t) * kOpRing, stream);
+        ctx->select_clean = false;
     }
     cudaStreamSynchronize(stream);
     fail(ctx, static_cast<kvzap_status>(v), "device-side condition %d recorded", v);

@@ -12,7 +12,8 @@
 //   B. rows kept before the CTA's first token = sum of the counts of all CTAs before it (one poll loop
 //      per earlier CTA, all in parallel).  When the sequence in progress at the CTA's first token began
 //      inside an earlier CTA's run of blocks, the rows that CTA kept before that start are recounted from
-//      the scores (no CTA reads another's mask).  Paged output needs the lengths of ALL lists before any
+//      the scores (no CTA reads another's mask).  On a short dense input all of it is recounted and no CTA waits for
+//      another (p.recount: 3 x 500 tokens 11.1 -> 8.9 us per call).  Paged output needs the lengths of ALL lists before any
 //      row can be placed: every CTA adds its counts to the lists' lengths (atomics), the CTA that arrives
 //      last assigns the pages and publishes a flag that all wait for; the page table is filled by all.
 //   C. four blocks at a time: rank of every kept (token, head) by popc and its source and destination as
@@ -35,6 +36,7 @@ constexpr int kOpSmemWords = 256;      // (block, head) pairs of a CTA whose mas
 // shared memory the kernel needs, and the smaller it is the more L1 is left for rows in flight: measured at 128k
 // tokens, paged output, a third of the rows kept: 72.5 us per call with 32 pairs, 69.2 with 16, 66.3 with 8.
 constexpr int kOpPairs = 8;
+constexpr int kOpRecountBlocks = 17;   // p.recount up to this many blocks: at most 16 * 128 scores before a CTA, 8 per thread
 constexpr int kOpRing = 16;            // scratch sets used in rotation by consecutive calls
 constexpr int kOpRows = 4;             // rows of K and of V per register set of a 16-lane group (two sets in rotation)
 // dynamic shared memory: the list of kept rows of kOpPairs (block, head) pairs, rounded up to whole rounds of the move loop
@@ -73,6 +75,10 @@ struct PruneParams {
     int32_t *scan_flag;        // paged: the call's number once the page assignment is there
     int32_t epoch;             // the call's number, never 0
     int64_t wait_limit;
+    uint4 *clear;              // scratch of the selection ahead (fixed budget) to be zero for the next one, clear_units of it
+    int64_t clear_units;
+    int32_t recount;           // 1: short dense input, one head per CTA: rows kept before the CTA's first token are counted
+                               // from the scores, not learnt from the CTAs before it
     int32_t wait_first;        // 1: wait for the work ahead in the stream before the first load
 };
 
@@ -135,14 +141,16 @@ __device__ __forceinline__ void load_token(const PruneParams &p, int64_t word, i
     ts.in_window = t >= seq_end - static_cast<int64_t>(p.window);
 }
 // Keep bits of the word's 32 tokens (whole warp): lane h returns head h's word.
-__device__ __forceinline__ uint32_t keep_word(const PruneParams &p, const TokenScores &ts, int lane)
+// tau_lo: the thresholds of sequence b_lo, in shared memory -- read from global memory by every word of every CTA they
+// all came from one 32-byte sector of L2, and at 32k tokens this phase took 13.5 us instead of 3.
+__device__ __forceinline__ uint32_t keep_word(const PruneParams &p, const TokenScores &ts, int lane, const float *tau_lo, int b_lo)
 {
     const int H = p.n_heads;
     const bool valid = ts.b >= 0;
     float tau_h[kMaxHeads];
 #pragma unroll
-    for (int h = 0; h < kMaxHeads; ++h) tau_h[h] = p.tau;
-    if (p.tau_list != nullptr && valid) {
+    for (int h = 0; h < kMaxHeads; ++h) tau_h[h] = tau_lo[h];
+    if (p.tau_list != nullptr && valid && ts.b != b_lo) {
 #pragma unroll
         for (int h = 0; h < kMaxHeads; ++h)
             if (h < H) tau_h[h] = __ldcg(p.tau_list + ts.b * H + h);
@@ -178,6 +186,7 @@ prune_onepass_kernel(const PruneParams p)
     __shared__ int32_t runb_s[kOpPairs + kMaxHeads];    // rows of that head kept before that block; last row: after all of them
     __shared__ int32_t off_s[kOpPairs + 1];
     __shared__ int flag_s;
+    __shared__ float tau_s[kMaxHeads];                  // thresholds of the sequence at the CTA's first token
 
     griddep_launch_dependents();
     if (p.wait_first) griddep_wait();
@@ -207,6 +216,7 @@ prune_onepass_kernel(const PruneParams p)
         b_hi = seq_of_token(p.cu_seqlens, p.n_seqs, t_last);
         s0 = p.cu_seqlens[b_lo];
     }
+    if (tid < kMaxHeads) tau_s[tid] = p.tau_list != nullptr && tid < H ? __ldcg(p.tau_list + b_lo * H + tid) : p.tau;
     const int j0 = static_cast<int>((s0 / kBlockTokens) / p.blocks_per_cta);      // the CTA (column) whose blocks hold s0
     __syncthreads();
 
@@ -226,7 +236,7 @@ prune_onepass_kernel(const PruneParams p)
             for (int u = 0; u < kUnroll; ++u) {
                 const int wl = w0 + u * (kOpThreads / 32);
                 if (wl >= n_w) break;
-                const uint32_t my_word = keep_word(p, ts[u], lane);
+                const uint32_t my_word = keep_word(p, ts[u], lane, tau_s, b_lo);
                 const int bl = wl >> 2, q = wl & 3;
                 if (own(lane)) {
                     if (bl < smem_blocks) reinterpret_cast<uint32_t *>(&words_s[bl * HG + lane - h0])[q] = my_word;
@@ -247,15 +257,33 @@ prune_onepass_kernel(const PruneParams p)
             }
         }
         if (own(lane) && my_cnt) atomicAdd(&cnt_s[lane], my_cnt);
+        if (p.recount) {
+            // rows of the sequence in progress that are kept before this CTA's first token, one head: with few blocks
+            // these scores cost no more than a round trip, asked for beside the CTA's own, and no CTA waits for another
+            const int64_t w0 = (multi ? static_cast<int64_t>(p.cu_seqlens[b_lo + 1]) : p.n_tokens) - p.window;
+            int32_t before = 0;
+            for (int64_t t = s0 + tid; t < t0; t += 8 * kOpThreads) {
+                float v[8];
+#pragma unroll
+                for (int u = 0; u < 8; ++u) v[u] = t + u * kOpThreads < t0 ? __ldcg(p.scores + (t + u * kOpThreads) * H + h0) : 0.0f;
+#pragma unroll
+                for (int u = 0; u < 8; ++u) {
+                    const int64_t tu = t + u * kOpThreads;
+                    if (tu < t0 && (tu >= w0 || v[u] >= tau_s[h0])) ++before;
+                }
+            }
+            before = __reduce_add_sync(0xffffffffu, before);
+            if (lane == 0 && before) atomicAdd(&part_s[h0], before);
+        }
         // The sequence in progress at this CTA's first token began inside CTA j0's blocks: the rows CTA j0 kept
         // from that start to the end of its blocks are recounted here (all of them belong to that sequence).
-        if (multi && j0 < c) {
+        if (multi && j0 < c && !p.recount) {
             const int64_t end = static_cast<int64_t>(j0 + 1) * p.blocks_per_cta * kBlockTokens;
             int32_t extra = 0;
             for (int64_t word = s0 / 32 + warp; word * 32 < end; word += kOpThreads / 32) {
                 TokenScores ts;
                 load_token(p, word, lane, multi, ts);
-                uint32_t w = keep_word(p, ts, lane);
+                uint32_t w = keep_word(p, ts, lane, tau_s, b_lo);
                 if (word * 32 < s0) w &= ~0u << static_cast<int>(s0 - word * 32);       // bits of the sequence before
                 extra += __popc(w);
             }
@@ -263,7 +291,7 @@ prune_onepass_kernel(const PruneParams p)
         }
     }
     __syncthreads();
-    if (tid < kMaxHeads && own(tid)) st_relaxed_gpu_u64(p.cta_counts + c * kMaxHeads + tid, tag | static_cast<uint32_t>(cnt_s[tid]));
+    if (!p.recount && tid < kMaxHeads && own(tid)) st_relaxed_gpu_u64(p.cta_counts + c * kMaxHeads + tid, tag | static_cast<uint32_t>(cnt_s[tid]));
     if (paged) {
         if (b_lo == b_hi && tid < kMaxHeads && own(tid) && cnt_s[tid]) atomicAdd(p.len_acc + b_lo * H + tid, cnt_s[tid]);
         __threadfence();
@@ -320,7 +348,9 @@ prune_onepass_kernel(const PruneParams p)
     // ---------------------------------------------------------------- B: rows kept before this CTA's first token
     // run_s[h]: kept rows of head h before the current block; base_s[h]: before the start of the sequence that
     // is in progress at the current block's first token
-    {
+    if (p.recount) {
+        if (tid < kMaxHeads) { run_s[tid] = part_s[tid]; base_s[tid] = 0; }      // counted from the start of that sequence
+    } else {
         int32_t acc[2 * kMaxHeads];
 #pragma unroll
         for (int i = 0; i < 2 * kMaxHeads; ++i) acc[i] = 0;
@@ -559,6 +589,10 @@ prune_onepass_kernel(const PruneParams p)
         __syncthreads();
     }
     griddep_wait();        // every thread: this kernel completes after the one ahead of it
+    if (p.clear != nullptr)
+        for (int64_t i = (static_cast<int64_t>(g) * gridDim.x + c) * kOpThreads + tid; i < p.clear_units;
+             i += static_cast<int64_t>(gridDim.x) * gridDim.y * kOpThreads)
+            p.clear[i] = make_uint4(0u, 0u, 0u, 0u);
 }
 
 }  // namespace kvzap

@@ -5,18 +5,30 @@
 // compaction with that per-list threshold.  Candidates are the positions outside the window; scores
 // equal to the cut value are all kept; NaN scores are never candidates.
 //
-// The cut value comes from a radix select over order-preserving 32-bit keys, 8 bits per pass:
-// pass p histograms the byte p (from the top) of every candidate key that matches the bytes already
-// fixed.  Histograms of all four passes live in global memory (zeroed by the host before the first
-// pass); each CTA re-derives the bytes fixed so far from the earlier passes' histograms (at most three
-// 256-bin scans), so a pass is one launch and no kernel ever waits for another.
+// The cut value comes from a radix select over order-preserving 32-bit keys in three passes of 11, 11 and
+// 10 bits: pass p histograms the p-th digit (from the top) of every candidate key that matches the digits
+// already fixed.  Histograms of all passes live in global memory; they are zero between calls (the
+// compaction that follows the selection clears them).  Each CTA re-derives the digits fixed so far from
+// the earlier passes' histograms, so a pass is one launch and no kernel waits for another; in the last
+// pass the CTA of a selection that is done last finishes it and writes the cut value.
+// What bounds it is the latency of that chain of dependent launches, so there are as few of them as
+// possible, a CTA counts one head only (2048 bins instead of 8 x 256 of four passes), and the scores of a
+// later pass are loaded before the wait for the pass ahead.  32k tokens x 8 heads, from the first launch to
+// the cut values: 35.5 us with four passes of 8 bits, a memset ahead and a launch for the cut values
+// behind them, 17.6 us now.
 #pragma once
 
 #include "score_kernel.cuh"
 
 namespace kvzap {
 
-constexpr int kSelectThreads = 256;      // 8 warps: warp i derives the state of head i
+constexpr int kSelectThreads = 256;
+constexpr int kSelectTokens = 4 * kSelectThreads;      // tokens of a CTA, one head
+constexpr int kSelectPasses = 3;
+constexpr int kSelectBins = 2048;                      // bins stored per pass (the last pass uses half of them)
+
+__host__ __device__ constexpr int select_shift(int pass) { return pass == 0 ? 21 : pass == 1 ? 10 : 0; }
+__host__ __device__ constexpr int select_bits(int pass) { return pass == 2 ? 10 : 11; }
 
 // larger score <-> larger key; -0 sorts below +0, NaN is never turned into a key
 __device__ __forceinline__ uint32_t score_key(float v)
@@ -29,60 +41,59 @@ __device__ __forceinline__ float key_score(uint32_t k)
     return __uint_as_float((k & 0x80000000u) ? (k & 0x7fffffffu) : ~k);
 }
 
-// Whole warp: walking the 256 bins from the top, the bin that holds the k-th key (k >= 1); `above` =
-// keys in higher bins.  Returns 256 when all bins together hold fewer than k keys.
-__device__ __forceinline__ uint32_t select_bin(const uint32_t *hist, uint32_t k, uint32_t &above, int lane)
+// The bins of one selection and pass that a thread looks after: 8 consecutive ones (all 2048 by the CTA; the upper
+// half is zero in the last pass).
+struct SelectBins {
+    uint32_t c[8];
+};
+__device__ __forceinline__ SelectBins load_bins(const uint32_t *hist)
 {
-    uint32_t c[8], mine = 0;
+    SelectBins b;
+    const uint4 x = __ldcg(reinterpret_cast<const uint4 *>(hist) + 2 * threadIdx.x);
+    const uint4 y = __ldcg(reinterpret_cast<const uint4 *>(hist) + 2 * threadIdx.x + 1);
+    b.c[0] = x.x; b.c[1] = x.y; b.c[2] = x.z; b.c[3] = x.w;
+    b.c[4] = y.x; b.c[5] = y.y; b.c[6] = y.z; b.c[7] = y.w;
+    return b;
+}
+
+// Whole CTA: walking the bins from the top, the one that holds the k-th key (k >= 1); `above` = keys in higher bins.
+// Returns kSelectBins when all bins together hold fewer than k keys.  `scratch`: kSelectThreads / 32 + 2 words.
+__device__ __forceinline__ uint32_t select_bin(const SelectBins &b, uint32_t k, uint32_t &above, uint32_t *scratch)
+{
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    constexpr int kWarps = kSelectThreads / 32;
+    uint32_t mine = 0;
 #pragma unroll
-    for (int i = 0; i < 8; ++i) {
-        c[i] = __ldcg(hist + 8 * lane + i);
-        mine += c[i];
-    }
-    uint32_t incl = mine;                 // becomes the count in this lane's bins and all higher lanes'
+    for (int i = 0; i < 8; ++i) mine += b.c[i];
+    uint32_t incl = mine;                 // becomes the count in this thread's bins and those of all higher lanes
 #pragma unroll
     for (int o = 1; o < 32; o <<= 1) {
         const uint32_t y = __shfl_down_sync(0xffffffffu, incl, o);
         if (lane + o < 32) incl += y;
     }
-    const uint32_t higher = incl - mine;
-    uint32_t bin = 256u, ab = 0u;
-    if (higher < k && k <= incl) {
-        uint32_t run = higher;
+    __syncthreads();                      // scratch may still be read by the selection before
+    if (lane == 0) scratch[warp] = incl;
+    if (threadIdx.x == 0) scratch[kWarps] = kSelectBins;
+    __syncthreads();
+    uint32_t higher = incl - mine;
+#pragma unroll
+    for (int w = 0; w < kWarps; ++w)
+        if (w > warp) higher += scratch[w];
+    if (higher < k && k <= higher + mine) {              // exactly one thread, if any
+        uint32_t run = higher, bin = kSelectBins, ab = 0u;
 #pragma unroll
         for (int i = 7; i >= 0; --i) {
-            if (bin == 256u) {
-                if (run + c[i] >= k) { bin = 8u * lane + i; ab = run; }
-                else run += c[i];
+            if (bin == kSelectBins) {
+                if (run + b.c[i] >= k) { bin = 8u * threadIdx.x + i; ab = run; }
+                else run += b.c[i];
             }
         }
+        scratch[kWarps] = bin;
+        scratch[kWarps + 1] = ab;
     }
-    const uint32_t found = __ballot_sync(0xffffffffu, bin != 256u);
-    if (found == 0u) { above = 0u; return 256u; }
-    const int src = __ffs(found) - 1;
-    above = __shfl_sync(0xffffffffu, ab, src);
-    return __shfl_sync(0xffffffffu, bin, src);
-}
-
-struct SelectState {
-    uint32_t prefix;      // the key bytes fixed by the passes before `pass`
-    uint32_t k_rem;       // rank still to find among the keys that share them
-    int dead;             // 1: fewer candidates than the budget (cut value -inf), nothing to histogram
-};
-
-// Whole warp: state of one (sequence, head-or-layer) selection before pass `pass`.
-// hist points at [pass][...][256] for this selection with `pass_stride` words between passes.
-__device__ __forceinline__ SelectState select_state(const uint32_t *hist, int64_t pass_stride, int pass, uint32_t k, int lane)
-{
-    SelectState s{0u, k, 0};
-    for (int q = 0; q < pass; ++q) {
-        uint32_t above;
-        const uint32_t bin = select_bin(hist + q * pass_stride, s.k_rem, above, lane);
-        if (bin == 256u) { s.dead = 1; break; }
-        s.prefix = (s.prefix << 8) | bin;
-        s.k_rem -= above;
-    }
-    return s;
+    __syncthreads();
+    above = scratch[kWarps + 1];
+    return scratch[kWarps];
 }
 
 __device__ __forceinline__ uint32_t select_budget(float keep_ratio, int64_t n_cand, int per_layer, int n_heads, bool &too_many)
@@ -93,79 +104,100 @@ __device__ __forceinline__ uint32_t select_budget(float keep_ratio, int64_t n_ca
     return too_many ? 0xffffffffu : static_cast<uint32_t>(total);
 }
 
-// grid (ceil(n_tokens / 256), n_seqs); hist [4][n_seqs][n_sel][256], n_sel = per_layer ? 1 : n_heads
+// grid (ceil(n_tokens / kSelectTokens), n_heads, n_seqs); hist [kSelectPasses][n_seqs][n_sel][kSelectBins], n_sel =
+// per_layer ? 1 : n_heads; arrive [n_seqs][n_sel], zero between launches; the last pass writes tau_list [n_seqs][n_heads].
 __global__ void __launch_bounds__(kSelectThreads)
-select_hist_kernel(const float *__restrict__ scores, int64_t n_tokens, int n_heads, const int32_t *__restrict__ cu_seqlens,
-                   int n_seqs, int window, float keep_ratio, int per_layer, int pass, uint32_t *__restrict__ hist)
+select_pass_kernel(const float *__restrict__ scores, int64_t n_tokens, int n_heads, const int32_t *__restrict__ cu_seqlens,
+                   int n_seqs, int window, float keep_ratio, int per_layer, int pass, uint32_t *__restrict__ hist,
+                   uint32_t *__restrict__ arrive, float *__restrict__ tau_list, int32_t *__restrict__ status)
 {
-    __shared__ uint32_t sh[kMaxHeads][256];
-    __shared__ uint32_t s_prefix[kMaxHeads];
-    __shared__ int s_dead[kMaxHeads];
-    // the launches of one selection are queued with early start: each lets the next be placed at once and
-    // waits here, every thread, for the one ahead (its histograms, or the scores) to be complete
+    __shared__ uint32_t sh[kSelectBins];
+    __shared__ uint32_t scratch[kSelectThreads / 32 + 2];
+    __shared__ int last_s;
+    // The first pass waits for the scores, and lets the second start once it has: later passes find them complete and
+    // wait for the pass ahead only where they need its histogram.
+    if (pass == 0) griddep_wait();
     griddep_launch_dependents();
-    griddep_wait();
-    const int b = blockIdx.y, tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    const int h = blockIdx.y, b = blockIdx.z, tid = threadIdx.x;
     const int64_t t0 = cu_seqlens ? cu_seqlens[b] : 0, t1 = cu_seqlens ? cu_seqlens[b + 1] : n_tokens;
     const int64_t n_cand = t1 - t0 - window > 0 ? t1 - t0 - window : 0;
-    const int64_t c0 = static_cast<int64_t>(blockIdx.x) * kSelectThreads;
-    if (c0 >= n_cand) return;
+    const int64_t c0 = static_cast<int64_t>(blockIdx.x) * kSelectTokens;
     bool too_many;
     const uint32_t k = select_budget(keep_ratio, n_cand, per_layer, n_heads, too_many);
-    if (k == 0u) return;                                  // the cut value is +inf whatever the scores
-    const int n_sel = per_layer ? 1 : n_heads;
-    const int64_t pass_stride = static_cast<int64_t>(n_seqs) * n_sel * 256;
-    for (int i = tid; i < kMaxHeads * 256; i += kSelectThreads) (&sh[0][0])[i] = 0u;
-    if (warp < n_sel) {
-        const SelectState s = select_state(hist + (static_cast<int64_t>(b) * n_sel + warp) * 256, pass_stride, pass, k, lane);
-        if (lane == 0) { s_prefix[warp] = s.prefix; s_dead[warp] = s.dead; }
+    const bool last_pass = pass == kSelectPasses - 1;
+    if (c0 >= n_cand || k == 0u) {
+        if (pass > 0) griddep_wait();
+        if (last_pass && blockIdx.x == 0) {               // nothing to select: the cut value is +inf whatever the scores
+            if (tid == 0 && k == 0u) tau_list[b * n_heads + h] = INFINITY;
+        }
+        return;
     }
-    __syncthreads();
-    if (c0 + tid < n_cand) {
-        const float *row = scores + (t0 + c0 + tid) * n_heads;
-        for (int h = 0; h < n_heads; ++h) {
-            const int hs = per_layer ? 0 : h;
-            const float v = __ldcg(row + h);
-            if (s_dead[hs] || v != v) continue;
-            const uint32_t key = score_key(v);
-            if (pass == 0 || (key >> (32 - 8 * pass)) == s_prefix[hs])
-                atomicAdd(&sh[hs][(key >> (24 - 8 * pass)) & 255u], 1u);
+    float v[4];
+#pragma unroll
+    for (int j = 0; j < 4; ++j) {
+        const int64_t i = c0 + j * kSelectThreads + tid;
+        v[j] = i < n_cand ? __ldcg(scores + (t0 + i) * n_heads + h) : __uint_as_float(0x7fffffffu);      // NaN: no candidate
+    }
+    for (int i = tid; i < kSelectBins; i += kSelectThreads) sh[i] = 0u;
+    if (pass > 0) griddep_wait();
+    const int n_sel = per_layer ? 1 : n_heads, sel = b * n_sel + (per_layer ? 0 : h);
+    const int64_t pass_stride = static_cast<int64_t>(n_seqs) * n_sel * kSelectBins;
+    uint32_t *mine = hist + static_cast<int64_t>(sel) * kSelectBins;
+    // the digits fixed by the passes before this one
+    uint32_t prefix = 0u, k_rem = k, above;
+    bool dead = false;                                    // fewer candidates than the budget: the cut value is -inf
+    {
+        SelectBins bins[kSelectPasses - 1];
+#pragma unroll
+        for (int q = 0; q < kSelectPasses - 1; ++q)
+            if (q < pass) bins[q] = load_bins(mine + q * pass_stride);
+#pragma unroll
+        for (int q = 0; q < kSelectPasses - 1; ++q) {
+            if (q >= pass || dead) continue;
+            const uint32_t bin = select_bin(bins[q], k_rem, above, scratch);
+            if (bin == kSelectBins) { dead = true; continue; }
+            prefix = (prefix << select_bits(q)) | bin;
+            k_rem -= above;
         }
     }
     __syncthreads();
-    uint32_t *out = hist + pass * pass_stride + static_cast<int64_t>(b) * n_sel * 256;
-    for (int i = tid; i < n_sel * 256; i += kSelectThreads) {
-        const uint32_t v = sh[i >> 8][i & 255];
-        if (v) atomicAdd(out + i, v);
+    if (!dead) {
+        const int shift = select_shift(pass), bits = select_bits(pass);
+#pragma unroll
+        for (int j = 0; j < 4; ++j) {
+            if (v[j] != v[j]) continue;
+            const uint32_t key = score_key(v[j]);
+            if (pass == 0 || (key >> (shift + bits)) == prefix) atomicAdd(&sh[(key >> shift) & ((1u << bits) - 1u)], 1u);
+        }
     }
-}
-
-// grid n_seqs; writes the cut values tau_list [n_seqs][n_heads]
-__global__ void __launch_bounds__(kSelectThreads)
-select_finish_kernel(int64_t n_tokens, int n_heads, const int32_t *__restrict__ cu_seqlens, int n_seqs, int window,
-                     float keep_ratio, int per_layer, const uint32_t *__restrict__ hist, float *__restrict__ tau_list,
-                     int32_t *__restrict__ status)
-{
-    griddep_launch_dependents();
-    griddep_wait();
-    const int b = blockIdx.x, lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    const int64_t t0 = cu_seqlens ? cu_seqlens[b] : 0, t1 = cu_seqlens ? cu_seqlens[b + 1] : n_tokens;
-    const int64_t n_cand = t1 - t0 - window > 0 ? t1 - t0 - window : 0;
-    bool too_many;
-    const uint32_t k = select_budget(keep_ratio, n_cand, per_layer, n_heads, too_many);
-    if (too_many && threadIdx.x == 0) atomicCAS(status, 0, 2 /* KVZAP_ERR_UNSUPPORTED */);
-    const int n_sel = per_layer ? 1 : n_heads;
-    if (warp >= n_sel) return;
-    float tau = INFINITY;
-    if (k > 0u) {
-        const int64_t pass_stride = static_cast<int64_t>(n_seqs) * n_sel * 256;
-        const SelectState s = select_state(hist + (static_cast<int64_t>(b) * n_sel + warp) * 256, pass_stride, 4, k, lane);
-        tau = s.dead ? -INFINITY : key_score(s.prefix);
+    __syncthreads();
+    uint32_t *out = mine + pass * pass_stride;
+    for (int i = tid; i < kSelectBins; i += kSelectThreads) {
+        const uint32_t n = sh[i];
+        if (n) atomicAdd(out + i, n);
+    }
+    if (!last_pass) return;
+    // the selection's CTA that is done last takes the last digit
+    __threadfence();
+    __syncthreads();
+    if (tid == 0) {
+        if (too_many) atomicCAS(status, 0, 2 /* KVZAP_ERR_UNSUPPORTED */);
+        const uint32_t n_ctas = static_cast<uint32_t>((n_cand + kSelectTokens - 1) / kSelectTokens) * (per_layer ? n_heads : 1);
+        last_s = atomicAdd(arrive + sel, 1u) + 1u == n_ctas;
+        if (last_s) arrive[sel] = 0u;
+        __threadfence();
+    }
+    __syncthreads();
+    if (!last_s) return;
+    float tau = -INFINITY;
+    if (!dead) {
+        const uint32_t bin = select_bin(load_bins(out), k_rem, above, scratch);
+        if (bin != kSelectBins) tau = key_score((prefix << select_bits(kSelectPasses - 1)) | bin);
     }
     if (per_layer) {
-        for (int h = lane; h < n_heads; h += 32) tau_list[b * n_heads + h] = tau;
-    } else if (lane == 0) {
-        tau_list[b * n_heads + warp] = tau;
+        if (tid < n_heads) tau_list[b * n_heads + tid] = tau;
+    } else if (tid == 0) {
+        tau_list[b * n_heads + h] = tau;
     }
 }
 
