@@ -18,8 +18,8 @@
 // With fewer lists than resident CTAs (a small batch, layer by layer) there is one wave, and it lasts as
 // long as its longest part: equal parts of lists whose lengths spread over 1 : 7 (contexts of one batch x
 // what each head keeps) leave most of it idle.  There the CTAs share the lists out themselves (attn_unit):
-// every CTA reads all list lengths, finds the shortest part length for which all parts fit the grid, and
-// takes the part of its index.  8 sequences x 8 heads, 2176 rows on average: 26.0 -> 20.4 us per call.
+// every CTA reads all list lengths, finds the shortest part length (of at least four tiles a warp) for which
+// all parts fit the grid, and takes the part of its index.  8 sequences x 8 heads, 2176 rows on average: 26.0 -> 20.4 us per call.
 //
 // Math per tile, on the warp-level tensor-core path (the work is HBM-bound; 16-row MMAs are enough):
 //   S[16 x 16]  = Q[16 x D] K^T      m16n8k16, Q rows 0..G-1 real, the rest zero
@@ -54,7 +54,11 @@
 namespace kvzap {
 
 constexpr int kAttnWarps = 4;
-constexpr int kAttnStages = 3;
+// Stages of a warp's ring.  bf16 rows: two, so that three CTAs fit an SM (168 registers, 66 KB) -- the same bytes in flight as
+// two CTAs with three stages, but the serial parts of a CTA (counts, pages, first tiles, merge: some 3 us) run beside two
+// others: 128 sequences x 4 layers, layer by layer, 1553 -> 1527 us; 80 x 8 layers 1245 -> 1175 us.  8-bit rows: three,
+// four CTAs fit either way.
+__host__ __device__ constexpr int attn_stages(bool fp8) { return fp8 ? 3 : 2; }
 constexpr int kAttnTileRows = 16;
 constexpr int kAttnThreads = kAttnWarps * 32;
 constexpr int kAttnMaxGroup = 8;                 // query heads per KV head (rows 0..7 of the 16-row MMA)
@@ -79,6 +83,7 @@ struct AttnParams {
 // fp32: whatever their rounding, every warp rounds alike).  Returns the number of parts of the list that `unit` falls
 // into, 0 if there is no such unit; `list` and `part` say which.
 constexpr int kAttnListsPerLane = 20;       // n <= 32 * this
+constexpr float kAttnMinPart = 16.0f;       // tiles
 __device__ __forceinline__ int attn_unit(const int32_t *lengths, int n, int n_units, int unit, int lane, int &list, int &part)
 {
     // lane l owns lists [l * per, (l + 1) * per), in registers
@@ -106,7 +111,7 @@ __device__ __forceinline__ int attn_unit(const int32_t *lengths, int n, int n_un
         }
         return parts;
     };
-    float lo = fmaxf(1.0f, static_cast<float>(sum) / static_cast<float>(n_units)), hi = static_cast<float>(longest);
+    float lo = fmaxf(kAttnMinPart, static_cast<float>(sum) / static_cast<float>(n_units)), hi = fmaxf(lo, static_cast<float>(longest));
     if (n * 2 <= n_units) hi = fminf(hi, 2.02f * lo);       // at most sum / hi + n parts
     constexpr float kDown = 1.0f - 1.0f / (1 << 20);        // a list of exactly the target length is one part
     float inv = kDown / hi;                                 // fits: one part each, or half of the units plus one each
@@ -147,7 +152,7 @@ __host__ __device__ constexpr uint32_t attn_stage_bytes(int head_dim, bool fp8 =
 }
 __host__ __device__ constexpr uint32_t attn_smem_bytes(int head_dim, bool fp8 = false)
 {
-    return kAttnWarps * kAttnStages * attn_stage_bytes(head_dim, fp8) + (fp8 ? 128u : 1024u) /* alignment */ + 256u /* barriers */;
+    return kAttnWarps * attn_stages(fp8) * attn_stage_bytes(head_dim, fp8) + (fp8 ? 128u : 1024u) /* alignment */ + 256u /* barriers */;
 }
 
 // four E4M3 codes (a 32-bit word, lowest byte first) -> two packed f16 pairs (exact: f16 holds every E4M3 value)
@@ -173,12 +178,13 @@ __device__ __forceinline__ void attn_store(uint16_t *out, const float4 &num, flo
 }
 
 template <int kD, bool kFp8>
-__global__ void __launch_bounds__(kAttnThreads, kFp8 ? 4 : 1)
+__global__ void __launch_bounds__(kAttnThreads, kFp8 ? 4 : 3)
 decode_attn_kernel(const __grid_constant__ CUtensorMap tmap_kpool, const __grid_constant__ CUtensorMap tmap_vpool,
                    const __grid_constant__ CUtensorMap tmap_kring, const __grid_constant__ CUtensorMap tmap_vring,
                    const AttnParams p)
 {
     constexpr int kHalves = kD / 64;
+    constexpr int kAttnStages = attn_stages(kFp8);
     constexpr uint32_t kStageBytes = attn_stage_bytes(kD, kFp8);
     constexpr int kRowBytes8 = kD + kAttnTrailerBytes;              // 8-bit rows
     constexpr uint32_t kTileBytes8 = kAttnTileRows * kRowBytes8;

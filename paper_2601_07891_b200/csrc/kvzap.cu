@@ -2414,18 +2414,22 @@ static kvzap_status attention_impl(kvzap_ctx *ctx, kvzap_cache *cache, int32_t l
     p.status = ctx->status_dev;
     const int64_t n_lists_call = static_cast<int64_t>(p.n_layers_call) * v.n_seqs * v.n_heads;
     if (n_lists_call > 0x7fffffffLL) return fail(ctx, KVZAP_ERR_UNSUPPORTED, "attention: too many lists for one launch");
-    // Two CTAs fit an SM (four of the 8-bit kernel's).  Fewer lists than that: one wave, whose CTAs share the lists out
-    // by their lengths.  With fewer than sixteen CTAs per slot the last, longest lists leave most SMs idle: cut
-    // every list into up to 16 parts so that there are about that many units.
-    const int64_t slots = static_cast<int64_t>(ctx->sm_count) * (fp8 && d_attn == 128 ? 4 : 2);
+    // Three CTAs fit an SM (four of the 8-bit kernel's).  Fewer lists than that: one wave, whose CTAs share the lists out
+    // by their lengths.  More: every list in as many parts as make some 24 CTAs per SM -- a CTA costs about 3 us beside its
+    // share of the rows, the last ones leave SMs idle -- but none shorter than 1200 rows of the longest list the cache can
+    // hold.  512 lists of 1600 rows: 9 parts 1062 us, 2 parts 763 us (8 layers, with their steps); 1024 lists of 750 rows:
+    // 4 parts 490 us, 1 part 355 us, of 4700 rows: 1 part 1678 us, 3 parts 1527 us (4 layers).  320 lists, by their
+    // lengths: 898 us against 1115 us in 14 equal parts (8 layers).
+    const int64_t slots = static_cast<int64_t>(ctx->sm_count) * (fp8 && d_attn == 128 ? 4 : 3);
     int64_t n_ctas = n_lists_call;
     p.n_parts = 1;
-    if (n_lists_call < slots) {
+    if (n_lists_call < slots && n_lists_call <= 32 * kAttnListsPerLane) {
         p.n_parts = 0;
         n_ctas = slots;
     } else {
-        const int64_t want_units = static_cast<int64_t>(ctx->sm_count) * 32;
-        int64_t parts = want_units / n_lists_call;
+        const int64_t longest = static_cast<int64_t>(v.max_pages) * v.page_tokens + v.window;
+        int64_t parts = static_cast<int64_t>(ctx->sm_count) * 24 / n_lists_call;
+        if (parts > longest / 1200) parts = longest / 1200;
         if (parts > 16) parts = 16;
         if (parts > 1) p.n_parts = static_cast<int32_t>(parts);
         n_ctas = n_lists_call * p.n_parts;

@@ -77,3 +77,26 @@ def test_alone_and_beside_scoring(T, lens, D, proj, paged, window):
                 page += k
     if paged:
         assert int(got[5]) == page - 3
+
+
+@pytest.mark.parametrize("T,n_pages,max_pages", [(777, 40, 60), (777, 4000, 5), (9001, 40, 700)])
+@pytest.mark.parametrize("trusted", [False, True])
+def test_paged_pool_or_table_too_small(T, n_pages, max_pages, trusted):
+    """Pages assigned inside the compaction (short) and by a launch of its own (long): the status word says so, the lengths
+    are there, no page is used and nothing is written."""
+    ctx = binding.Kvzap(D_MODEL, HIDDEN, H, 64, 1, max_tokens=T, trusted_producers=trusted)
+    ctx.set_weights(0, *[x.cuda() for x in synth.mlp_weights(D_MODEL, HIDDEN, H, 5, "cpu", 0.3)])
+    X = synth.hidden_states(T, D_MODEL, seed=T).cuda()
+    K, V = (t.cuda() for t in synth.keys_values(H, T, 64, seed=3))
+    out = [torch.full((n_pages, 16, 64), 7.0, dtype=torch.bfloat16, device="cuda") for _ in range(2)]
+    table = torch.full((H, max_pages), -1, dtype=torch.int32, device="cuda")
+    used, lengths = torch.full((1,), 9, dtype=torch.int32, device="cuda"), torch.zeros(1, H, dtype=torch.int32, device="cuda")
+    scores = torch.zeros(T, H, dtype=torch.float32, device="cuda")
+    binding.kvzap_prefill_fused_paged(ctx.handle, 0, X, K, V, None, 1, TAU, 128, *out, 16, 0, table, lengths, used, scores)
+    torch.cuda.synchronize()
+    assert ctx.poll_status() == 4                       # KVZAP_ERR_OOM_PAGES
+    keep = scores >= TAU
+    keep[-128:] = True
+    assert torch.equal(lengths[0], keep.sum(0).int())
+    assert int(used) == 0 and (table == -1).all() and all((x == 7.0).all() for x in out)
+    ctx.close()
