@@ -638,16 +638,18 @@ static kvzap_status launch_score(kvzap_ctx *ctx, int32_t layer, int32_t n_layers
         // Early start.  Without the fused part the kernel reads nothing but weights, and hidden states of trusted
         // producers, until every thread has waited for the kernel ahead, and writes only after.  The fused decode
         // step touches the cache (counters, page allocator, rows): its clusters order themselves through `done`,
-        // which covers earlier fused steps of the same layout only, so it does that before the wait only directly
-        // behind such a step of the previous call on the same cache (fuse_chain) -- never behind a prompt chunk's
-        // page assignment, a release or an export, whose kernels it would race with -- and with a grid of at least
+        // which covers earlier fused steps of the same layers in the same layout only, so it does that before the wait
+        // only directly behind such a step of the previous call on the same cache (fuse_chain), with a grid of at least
         // half the SMs and its own scores buffer; else all it does before the wait is to fetch its first W1 tiles.
-        // Directly behind the call that wrote the weights not even that is allowed.
+        // That is sound only if whatever precedes the first step of such a chain -- a prompt chunk's page assignment, a
+        // release, a step in another layout -- is complete before the second starts, which may be of other layers and
+        // then waits for nothing: a step that waits lets the next launch be placed only after its wait (late_trigger).
+        // Directly behind the call that wrote the weights not even the early W1 tiles are allowed.
         const bool overlap = fuse_ok && fuse_chain != nullptr && *fuse_chain == layout_i && !clash &&
                              p.n_tiles * n_ctas * 2 >= ctx->sm_count;
         const bool early = !ctx->profiling && ctx->weights_seq + 1 != ctx->op_seq;
         p.wait_before_load = ctx->trusted && (!fuse_ok || overlap) ? 0 : 1;
-        p.late_trigger = late_trigger && p.wait_before_load;
+        p.late_trigger = (late_trigger || fuse_ok) && p.wait_before_load;
         ctx->last_score_late = p.late_trigger != 0;
         ctx->last_score_early = early;
         {
