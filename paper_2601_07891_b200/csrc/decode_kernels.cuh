@@ -86,9 +86,10 @@ constexpr int kDecodeLanes = 8;        // lanes that share one list (a 256-byte 
 // The kernel is launched so that it may be placed while the scoring kernel ahead of it in the stream
 // is still running.  With a window, the fate of the token that leaves it depends only on its
 // BUFFERED score, so the row traffic (old row to its page, new rows into the ring) needs nothing
-// from that kernel and only the new scores wait for it.  `wait_first` != 0 makes the whole kernel
-// wait instead: required when the scoring kernel itself was started before the previous step's
-// update had finished (two updates must never touch the cache at the same time).
+// from that kernel and only the new scores wait for it.  That is sound only if the scoring launch lets
+// this one start after its own wait: everything ahead of it -- the previous step's update, a prompt chunk's
+// page assignment, a release -- is then complete before a list or the allocator is touched here.
+// `wait_first` != 0 makes the whole kernel wait instead (scoring kernels that trigger at once).
 __global__ void __launch_bounds__(kDecodeThreads)
 decode_update_kernel(const CacheView c, int layer0, int n_layers_call, const float *__restrict__ scores,
                      const uint4 *__restrict__ K_new, const uint4 *__restrict__ V_new, float tau,
@@ -208,8 +209,7 @@ decode_update_kernel(const CacheView c, int layer0, int n_layers_call, const flo
 __global__ void __launch_bounds__(32)
 release_seq_kernel(const CacheView c, int32_t seq)
 {
-    griddep_wait();              // every kernel that touches the cache waits for the one ahead before it does
-    griddep_launch_dependents();
+    griddep_wait();              // and lets nothing start before it is done
     const int64_t li = static_cast<int64_t>(seq) * c.n_layers * c.n_heads + blockIdx.x;
     const int lane = threadIdx.x;
     const int32_t n_pages = (c.prefix_len[li] + c.page_tokens - 1) / c.page_tokens;

@@ -76,7 +76,7 @@ struct ScoreParams {
     int32_t *status;      // device status word
     int32_t wait_before_write;    // 1: the epilogue waits for the kernel ahead in the stream before its first store
     int32_t wait_before_load;     // 1: every thread waits for the work ahead in the stream before caller data is read
-    int32_t late_trigger;         // few-token kernel: 1: the next launch may start once that wait is over (else at once)
+    int32_t late_trigger;         // 1: the next launch may start once that wait is over (else at once)
     int32_t *tile_counter;        // work tiles handed out beyond the first one of every CTA (or pair); starts at 0
     int32_t *tile_counter_reset;  // the counter of the launch after next: set to 0 by this launch
     // 8-bit inputs (score_kernel<.., .., true>): hidden states and first-layer weights are E4M3 bytes, a 128-byte
@@ -263,8 +263,9 @@ score_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_constant__
     const uint32_t tile_ring_addr = bars + 16 * kMaxStages + 80 + 16 * kSchedSlots;
 
     // Let the kernel behind this one in the stream (the compaction) be placed right away; it waits
-    // for this kernel's results itself.
-    griddep_launch_dependents();
+    // for this kernel's results itself.  The update of a decode step in two launches moves rows before
+    // that wait, so it is let in only when all work ahead of this launch is complete (late_trigger).
+    if (!p.late_trigger) griddep_launch_dependents();
     const int warp = threadIdx.x >> 5;
     const int lane = threadIdx.x & 31;
     constexpr int kEpiWarps = kMlp ? 8 : 4;
@@ -314,6 +315,7 @@ score_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_constant__
     // The set-up above overlaps the tail of the work ahead in the stream either way; unless the caller
     // vouches for the producers of its inputs, nothing of them is read before that work has completed.
     if (p.wait_before_load) griddep_wait();
+    if (p.late_trigger) griddep_launch_dependents();
 
     const int k_blocks = p.k_blocks > 0 ? p.k_blocks : p.d_model / kBlockK;
     const int k_elems = p.k_elems > 0 ? p.k_elems : kBlockK;

@@ -1,7 +1,8 @@
 """Decode steps enqueued, without a synchronisation anywhere, behind work that they must not run beside: a prompt chunk's
-page assignment and compaction, a release, a step in another layout.  The step directly behind is followed by steps of
-other layers of the same layout, on grids large enough to overlap.  Every list is compared with the selection by score
-of its whole stream, and no page is owned twice."""
+page assignment and compaction, a release, a step in another layout.  In one launch: the step directly behind is followed
+by steps of other layers of the same layout, on grids large enough to overlap.  In two launches (more tiles than the
+few-token kernel takes; linear surrogate; 8-bit inputs without a few-token layout): the update moves rows beside the
+scoring.  Every list is compared with the selection by score of its whole stream, and no page is owned twice."""
 import numpy as np
 import pytest
 import torch
@@ -16,12 +17,15 @@ D_MODEL, H, D, W, P, TAU = 512, 8, 64, 32, 4, 0.1
 class _Server:
     """A cache, its streams of tokens per (slot, layer), and calls that are made only when all inputs are there."""
 
-    def __init__(self, hidden, B, L, trusted, n_rows):
-        self.B, self.L = B, L
+    def __init__(self, hidden, B, L, trusted, n_rows, fp8=False):
+        self.B, self.L, self.fp8 = B, L, fp8
         self.ctx = binding.Kvzap(D_MODEL, hidden, H, D, L, max_tokens=512, trusted_producers=trusted)
         for l in range(L):
             w = synth.mlp_weights(D_MODEL, hidden, H, 70 + l, "cuda", 0.3) if hidden else synth.linear_weights(D_MODEL, H, 70 + l, "cuda", 0.3)
-            self.ctx.set_weights(l, *w)
+            if fp8:
+                binding.kvzap_set_weights_fp8(self.ctx.handle, l, *synth.quantize_e4m3(w[0]), *w[1:])
+            else:
+                self.ctx.set_weights(l, *w)
         self.max_pages = n_rows // P + 2
         self.n_pool = B * L * H * self.max_pages
         self.pools = [torch.zeros(self.n_pool, P, D, dtype=torch.bfloat16, device="cuda") for _ in range(2)]
@@ -53,7 +57,12 @@ class _Server:
         X = self._inputs(n * B)[0].view(n, B, D_MODEL)
         K, V = (t.view(n, B, H, D) for t in synth.keys_values(n * B, H, D, 9000 + self.seed, "cuda"))
         s = torch.zeros(n, B, H, dtype=torch.float32, device="cuda")
-        self.calls.append(lambda: binding.kvzap_decode_step(self.ctx.handle, self.cache, a, e, X, K, V, TAU, s))
+        if self.fp8:
+            x, scale = synth.quantize_e4m3(X.view(n * B, D_MODEL))
+            x, scale = x.view(n, B, D_MODEL), scale.view(n, B)
+            self.calls.append(lambda: binding.kvzap_decode_step_fp8(self.ctx.handle, self.cache, a, e, x, scale, K, V, TAU, s))
+        else:
+            self.calls.append(lambda: binding.kvzap_decode_step(self.ctx.handle, self.cache, a, e, X, K, V, TAU, s))
         for b in range(B):
             if self.active[b]:
                 for l in range(a, e):
@@ -122,4 +131,32 @@ def test_steps_of_layer_groups_behind_other_work(B, L, group, trusted):
         srv.prompt((r + 1) % 3, 60)
         srv.step(0, L)                      # in another layout than its groups
         groups(3)
+    srv.check()
+
+
+@pytest.mark.parametrize("trusted", [True, False])
+@pytest.mark.parametrize("hidden,B,L", [(512, 130, 20), (512, 6, 40), (0, 130, 20), (64, 6, 38)])
+def test_steps_in_two_launches_behind_other_work(hidden, B, L, trusted):
+    srv = _Server(hidden, B, L, trusted, 320)
+    for b in range(3):
+        srv.prompt(b, 70 + 30 * b)
+    for r in range(5):
+        srv.prompt(r % 3, 41)
+        for _ in range(3):                  # behind the chunk, then behind one another
+            srv.step(0, L)
+        srv.release((r + 1) % 3)
+        for _ in range(3):
+            srv.step(0, L)
+        srv.prompt((r + 1) % 3, 60)
+    srv.check()
+
+
+@pytest.mark.parametrize("trusted", [True, False])
+def test_eight_bit_steps_in_two_launches_behind_a_release(trusted):
+    srv = _Server(512, 130, 20, trusted, 320, fp8=True)
+    for b in range(12):
+        for _ in range(6):                  # from the 33rd step on rows leave the window and take pages
+            srv.step(0, 20)
+        srv.release(b)
+    srv.step(0, 20)
     srv.check()
