@@ -58,7 +58,7 @@ chunk_ring_kernel(const CacheView c, const __grid_constant__ ChunkSeqs seqs, int
     V += tok0 * c.row_units;
     scores += tok0 * H;
     const int64_t n_old = __ldcg(c.n_tokens + li);
-    if (tid == 0) { len_s = __ldcg(c.prefix_len + li); ok_s = 1; kept_s = 0; }
+    if (tid == 0) { len_s = __ldcg(c.prefix_len + li); kept_s = 0; }
     __syncthreads();
     const int64_t in_ring = n_old < c.window ? n_old : c.window;
     const int64_t first = n_old - in_ring;                         // oldest position still in the window
@@ -68,7 +68,7 @@ chunk_ring_kernel(const CacheView c, const __grid_constant__ ChunkSeqs seqs, int
     int32_t *table = c.page_table + li * c.max_pages;
     const int group = tid >> 4, gl = tid & 15;
     constexpr int kGroups = kChunkThreads / 16, kRows = 2;         // 16 lanes per row, two rows per lane group in flight
-    for (int64_t base = 0; base < n_exit && ok_s; base += 128) {
+    for (int64_t base = 0; base < n_exit; base += 128) {
         if (warp == 0) {
             const int64_t len = len_s;
             uint32_t kept[4];
@@ -122,6 +122,7 @@ chunk_ring_kernel(const CacheView c, const __grid_constant__ ChunkSeqs seqs, int
             }
         }
         __syncthreads();
+        const bool more = ok_s != 0;        // read between two barriers: all threads leave the loop together
         const int n_batch = n_exit - base < 128 ? static_cast<int>(n_exit - base) : 128;
         for (int i0 = group; i0 < n_batch; i0 += kRows * kGroups) {
             for (int u = gl; u < c.row_units; u += 16) {
@@ -145,6 +146,7 @@ chunk_ring_kernel(const CacheView c, const __grid_constant__ ChunkSeqs seqs, int
             }
         }
         __syncthreads();
+        if (!more) break;                   // no page left: the exits behind these are dropped
     }
     // the chunk's last min(m, w) tokens into the ring (the slots they take were read above)
     const int64_t n_win = m < c.window ? m : c.window;

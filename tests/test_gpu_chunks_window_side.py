@@ -67,3 +67,43 @@ def test_chunks_against_selection(trusted, n_seqs, window, P, rounds):
             binding.kvzap_cache_release_seq(ctx.handle, cache, s)
     binding.kvzap_cache_destroy(cache)
     ctx.close()
+
+
+@pytest.mark.parametrize("trusted", [False, True])
+@pytest.mark.parametrize("max_pages,pool_pages,second", [(40, 4000, 260), (40, 4000, 300), (100, 700, 260), (100, 1, 200)])
+def test_pages_run_out_among_several_batches_of_exits(trusted, max_pages, pool_pages, second):
+    """A window of 272 tokens pushed out in batches of 128 until the table (160 rows) or the pool is full: a list holds the
+    exits that found a page, oldest first, and its window the newest tokens, in every repetition."""
+    n_seqs, window, P = 3, 272, 4
+    ctx = binding.Kvzap(D_MODEL, HIDDEN, H, D, 1, max_tokens=n_seqs * 400, max_seqs=n_seqs, trusted_producers=trusted)
+    ctx.set_weights(0, *[x.cuda() for x in synth.mlp_weights(D_MODEL, HIDDEN, H, 9, "cpu", 0.3)])
+    pools = [torch.zeros(pool_pages, P, D, dtype=torch.bfloat16, device="cuda") for _ in range(2)]
+    lens = [[window] * n_seqs, [second] * n_seqs]
+    inputs = []
+    for r in range(2):
+        n = sum(lens[r])
+        inputs.append((torch.from_numpy(synth.cu_seqlens(lens[r])).cuda(), synth.hidden_states(n, D_MODEL, seed=r).cuda(),
+                       *(t.cuda() for t in synth.keys_values(H, n, D, seed=10 + r)), torch.zeros(n, H, device="cuda")))
+    out = [torch.zeros(max_pages * P + window, D, dtype=torch.bfloat16, device="cuda") for _ in range(2)]
+    n = torch.zeros(1, dtype=torch.int32, device="cuda")
+    for _ in range(4):
+        cache = binding.kvzap_cache_create(ctx.handle, n_seqs, window, P, *pools, max_pages)
+        for cu, X, K, V, s in inputs:
+            binding.kvzap_prefill_to_cache_batch(ctx.handle, cache, 0, list(range(n_seqs)), cu, X, K, V, float("-inf"), s)
+        torch.cuda.synchronize()
+        assert ctx.poll_status() == 4                  # KVZAP_ERR_OOM_PAGES
+        owned = 0
+        for b in range(n_seqs):
+            stream = [torch.cat([inputs[r][i][:, b * lens[r][b]:(b + 1) * lens[r][b]] for r in range(2)], dim=1) for i in (2, 3)]
+            for h in range(H):
+                binding.kvzap_cache_export(ctx.handle, cache, b, 0, h, *out, n)
+                prefix = int(n) - window
+                owned += (prefix + P - 1) // P
+                assert 0 <= prefix <= second and (prefix == 160 or max_pages != 40)
+                for x, o in zip(stream, out):
+                    want = torch.cat([x[h, :prefix], x[h, -window:]])
+                    assert torch.equal(o[:int(n)].view(torch.int16), want.view(torch.int16))
+        if max_pages != 40:
+            assert owned == pool_pages         # every page of the pool went to a list
+        binding.kvzap_cache_destroy(cache)
+    ctx.close()
