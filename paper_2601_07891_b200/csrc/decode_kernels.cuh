@@ -38,7 +38,9 @@ struct CacheView {
 
 // One more page for a list: a released one if the stack has any, else the next never-used page of the
 // pool; -1 (and the status word) when neither is left.  Kernels that take pages never release any, so the
-// stack only shrinks while they run: an index handed out by the atomic below is stable.
+// stack only shrinks while they run: an index handed out by the atomic below is stable.  What a taker moved the cursor
+// past the pool it moves back: while it is past the pool every page below is handed out, so nobody gets one twice, and it
+// ends where the pages end -- a later page assignment reads it, and it cannot run away over many failing steps.
 __device__ __forceinline__ int32_t cache_take_page(const CacheView &c, int32_t *status)
 {
     if (__ldcg(c.free_top) > 0) {                       // the usual case, an empty stack, costs one load
@@ -48,6 +50,7 @@ __device__ __forceinline__ int32_t cache_take_page(const CacheView &c, int32_t *
     }
     const int32_t got = atomicAdd(c.page_cursor, 1);
     if (got >= c.n_pages_pool) {
+        atomicSub(c.page_cursor, 1);
         atomicCAS(status, 0, 4 /* KVZAP_ERR_OOM_PAGES */);
         return -1;
     }
@@ -72,7 +75,10 @@ __device__ __forceinline__ int cache_take_pages(const CacheView &c, int32_t *sta
     cur = __shfl_sync(0xffffffffu, cur, 0);
     const int64_t left = c.n_pages_pool - cur;
     const int fresh = got == n || left <= 0 ? 0 : left < n - got ? static_cast<int>(left) : n - got;
-    if (got + fresh < n && lane == 0) atomicCAS(status, 0, 4 /* KVZAP_ERR_OOM_PAGES */);
+    if (got + fresh < n && lane == 0) {
+        atomicSub(c.page_cursor, n - got - fresh);
+        atomicCAS(status, 0, 4 /* KVZAP_ERR_OOM_PAGES */);
+    }
     for (int i = lane; i < got + fresh; i += 32) pages[i] = i < got ? __ldcg(c.free_stack + top - 1 - i) : cur + (i - got);
     return got + fresh;
 }

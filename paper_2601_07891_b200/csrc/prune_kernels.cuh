@@ -188,7 +188,10 @@ assign_pages(int n_heads, int n_seqs, int32_t *__restrict__ lengths, int page_to
     const int32_t used = carry_s;
     if (n_free < 0) n_free = 0;
     const int32_t from_stack = used < n_free ? used : n_free;
-    const bool fail = fail_s != 0 || static_cast<int64_t>(first_page) + (used - from_stack) > n_pages_pool;
+    // a cache (page_cursor): what comes from the stack, or an append that needs no page, fits wherever the cursor stands
+    const bool fits = static_cast<int64_t>(first_page) + (used - from_stack) <= n_pages_pool ||
+                      (page_cursor != nullptr && used == from_stack);
+    const bool fail = fail_s != 0 || !fits;
     if (fail) {
         for (int idx = tid; idx < n_lists; idx += NT) {
             list_page0[idx] = -1;

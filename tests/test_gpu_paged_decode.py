@@ -388,3 +388,47 @@ def test_release_seq_hands_its_pages_out_again(binding, oracle, hidden):
     check()
     cache.close()
     ctx.close()
+
+
+@pytest.mark.parametrize("how", ["chunk", "steps"])
+def test_cache_that_ran_out_of_pages_takes_prompts_again_after_a_release(binding, how):
+    """The window side of a chunk, or decode steps, ask for more pages than the pool has; then a sequence is released and
+    its slot gets a prompt that fits the pages given back."""
+    d_model, hidden, H, D, w, P, tau, n_pool, max_pages = 256, 128, 8, 64, 16, 4, float("-inf"), 200, 60
+    ctx = binding.Kvzap(d_model, hidden, H, D, 1, max_tokens=256)
+    ctx.set_weights(0, *[parity.dev(x) for x in _weights(d_model, hidden, H, seed=3)])
+    pools = [torch.zeros(n_pool, P, D, dtype=torch.bfloat16, device="cuda") for _ in range(2)]
+    cache = ctx.create_cache(2, w, P, *pools, max_pages)
+
+    def prompt(slot, n, seed):
+        K, V = (parity.dev(t) for t in synth.keys_values(H, n, D, seed=seed))
+        cache.prefill(0, slot, parity.dev(synth.hidden_states(n, d_model, seed=seed)), K, V, tau)
+        return K, V
+
+    prompt(0, w + 88, 1)                                # 22 pages a list: 176 of the 200
+    prompt(1, w, 2)
+    for i in range(20):
+        if how == "chunk":
+            prompt(1, w, 3 + i)                         # 4 pages a list
+        else:
+            K, V = (parity.dev(t).view(1, 2, H, D) for t in synth.keys_values(2 * H, 1, D, seed=30 + i))
+            cache.decode_step(0, 1, parity.dev(synth.hidden_states(2, d_model, seed=30 + i)).view(1, 2, d_model), K, V, tau)
+    torch.cuda.synchronize()
+    assert ctx.poll_status() == 4                       # KVZAP_ERR_OOM_PAGES
+    cache.release_seq(0)
+    kv = prompt(0, w + 80, 90)                          # 20 pages a list: 160 of the 176 given back
+    torch.cuda.synchronize()
+    assert ctx.poll_status() == 0
+    for h in range(H):
+        out = _export(binding, ctx, cache.handle, 0, 0, h, w + 80, D)
+        for got, x in zip(out[:2], kv):
+            np.testing.assert_array_equal(got, synth.bits(x[h].cpu()))
+    prefix = torch.zeros(2 * H, dtype=torch.int32, device="cuda")
+    table = torch.zeros(2 * H, max_pages, dtype=torch.int32, device="cuda")
+    cursor = torch.zeros(1, dtype=torch.int32, device="cuda")
+    binding.kvzap_cache_snapshot(ctx.handle, cache.handle, prefix, table, cursor)
+    pages = (prefix.cpu().numpy() + P - 1) // P
+    owned = np.concatenate([t[:k] for t, k in zip(table.cpu().numpy(), pages)])
+    assert len(np.unique(owned)) == len(owned) and int(cursor) == n_pool
+    cache.close()
+    ctx.close()
