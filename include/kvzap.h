@@ -13,7 +13,8 @@
  * General conventions
  *   - Every tensor argument is a DEVICE pointer owned by the caller, unless a
  *     comment says "host".  The library owns only its context (a private
- *     copy of the surrogate weights and a few MB of scratch).
+ *     copy of the surrogate weights and a few MB of scratch; a fixed-budget call
+ *     of many sequences adds up to 50 MB on first use).
  *   - bf16 tensors are passed as `const void*` (raw 16-bit patterns),
  *     row-major, innermost dimension last.  Pointers must be 16-byte aligned.
  *   - `stream` is a cudaStream_t passed as `void*` (NULL = default stream).

@@ -87,8 +87,9 @@ struct kvzap_ctx {
     uint32_t *maskbits = nullptr;    // [kMaskRing][H][max_words]: consecutive calls use different slices
     uint64_t mask_turn = 0;
     int32_t *tile_counters = nullptr;    // [kMaskRing] work-tile counters of the scoring launches, used in rotation
-    uint32_t *select_hist = nullptr;     // fixed-budget selection: [passes][max_seqs][H][bins] histograms, zero between calls
-    bool select_clean = false;           //                         ... as far as the host knows
+    uint32_t *select_hist = nullptr;     // fixed-budget selection: [passes][select_seqs][H][bins] histograms, zero between calls
+    int32_t select_seqs = 0;             //                         sequences they have room for, grown by the calls
+    bool select_clean = false;           //                         all zero as far as the host knows
     uint32_t *select_arrive = nullptr;   //                         [max_seqs][H] CTAs that are done, zero between launches
     float *select_tau = nullptr;         //                         [max_seqs][H] cut values when the caller wants none
     float *plan_scores = nullptr;        // kvzap_prefill_plan without scores_out: [max_tokens][H] (allocated on first use)
@@ -465,9 +466,26 @@ static kvzap_status hidden_tmap(kvzap_ctx *ctx, CUtensorMap *out, const void *ba
     return KVZAP_OK;
 }
 
-static size_t select_hist_bytes(const kvzap_config &c)
+static size_t select_hist_bytes(const kvzap_config &c, int64_t n_seqs)
 {
-    return sizeof(uint32_t) * kSelectPasses * static_cast<size_t>(c.max_seqs) * c.n_kv_heads * kSelectBins;
+    return sizeof(uint32_t) * kSelectPasses * static_cast<size_t>(n_seqs) * c.n_kv_heads * kSelectBins;
+}
+
+// Room for the selections of n_seqs sequences (at most kSelectSeqs, a call of more takes them in turns): 192 KB each at
+// 8 heads, so a context starts with a few and grows by the calls that come.
+static kvzap_status reserve_select(kvzap_ctx *ctx, int32_t n_seqs)
+{
+    if (n_seqs <= ctx->select_seqs) return KVZAP_OK;
+    int32_t room = ctx->select_seqs > 0 ? ctx->select_seqs : kSelectSeqsFirst;
+    while (room < n_seqs) room *= 2;
+    if (room > kSelectSeqs) room = kSelectSeqs;
+    if (ctx->select_hist) KVZAP_CUDA(ctx, cudaFree(ctx->select_hist));      // waits for the launches that use it
+    ctx->select_hist = nullptr;
+    ctx->select_seqs = 0;
+    ctx->select_clean = false;
+    KVZAP_CUDA(ctx, cudaMalloc(&ctx->select_hist, select_hist_bytes(ctx->cfg, room)));
+    ctx->select_seqs = room;
+    return KVZAP_OK;
 }
 
 static uint32_t *next_mask_slice(kvzap_ctx *ctx)
@@ -1375,7 +1393,12 @@ kvzap_status kvzap_create(kvzap_ctx **out, const kvzap_config *cfg)
     CREATE_CUDA(cudaMemset(ctx->chunk_arrive, 0, sizeof(uint32_t)));
     CREATE_CUDA(cudaMalloc(&ctx->tile_counters, sizeof(int32_t) * kMaskRing));
     CREATE_CUDA(cudaMemset(ctx->tile_counters, 0, sizeof(int32_t) * kMaskRing));
-    CREATE_CUDA(cudaMalloc(&ctx->select_hist, select_hist_bytes(c)));
+    if (reserve_select(ctx, 1) != KVZAP_OK) {
+        snprintf(g_create_error, sizeof g_create_error, "%s", ctx->err);
+        free_all(ctx);
+        delete ctx;
+        return KVZAP_ERR_CUDA;
+    }
     CREATE_CUDA(cudaMalloc(&ctx->select_arrive, sizeof(uint32_t) * static_cast<size_t>(c.max_seqs) * c.n_kv_heads));
     CREATE_CUDA(cudaMemset(ctx->select_arrive, 0, sizeof(uint32_t) * static_cast<size_t>(c.max_seqs) * c.n_kv_heads));
     CREATE_CUDA(cudaMalloc(&ctx->select_tau, sizeof(float) * static_cast<size_t>(c.max_seqs) * c.n_kv_heads));
@@ -1666,23 +1689,32 @@ kvzap_status kvzap_prune_prefill_topk(kvzap_ctx *ctx, const void *K, const void 
     if (st != KVZAP_OK) return st;
     if (!scores) return fail(ctx, KVZAP_ERR_INVALID_ARG, "scores is NULL");
     const int n_sel = per_layer ? 1 : c.n_kv_heads;
-    if (!ctx->select_clean) KVZAP_CUDA(ctx, cudaMemsetAsync(ctx->select_hist, 0, select_hist_bytes(c), stream));
+    const int32_t group = n_seqs < kSelectSeqs ? n_seqs : kSelectSeqs;
+    st = reserve_select(ctx, group);
+    if (st != KVZAP_OK) return st;
+    if (!ctx->select_clean) KVZAP_CUDA(ctx, cudaMemsetAsync(ctx->select_hist, 0, select_hist_bytes(c, ctx->select_seqs), stream));
     ctx->select_clean = false;               // until the launch that clears them is in the stream
-    const dim3 grid(static_cast<unsigned>((n_tokens + kSelectTokens - 1) / kSelectTokens), static_cast<unsigned>(c.n_kv_heads),
-                    static_cast<unsigned>(n_seqs));
-    for (int pass = 0; pass < kSelectPasses; ++pass) {
-        cudaLaunchConfig_t cfg;
-        cudaLaunchAttribute attrs[2];
-        make_launch(&cfg, attrs, grid, dim3(kSelectThreads), 0, stream, !ctx->profiling, 1);
-        KVZAP_CUDA(ctx, cudaLaunchKernelEx(&cfg, select_pass_kernel, scores, n_tokens, static_cast<int>(c.n_kv_heads), cu_seqlens,
-                                           static_cast<int>(n_seqs), static_cast<int>(w), keep_ratio, per_layer ? 1 : 0, pass,
-                                           ctx->select_hist, ctx->select_arrive, tau_list, ctx->status_dev));
-        ctx->launches += 1;
+    int32_t n_now = 0;
+    for (int32_t b0 = 0; b0 < n_seqs; b0 += n_now) {
+        if (b0 > 0) KVZAP_CUDA(ctx, cudaMemsetAsync(ctx->select_hist, 0, select_hist_bytes(c, n_now), stream));
+        n_now = n_seqs - b0 < group ? n_seqs - b0 : group;
+        const dim3 grid(static_cast<unsigned>((n_tokens + kSelectTokens - 1) / kSelectTokens), static_cast<unsigned>(c.n_kv_heads),
+                        static_cast<unsigned>(n_now));
+        for (int pass = 0; pass < kSelectPasses; ++pass) {
+            cudaLaunchConfig_t cfg;
+            cudaLaunchAttribute attrs[2];
+            make_launch(&cfg, attrs, grid, dim3(kSelectThreads), 0, stream, !ctx->profiling, 1);
+            KVZAP_CUDA(ctx, cudaLaunchKernelEx(&cfg, select_pass_kernel, scores, n_tokens, static_cast<int>(c.n_kv_heads),
+                                               cu_seqlens ? cu_seqlens + b0 : nullptr, static_cast<int>(n_now), static_cast<int>(w),
+                                               keep_ratio, per_layer ? 1 : 0, pass, ctx->select_hist, ctx->select_arrive,
+                                               tau_list + static_cast<int64_t>(b0) * c.n_kv_heads, ctx->status_dev));
+            ctx->launches += 1;
+        }
     }
     // the same mask + compaction launch as kvzap_prune_prefill, with the cut values as per-list thresholds
     st = launch_prune_onepass(ctx, scores, tau_list, 0.0f, w, K, V, cu_seqlens, n_seqs, n_tokens, K_out, V_out, lengths, 0,
                               0, 0, 0, nullptr, nullptr, stream, nullptr, false, ctx->select_hist,
-                              static_cast<int64_t>(kSelectPasses) * n_seqs * n_sel * kSelectBins);
+                              static_cast<int64_t>(kSelectPasses) * n_now * n_sel * kSelectBins);
     ctx->select_clean = st == KVZAP_OK;
     return st;
 }

@@ -26,6 +26,10 @@ constexpr int kSelectThreads = 256;
 constexpr int kSelectTokens = 4 * kSelectThreads;      // tokens of a CTA, one head
 constexpr int kSelectPasses = 3;
 constexpr int kSelectBins = 2048;                      // bins stored per pass (the last pass uses half of them)
+// Sequences whose selections run at once: the histograms (kSelectPasses * kSelectBins words per sequence and head) are
+// then at most 50 MB at 8 heads.  A context has room for kSelectSeqsFirst of them from the start.
+constexpr int kSelectSeqs = 256;
+constexpr int kSelectSeqsFirst = 8;
 
 __host__ __device__ constexpr int select_shift(int pass) { return pass == 0 ? 21 : pass == 1 ? 10 : 0; }
 __host__ __device__ constexpr int select_bits(int pass) { return pass == 2 ? 10 : 11; }
@@ -104,7 +108,7 @@ __device__ __forceinline__ uint32_t select_budget(float keep_ratio, int64_t n_ca
     return too_many ? 0xffffffffu : static_cast<uint32_t>(total);
 }
 
-// grid (ceil(n_tokens / kSelectTokens), n_heads, n_seqs); hist [kSelectPasses][n_seqs][n_sel][kSelectBins], n_sel =
+// grid (ceil(n_tokens / kSelectTokens), n_heads, n_seqs), the sequences being cu_seqlens[0 .. n_seqs]; hist [kSelectPasses][n_seqs][n_sel][kSelectBins], n_sel =
 // per_layer ? 1 : n_heads; arrive [n_seqs][n_sel], zero between launches; the last pass writes tau_list [n_seqs][n_heads].
 __global__ void __launch_bounds__(kSelectThreads)
 select_pass_kernel(const float *__restrict__ scores, int64_t n_tokens, int n_heads, const int32_t *__restrict__ cu_seqlens,

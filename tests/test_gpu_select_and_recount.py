@@ -112,3 +112,15 @@ def test_fixed_budget(ctx, lens, window, kind, ratio, per_layer):
         keep[start + n_cand:start + n] = True
         start += n
     _check(K, V, s, lens, window, keep, out)
+
+
+def test_scratch_grows_with_the_calls_not_with_max_seqs():
+    """A context made for many sequences starts small, takes calls of ever more sequences, and still takes small ones."""
+    free = torch.cuda.mem_get_info()[0]
+    c = binding.Kvzap(256, 0, H, D, 1, max_tokens=20000, max_seqs=4096)
+    assert free - torch.cuda.mem_get_info()[0] < 64 << 20
+    rng = np.random.default_rng(4)
+    for n_seqs in (3, 9, 255, 256, 257, 700, 2):
+        lens = [int(x) for x in rng.integers(0, 40 if n_seqs > 9 else 900, n_seqs)]
+        test_fixed_budget(c, lens, 4, "normal", 0.25, n_seqs % 2 == 0)
+    c.close()
