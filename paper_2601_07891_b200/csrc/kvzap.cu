@@ -1698,13 +1698,17 @@ kvzap_status kvzap_prune_prefill_topk(kvzap_ctx *ctx, const void *K, const void 
     for (int32_t b0 = 0; b0 < n_seqs; b0 += n_now) {
         if (b0 > 0) KVZAP_CUDA(ctx, cudaMemsetAsync(ctx->select_hist, 0, select_hist_bytes(c, n_now), stream));
         n_now = n_seqs - b0 < group ? n_seqs - b0 : group;
-        const dim3 grid(static_cast<unsigned>((n_tokens + kSelectTokens - 1) / kSelectTokens), static_cast<unsigned>(c.n_kv_heads),
-                        static_cast<unsigned>(n_now));
+        int64_t per_seq = static_cast<int64_t>(ctx->sm_count) * kSelectCtasPerSm / (static_cast<int64_t>(c.n_kv_heads) * n_now);
+        if (per_seq < 1) per_seq = 1;
+        const int64_t n_blocks = (n_tokens + kSelectTokens - 1) / kSelectTokens;
+        const bool strided = per_seq < n_blocks;
+        if (!strided) per_seq = n_blocks;
+        const dim3 grid(static_cast<unsigned>(per_seq), static_cast<unsigned>(c.n_kv_heads), static_cast<unsigned>(n_now));
         for (int pass = 0; pass < kSelectPasses; ++pass) {
             cudaLaunchConfig_t cfg;
             cudaLaunchAttribute attrs[2];
             make_launch(&cfg, attrs, grid, dim3(kSelectThreads), 0, stream, !ctx->profiling, 1);
-            KVZAP_CUDA(ctx, cudaLaunchKernelEx(&cfg, select_pass_kernel, scores, n_tokens, static_cast<int>(c.n_kv_heads),
+            KVZAP_CUDA(ctx, cudaLaunchKernelEx(&cfg, strided ? select_pass_kernel<true> : select_pass_kernel<false>, scores, n_tokens, static_cast<int>(c.n_kv_heads),
                                                cu_seqlens ? cu_seqlens + b0 : nullptr, static_cast<int>(n_now), static_cast<int>(w),
                                                keep_ratio, per_layer ? 1 : 0, pass, ctx->select_hist, ctx->select_arrive,
                                                tau_list + static_cast<int64_t>(b0) * c.n_kv_heads, ctx->status_dev));

@@ -23,13 +23,17 @@
 namespace kvzap {
 
 constexpr int kSelectThreads = 256;
-constexpr int kSelectTokens = 4 * kSelectThreads;      // tokens of a CTA, one head
+constexpr int kSelectTokens = 4 * kSelectThreads;      // tokens that a CTA counts at a time, one head
 constexpr int kSelectPasses = 3;
 constexpr int kSelectBins = 2048;                      // bins stored per pass (the last pass uses half of them)
 // Sequences whose selections run at once: the histograms (kSelectPasses * kSelectBins words per sequence and head) are
 // then at most 50 MB at 8 heads.  A context has room for kSelectSeqsFirst of them from the start.
 constexpr int kSelectSeqs = 256;
 constexpr int kSelectSeqsFirst = 8;
+// CTAs of a launch per SM, at most: the host does not know how long each sequence is, and a CTA for every block of the whole
+// input in every sequence is mostly CTAs with nothing to do (64 x 1000 tokens: 32256 of them a pass, the call 163 us; now
+// 75 us).  Two launches' worth of resident CTAs, so up to a few sequences every block still has one of its own.
+constexpr int kSelectCtasPerSm = 16;
 
 __host__ __device__ constexpr int select_shift(int pass) { return pass == 0 ? 21 : pass == 1 ? 10 : 0; }
 __host__ __device__ constexpr int select_bits(int pass) { return pass == 2 ? 10 : 11; }
@@ -108,8 +112,11 @@ __device__ __forceinline__ uint32_t select_budget(float keep_ratio, int64_t n_ca
     return too_many ? 0xffffffffu : static_cast<uint32_t>(total);
 }
 
-// grid (ceil(n_tokens / kSelectTokens), n_heads, n_seqs), the sequences being cu_seqlens[0 .. n_seqs]; hist [kSelectPasses][n_seqs][n_sel][kSelectBins], n_sel =
+// grid (n, n_heads, n_seqs), the sequences being cu_seqlens[0 .. n_seqs]: CTA x of a sequence counts its blocks of kSelectTokens
+// tokens x, x + n, x + 2n, ... (kStrided: n may be less than the blocks of the input; the loop over them alone costs 1 us a
+// call where it is not needed); hist [kSelectPasses][n_seqs][n_sel][kSelectBins], n_sel =
 // per_layer ? 1 : n_heads; arrive [n_seqs][n_sel], zero between launches; the last pass writes tau_list [n_seqs][n_heads].
+template <bool kStrided>
 __global__ void __launch_bounds__(kSelectThreads)
 select_pass_kernel(const float *__restrict__ scores, int64_t n_tokens, int n_heads, const int32_t *__restrict__ cu_seqlens,
                    int n_seqs, int window, float keep_ratio, int per_layer, int pass, uint32_t *__restrict__ hist,
@@ -137,11 +144,14 @@ select_pass_kernel(const float *__restrict__ scores, int64_t n_tokens, int n_hea
         return;
     }
     float v[4];
+    auto load = [&](int64_t c) {
 #pragma unroll
-    for (int j = 0; j < 4; ++j) {
-        const int64_t i = c0 + j * kSelectThreads + tid;
-        v[j] = i < n_cand ? __ldcg(scores + (t0 + i) * n_heads + h) : __uint_as_float(0x7fffffffu);      // NaN: no candidate
-    }
+        for (int j = 0; j < 4; ++j) {
+            const int64_t i = c + j * kSelectThreads + tid;
+            v[j] = i < n_cand ? __ldcg(scores + (t0 + i) * n_heads + h) : __uint_as_float(0x7fffffffu);      // NaN: no candidate
+        }
+    };
+    load(c0);
     for (int i = tid; i < kSelectBins; i += kSelectThreads) sh[i] = 0u;
     if (pass > 0) griddep_wait();
     const int n_sel = per_layer ? 1 : n_heads, sel = b * n_sel + (per_layer ? 0 : h);
@@ -167,11 +177,21 @@ select_pass_kernel(const float *__restrict__ scores, int64_t n_tokens, int n_hea
     __syncthreads();
     if (!dead) {
         const int shift = select_shift(pass), bits = select_bits(pass);
+        auto count = [&]() {
 #pragma unroll
-        for (int j = 0; j < 4; ++j) {
-            if (v[j] != v[j]) continue;
-            const uint32_t key = score_key(v[j]);
-            if (pass == 0 || (key >> (shift + bits)) == prefix) atomicAdd(&sh[(key >> shift) & ((1u << bits) - 1u)], 1u);
+            for (int j = 0; j < 4; ++j) {
+                if (v[j] != v[j]) continue;
+                const uint32_t key = score_key(v[j]);
+                if (pass == 0 || (key >> (shift + bits)) == prefix) atomicAdd(&sh[(key >> shift) & ((1u << bits) - 1u)], 1u);
+            }
+        };
+        count();
+        if constexpr (kStrided) {
+            const int64_t stride = static_cast<int64_t>(gridDim.x) * kSelectTokens;
+            for (int64_t c = c0 + stride; c < n_cand; c += stride) {
+                load(c);
+                count();
+            }
         }
     }
     __syncthreads();
@@ -186,7 +206,9 @@ select_pass_kernel(const float *__restrict__ scores, int64_t n_tokens, int n_hea
     __syncthreads();
     if (tid == 0) {
         if (too_many) atomicCAS(status, 0, 2 /* KVZAP_ERR_UNSUPPORTED */);
-        const uint32_t n_ctas = static_cast<uint32_t>((n_cand + kSelectTokens - 1) / kSelectTokens) * (per_layer ? n_heads : 1);
+        uint32_t n_ctas = static_cast<uint32_t>((n_cand + kSelectTokens - 1) / kSelectTokens);
+        if constexpr (kStrided) n_ctas = min(n_ctas, gridDim.x);
+        if (per_layer) n_ctas *= n_heads;
         last_s = atomicAdd(arrive + sel, 1u) + 1u == n_ctas;
         if (last_s) arrive[sel] = 0u;
         __threadfence();

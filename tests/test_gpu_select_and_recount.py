@@ -124,3 +124,16 @@ def test_scratch_grows_with_the_calls_not_with_max_seqs():
         lens = [int(x) for x in rng.integers(0, 40 if n_seqs > 9 else 900, n_seqs)]
         test_fixed_budget(c, lens, 4, "normal", 0.25, n_seqs % 2 == 0)
     c.close()
+
+
+def test_few_blocks_in_flight_per_sequence():
+    """So many sequences that a long one's blocks are counted by fewer CTAs than it has blocks, one after the other."""
+    c = binding.Kvzap(256, 0, H, D, 1, max_tokens=40000, max_seqs=400)
+    for n_seqs, longest in ((60, 9000), (150, 5121), (400, 17000)):
+        rng = np.random.default_rng(n_seqs)
+        lens = [int(x) for x in rng.integers(0, 30, n_seqs)]
+        lens[n_seqs // 2], lens[7] = longest, 2048 + 16
+        for per_layer in (False, True):
+            test_fixed_budget(c, lens, 16, "normal", 0.25, per_layer)
+        test_fixed_budget(c, lens, 16, "low bits", 0.37, False)
+    c.close()
