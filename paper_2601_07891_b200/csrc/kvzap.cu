@@ -62,7 +62,7 @@ struct kvzap_ctx {
         CUtensorMap tmap_w;
         CUtensorMap tmap_w8;             // the 8-bit copy of the weights, same slices (set by kvzap_set_weights_fp8)
         bool ok8 = false;
-        uint32_t *arrive = nullptr;      // [sm_count] arrivals per tile over all launches (taken modulo the slices)
+        uint32_t *arrive = nullptr;      // [sm_count] slices of a tile that have arrived, zero between launches
     };
     static constexpr int kMaxLayouts = 4;
     SplitLayout layouts[kMaxLayouts];

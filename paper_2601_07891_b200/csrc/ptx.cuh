@@ -309,6 +309,14 @@ __device__ __forceinline__ void st_release_gpu(int32_t *p, int32_t v)
     asm volatile("st.release.gpu.global.s32 [%0], %1;" ::"l"(p), "r"(v) : "memory");
 }
 
+// Counts one of n arrivals in: true for the last one, and the counter is back at zero with it.  (A count that runs on over
+// all launches and is taken modulo n goes wrong for good when it wraps, unless n is a power of two: 2^32 arrivals of five
+// per launch are some hours of decoding.)
+__device__ __forceinline__ bool arrive_last(uint32_t *counter, uint32_t n)
+{
+    return atomicInc(counter, n - 1u) == n - 1u;
+}
+
 // ---------------------------------------------------------------- programmatic dependent launch
 // A kernel launched with the programmatic-stream-serialization attribute may start once every CTA
 // of the kernel before it in the stream has executed griddep_launch_dependents() (or exited);

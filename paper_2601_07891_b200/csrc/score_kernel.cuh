@@ -87,7 +87,7 @@ struct ScoreParams {
     const float *w1_scale;        // stacked over all layers [L][w_rows], one scale per first-layer output row
     // few-token kernel only: the clusters of one tile combine their partial scores through global memory
     float *split_part;            // [n_tiles][n_split][128][8]
-    uint32_t *split_arrive;       // [n_tiles] arrivals so far, over all launches (never reset in normal use)
+    uint32_t *split_arrive;       // [n_tiles] slices that have arrived, zero between launches
 };
 
 // Byte offsets inside the dynamic shared memory block (after 1024-byte alignment).

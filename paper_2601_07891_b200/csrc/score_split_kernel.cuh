@@ -513,8 +513,7 @@ score_split_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_cons
             __threadfence();
             named_barrier_sync(2, 128);
             if (threadIdx.x == 64) {
-                const uint32_t before = atomicAdd(p.split_arrive + tile, 1u);
-                *last_flag = (before + 1u) % static_cast<uint32_t>(n_split) == 0u ? 1 : 0;
+                *last_flag = arrive_last(p.split_arrive + tile, static_cast<uint32_t>(n_split)) ? 1 : 0;
                 __threadfence();
             }
             named_barrier_sync(2, 128);

@@ -1,6 +1,11 @@
 """GPU parity of the few-token scoring kernel over the layouts it chooses by the number of 128-token tiles: scores at
 the sizes where one layout gives way to the next, and decode steps of one cache that change layout from call to call
 (all layers in one call, then layer by layer), against the CPU oracle."""
+import ctypes
+import os
+import shutil
+import subprocess
+
 import numpy as np
 import pytest
 import torch
@@ -9,6 +14,8 @@ from paper_2601_07891_b200 import binding, synth
 from tests import parity
 
 pytestmark = pytest.mark.gpu
+
+HERE = os.path.dirname(os.path.abspath(__file__))
 
 # An fp32 pre-activation is a chain of at most d_model / 16 + 8 additions of partial sums below 6 in magnitude, each off
 # by at most 2^-23 of it; the second layer adds up |w2| of `hidden` of them: 0.8 sqrt(hidden) * 6 * 2^-23 * 72 at
@@ -86,3 +93,23 @@ def test_decode_steps_that_change_layout(oracle, B, L, trusted):
                     np.testing.assert_array_equal(synth.bits(out[1])[:m], Vd)
     binding.kvzap_cache_destroy(cache)
     ctx.close()
+
+
+@pytest.mark.parametrize("n", [2, 4, 5, 8])
+def test_arrivals_of_the_slices_do_not_add_up_over_launches(n):
+    """Every n-th arrival is the last of its launch and leaves the counter at zero, so that no number of launches wraps it."""
+    lib = os.path.join(HERE, "_build", "libarrivals.so")
+    os.makedirs(os.path.dirname(lib), exist_ok=True)
+    subprocess.run([shutil.which("nvcc") or "/usr/local/cuda/bin/nvcc", "-gencode", "arch=compute_100a,code=sm_100a", "-O2",
+                    "-std=c++17", "-shared", "-Xcompiler", "-fPIC", "-o", lib, os.path.join(HERE, "helpers", "arrivals.cu")],
+                   check=True)
+    launch = ctypes.CDLL(lib).launch_arrivals
+    launch.argtypes = [ctypes.c_void_p, ctypes.c_uint, ctypes.c_int] + 3 * [ctypes.c_void_p]
+    rounds = 7
+    counter = torch.zeros(1, dtype=torch.int32, device="cuda")
+    last, after = (torch.full((rounds * n,), -1, dtype=torch.int32, device="cuda") for _ in range(2))
+    for _ in range(2):
+        assert launch(counter.data_ptr(), n, rounds, last.data_ptr(), after.data_ptr(), torch.cuda.current_stream().cuda_stream) == 0
+        torch.cuda.synchronize()
+        assert last.tolist() == ([0] * (n - 1) + [1]) * rounds
+        assert after.tolist() == (list(range(1, n)) + [0]) * rounds
