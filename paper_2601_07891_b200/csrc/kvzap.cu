@@ -1086,7 +1086,11 @@ static kvzap_status launch_prune_onepass(kvzap_ctx *ctx, const float *scores, co
     }
     // A launch that waits for the work ahead takes every slot of the device (32k tokens, a quarter kept: 40 -> 31 us); one
     // that may run beside the launch ahead (and the one behind it beside this one) half of them, and so does the paged
-    // output, whose CTAs all wait for one another: two such launches on two streams still fit side by side.
+    // output, whose CTAs all wait for one another: two such launches on two streams still fit side by side.  Half of them
+    // too where one block per CTA of one sequence would leave an eighth of the slots empty: some SMs then work on two CTAs
+    // and the others idle, which half as many CTAs of two blocks do not (8 heads: 3000 tokens 11.2 -> 10.0 us, 4000 tokens
+    // 11.5 -> 10.5 us; 4 heads, 9000 tokens, 284 CTAs: 9.9 us with all slots, 11.0 us with half; 64 x 250 tokens, 2 heads,
+    // 250 CTAs: 15.2 and 15.8 us).
     // Heads per CTA: as many as still leave a CTA a dozen blocks or more.  The one CTA that holds a sequence's window
     // keeps all rows of a block where the others keep a quarter or a third; with many blocks per CTA that is a small
     // surplus, with two or three it would make that CTA the last to finish by far.
@@ -1095,7 +1099,10 @@ static kvzap_status launch_prune_onepass(kvzap_ctx *ctx, const float *scores, co
     for (int hg = kMaxHeads; hg >= 1; hg >>= 1) {
         heads_per_cta = hg;
         groups = (c.n_kv_heads + hg - 1) / hg;
-        grid = ctx->op_capacity * (wait_first && page_tokens == 0 ? 2 : 1) / groups;
+        const bool all_slots = wait_first && page_tokens == 0 &&
+                               (n_seqs > 1 || 2 * (ctx->op_capacity / groups) < n_blocks ||
+                                n_blocks * groups * 8 >= 14 * static_cast<int64_t>(ctx->op_capacity));
+        grid = ctx->op_capacity * (all_slots ? 2 : 1) / groups;
         if (grid < 1) grid = 1;
         if (grid > n_blocks) grid = n_blocks;
         per_cta = (n_blocks + grid - 1) / grid;

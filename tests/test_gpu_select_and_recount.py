@@ -61,7 +61,8 @@ def _inputs(T, lens, kind):
 
 @pytest.mark.parametrize("lens,window", [
     ([1], 0), ([127], 16), ([129], 200), ([2176], 128), ([2177], 128), ([2305], 0), ([500, 501, 500], 128), ([3, 0, 700, 0, 1, 900, 128], 16),
-    ([128, 128, 256], 128), ([1000, 1176], 64), ([1000, 1305], 64), ([20000], 128)])
+    ([128, 128, 256], 128), ([1000, 1176], 64), ([1000, 1305], 64), ([3000], 128), ([4097], 128), ([4200], 16), ([9000], 128),
+    ([20000], 128)])
 @pytest.mark.parametrize("kind", ["normal", "special"])
 def test_threshold(ctx, lens, window, kind):
     T, tau = sum(lens), 0.5
