@@ -537,10 +537,17 @@ struct CompactArgs {
 // at 4096 -> 512 -> 8, one launch: a decode step of one tile 27.5 us with 2 x 2 CTAs, 15.0 us with 4 x 8; the scoring of
 // 7 tiles 20.3 us with 4 x 2, 13.5 us with 4 x 4.  What bounds a launch is one CTA's load, (128 + hidden / n) * d_model / k
 // elements at about 55 bytes per clock, on top of some 8 us for its serial parts.
-static int split_layout(const kvzap_ctx *ctx, int64_t n_tiles, bool fp8)
+// beside: a launch that may run beside the ones ahead of it and behind it (prompts of a context that trusts its producers):
+// more than eight CTAs per tile only where a third of the SMs hold them, or its neighbours find no room.  Six layers of
+// a prompt in a row, widest layout against this rule: 777 tokens 71.5 -> 63.7 us at 4096 -> 512, 90.8 -> 64.1 us at
+// 4096 -> 1024, 300 tokens 67.0 -> 56.6 us at 4096 -> 640; with a synchronisation behind the six 88.2 -> 82.8, 108.6 -> 96.8,
+// 83.2 -> 77.0 us.  Not for the scoring of a chunk, behind which the window side and the compaction wait (a chunk of 1000
+// tokens through four layers, three times: 378 us, 418 us by this rule), nor for decode steps in one launch.
+static int split_layout(const kvzap_ctx *ctx, int64_t n_tiles, bool fp8, bool beside = false)
 {
     for (int i = 1; i < ctx->n_layouts; ++i) {
         const kvzap_ctx::SplitLayout &l = ctx->layouts[i];
+        if (beside && l.n * l.k > 8 && n_tiles * l.n * l.k * 3 > ctx->sm_count) continue;
         if ((!fp8 || l.ok8) && n_tiles * l.n * l.k <= ctx->sm_count && n_tiles * l.n <= l.max_clusters) return i;
     }
     if (ctx->n_layouts > 0 && (!fp8 || ctx->layouts[0].ok8) &&
@@ -582,7 +589,7 @@ static kvzap_status launch_score(kvzap_ctx *ctx, int32_t layer, int32_t n_layers
     // range) the same kernel serves launches of up to half as many tiles as there are SMs, where CTA pairs
     // would leave most SMs idle.
     const int64_t few_tiles = blocks_per_layer * n_layers;
-    const int layout_i = split_layout(ctx, few_tiles, fp8);
+    const int layout_i = split_layout(ctx, few_tiles, fp8, ctx->trusted && fuse == nullptr && !late_trigger);
     const bool slices_only = layout_i < 0 && ctx->n_layouts > 0 && ctx->layouts[0].n == 2 && ctx->layouts[0].k == 2 &&
                              fuse == nullptr && !fp8 && few_tiles * 2 <= ctx->sm_count;
     if (fp8 && layout_i < 0)

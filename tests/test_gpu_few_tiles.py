@@ -113,3 +113,27 @@ def test_arrivals_of_the_slices_do_not_add_up_over_launches(n):
         torch.cuda.synchronize()
         assert last.tolist() == ([0] * (n - 1) + [1]) * rounds
         assert after.tolist() == (list(range(1, n)) + [0]) * rounds
+
+
+@pytest.mark.parametrize("hidden", [256, 512, 640, 1024])
+@pytest.mark.parametrize("T", [1, 128, 129, 300, 640, 777, 2305])
+def test_scores_of_the_layouts_that_leave_room_for_other_launches(oracle, hidden, T):
+    """Contexts that trust their producers take narrower layouts for prompts: layers back to back, each its own buffers."""
+    d_model, H, L = 1024, 8, 3
+    ctx = binding.Kvzap(d_model, hidden, H, 64, L, max_tokens=T, trusted_producers=True)
+    X = synth.hidden_states(T, d_model, seed=T + hidden)
+    wts = [synth.mlp_weights(d_model, hidden, H, 50 + l, "cpu", 0.3) for l in range(L)]
+    for l in range(L):
+        ctx.set_weights(l, *[parity.dev(x) for x in wts[l]])
+    Xd = parity.dev(X)
+    scores = [torch.full((T, H), 7.0, dtype=torch.float32, device="cuda") for _ in range(L)]
+    torch.cuda.synchronize()
+    for l in range(L):
+        ctx.score(l, Xd, out=scores[l])
+    torch.cuda.synchronize()
+    assert ctx.poll_status() == 0
+    rows = np.unique(np.concatenate([np.arange(min(T, 160)), np.arange(max(0, T - 160), T)]))
+    for l in range(L):
+        _, err = parity.check_scores(oracle, scores[l], X, wts[l], rows)
+        assert err <= ATOL
+    ctx.close()
