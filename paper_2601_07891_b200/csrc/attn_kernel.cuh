@@ -56,8 +56,10 @@ namespace kvzap {
 constexpr int kAttnWarps = 4;
 // Stages of a warp's ring.  bf16 rows: two, so that three CTAs fit an SM (168 registers, 66 KB) -- the same bytes in flight as
 // two CTAs with three stages, but the serial parts of a CTA (counts, pages, first tiles, merge: some 3 us) run beside two
-// others: 128 sequences x 4 layers, layer by layer, 1553 -> 1527 us; 80 x 8 layers 1245 -> 1175 us.  8-bit rows: three,
-// four CTAs fit either way.
+// others: 128 sequences x 4 layers, layer by layer, 1553 -> 1527 us; 80 x 8 layers 1245 -> 1175 us.  Rows of 64 elements (122
+// registers, half the bytes a stage): two or three make 0 to 5 % either way (8 sequences x 2000 rows 13.6 / 14.3 us, 64 x
+// 300 12.9 / 13.3, 128 x 4000 169.8 / 169.6, 512 x 200 50.2 / 49.2), so they have two as well.  8-bit rows: three, four CTAs
+// fit either way.
 __host__ __device__ constexpr int attn_stages(bool fp8) { return fp8 ? 3 : 2; }
 constexpr int kAttnTileRows = 16;
 constexpr int kAttnThreads = kAttnWarps * 32;

@@ -2472,12 +2472,15 @@ static kvzap_status attention_impl(kvzap_ctx *ctx, kvzap_cache *cache, int32_t l
     p.status = ctx->status_dev;
     const int64_t n_lists_call = static_cast<int64_t>(p.n_layers_call) * v.n_seqs * v.n_heads;
     if (n_lists_call > 0x7fffffffLL) return fail(ctx, KVZAP_ERR_UNSUPPORTED, "attention: too many lists for one launch");
-    // Three CTAs fit an SM (four of the 8-bit kernel's).  Fewer lists than that: one wave, whose CTAs share the lists out
-    // by their lengths.  More: every list in as many parts as make some 24 CTAs per SM -- a CTA costs about 3 us beside its
+    // Three CTAs fit an SM (four of the 8-bit kernel's; of both kernels' for rows of 64 elements, where three are counted all
+    // the same: with four, 8-bit rows, 56 sequences x 300 rows 31.7 -> 17.7 us, 55 x 1500 50 -> 43 us, but 64 x 300 13.8 ->
+    // 20.1 us, one of 20000 rows 19.6 -> 21.0 us).  Fewer lists than that: one wave, whose CTAs share the lists out by their
+    // lengths.  More: every list in as many parts as make some 24 CTAs per SM -- a CTA costs about 3 us beside its
     // share of the rows, the last ones leave SMs idle -- but none shorter than 1200 rows of the longest list the cache can
     // hold.  512 lists of 1600 rows: 9 parts 1062 us, 2 parts 763 us (8 layers, with their steps); 1024 lists of 750 rows:
     // 4 parts 490 us, 1 part 355 us, of 4700 rows: 1 part 1678 us, 3 parts 1527 us (4 layers).  320 lists, by their
-    // lengths: 898 us against 1115 us in 14 equal parts (8 layers).
+    // lengths: 898 us against 1115 us in 14 equal parts (8 layers).  The capacity stands for the lengths, which the host does
+    // not know: 1024 lists of 300 rows take 32.8 us in a table for as many, 51.8 us in one for 32768.
     const int64_t slots = static_cast<int64_t>(ctx->sm_count) * (fp8 && d_attn == 128 ? 4 : 3);
     int64_t n_ctas = n_lists_call;
     p.n_parts = 1;

@@ -20,9 +20,11 @@
 //      byte offsets, listed in shared memory; then one loop moves whole rows with 16-byte accesses, 16
 //      lanes per row, two register sets per lane group so that loads are in flight while the rows before
 //      them are stored.
-// The grid never exceeds half the CTAs the device holds at once: a CTA that waits for another waits for
-// one that is running or about to, and the next call's kernel finds room to do its steps A and B while
-// this one moves rows.  Every wait is bounded all the same (status word, KVZAP_ERR_TIMEOUT, nothing
+// The grid never exceeds what the device holds at once.  Paged output, where all CTAs wait for one another, and launches that
+// may start beside the one ahead take half of that at most: two such launches on two streams fit side by side, and the next
+// call's kernel finds room to do its steps A and B while this one moves rows.  Dense output that waits for the work ahead may
+// take all of it: a CTA there waits only for CTAs of its head group with a lower column, which the device dispatches before
+// it, so whatever else holds slots, the lowest column not yet done is always running.  Every wait is bounded all the same (status word, KVZAP_ERR_TIMEOUT, nothing
 // written).  The scratch of consecutive calls rotates (the host explains the overlap rules).
 #pragma once
 

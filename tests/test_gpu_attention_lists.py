@@ -1,5 +1,5 @@
-"""Attention over few lists of very unequal length, where the CTAs share the lists out by their lengths: around the
-number of resident CTAs at which that rule ends, empty lists, one list that holds nearly all rows, a layer range, both
+"""Attention over few lists of very unequal length, where the CTAs share the lists out by their lengths: on both sides of
+the number of resident CTAs at which that rule ends, empty lists, one list that holds nearly all rows, a layer range, both
 row formats.  Against softmax attention in fp64 over the rows that were imported."""
 import numpy as np
 import pytest
@@ -77,3 +77,12 @@ def test_attention_over_unequal_lists(fp8, D, B, L, layers, kind):
     assert float((O.double() - want).abs().max()) <= ATTN_ATOL
     binding.kvzap_cache_destroy(cache)
     ctx.close()
+
+
+@pytest.mark.parametrize("fp8,D", [(False, 128), (False, 64), (True, 128), (True, 64)])
+@pytest.mark.parametrize("kind", ["log", "equal", "one"])
+@pytest.mark.parametrize("past", [0, 1])
+def test_attention_where_sharing_by_length_ends(fp8, D, kind, past):
+    """The largest batch with fewer lists than resident CTAs (three per SM, four of the 8-bit kernel's at 128), and the next."""
+    slots = torch.cuda.get_device_properties(0).multi_processor_count * (4 if fp8 and D == 128 else 3)
+    test_attention_over_unequal_lists(fp8, D, (slots - 1) // H + past, 1, (0, 1), kind)
