@@ -478,7 +478,7 @@ static kvzap_status reserve_select(kvzap_ctx *ctx, int32_t n_seqs)
     if (n_seqs <= ctx->select_seqs) return KVZAP_OK;
     int32_t room = ctx->select_seqs > 0 ? ctx->select_seqs : kSelectSeqsFirst;
     while (room < n_seqs) room *= 2;
-    if (room > kSelectSeqs) room = kSelectSeqs;
+    room = std::min({room, kSelectSeqs, ctx->cfg.max_seqs});      // n_seqs is above neither
     if (ctx->select_hist) KVZAP_CUDA(ctx, cudaFree(ctx->select_hist));      // waits for the launches that use it
     ctx->select_hist = nullptr;
     ctx->select_seqs = 0;
