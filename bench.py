@@ -45,8 +45,8 @@ NCU_TRAFFIC_FP8 = {
     "qwen3_8b_prefill_32k": (140.4e6, "profiles/score_kernel_mlp_fp8_qwen3_8b_prefill_32k.md"),
 }
 # attention over the pruned cache: DRAM bytes per ALGORITHMIC byte, from a one-layer capture (traffic grows with the rows read)
-NCU_ATTENTION_TRAFFIC_RATIO = 2.4093 / 2.3986
-NCU_ATTENTION_FP8_TRAFFIC_RATIO = 1.3609 / 1.3501
+NCU_ATTENTION_TRAFFIC_RATIO = 2.4087 / 2.3986
+NCU_ATTENTION_FP8_TRAFFIC_RATIO = 1.3626 / 1.3501
 
 
 def load_peaks():
