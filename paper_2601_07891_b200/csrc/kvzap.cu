@@ -555,6 +555,49 @@ static int split_layout(const kvzap_ctx *ctx, int64_t n_tiles, bool fp8, bool be
     return -1;
 }
 
+// Blocks of a prompt that whole waves of CTA pairs leave over and that the few-token kernel takes instead, in a launch of its
+// own behind them (launch_score_rest): a wave lasts as long for one tile as for all of them.  4096 -> 512 -> 8, calls in a
+// row: 19500 tokens (5 blocks more than a wave) 114 -> 89 us a call, 22000 tokens (24 blocks more) 116 -> 103 us; with 8-bit
+// inputs 77 -> 61 us and 79 -> 70 us.  0 where there are more blocks than that kernel takes, or no whole wave; and on contexts
+// that trust their producers, whose next launch fills the last wave.
+static int64_t rest_blocks(const kvzap_ctx *ctx, int64_t blocks, bool fp8)
+{
+    const int64_t wave = 2 * static_cast<int64_t>(ctx->pair_clusters);
+    if (ctx->trusted || ctx->profiling || ctx->cfg.hidden == 0 || wave == 0 || blocks <= wave) return 0;
+    const int64_t rest = blocks % wave;
+    return rest > 0 && split_layout(ctx, rest, fp8) >= 0 ? rest : 0;
+}
+
+// The few-token kernel over the blocks from block0 on, directly behind the launch over those before (p, one layer), which lets
+// it start once all work ahead of that launch has completed: it loads at once and waits before it writes.
+static kvzap_status launch_score_rest(kvzap_ctx *ctx, ScoreParams p, const CUtensorMap &tmap_x, int64_t block0, bool fp8, cudaStream_t stream)
+{
+    const int64_t rest = p.blocks_per_layer - block0;
+    const kvzap_ctx::SplitLayout &layout = ctx->layouts[split_layout(ctx, rest, fp8)];
+    p.block0 = static_cast<int32_t>(block0);
+    p.n_tiles = p.tiles_per_layer = static_cast<int32_t>(rest);
+    p.group_w = p.chunk_n = ctx->cfg.hidden / layout.n;
+    p.n_groups = p.n_chunks = 1;
+    p.n_stages = layout.stages;
+    p.acc_bufs = 1;
+    p.tmem_cols = layout.tmem_cols;
+    p.wait_before_load = p.late_trigger = 0;
+    p.split_part = ctx->split_part;
+    p.split_arrive = layout.arrive;
+    DecodeFuse f;
+    memset(&f, 0, sizeof f);
+    ProfScope prof(ctx, KVZAP_KERNEL_SCORE, stream);
+    cudaLaunchConfig_t cfg;
+    cudaLaunchAttribute attrs[2];
+    make_launch(&cfg, attrs, dim3(static_cast<unsigned>(rest * layout.n * layout.k)), dim3(kScoreThreads), layout.smem, stream, true, layout.k);
+    if (fp8)
+        KVZAP_CUDA(ctx, cudaLaunchKernelEx(&cfg, score_split_kernel<true>, tmap_x, layout.tmap_w8, p, layout.n, layout.k, f));
+    else
+        KVZAP_CUDA(ctx, cudaLaunchKernelEx(&cfg, score_split_kernel<false>, tmap_x, layout.tmap_w, p, layout.n, layout.k, f));
+    ctx->launches += 1;
+    return KVZAP_OK;
+}
+
 // Launches the scoring kernel over layers [layer, layer + n_layers); hidden is [n_layers][n_tokens][d_model],
 // scores [n_layers][n_tokens][H]; maskbits != nullptr fuses the threshold/window test.
 static kvzap_status launch_score(kvzap_ctx *ctx, int32_t layer, int32_t n_layers, const void *hidden, int64_t n_tokens,
@@ -803,7 +846,8 @@ static kvzap_status launch_score(kvzap_ctx *ctx, int32_t layer, int32_t n_layers
     const bool pair = c.hidden > 0 && ctx->pair_clusters > 0 && blocks_per_layer >= 2;
     const kvzap_ctx::Schedule &sc = ctx->sched[pair ? 1 : 0];
     const int64_t tiles_per_layer = pair ? (blocks_per_layer + 1) / 2 : blocks_per_layer;
-    const int64_t n_tiles = tiles_per_layer * n_layers;
+    const int64_t rest = pair && n_layers == 1 && fuse_chain == nullptr ? rest_blocks(ctx, blocks_per_layer, false) : 0;
+    const int64_t n_tiles = rest > 0 ? (blocks_per_layer - rest) / 2 : tiles_per_layer * n_layers;
     CUtensorMap tmap_x;
     kvzap_status st = hidden_tmap(ctx, &tmap_x, hidden, n_tokens, n_layers);
     if (st != KVZAP_OK) return st;
@@ -843,7 +887,7 @@ static kvzap_status launch_score(kvzap_ctx *ctx, int32_t layer, int32_t n_layers
     // A decode step in two launches: behind a launch that waits, the update moves its rows beside the scoring (see
     // decode_update_kernel).  Trusted producers: this launch runs beside the step before instead and the update waits;
     // 64 layers x 8 sequences 68 us a step against 75 us with both steps in a row, default contexts 75 against 80 us.
-    p.late_trigger = fuse_chain != nullptr && p.wait_before_load;
+    p.late_trigger = (fuse_chain != nullptr || rest > 0) && p.wait_before_load;
     // every launch finds its counter at zero: it was cleared by the launch before the previous one
     p.tile_counter = ctx->tile_counters + ctx->score_turn % kMaskRing;
     p.tile_counter_reset = ctx->tile_counters + (ctx->score_turn + 2) % kMaskRing;
@@ -881,21 +925,30 @@ static kvzap_status launch_score(kvzap_ctx *ctx, int32_t layer, int32_t n_layers
     }
     KVZAP_CUDA(ctx, cudaGetLastError());
     ctx->launches += 1;
-    return KVZAP_OK;
+    if (rest == 0) return KVZAP_OK;
+    ctx->last_score_late = true;
+    return launch_score_rest(ctx, p, tmap_x, blocks_per_layer - rest, false, stream);
 }
 
 // Scoring with 8-bit inputs: hidden [n_tokens][d_model] E4M3 bytes with one scale per token, the layer's first-layer
-// weights given by kvzap_set_weights_fp8.  Always the persistent kernel (CTA pairs for the MLP from two blocks on);
-// the waits before loads and stores follow the rules of launch_score.
+// weights given by kvzap_set_weights_fp8.  Few tiles go to the few-token kernel as in launch_score, others to the persistent
+// kernel (CTA pairs for the MLP from two blocks on); the waits before loads and stores follow the rules of launch_score.
 static kvzap_status launch_score_fp8(kvzap_ctx *ctx, int32_t layer, const void *hidden8, const float *x_scale, int64_t n_tokens,
                                      float *scores, uint32_t *maskbits, const int32_t *cu_seqlens, int32_t n_seqs, float tau,
                                      int32_t w, cudaStream_t stream, bool update_behind = false)
 {
     const kvzap_config &c = ctx->cfg;
     const int64_t blocks_per_layer = (n_tokens + kTileM - 1) / kTileM;
+    // On a context that trusts its producers the small grids of the persistent kernel run beside one another instead (777
+    // tokens 9.7 us a call, with the few-token kernel 10.9); elsewhere a call waits for the one before, and 200 / 777 / 2200 /
+    // 3900 tokens take 13.5 / 15 / 18 / 25 us where one CTA pair per 256 tokens takes 36 to 38 (4096 -> 512 -> 8).
+    if (!ctx->trusted && split_layout(ctx, blocks_per_layer, true) >= 0)
+        return launch_score(ctx, layer, 1, hidden8, n_tokens, scores, maskbits, cu_seqlens, n_seqs, tau, w, stream, 1, nullptr, nullptr,
+                            nullptr, nullptr, nullptr, true, x_scale);
     const bool pair = c.hidden > 0 && ctx->pair_clusters > 0 && blocks_per_layer >= 2;
     const kvzap_ctx::Schedule &sc = ctx->sched[pair ? 1 : 0];
-    const int64_t n_tiles = pair ? (blocks_per_layer + 1) / 2 : blocks_per_layer;
+    const int64_t rest = pair && !update_behind ? rest_blocks(ctx, blocks_per_layer, true) : 0;
+    const int64_t n_tiles = pair ? (blocks_per_layer - rest + 1) / 2 : blocks_per_layer;
     CUtensorMap tmap_x;
     kvzap_status st = make_tmap8(ctx, &tmap_x, hidden8, static_cast<uint64_t>(n_tokens), static_cast<uint64_t>(c.d_model), kTileM, 1, false);
     if (st != KVZAP_OK) return st;
@@ -932,7 +985,7 @@ static kvzap_status launch_score_fp8(kvzap_ctx *ctx, int32_t layer, const void *
     p.tau = tau;
     p.status = ctx->status_dev;
     p.wait_before_load = ctx->trusted ? 0 : 1;
-    p.late_trigger = update_behind && p.wait_before_load;      // as in launch_score
+    p.late_trigger = (update_behind || rest > 0) && p.wait_before_load;      // as in launch_score
     p.k_blocks = c.d_model / 128;
     p.k_elems = 128;
     p.x_scale = x_scale;
@@ -970,7 +1023,7 @@ static kvzap_status launch_score_fp8(kvzap_ctx *ctx, int32_t layer, const void *
         }
     }
     ctx->launches += 1;
-    return KVZAP_OK;
+    return rest == 0 ? KVZAP_OK : launch_score_rest(ctx, p, tmap_x, blocks_per_layer - rest, true, stream);
 }
 
 // The launch of the compaction kernel over n_blocks blocks of every head.

@@ -124,7 +124,7 @@ score_split_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_cons
     const int pos = nh * k_split + kh;                   // this CTA among the n_ctas of its tile
     const int tile = static_cast<int>(blockIdx.x) / n_ctas;
     const int l_rel = tile / p.tiles_per_layer;
-    const int m_tile = tile - l_rel * p.tiles_per_layer;
+    const int m_tile = tile - l_rel * p.tiles_per_layer + p.block0;
     const int layer = p.layer0 + l_rel;
     if (f.enabled) {
         // the step number, drawn before any thread of this CTA lets the next launch be placed: a CTA of that launch
