@@ -796,13 +796,16 @@ static kvzap_status launch_score(kvzap_ctx *ctx, int32_t layer, int32_t n_layers
             // the same rule as for the one-launch pruning kernel: rows and counts are written before the work
             // ahead has completed only directly behind launches whose memory is on the pending list and does
             // not conflict
-            bool wait_first = !ctx->trusted || ctx->profiling || ctx->op_last_seq + 1 != ctx->op_seq || ctx->op_chain >= kOpRing - 2 ||
-                              clash;
+            bool wait_first = !ctx->trusted || ctx->profiling || ctx->op_last_seq + 1 != ctx->op_seq || ctx->op_chain >= kOpRing - 2;
             if (!wait_first)
                 wait_first = hazard(ctx, hidden, static_cast<size_t>(n_tokens) * c.d_model * 2, false) ||
-                             hazard(ctx, compact->K, kv_bytes, false) || hazard(ctx, compact->V, kv_bytes, false) ||
-                             hazard(ctx, compact->K_out, kv_bytes, true) || hazard(ctx, compact->V_out, kv_bytes, true) ||
-                             hazard(ctx, compact->lengths, sizeof(int32_t) * c.n_kv_heads, true);
+                             hazard(ctx, compact->K, kv_bytes, false) || hazard(ctx, compact->V, kv_bytes, false);
+            // Only what it writes is still in use (an output buffer of one of the last calls again): everything up to the
+            // loads of the rows goes ahead, its stores wait.  It stays a link of the chain: what follows may still meet the
+            // launches ahead of it.  4096 tokens, three contexts in turn, each with its own outputs: 15.4 -> 10.7 us per call.
+            const bool wait_stores = !wait_first && (clash || hazard(ctx, compact->K_out, kv_bytes, true) ||
+                                                     hazard(ctx, compact->V_out, kv_bytes, true) ||
+                                                     hazard(ctx, compact->lengths, sizeof(int32_t) * c.n_kv_heads, true));
             if (wait_first) serial_point(ctx);
             else ctx->op_chain += 1;
             ctx->op_last_seq = ctx->op_seq;
@@ -826,7 +829,8 @@ static kvzap_status launch_score(kvzap_ctx *ctx, int32_t layer, int32_t n_layers
             fc.epoch = ctx->op_epoch;
             fc.n_stages = kLinStagesCompact;
             fc.wait_limit = ctx->wait_limit;
-            p.wait_before_write = wait_first ? 1 : 0;
+            p.wait_before_write = wait_first ? 1 : wait_stores ? 2 : 0;
+            p.late_trigger = wait_first && ctx->trusted;     // what starts behind finds all work ahead of this launch complete
             p.maskbits = nullptr;
             smem = lin_smem_bytes(kLinStagesCompact);
             if (compacted) *compacted = true;

@@ -10,7 +10,7 @@
 // Warp roles as in score_kernel: warp 0 TMA producer, warp 1 MMA issuer / TMEM owner, warps 2..5
 // epilogue (TMEM lane quarter = warp % 4).  The kernel may be placed before the kernel ahead of it in
 // the stream has finished: it reads only hidden states and weights, every thread waits for that
-// kernel before it exits, and with p.wait_before_write set nothing is written before that wait either
+// kernel before it exits, and with p.wait_before_write set nothing of the caller is written before that wait either
 // (the host sets it unless the mask slice and the scores buffer written here are known to be free).
 #pragma once
 
@@ -77,7 +77,7 @@ score_linear_split_kernel(const __grid_constant__ CUtensorMap tmap_x, const __gr
     volatile uint32_t *tmem_slot = reinterpret_cast<volatile uint32_t *>(smem + bars_off + 16 * kLinStages + 16);
     volatile int *abort_flag = reinterpret_cast<volatile int *>(smem + bars_off + 16 * kLinStages + 20);
 
-    griddep_launch_dependents();
+    if (!p.late_trigger) griddep_launch_dependents();
     if (p.wait_before_load) griddep_wait();     // caller data is read only after the work ahead in the stream is complete
     const int warp = threadIdx.x >> 5;
     const int lane = threadIdx.x & 31;
@@ -206,7 +206,8 @@ score_linear_split_kernel(const __grid_constant__ CUtensorMap tmap_x, const __gr
     // nothing has been written so far
     if (fc.enabled) {
         // ------------------------------------------------------------ scoring and compaction in one launch
-        if (p.wait_before_write) griddep_wait();           // every thread: outputs may still be in use by the work ahead
+        if (p.wait_before_write == 1) griddep_wait();      // every thread; 2: only its stores wait, further down
+        if (p.late_trigger) griddep_launch_dependents();
         const uint32_t wt_addr = smem_u32(&wt_s[0][0]);
         if (rank == 0 && epi) {
 #pragma unroll
@@ -220,17 +221,6 @@ score_linear_split_kernel(const __grid_constant__ CUtensorMap tmap_x, const __gr
             for (int h = 0; h < kMaxHeads; ++h) s[h] += __ldg(p.b1 + layer * p.w_rows + h);
             const int64_t t = static_cast<int64_t>(m_tile) * kTileM + row;
             const bool valid = t < p.n_tokens;
-            if (valid && p.scores != nullptr) {
-                float *dst = p.scores + t * p.n_heads;
-                if (p.n_heads == kMaxHeads) {
-                    reinterpret_cast<float4 *>(dst)[0] = make_float4(s[0], s[1], s[2], s[3]);
-                    reinterpret_cast<float4 *>(dst)[1] = make_float4(s[4], s[5], s[6], s[7]);
-                } else {
-#pragma unroll
-                    for (int h = 0; h < kMaxHeads; ++h)
-                        if (h < p.n_heads) dst[h] = s[h];
-                }
-            }
             const bool in_window = valid && t >= p.n_tokens - static_cast<int64_t>(p.window);      // one sequence
             uint32_t my_word = 0;
 #pragma unroll
@@ -315,17 +305,33 @@ score_linear_split_kernel(const __grid_constant__ CUtensorMap tmap_x, const __gr
                 ent_dst_s[idx] = (static_cast<int64_t>(h) * p.n_tokens + n) * fc.row_bytes;
             }
         }
-        if (rank == 0 && m_tile == p.tiles_per_layer - 1 && threadIdx.x < p.n_heads) {
-            const int h = threadIdx.x;
-            fc.lengths[h] = run_s[h] + __popc(wt_s[h][0]) + __popc(wt_s[h][1]) + __popc(wt_s[h][2]) + __popc(wt_s[h][3]);
-        }
         __syncthreads();
-        // rows travel global -> the idle pipeline stages -> global; as many per round as the stages hold
-        const int cap = static_cast<int>(static_cast<uint32_t>(n_st) * kLinStageBytes / (2u * fc.row_bytes));
+        // the tile's scores and, at the end of the sequence, its lengths
+        auto store_scores = [&]() {
+            const int64_t t = static_cast<int64_t>(m_tile) * kTileM + row;
+            if (rank == 0 && epi && t < p.n_tokens && p.scores != nullptr) {
+                float *dst = p.scores + t * p.n_heads;
+                if (p.n_heads == kMaxHeads) {
+                    reinterpret_cast<float4 *>(dst)[0] = make_float4(s[0], s[1], s[2], s[3]);
+                    reinterpret_cast<float4 *>(dst)[1] = make_float4(s[4], s[5], s[6], s[7]);
+                } else {
+#pragma unroll
+                    for (int h = 0; h < kMaxHeads; ++h)
+                        if (h < p.n_heads) dst[h] = s[h];
+                }
+            }
+            if (rank == 0 && m_tile == p.tiles_per_layer - 1 && threadIdx.x < p.n_heads) {
+                const int h = threadIdx.x;
+                fc.lengths[h] = run_s[h] + __popc(wt_s[h][0]) + __popc(wt_s[h][1]) + __popc(wt_s[h][2]) + __popc(wt_s[h][3]);
+            }
+        };
+        // rows travel global -> the idle pipeline stages (and the partial sums behind them, summed up by now) -> global; as
+        // many per round as they hold: 96 rows of 256 bytes, where a quarter of a tile keeps 85 on average
+        const int cap = static_cast<int>(bars_off / (2u * fc.row_bytes));
         // as asynchronous 16-byte copies into shared memory (they pass by the L1 and the registers, so the rows of
         // a round are all in flight at once), 16 lanes per row, then ordinary loads from there and stores
         const int group = threadIdx.x >> 4, gl = threadIdx.x & 15;
-        for (int c0 = 0; c0 < n_rows; c0 += cap) {
+        for (int c0 = 0; c0 == 0 || c0 < n_rows; c0 += cap) {
             const int n_chunk = n_rows - c0 < cap ? n_rows - c0 : cap;
             for (int i = group; i < n_chunk; i += kLinThreads / 16) {
                 const uint32_t slot = smem_base + static_cast<uint32_t>(i) * 2u * fc.row_bytes;
@@ -335,7 +341,13 @@ score_linear_split_kernel(const __grid_constant__ CUtensorMap tmap_x, const __gr
                     asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(slot + fc.row_bytes + u), "l"(fc.V + src + u) : "memory");
                 }
             }
-            asm volatile("cp.async.commit_group;\n\tcp.async.wait_group 0;" ::: "memory");
+            asm volatile("cp.async.commit_group;" ::: "memory");
+            if (c0 == 0) {
+                // the first round's rows are on their way; outputs may be in use by the work ahead up to here
+                if (p.wait_before_write == 2) griddep_wait();
+                store_scores();
+            }
+            asm volatile("cp.async.wait_group 0;" ::: "memory");
             __syncthreads();
             for (int i = group; i < n_chunk; i += kLinThreads / 16) {
                 const uint8_t *slot = smem + static_cast<uint32_t>(i) * 2u * fc.row_bytes;
