@@ -64,9 +64,12 @@ struct kvzap_ctx {
         bool ok8 = false;
         uint32_t *arrive = nullptr;      // [sm_count] slices of a tile that have arrived, zero between launches
     };
-    static constexpr int kMaxLayouts = 4;
+    static constexpr int kMaxLayouts = 4, kMaxPairLayouts = 6;
     SplitLayout layouts[kMaxLayouts];
     int n_layouts = 0;
+    // the same with CTA pairs that share the W1 tiles (two blocks a tile, clusters of 2 k), for prompts and chunks
+    SplitLayout pair_layouts[kMaxPairLayouts];
+    int n_pair_layouts = 0;
     int split_smem_limit = 0;            // dynamic shared memory the few-token kernel may use
     uint64_t weights_seq = 0;            // op_seq of the last call that set weights
     // weights of all layers, stacked so that one tensor map / one base pointer serves any layer range
@@ -413,6 +416,7 @@ static void free_all(kvzap_ctx *ctx)
     cudaFree(ctx->select_tau);
     cudaFree(ctx->select_arrive);
     for (auto &l : ctx->layouts) cudaFree(l.arrive);
+    for (auto &l : ctx->pair_layouts) cudaFree(l.arrive);
     cudaFree(ctx->list_page0);
     cudaFree(ctx->list_base);
     cudaFree(ctx->op_mask); cudaFree(ctx->op_counts); cudaFree(ctx->op_len_acc);
@@ -555,6 +559,57 @@ static int split_layout(const kvzap_ctx *ctx, int64_t n_tiles, bool fp8, bool be
     return -1;
 }
 
+// What one CTA of a layout loads, in rows times parts of K: what bounds a launch of few tiles.
+static double split_load(const kvzap_ctx *ctx, const kvzap_ctx::SplitLayout &l, int k, bool pair)
+{
+    return (kTileM + static_cast<double>(ctx->cfg.hidden) / l.n / (pair ? 2 : 1)) / k;
+}
+
+// The layout with CTA pairs for a prompt of that many blocks whose CTAs load least, if they load a tenth less than `other`;
+// nullptr if there is none whose clusters the device holds at once, and for launches that run beside their neighbours
+// (`beside`), where it made nothing faster for sure.  4096 -> 512 -> 8, calls in a row on a default context, us a call: 1700
+// tokens 21.0 -> 20.0, 3000 tokens 29.2 -> 27.4, 5000 tokens 41.0 -> 36.3, 9400 tokens 45.0 -> 40.3; 8-bit 5000 tokens 40.2 ->
+// 27.8, 9400 tokens 43.3 -> 30.9; 5120 -> 640 -> 8, 3000 tokens 34.3 -> 28.0.
+static const kvzap_ctx::SplitLayout *pair_layout(const kvzap_ctx *ctx, int64_t blocks, bool fp8, bool beside, double other)
+{
+    const kvzap_ctx::SplitLayout *best = nullptr;
+    double least = 0.9 * other;
+    const int64_t pairs = (blocks + 1) / 2;
+    for (int i = 0; i < (beside ? 0 : ctx->n_pair_layouts); ++i) {
+        const kvzap_ctx::SplitLayout &l = ctx->pair_layouts[i];
+        const int64_t ctas = pairs * 2 * l.n * l.k;
+        if ((fp8 && !l.ok8) || ctas > ctx->sm_count || pairs * l.n > l.max_clusters) continue;
+        const double load = split_load(ctx, l, l.k, true);
+        if (load < least) { least = load; best = &l; }
+    }
+    return best;
+}
+
+// The few-token layout of a prompt: one of split_layout() or pair_layout(); nullptr if there are too many blocks.
+static const kvzap_ctx::SplitLayout *prompt_layout(const kvzap_ctx *ctx, int64_t blocks, bool fp8, bool beside, bool *pair)
+{
+    const int i = split_layout(ctx, blocks, fp8, beside);
+    const kvzap_ctx::SplitLayout *l =
+        pair_layout(ctx, blocks, fp8, beside, i >= 0 ? split_load(ctx, ctx->layouts[i], ctx->layouts[i].k, false) : 1e9);
+    *pair = l != nullptr;
+    return l ? l : i >= 0 ? &ctx->layouts[i] : nullptr;
+}
+
+// Enqueues the few-token kernel over p.n_tiles tiles (of two blocks for a layout with CTA pairs).
+static cudaError_t launch_split(const kvzap_ctx::SplitLayout &l, int k, bool pair, bool fp8, const CUtensorMap &tmap_x, const ScoreParams &p,
+                                const DecodeFuse &f, bool early, cudaStream_t stream)
+{
+    const int ctas = pair ? 2 : 1;
+    cudaLaunchConfig_t cfg;
+    cudaLaunchAttribute attrs[2];
+    make_launch(&cfg, attrs, dim3(static_cast<unsigned>(p.n_tiles * ctas * l.n * k)), dim3(kScoreThreads), l.smem, stream, early, ctas * k);
+    const CUtensorMap &tmap_w = fp8 ? l.tmap_w8 : l.tmap_w;
+    if (pair) return fp8 ? cudaLaunchKernelEx(&cfg, score_split_kernel<true, true>, tmap_x, tmap_w, p, l.n, k, f)
+                         : cudaLaunchKernelEx(&cfg, score_split_kernel<false, true>, tmap_x, tmap_w, p, l.n, k, f);
+    return fp8 ? cudaLaunchKernelEx(&cfg, score_split_kernel<true, false>, tmap_x, tmap_w, p, l.n, k, f)
+               : cudaLaunchKernelEx(&cfg, score_split_kernel<false, false>, tmap_x, tmap_w, p, l.n, k, f);
+}
+
 // Blocks of a prompt that whole waves of CTA pairs leave over and that the few-token kernel takes instead, in a launch of its
 // own behind them (launch_score_rest): a wave lasts as long for one tile as for all of them.  4096 -> 512 -> 8, calls in a
 // row: 19500 tokens (5 blocks more than a wave) 114 -> 89 us a call, 22000 tokens (24 blocks more) 116 -> 103 us; with 8-bit
@@ -565,7 +620,8 @@ static int64_t rest_blocks(const kvzap_ctx *ctx, int64_t blocks, bool fp8)
     const int64_t wave = 2 * static_cast<int64_t>(ctx->pair_clusters);
     if (ctx->trusted || ctx->profiling || ctx->cfg.hidden == 0 || wave == 0 || blocks <= wave) return 0;
     const int64_t rest = blocks % wave;
-    return rest > 0 && split_layout(ctx, rest, fp8) >= 0 ? rest : 0;
+    bool pair;
+    return rest > 0 && prompt_layout(ctx, rest, fp8, false, &pair) != nullptr ? rest : 0;
 }
 
 // The few-token kernel over the blocks from block0 on, directly behind the launch over those before (p, one layer), which lets
@@ -573,9 +629,10 @@ static int64_t rest_blocks(const kvzap_ctx *ctx, int64_t blocks, bool fp8)
 static kvzap_status launch_score_rest(kvzap_ctx *ctx, ScoreParams p, const CUtensorMap &tmap_x, int64_t block0, bool fp8, cudaStream_t stream)
 {
     const int64_t rest = p.blocks_per_layer - block0;
-    const kvzap_ctx::SplitLayout &layout = ctx->layouts[split_layout(ctx, rest, fp8)];
+    bool pair;
+    const kvzap_ctx::SplitLayout &layout = *prompt_layout(ctx, rest, fp8, false, &pair);
     p.block0 = static_cast<int32_t>(block0);
-    p.n_tiles = p.tiles_per_layer = static_cast<int32_t>(rest);
+    p.n_tiles = p.tiles_per_layer = static_cast<int32_t>(pair ? (rest + 1) / 2 : rest);
     p.group_w = p.chunk_n = ctx->cfg.hidden / layout.n;
     p.n_groups = p.n_chunks = 1;
     p.n_stages = layout.stages;
@@ -587,13 +644,7 @@ static kvzap_status launch_score_rest(kvzap_ctx *ctx, ScoreParams p, const CUten
     DecodeFuse f;
     memset(&f, 0, sizeof f);
     ProfScope prof(ctx, KVZAP_KERNEL_SCORE, stream);
-    cudaLaunchConfig_t cfg;
-    cudaLaunchAttribute attrs[2];
-    make_launch(&cfg, attrs, dim3(static_cast<unsigned>(rest * layout.n * layout.k)), dim3(kScoreThreads), layout.smem, stream, true, layout.k);
-    if (fp8)
-        KVZAP_CUDA(ctx, cudaLaunchKernelEx(&cfg, score_split_kernel<true>, tmap_x, layout.tmap_w8, p, layout.n, layout.k, f));
-    else
-        KVZAP_CUDA(ctx, cudaLaunchKernelEx(&cfg, score_split_kernel<false>, tmap_x, layout.tmap_w, p, layout.n, layout.k, f));
+    KVZAP_CUDA(ctx, launch_split(layout, layout.k, pair, fp8, tmap_x, p, f, true, stream));
     ctx->launches += 1;
     return KVZAP_OK;
 }
@@ -635,11 +686,15 @@ static kvzap_status launch_score(kvzap_ctx *ctx, int32_t layer, int32_t n_layers
     const int layout_i = split_layout(ctx, few_tiles, fp8, ctx->trusted && fuse == nullptr && !late_trigger);
     const bool slices_only = layout_i < 0 && ctx->n_layouts > 0 && ctx->layouts[0].n == 2 && ctx->layouts[0].k == 2 &&
                              fuse == nullptr && !fp8 && few_tiles * 2 <= ctx->sm_count;
-    if (fp8 && layout_i < 0)
+    const double single_load = layout_i >= 0 ? split_load(ctx, ctx->layouts[layout_i], ctx->layouts[layout_i].k, false)
+                               : slices_only ? split_load(ctx, ctx->layouts[0], 1, false) : 1e9;
+    const kvzap_ctx::SplitLayout *pairs =
+        n_layers == 1 && fuse_chain == nullptr ? pair_layout(ctx, few_tiles, fp8, ctx->trusted && !late_trigger, single_load) : nullptr;
+    if (fp8 && layout_i < 0 && pairs == nullptr)
         return fail(ctx, KVZAP_ERR_UNSUPPORTED, "8-bit few-token scoring: this shape has no four-CTA layout");
-    if (layout_i >= 0 || slices_only) {
-        const kvzap_ctx::SplitLayout &layout = ctx->layouts[slices_only ? 0 : layout_i];
-        const int split_n = layout.n, split_k = slices_only ? 1 : layout.k;
+    if (layout_i >= 0 || slices_only || pairs != nullptr) {
+        const kvzap_ctx::SplitLayout &layout = pairs ? *pairs : ctx->layouts[slices_only ? 0 : layout_i];
+        const int split_n = layout.n, split_k = slices_only && !pairs ? 1 : layout.k;
         CUtensorMap tmap_x;
         kvzap_status st = fp8 ? make_tmap8(ctx, &tmap_x, hidden, static_cast<uint64_t>(n_tokens), static_cast<uint64_t>(c.d_model),
                                            kTileM, static_cast<uint64_t>(n_layers), false)
@@ -650,8 +705,8 @@ static kvzap_status launch_score(kvzap_ctx *ctx, int32_t layer, int32_t n_layers
         p.x_scale = x_scale;
         p.w1_scale = ctx->w1_scale_all;
         p.n_tokens = n_tokens;
-        p.n_tiles = static_cast<int32_t>(blocks_per_layer * n_layers);
-        p.tiles_per_layer = static_cast<int32_t>(blocks_per_layer);
+        p.n_tiles = static_cast<int32_t>(pairs ? (blocks_per_layer + 1) / 2 : blocks_per_layer * n_layers);
+        p.tiles_per_layer = static_cast<int32_t>(pairs ? (blocks_per_layer + 1) / 2 : blocks_per_layer);
         p.blocks_per_layer = static_cast<int32_t>(blocks_per_layer);
         p.n_layers_call = n_layers;
         p.layer0 = layer;
@@ -722,14 +777,7 @@ static kvzap_status launch_score(kvzap_ctx *ctx, int32_t layer, int32_t n_layers
         ctx->last_score_early = early;
         {
             ProfScope prof(ctx, KVZAP_KERNEL_SCORE, stream);
-            cudaLaunchConfig_t cfg;
-            cudaLaunchAttribute attrs[2];
-            make_launch(&cfg, attrs, dim3(static_cast<unsigned>(p.n_tiles * n_ctas)), dim3(kScoreThreads), layout.smem, stream, early,
-                        split_k);
-            if (fp8)
-                KVZAP_CUDA(ctx, cudaLaunchKernelEx(&cfg, score_split_kernel<true>, tmap_x, layout.tmap_w8, p, split_n, split_k, f));
-            else
-                KVZAP_CUDA(ctx, cudaLaunchKernelEx(&cfg, score_split_kernel<false>, tmap_x, layout.tmap_w, p, split_n, split_k, f));
+            KVZAP_CUDA(ctx, launch_split(layout, split_k, pairs != nullptr, fp8, tmap_x, p, f, early, stream));
         }
         ctx->launches += 1;
         return KVZAP_OK;
@@ -946,7 +994,8 @@ static kvzap_status launch_score_fp8(kvzap_ctx *ctx, int32_t layer, const void *
     // On a context that trusts its producers the small grids of the persistent kernel run beside one another instead (777
     // tokens 9.7 us a call, with the few-token kernel 10.9); elsewhere a call waits for the one before, and 200 / 777 / 2200 /
     // 3900 tokens take 13.5 / 15 / 18 / 25 us where one CTA pair per 256 tokens takes 36 to 38 (4096 -> 512 -> 8).
-    if (!ctx->trusted && split_layout(ctx, blocks_per_layer, true) >= 0)
+    bool pairs;
+    if (!ctx->trusted && prompt_layout(ctx, blocks_per_layer, true, false, &pairs) != nullptr)
         return launch_score(ctx, layer, 1, hidden8, n_tokens, scores, maskbits, cu_seqlens, n_seqs, tau, w, stream, 1, nullptr, nullptr,
                             nullptr, nullptr, nullptr, true, x_scale);
     const bool pair = c.hidden > 0 && ctx->pair_clusters > 0 && blocks_per_layer >= 2;
@@ -1375,7 +1424,7 @@ kvzap_status kvzap_create(kvzap_ctx **out, const kvzap_config *cfg)
     CREATE_CUDA(cudaFuncSetAttribute(decode_update_kernel, cudaFuncAttributePreferredSharedMemoryCarveout,
                                      static_cast<int>(cudaSharedmemCarveoutMaxShared)));
     if (c.hidden > 0)
-        CREATE_CUDA(cudaFuncSetAttribute(score_split_kernel<false>, cudaFuncAttributePreferredSharedMemoryCarveout,
+        CREATE_CUDA(cudaFuncSetAttribute(score_split_kernel<false, false>, cudaFuncAttributePreferredSharedMemoryCarveout,
                                          static_cast<int>(cudaSharedmemCarveoutMaxShared)));
     if (c.hidden > 0) {
         CREATE_CUDA(cudaFuncSetAttribute(score_kernel<true, false>, cudaFuncAttributePreferredSharedMemoryCarveout,
@@ -1421,7 +1470,10 @@ kvzap_status kvzap_create(kvzap_ctx **out, const kvzap_config *cfg)
     if (c.hidden > 0) {
         ctx->split_smem_limit = budget + 1024 - 4608;       // the kernel has 4112 bytes of static shared memory
         // the limit is the function's, not the context's: the most that any layout of any context takes
-        CREATE_CUDA(cudaFuncSetAttribute(score_split_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, ctx->split_smem_limit));
+        CREATE_CUDA(cudaFuncSetAttribute(score_split_kernel<false, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, ctx->split_smem_limit));
+        CREATE_CUDA(cudaFuncSetAttribute(score_split_kernel<false, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, ctx->split_smem_limit));
+        CREATE_CUDA(cudaFuncSetAttribute(score_split_kernel<false, true>, cudaFuncAttributePreferredSharedMemoryCarveout,
+                                         static_cast<int>(cudaSharedmemCarveoutMaxShared)));
         // Few-token layouts.  The first takes the largest launches: four CTAs per tile, 2 x 2 (two slices of hidden
         // units, two parts of K) when a slice of hidden / 2 units fits one MMA and the K blocks divide evenly, else
         // four slices.  The others spread a tile over more CTAs, widest first; of two of the same width the one whose
@@ -1429,29 +1481,45 @@ kvzap_status kvzap_create(kvzap_ctx **out, const kvzap_config *cfg)
         const int kb = c.d_model / kBlockK;
         const bool two_by_two = c.hidden / 2 <= 256 && (c.hidden / 4) % 16 == 0 && kb % 2 == 0;
         const int shapes[][2] = {{two_by_two ? 2 : 4, two_by_two ? 2 : 1}, {8, 8}, {5, 8}, {4, 8}, {5, 4}, {4, 4}, {4, 2}};
-        for (const auto &sh : shapes) {
-            const int n = sh[0], k = sh[1], ns = c.hidden / n, i = ctx->n_layouts;
-            if (i == kvzap_ctx::kMaxLayouts || c.hidden % (16 * n * k) != 0 || ns > 256 || kb % k != 0) continue;
-            if (i > 1 && n * k > ctx->layouts[i - 1].n * ctx->layouts[i - 1].k / 2) continue;
-            kvzap_ctx::SplitLayout &l = ctx->layouts[i];
+        // fills in a layout; false where the shape cannot be served
+        auto make_layout = [&](kvzap_ctx::SplitLayout &l, int n, int k, bool pair) -> bool {
+            const int ns = c.hidden / n, b_rows = pair ? ns / 2 : ns;
             l.n = n;
             l.k = k;
             for (l.stages = kMaxStages; l.stages >= 2; --l.stages)
-                if (split_smem_fits(ns, l.stages, k, ctx->split_smem_limit - 1024)) break;
-            if (l.stages < 2) { if (i == 0) break; else continue; }
-            l.smem = split_smem_layout(ns, l.stages, k).total + 1024;
+                if (split_smem_fits(ns, l.stages, k, b_rows, ctx->split_smem_limit - 1024)) break;
+            if (l.stages < 2) return false;
+            l.smem = split_smem_layout(ns, l.stages, k, b_rows).total + 1024;
             l.tmem_cols = next_pow2(ns);
             if (make_tmap_w(ctx, &l.tmap_w, ctx->w1_all, static_cast<uint64_t>(c.n_layers) * ctx->w1_rows,
-                            static_cast<uint64_t>(kb), static_cast<uint32_t>(ns)) != KVZAP_OK) {
-                if (i == 0) break; else continue;
-            }
+                            static_cast<uint64_t>(kb), static_cast<uint32_t>(b_rows)) != KVZAP_OK) return false;
             cudaLaunchConfig_t cfg;
             cudaLaunchAttribute attrs[2];
-            make_launch(&cfg, attrs, dim3(static_cast<unsigned>(n * k)), dim3(kScoreThreads), l.smem, nullptr, false, k);
-            CREATE_CUDA(cudaOccupancyMaxActiveClusters(&l.max_clusters, score_split_kernel<false>, &cfg));
-            CREATE_CUDA(cudaMalloc(&l.arrive, sizeof(uint32_t) * static_cast<size_t>(ctx->sm_count)));
-            CREATE_CUDA(cudaMemset(l.arrive, 0, sizeof(uint32_t) * static_cast<size_t>(ctx->sm_count)));
-            ctx->n_layouts = i + 1;
+            const int cluster = pair ? 2 * k : k;
+            make_launch(&cfg, attrs, dim3(static_cast<unsigned>(n * cluster)), dim3(kScoreThreads), l.smem, nullptr, false, cluster);
+            return (pair ? cudaOccupancyMaxActiveClusters(&l.max_clusters, score_split_kernel<false, true>, &cfg)
+                         : cudaOccupancyMaxActiveClusters(&l.max_clusters, score_split_kernel<false, false>, &cfg)) == cudaSuccess &&
+                   (l.arrive != nullptr || cudaMalloc(&l.arrive, sizeof(uint32_t) * static_cast<size_t>(ctx->sm_count)) == cudaSuccess) &&
+                   cudaMemset(l.arrive, 0, sizeof(uint32_t) * static_cast<size_t>(ctx->sm_count)) == cudaSuccess;
+        };
+        for (const auto &sh : shapes) {
+            const int n = sh[0], k = sh[1], i = ctx->n_layouts;
+            if (i == kvzap_ctx::kMaxLayouts || c.hidden % (16 * n * k) != 0 || c.hidden / n > 256 || kb % k != 0) continue;
+            if (i > 1 && n * k > ctx->layouts[i - 1].n * ctx->layouts[i - 1].k / 2) continue;
+            if (make_layout(ctx->layouts[i], n, k, false)) ctx->n_layouts = i + 1;
+            else if (i == 0) break;
+        }
+        // With CTA pairs: of two layouts with as many CTAs the one whose CTAs load less.  Slices of whole 32 units.  Clusters of
+        // four CTAs at most: with clusters of eight, which the MMAs and the exchange of a slice then wait for, 1300 and 1700
+        // tokens took 21.7 and 22.2 us instead of 21.4 and 21.0 (8-bit: 18.9 and 19.5 instead of 17.2 and 17.4).
+        const int pair_shapes[][2] = {{4, 2}, {5, 2}, {2, 2}, {4, 1}, {5, 1}, {1, 2}, {2, 1}, {1, 1}};
+        for (const auto &sh : pair_shapes) {
+            const int n = sh[0], k = sh[1], i = ctx->n_pair_layouts;
+            if (ctx->n_layouts == 0 || ctx->pair_clusters == 0 || i == kvzap_ctx::kMaxPairLayouts) break;
+            if (c.hidden % (32 * n) != 0 || c.hidden % (16 * n * k) != 0 || c.hidden / n > 256 || kb % k != 0) continue;
+            bool taken = false;
+            for (int j = 0; j < i; ++j) taken = taken || ctx->pair_layouts[j].n * ctx->pair_layouts[j].k == n * k;
+            if (!taken && make_layout(ctx->pair_layouts[i], n, k, true)) ctx->n_pair_layouts = i + 1;
         }
     }
     ctx->max_blocks = (c.max_tokens + kBlockTokens - 1) / kBlockTokens;
@@ -1596,17 +1664,20 @@ kvzap_status kvzap_set_weights_fp8(kvzap_ctx *ctx, int32_t layer, const void *W1
                                          static_cast<uint64_t>(c.d_model), static_cast<uint32_t>(ctx->sched[mode].chunk_n / (mode + 1)), 0, true);
             if (st != KVZAP_OK) return st;
         }
-        for (int i = 0; i < ctx->n_layouts; ++i) {
+        for (int i = 0; i < ctx->n_layouts + ctx->n_pair_layouts; ++i) {
             // the few-token layouts: the same slices of hidden units, K blocks of 128 codes
-            kvzap_ctx::SplitLayout &l = ctx->layouts[i];
+            const bool pair = i >= ctx->n_layouts;
+            kvzap_ctx::SplitLayout &l = pair ? ctx->pair_layouts[i - ctx->n_layouts] : ctx->layouts[i];
             if ((c.d_model / 128) % l.k != 0) continue;
             l.ok8 = make_tmap8(ctx, &l.tmap_w8, ctx->w1_fp8_all, static_cast<uint64_t>(rows_total), static_cast<uint64_t>(c.d_model),
-                               static_cast<uint32_t>(c.hidden / l.n), 0, true) == KVZAP_OK;
+                               static_cast<uint32_t>(c.hidden / l.n / (pair ? 2 : 1)), 0, true) == KVZAP_OK;
         }
         if (ctx->n_layouts > 0) {
-            KVZAP_CUDA(ctx, cudaFuncSetAttribute(score_split_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, ctx->split_smem_limit));
-            KVZAP_CUDA(ctx, cudaFuncSetAttribute(score_split_kernel<true>, cudaFuncAttributePreferredSharedMemoryCarveout,
-                                                 static_cast<int>(cudaSharedmemCarveoutMaxShared)));
+            for (auto kernel : {score_split_kernel<true, false>, score_split_kernel<true, true>}) {
+                KVZAP_CUDA(ctx, cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, ctx->split_smem_limit));
+                KVZAP_CUDA(ctx, cudaFuncSetAttribute(kernel, cudaFuncAttributePreferredSharedMemoryCarveout,
+                                                     static_cast<int>(cudaSharedmemCarveoutMaxShared)));
+            }
         }
         if (c.hidden > 0) {
             KVZAP_CUDA(ctx, cudaFuncSetAttribute(score_kernel<true, false, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(ctx->sched[0].smem)));
@@ -1894,6 +1965,8 @@ kvzap_status kvzap_poll_status(kvzap_ctx *ctx, void *stream_)
     cudaMemsetAsync(ctx->tile_counters, 0, sizeof(int32_t) * kMaskRing, stream);
     for (int i = 0; i < ctx->n_layouts; ++i)
         cudaMemsetAsync(ctx->layouts[i].arrive, 0, sizeof(uint32_t) * static_cast<size_t>(ctx->sm_count), stream);
+    for (int i = 0; i < ctx->n_pair_layouts; ++i)
+        cudaMemsetAsync(ctx->pair_layouts[i].arrive, 0, sizeof(uint32_t) * static_cast<size_t>(ctx->sm_count), stream);
     if (v == KVZAP_ERR_TIMEOUT) {
         reset_step_counters(ctx, stream);
         // a one-launch pruning call that gave up may have left its list-length sums and arrival count behind

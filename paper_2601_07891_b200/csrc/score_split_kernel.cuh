@@ -56,10 +56,11 @@ struct SplitSmemLayout {
 };
 // The parts received from the other CTAs of the cluster ([k_split - 1][own / 4][128 rows] float4) lie over the
 // stages, idle by then, and behind them the sums that the cluster's CTAs leave with its first one ([k_split][128][8]).
-__host__ __device__ inline SplitSmemLayout split_smem_layout(int ns, int n_stages, int k_split)
+// b_rows: rows of W1 that a CTA stages, ns or, for CTA pairs, half of them.
+__host__ __device__ inline SplitSmemLayout split_smem_layout(int ns, int n_stages, int k_split, int b_rows)
 {
     SplitSmemLayout L;
-    L.stage_bytes = kATileBytes + static_cast<uint32_t>(ns) * kBlockK * 2;
+    L.stage_bytes = kATileBytes + static_cast<uint32_t>(b_rows) * kBlockK * 2;
     L.stages_end = L.stage_bytes * n_stages;
     L.w2s = L.stages_end;
     L.b1s = L.w2s + static_cast<uint32_t>(ns) * kMaxHeads * 4;
@@ -70,9 +71,9 @@ __host__ __device__ inline SplitSmemLayout split_smem_layout(int ns, int n_stage
     L.total = L.bars + 256;
     return L;
 }
-__host__ inline bool split_smem_fits(int ns, int n_stages, int k_split, int budget)
+__host__ inline bool split_smem_fits(int ns, int n_stages, int k_split, int b_rows, int budget)
 {
-    const SplitSmemLayout L = split_smem_layout(ns, n_stages, k_split);
+    const SplitSmemLayout L = split_smem_layout(ns, n_stages, k_split, b_rows);
     return static_cast<int>(L.total) <= budget &&
            L.xpart + static_cast<uint32_t>(k_split) * kTileM * kMaxHeads * 4 <= L.stages_end;
 }
@@ -82,12 +83,17 @@ __host__ inline bool split_smem_fits(int ns, int n_stages, int k_split, int budg
 // A CTA ends up owning Ns / k_split hidden units.
 // kFp8: hidden states and W1 are E4M3 bytes (K blocks of 128 codes, tcgen05.mma kind::f8f6f4); the scales
 // x_scale[token] * w1_scale[hidden unit] multiply the summed pre-activation before the bias.
-template <bool kFp8>
+// kPair (prompts, not the fused step): two blocks of 128 tokens share every W1 tile.  A work tile is a pair of blocks, the
+// cluster has 2 * k_split CTAs, CTA 2 r + i holds block i's rows of K part r and half of the slice's W1 rows, and its first
+// one issues the MMAs of both (cta_group::2, as in score_kernel); everything behind the accumulators is per block, as without
+// pairs.  A CTA then loads (128 + Ns / 2) rows per K element instead of 128 + Ns, which is what bounds this kernel.
+template <bool kFp8, bool kPair>
 __global__ void __maxnreg__(128)
 score_split_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_constant__ CUtensorMap tmap_w,
                    const ScoreParams p, const int n_split, const int k_split, const DecodeFuse f)
 {
     constexpr int kElems = kFp8 ? 2 * kBlockK : kBlockK;         // elements per 128-byte K block
+    constexpr int kCtas = kPair ? 2 : 1;
     __shared__ int64_t fuse_dst[256];       // fused decode step: page row of the evicted token (-1 = dropped)
     __shared__ int64_t fuse_ring[256];      //                     ring row of the list's current slot (-1 = no list)
     __shared__ int32_t fuse_step;           //                     number of the step this CTA works on (its ticket)
@@ -98,7 +104,7 @@ score_split_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_cons
     const uint32_t smem_base = raw_addr + pad;
     const int ns = p.chunk_n;
     const int n_ctas = n_split * k_split;
-    const SplitSmemLayout L = split_smem_layout(ns, p.n_stages, k_split);
+    const SplitSmemLayout L = split_smem_layout(ns, p.n_stages, k_split, ns / kCtas);
 
     ulonglong2 *w2p = reinterpret_cast<ulonglong2 *>(smem + L.w2s);
     float *w2f = reinterpret_cast<float *>(smem + L.w2s);
@@ -118,13 +124,16 @@ score_split_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_cons
 
     const int warp = threadIdx.x >> 5;
     const int lane = threadIdx.x & 31;
-    const uint32_t rank = cluster_cta_rank();            // 0 .. k_split - 1
+    const uint32_t cta = cluster_cta_rank();
+    const uint32_t half = cta % kCtas;                   // which block of the pair
+    const uint32_t rank = cta / kCtas;                   // 0 .. k_split - 1
     const int kh = static_cast<int>(rank);               // which part of the K range
-    const int nh = (static_cast<int>(blockIdx.x) / k_split) % n_split;   // which slice of the hidden units
-    const int pos = nh * k_split + kh;                   // this CTA among the n_ctas of its tile
-    const int tile = static_cast<int>(blockIdx.x) / n_ctas;
+    const int nh = (static_cast<int>(blockIdx.x) / (kCtas * k_split)) % n_split;   // which slice of the hidden units
+    const int pos = nh * k_split + kh;                   // this CTA among the n_ctas of its block
+    const int tile = static_cast<int>(blockIdx.x) / (kCtas * n_ctas);
     const int l_rel = tile / p.tiles_per_layer;
-    const int m_tile = tile - l_rel * p.tiles_per_layer + p.block0;
+    const int m_tile = (tile - l_rel * p.tiles_per_layer) * kCtas + static_cast<int>(half) + p.block0;
+    const int part_tile = tile * kCtas + static_cast<int>(half);        // among all blocks of the launch
     const int layer = p.layer0 + l_rel;
     if (f.enabled) {
         // the step number, drawn before any thread of this CTA lets the next launch be placed: a CTA of that launch
@@ -155,26 +164,43 @@ score_split_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_cons
     const int kb_first = kh * k_blocks;
     const uint64_t pol_x = l2_policy_evict_last();        // the other CTAs of the cluster read the same X tile
     const uint64_t pol_w = l2_policy_evict_first();       // every W1 byte is read once per step
-    const int w_row = layer * p.w_rows + nh * ns;
+    const int w_row = layer * p.w_rows + nh * ns + static_cast<int>(half) * (ns / kCtas);
     const int row0 = m_tile * kTileM;
     const int n_pre = k_blocks < p.n_stages ? k_blocks : p.n_stages;
     // The first loads go out before the CTA-wide barrier below (TMEM allocation, the other warps): the
-    // stages are empty and their barriers were initialised by this warp's lane 0 just above.  W1 is the
-    // context's own copy and is not written by anything that may still be running ahead of this launch.
+    // stages are empty and their barriers were initialised by this warp's lane 0 just above (a pair: those of its first
+    // CTA, which count the copies of both).  W1 is the context's own copy and is not written by anything that may still be
+    // running ahead of this launch.
+    if constexpr (kPair) cluster_sync_all();
+    uint32_t full0 = bar_full;                           // the barriers that this CTA's copies complete on
+    if constexpr (kPair) full0 = map_to_cta(bar_full, cta - half);
+    auto load_w = [&](uint32_t st, uint32_t sa, int kb) {
+        if constexpr (kPair) {
+            if (half == 0) mbar_arrive_expect_tx(bar_full + 8 * st, 2u * L.stage_bytes);
+            tma_load_3d_pair(sa + kATileBytes, &tmap_w, full0 + 8 * st, 0, w_row, kb_first + kb, pol_w);
+        } else {
+            mbar_arrive_expect_tx(bar_full + 8 * st, L.stage_bytes);
+            tma_load_3d(sa + kATileBytes, &tmap_w, bar_full + 8 * st, 0, w_row, kb_first + kb, pol_w);
+        }
+    };
+    auto load_x = [&](uint32_t st, uint32_t sa, int kb) {
+        if constexpr (kPair) tma_load_3d_pair(sa, &tmap_x, full0 + 8 * st, (kb_first + kb) * kElems, row0, l_rel, pol_x);
+        else tma_load_3d(sa, &tmap_x, bar_full + 8 * st, (kb_first + kb) * kElems, row0, l_rel, pol_x);
+    };
     if (warp == 0) {
         __syncwarp();
-        if (elect_one()) {
-            for (int kb = 0; kb < n_pre; ++kb) {
-                const uint32_t sa = smem_base + kb * L.stage_bytes;
-                mbar_arrive_expect_tx(bar_full + 8 * kb, L.stage_bytes);
-                tma_load_3d(sa + kATileBytes, &tmap_w, bar_full + 8 * kb, 0, w_row, kb_first + kb, pol_w);
-            }
-        }
+        if (elect_one())
+            for (int kb = 0; kb < n_pre; ++kb) load_w(static_cast<uint32_t>(kb), smem_base + kb * L.stage_bytes, kb);
         __syncwarp();
     }
     if (warp == 1) {
-        tmem_alloc(smem_u32(const_cast<uint32_t *>(tmem_slot)), static_cast<uint32_t>(p.tmem_cols));
-        tmem_relinquish();
+        if constexpr (kPair) {
+            tmem_alloc_pair(smem_u32(const_cast<uint32_t *>(tmem_slot)), static_cast<uint32_t>(p.tmem_cols));
+            tmem_relinquish_pair();
+        } else {
+            tmem_alloc(smem_u32(const_cast<uint32_t *>(tmem_slot)), static_cast<uint32_t>(p.tmem_cols));
+            tmem_relinquish();
+        }
     }
     // unless the caller vouches for the producers of its inputs, nothing of them is read before the work
     // ahead in the stream has completed (every thread waits: the loads below are issued by several warps)
@@ -183,8 +209,7 @@ score_split_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_cons
     if (warp == 0) {
         __syncwarp();
         if (elect_one())
-            for (int kb = 0; kb < n_pre; ++kb)
-                tma_load_3d(smem_base + kb * L.stage_bytes, &tmap_x, bar_full + 8 * kb, (kb_first + kb) * kElems, row0, l_rel, pol_x);
+            for (int kb = 0; kb < n_pre; ++kb) load_x(static_cast<uint32_t>(kb), smem_base + kb * L.stage_bytes, kb);
         __syncwarp();
     }
     tc_fence_before_sync();
@@ -205,9 +230,8 @@ score_split_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_cons
                 break;
             }
             if (elected) {
-                mbar_arrive_expect_tx(bar_full + 8 * st, L.stage_bytes);
-                tma_load_3d(sa + kATileBytes, &tmap_w, bar_full + 8 * st, 0, w_row, kb_first + kb, pol_w);
-                tma_load_3d(sa, &tmap_x, bar_full + 8 * st, (kb_first + kb) * kElems, row0, l_rel, pol_x);
+                load_w(st, sa, kb);
+                load_x(st, sa, kb);
             }
             __syncwarp();
             sa += L.stage_bytes;
@@ -218,10 +242,11 @@ score_split_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_cons
             const long long t0 = clock64();
             while (clock64() - t0 < 2000000LL) { }
         }
-    } else if (warp == 1) {
-        // ------------------------------------------------------------ MMA issuer
-        const uint32_t idesc = kFp8 ? umma_idesc_e4m3_f32(kTileM, static_cast<uint32_t>(ns))
-                                    : umma_idesc_bf16_f32(kTileM, static_cast<uint32_t>(ns));
+    } else if (warp == 1 && half == 0) {
+        // ------------------------------------------------------------ MMA issuer (a pair: its first CTA)
+        const uint32_t idesc = kFp8 ? umma_idesc_e4m3_f32(kTileM * kCtas, static_cast<uint32_t>(ns))
+                                    : umma_idesc_bf16_f32(kTileM * kCtas, static_cast<uint32_t>(ns));
+        const uint16_t both = static_cast<uint16_t>(3u << cta);
         const uint64_t desc0 = umma_desc_k_major_sw128(smem_base);
         const uint32_t desc_hi = static_cast<uint32_t>(desc0 >> 32);
         const uint32_t desc_lo0 = static_cast<uint32_t>(desc0);
@@ -236,17 +261,22 @@ score_split_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_cons
             }
             tc_fence_after_sync();
             if (elected) {
-                issue_k_block<false, 1, kFp8>(tmem_base, a_lo, a_lo + (kATileBytes >> 4), desc_hi, 0, 0, idesc, kb == 0);
-                umma_commit(bar_empty + 8 * st);
+                issue_k_block<kPair, 1, kFp8>(tmem_base, a_lo, a_lo + (kATileBytes >> 4), desc_hi, 0, 0, idesc, kb == 0);
+                if constexpr (kPair) umma_commit_pair(bar_empty + 8 * st, both);
+                else umma_commit(bar_empty + 8 * st);
             }
             __syncwarp();
             a_lo += stage_units;
             if (++st == static_cast<uint32_t>(p.n_stages)) { st = 0; st_par ^= 1u; a_lo = desc_lo0; }
         }
-        if (ok && elected) umma_commit(bar_tfull);
+        if (ok && elected) {
+            if constexpr (kPair) umma_commit_pair(bar_tfull, both);
+            else umma_commit(bar_tfull);
+        }
         __syncwarp();
         if (!ok && elected) {
-            umma_commit(bar_done);
+            if constexpr (kPair) umma_commit_pair(bar_done, static_cast<uint16_t>(1u << cta));
+            else umma_commit(bar_done);
             const long long t0 = clock64();
             while (!mbar_try_wait(bar_done, 0))
                 if (clock64() - t0 > KVZAP_WAIT_LIMIT_CYCLES / 16) break;
@@ -391,7 +421,7 @@ score_split_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_cons
                 const uint32_t c = static_cast<uint32_t>(i % n16);
                 const uint32_t to = (rank + 1u + static_cast<uint32_t>(i / n16)) % static_cast<uint32_t>(k_split);
                 const uint32_t slot = rank < to ? rank : rank - 1u;         // the receiver's parts in rank order, itself left out
-                const uint32_t dst0 = map_to_cta(smem_base, to) + (slot * (static_cast<uint32_t>(own_n) >> 2) + c * 4) * kTileM * 16;
+                const uint32_t dst0 = map_to_cta(smem_base, to * kCtas + half) + (slot * (static_cast<uint32_t>(own_n) >> 2) + c * 4) * kTileM * 16;
                 uint32_t r[16];
                 tmem_ld_x16(t_row + to * own_n + c * 16, r);
                 tmem_wait_ld();
@@ -473,7 +503,7 @@ score_split_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_cons
             s[0] += pa.x; s[1] += pa.y; s[2] += pa.z; s[3] += pa.w;
             s[4] += pb.x; s[5] += pb.y; s[6] += pb.z; s[7] += pb.w;
             // hand this CTA's partial sums to its cluster's first CTA: xpart[rank][row][8]
-            const uint32_t dst = map_to_cta(smem_base + L.xpart + (rank * kTileM + row) * kMaxHeads * 4, 0);
+            const uint32_t dst = map_to_cta(smem_base + L.xpart + (rank * kTileM + row) * kMaxHeads * 4, half);
             st_shared_cluster_v4(dst, s[0], s[1], s[2], s[3]);
             st_shared_cluster_v4(dst + 16, s[4], s[5], s[6], s[7]);
         }
@@ -486,7 +516,8 @@ score_split_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_cons
     if (threadIdx.x == 0 && *abort_flag) atomicCAS(p.status, 0, 5 /* KVZAP_ERR_TIMEOUT */);
     if (warp == 1) {
         tc_fence_after_sync();
-        tmem_dealloc(tmem_base, static_cast<uint32_t>(p.tmem_cols));
+        if constexpr (kPair) tmem_dealloc_pair(tmem_base, static_cast<uint32_t>(p.tmem_cols));
+        else tmem_dealloc(tmem_base, static_cast<uint32_t>(p.tmem_cols));
     }
     // If this launch was allowed to start before the kernel ahead of it had finished (consecutive decode
     // steps), it still completes after it: every thread waits here.
@@ -507,13 +538,13 @@ score_split_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_cons
         const int32_t done_i = (layer * p.tiles_per_layer + m_tile) * n_split + nh;
         if (n_split > 1) {
             // the slices meet in global memory; whoever arrives last finishes the tile
-            float4 *mine = reinterpret_cast<float4 *>(p.split_part + ((static_cast<int64_t>(tile) * n_split + nh) * kTileM + row) * kMaxHeads);
+            float4 *mine = reinterpret_cast<float4 *>(p.split_part + ((static_cast<int64_t>(part_tile) * n_split + nh) * kTileM + row) * kMaxHeads);
             __stcg(mine, make_float4(s[0], s[1], s[2], s[3]));
             __stcg(mine + 1, make_float4(s[4], s[5], s[6], s[7]));
             __threadfence();
             named_barrier_sync(2, 128);
             if (threadIdx.x == 64) {
-                *last_flag = arrive_last(p.split_arrive + tile, static_cast<uint32_t>(n_split)) ? 1 : 0;
+                *last_flag = arrive_last(p.split_arrive + part_tile, static_cast<uint32_t>(n_split)) ? 1 : 0;
                 __threadfence();
             }
             named_barrier_sync(2, 128);
@@ -525,7 +556,7 @@ score_split_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_cons
 #pragma unroll
             for (int h = 0; h < kMaxHeads; ++h) s[h] = 0.0f;
             for (int r = 0; r < n_split; ++r) {
-                const float4 *src = reinterpret_cast<const float4 *>(p.split_part + ((static_cast<int64_t>(tile) * n_split + r) * kTileM + row) * kMaxHeads);
+                const float4 *src = reinterpret_cast<const float4 *>(p.split_part + ((static_cast<int64_t>(part_tile) * n_split + r) * kTileM + row) * kMaxHeads);
                 const float4 pa = __ldcg(src), pb = __ldcg(src + 1);
                 s[0] += pa.x; s[1] += pa.y; s[2] += pa.z; s[3] += pa.w;
                 s[4] += pb.x; s[5] += pb.y; s[6] += pb.z; s[7] += pb.w;
