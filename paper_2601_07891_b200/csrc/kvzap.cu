@@ -565,6 +565,13 @@ static double split_load(const kvzap_ctx *ctx, const kvzap_ctx::SplitLayout &l, 
     return (kTileM + static_cast<double>(ctx->cfg.hidden) / l.n / (pair ? 2 : 1)) / k;
 }
 
+// Whether a wave of the surrogate's tiles takes far longer than a launch (4096 -> 512: 52 us, so 13 us at this size): below,
+// neither pairs nor a launch of its own for left-over blocks gain anything.
+static bool long_waves(const kvzap_ctx *ctx)
+{
+    return static_cast<int64_t>(ctx->cfg.d_model) * ctx->cfg.hidden >= int64_t{1} << 19;
+}
+
 // The layout with CTA pairs for a prompt of that many blocks whose CTAs load least, if they load a tenth less than `other`;
 // nullptr if there is none whose clusters the device holds at once, and for launches that run beside their neighbours
 // (`beside`), where it made nothing faster for sure.  4096 -> 512 -> 8, calls in a row on a default context, us a call: 1700
@@ -575,7 +582,7 @@ static const kvzap_ctx::SplitLayout *pair_layout(const kvzap_ctx *ctx, int64_t b
     const kvzap_ctx::SplitLayout *best = nullptr;
     double least = 0.9 * other;
     const int64_t pairs = (blocks + 1) / 2;
-    for (int i = 0; i < (beside ? 0 : ctx->n_pair_layouts); ++i) {
+    for (int i = 0; i < (beside || !long_waves(ctx) ? 0 : ctx->n_pair_layouts); ++i) {
         const kvzap_ctx::SplitLayout &l = ctx->pair_layouts[i];
         const int64_t ctas = pairs * 2 * l.n * l.k;
         if ((fp8 && !l.ok8) || ctas > ctx->sm_count || pairs * l.n > l.max_clusters) continue;
@@ -618,7 +625,7 @@ static cudaError_t launch_split(const kvzap_ctx::SplitLayout &l, int k, bool pai
 static int64_t rest_blocks(const kvzap_ctx *ctx, int64_t blocks, bool fp8)
 {
     const int64_t wave = 2 * static_cast<int64_t>(ctx->pair_clusters);
-    if (ctx->trusted || ctx->profiling || ctx->cfg.hidden == 0 || wave == 0 || blocks <= wave) return 0;
+    if (ctx->trusted || ctx->profiling || !long_waves(ctx) || wave == 0 || blocks <= wave) return 0;
     const int64_t rest = blocks % wave;
     bool pair;
     return rest > 0 && prompt_layout(ctx, rest, fp8, false, &pair) != nullptr ? rest : 0;
