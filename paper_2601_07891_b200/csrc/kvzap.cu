@@ -92,6 +92,7 @@ struct kvzap_ctx {
     int32_t *tile_counters = nullptr;    // [kMaskRing] work-tile counters of the scoring launches, used in rotation
     uint32_t *select_hist = nullptr;     // fixed-budget selection: [passes][select_seqs][H][bins] histograms, zero between calls
     int32_t select_seqs = 0;             //                         sequences they have room for, grown by the calls
+    int select_cluster = 0;              // CTAs of a selection in one launch, at most (0: not available)
     bool select_clean = false;           //                         all zero as far as the host knows
     uint32_t *select_arrive = nullptr;   //                         [max_seqs][H] CTAs that are done, zero between launches
     float *select_tau = nullptr;         //                         [max_seqs][H] cut values when the caller wants none
@@ -1164,7 +1165,8 @@ static kvzap_status launch_prune_onepass(kvzap_ctx *ctx, const float *scores, co
                                          int64_t n_tokens, void *K_out, void *V_out, int32_t *lengths, int32_t page_tokens,
                                          int32_t first_page, int64_t n_pages_pool, int32_t max_pages, int32_t *page_table,
                                          int32_t *n_pages_used, cudaStream_t stream, int32_t *slot_out = nullptr,
-                                         bool scores_just_made = false, uint32_t *clear = nullptr, int64_t clear_words = 0)
+                                         bool scores_just_made = false, uint32_t *clear = nullptr, int64_t clear_words = 0,
+                                         bool tau_behind = false)
 {
     const kvzap_config &c = ctx->cfg;
     if (page_tokens > 0 && n_pages_pool * page_tokens >= 0xffffffffLL)
@@ -1270,7 +1272,7 @@ static kvzap_status launch_prune_onepass(kvzap_ctx *ctx, const float *scores, co
     p.scan_flag = ctx->op_scan_flag + set;
     p.epoch = ctx->op_epoch;
     p.wait_limit = ctx->wait_limit;
-    p.wait_first = wait_first ? 1 : 0;
+    p.wait_first = tau_behind ? 2 : wait_first ? 1 : 0;
     {
         ProfScope prof(ctx, KVZAP_KERNEL_COMPACT, stream);
         cudaLaunchConfig_t cfg;
@@ -1544,6 +1546,22 @@ kvzap_status kvzap_create(kvzap_ctx **out, const kvzap_config *cfg)
         free_all(ctx);
         delete ctx;
         return KVZAP_ERR_CUDA;
+    }
+    // clusters of 16 CTAs where the device takes them, else of 8
+    for (int cluster : {kSelectMaxCluster, 8}) {
+        if (cluster > 8 && cudaFuncSetAttribute(select_cluster_kernel, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) != cudaSuccess) {
+            cudaGetLastError();
+            continue;
+        }
+        cudaLaunchConfig_t cfg;
+        cudaLaunchAttribute attrs[2];
+        make_launch(&cfg, attrs, dim3(static_cast<unsigned>(cluster)), dim3(kSelectThreads), 0, nullptr, false, cluster);
+        int fit = 0;
+        if (cudaOccupancyMaxActiveClusters(&fit, select_cluster_kernel, &cfg) == cudaSuccess && fit >= c.n_kv_heads) {
+            ctx->select_cluster = cluster;
+            break;
+        }
+        cudaGetLastError();
     }
     CREATE_CUDA(cudaMalloc(&ctx->select_arrive, sizeof(uint32_t) * static_cast<size_t>(c.max_seqs) * c.n_kv_heads));
     CREATE_CUDA(cudaMemset(ctx->select_arrive, 0, sizeof(uint32_t) * static_cast<size_t>(c.max_seqs) * c.n_kv_heads));
@@ -1837,6 +1855,25 @@ kvzap_status kvzap_prune_prefill_topk(kvzap_ctx *ctx, const void *K, const void 
     st = check_prune_args(ctx, K, V, K_out, V_out, lengths, w);
     if (st != KVZAP_OK) return st;
     if (!scores) return fail(ctx, KVZAP_ERR_INVALID_ARG, "scores is NULL");
+    if (!per_layer && ctx->select_cluster > 0 && n_tokens <= kSelectClusterTokens * n_seqs && n_seqs <= 65535) {
+        // One launch: CTAs of some 2048 candidates of an average sequence, at most as many as a cluster may have; and more
+        // than that, for batches with one sequence far longer than the others, where all of them still fit in one wave.
+        int cluster = 1;
+        const int64_t lists = static_cast<int64_t>(c.n_kv_heads) * n_seqs;
+        while (cluster < ctx->select_cluster &&
+               (static_cast<int64_t>(cluster) * kSelectKept * kSelectThreads * n_seqs < n_tokens ||
+                (2 * cluster * lists <= 4 * static_cast<int64_t>(ctx->sm_count) && static_cast<int64_t>(cluster) * 2 * 8192 <= n_tokens)))
+            cluster *= 2;
+        cudaLaunchConfig_t cfg;
+        cudaLaunchAttribute attrs[2];
+        make_launch(&cfg, attrs, dim3(static_cast<unsigned>(cluster), static_cast<unsigned>(c.n_kv_heads), static_cast<unsigned>(n_seqs)),
+                    dim3(kSelectThreads), 0, stream, !ctx->profiling, cluster);
+        KVZAP_CUDA(ctx, cudaLaunchKernelEx(&cfg, select_cluster_kernel, scores, n_tokens, static_cast<int>(c.n_kv_heads), cu_seqlens,
+                                           static_cast<int>(w), keep_ratio, tau_list));
+        ctx->launches += 1;
+        return launch_prune_onepass(ctx, scores, tau_list, 0.0f, w, K, V, cu_seqlens, n_seqs, n_tokens, K_out, V_out, lengths, 0,
+                                    0, 0, 0, nullptr, nullptr, stream, nullptr, false, nullptr, 0, true);
+    }
     const int n_sel = per_layer ? 1 : c.n_kv_heads;
     const int32_t group = n_seqs < kSelectSeqs ? n_seqs : kSelectSeqs;
     st = reserve_select(ctx, group);

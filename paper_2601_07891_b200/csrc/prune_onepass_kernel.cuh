@@ -81,7 +81,8 @@ struct PruneParams {
     int64_t clear_units;
     int32_t recount;           // 1: short dense input, one head per CTA: rows kept before the CTA's first token are counted
                                // from the scores, not learnt from the CTAs before it
-    int32_t wait_first;        // 1: wait for the work ahead in the stream before the first load
+    int32_t wait_first;        // 1: wait for the work ahead in the stream before the first load; 2: before tau_list is read,
+                               // the launch ahead, which writes it, started only when everything ahead of it was complete
 };
 
 // Spins until *flag == want (acquire); false when the cycle budget runs out.
@@ -191,7 +192,7 @@ prune_onepass_kernel(const PruneParams p)
     __shared__ float tau_s[kMaxHeads];                  // thresholds of the sequence at the CTA's first token
 
     griddep_launch_dependents();
-    if (p.wait_first) griddep_wait();
+    if (p.wait_first == 1) griddep_wait();
 
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const int H = p.n_heads;
@@ -218,6 +219,19 @@ prune_onepass_kernel(const PruneParams p)
         b_hi = seq_of_token(p.cu_seqlens, p.n_seqs, t_last);
         s0 = p.cu_seqlens[b_lo];
     }
+    // the scores of the first words that this warp looks at, on their way during the wait for the thresholds
+    constexpr int kUnroll = 4;                                // words whose scores are in flight together
+    const int n_w = static_cast<int>(blk1 - blk0) * 4;        // 32-token words of this CTA
+    TokenScores ts[kUnroll];
+    auto load_words = [&](int w0) {
+#pragma unroll
+        for (int u = 0; u < kUnroll; ++u) {
+            const int wl = w0 + u * (kOpThreads / 32);
+            if (wl < n_w) load_token(p, blk0 * 4 + wl, lane, multi, ts[u]);
+        }
+    };
+    load_words(warp);
+    if (p.wait_first == 2) griddep_wait();
     if (tid < kMaxHeads) tau_s[tid] = p.tau_list != nullptr && tid < H ? __ldcg(p.tau_list + b_lo * H + tid) : p.tau;
     const int j0 = static_cast<int>((s0 / kBlockTokens) / p.blocks_per_cta);      // the CTA (column) whose blocks hold s0
     __syncthreads();
@@ -225,15 +239,8 @@ prune_onepass_kernel(const PruneParams p)
     // ---------------------------------------------------------------- A: keep bits and counts of the CTA's blocks
     {
         int32_t my_cnt = 0;                                   // lane h: kept rows of head h in the words this warp made
-        const int n_w = static_cast<int>(blk1 - blk0) * 4;    // 32-token words of this CTA
-        constexpr int kUnroll = 4;                            // words whose scores are in flight together
         for (int w0 = warp; w0 < n_w; w0 += (kOpThreads / 32) * kUnroll) {
-            TokenScores ts[kUnroll];
-#pragma unroll
-            for (int u = 0; u < kUnroll; ++u) {
-                const int wl = w0 + u * (kOpThreads / 32);
-                if (wl < n_w) load_token(p, blk0 * 4 + wl, lane, multi, ts[u]);
-            }
+            if (w0 != warp) load_words(w0);
 #pragma unroll
             for (int u = 0; u < kUnroll; ++u) {
                 const int wl = w0 + u * (kOpThreads / 32);

@@ -15,7 +15,8 @@
 // possible, a CTA counts one head only (2048 bins instead of 8 x 256 of four passes), and the scores of a
 // later pass are loaded before the wait for the pass ahead.  32k tokens x 8 heads, from the first launch to
 // the cut values: 35.5 us with four passes of 8 bits, a memset ahead and a launch for the cut values
-// behind them, 17.6 us now.
+// behind them, 17.6 us now.  That serves cut values per layer and very long sequences; others take one launch of clusters
+// (select_cluster_kernel).
 #pragma once
 
 #include "score_kernel.cuh"
@@ -225,6 +226,101 @@ select_pass_kernel(const float *__restrict__ scores, int64_t n_tokens, int n_hea
     } else if (tid == 0) {
         tau_list[b * n_heads + h] = tau;
     }
+}
+
+// The same selection in one launch, for cut values per head: a cluster of gridDim.x CTAs (a power of two, at most 16) per
+// (sequence, head), each with an equal share of the candidates, of which a thread keeps the first kSelectKept in registers
+// and reads the others again in every pass.  A pass counts its digit in shared memory, adds what there is to the bins of
+// the CTA that owns them (2048 / gridDim.x each, in distributed shared memory), and after one cluster barrier every CTA
+// reads all bins and takes the digit itself: no global memory, no launch and no grid-wide meeting between the passes.  The
+// pruning behind it reads its first scores before it waits for the cut values.  32k tokens x 8 heads, a quarter kept, the
+// whole call: 38.8 us with three launches, 37.6 us with this one, 36.2 us with the early scores; a first pass on new inputs
+// 74 -> 65 us.  (Bins owned in turn, so that neighbouring ones, which most keys share, spread over the CTAs: 65 us, a thread's
+// eight bins then come from eight CTAs.)
+constexpr int kSelectKept = 8;
+constexpr int kSelectMaxCluster = 16;
+// Tokens of an average sequence up to which it is taken.  The whole call, us: one sequence of 300 tokens 23.4 -> 17.8, 16000
+// tokens 29.9 -> 26.0, 32768 tokens 38.3 -> 36.5, but 65536 tokens 55.9 -> 57.4, 131072 tokens 87.5 -> 91.8 (16 CTAs a head are
+// too few for the counting); 4 x 32768 tokens 99 -> 88, 7 x 4681 tokens 49.2 -> 42.7, 60 x 546 tokens 63 -> 45.5.
+constexpr int64_t kSelectClusterTokens = 40960;
+
+__global__ void __launch_bounds__(kSelectThreads)
+select_cluster_kernel(const float *__restrict__ scores, int64_t n_tokens, int n_heads, const int32_t *__restrict__ cu_seqlens,
+                      int window, float keep_ratio, float *__restrict__ tau_list)
+{
+    __shared__ uint32_t sh[kSelectBins];
+    __shared__ __align__(16) uint32_t all[kSelectPasses][kSelectBins];      // of every pass, the bins that this CTA owns
+    __shared__ uint32_t scratch[kSelectThreads / 32 + 2];
+    griddep_wait();
+    griddep_launch_dependents();
+    const int h = blockIdx.y, b = blockIdx.z, tid = threadIdx.x;
+    const int64_t t0 = cu_seqlens ? cu_seqlens[b] : 0, t1 = cu_seqlens ? cu_seqlens[b + 1] : n_tokens;
+    const int64_t n_cand = t1 - t0 - window > 0 ? t1 - t0 - window : 0;
+    bool too_many;
+    const uint32_t k = select_budget(keep_ratio, n_cand, 0, n_heads, too_many);      // n_cand < 2^32: never too many
+    if (k == 0u) {                                        // the whole cluster
+        if (blockIdx.x == 0 && tid == 0) tau_list[b * n_heads + h] = INFINITY;
+        return;
+    }
+    const int64_t share = (n_cand + gridDim.x - 1) / gridDim.x;
+    const int64_t lo = blockIdx.x * share, hi = lo + share < n_cand ? lo + share : n_cand;
+    const float *mine = scores + t0 * n_heads + h;
+    float v[kSelectKept];
+#pragma unroll
+    for (int j = 0; j < kSelectKept; ++j) {
+        const int64_t i = lo + j * kSelectThreads + tid;
+        v[j] = i < hi ? __ldcg(mine + i * n_heads) : __uint_as_float(0x7fffffffu);      // NaN: no candidate
+    }
+    for (int i = tid; i < kSelectBins; i += kSelectThreads) {
+        sh[i] = 0u;
+#pragma unroll
+        for (int q = 0; q < kSelectPasses; ++q) all[q][i] = 0u;
+    }
+    cluster_sync_all();                                   // everybody's bins are zero
+    const int own_bits = 11 - (31 - __clz(static_cast<int>(gridDim.x)));      // log2 of the bins that a CTA owns
+    uint32_t prefix = 0u, k_rem = k, above;
+    bool dead = false;                                    // fewer candidates than the budget: the cut value is -inf
+#pragma unroll
+    for (int pass = 0; pass < kSelectPasses; ++pass) {
+        const int shift = select_shift(pass), bits = select_bits(pass);
+        auto count = [&](float x) {
+            if (x != x) return;
+            const uint32_t key = score_key(x);
+            if (pass == 0 || (key >> (shift + bits)) == prefix) atomicAdd(&sh[(key >> shift) & ((1u << bits) - 1u)], 1u);
+        };
+#pragma unroll
+        for (int j = 0; j < kSelectKept; ++j) count(v[j]);
+        for (int64_t base = lo + kSelectKept * kSelectThreads; base < hi; base += 4 * kSelectThreads) {
+            float x[4];
+#pragma unroll
+            for (int j = 0; j < 4; ++j) {
+                const int64_t i = base + j * kSelectThreads + tid;
+                x[j] = i < hi ? __ldcg(mine + i * n_heads) : __uint_as_float(0x7fffffffu);
+            }
+#pragma unroll
+            for (int j = 0; j < 4; ++j) count(x[j]);
+        }
+        __syncthreads();
+        const uint32_t bins_addr = smem_u32(&all[pass][0]);
+        for (int i = tid; i < kSelectBins; i += kSelectThreads) {
+            const uint32_t n = sh[i];
+            if (n) {
+                sh[i] = 0u;
+                red_shared_cluster_add(map_to_cta(bins_addr + 4 * i, static_cast<uint32_t>(i) >> own_bits), n);
+            }
+        }
+        cluster_sync_all();
+        SelectBins bins;                                  // 8 consecutive ones belong to one CTA
+        const uint32_t at = map_to_cta(bins_addr + 32 * tid, static_cast<uint32_t>(8 * tid) >> own_bits);
+        ld_shared_cluster_v4(at, bins.c[0], bins.c[1], bins.c[2], bins.c[3]);
+        ld_shared_cluster_v4(at + 16, bins.c[4], bins.c[5], bins.c[6], bins.c[7]);
+        const uint32_t bin = select_bin(bins, k_rem, above, scratch);
+        if (bin == kSelectBins) { dead = true; break; }   // in the first pass, and the same in every CTA
+        prefix = (prefix << bits) | bin;
+        k_rem -= above;
+    }
+    if (blockIdx.x == 0 && tid == 0) tau_list[b * n_heads + h] = dead ? -INFINITY : key_score(prefix);
+    cluster_sync_all();                                   // nobody leaves while its bins may still be read
 }
 
 }  // namespace kvzap
