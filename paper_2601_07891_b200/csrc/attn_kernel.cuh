@@ -21,6 +21,13 @@
 // every CTA reads all list lengths, finds the shortest part length (of at least four tiles a warp) for which
 // all parts fit the grid, and takes the part of its index.  8 sequences x 8 heads, 2176 rows on average: 26.0 -> 20.4 us per call.
 //
+// Layer by layer a small batch is a chain of two launches of about the same length, the step (round trips to memory on a
+// fifth of the SMs) and this one (round trips, then rows).  On a context that trusts its producers they run beside one another
+// (kBeside): the step behind an attention scores beside it and only its stores to the cache wait, and the attention behind
+// that step reads all rows that the lists held before it while it runs; what the step changes (the prefix's last tile, the
+// window) is read when it has completed, and so are the queries, once more -- if they are not what they were, the CTA starts
+// again.  36 layers x 8 sequences x 2176 rows 1238 -> 836 us, 4 layers x 128 sequences x 4736 rows 1596 -> 1524 us.
+//
 // Math per tile, on the warp-level tensor-core path (the work is HBM-bound; 16-row MMAs are enough):
 //   S[16 x 16]  = Q[16 x D] K^T      m16n8k16, Q rows 0..G-1 real, the rest zero
 //   P           = exp2(S * scale * log2(e) - running max), rows beyond the list's end masked
@@ -77,6 +84,8 @@ struct AttnParams {
     int32_t n_parts;            // CTAs per list (1 = the CTA writes the output itself); 0 = by length, see attn_unit
     float *part_scratch;        // [CTA] { m[8], l[8], O[8][D] }: the parts of a list are consecutive CTAs
     uint32_t *part_arrive;      // [list] parts that have stored their triple; back to 0 after the launch
+    int32_t beside_ctas;        // kBeside: CTAs [0, beside_ctas) run beside the step, as many as find room
+    int32_t beside_tiles;       // n_parts == 0: with more tiles than this in all lists all CTAs wait for the step
 };
 
 // The lists of a call, of lengths[0 .. n) tiles, cut into at most n_units (>= n) parts: a list of t tiles has
@@ -179,7 +188,9 @@ __device__ __forceinline__ void attn_store(uint16_t *out, const float4 &num, flo
     *reinterpret_cast<uint2 *>(out) = v;
 }
 
-template <int kD, bool kFp8>
+// kBeside: the launch may run beside the step ahead of it (p.after_step); a kernel of its own, since what that takes (the rest
+// of a list learnt late, queries read twice) costs a launch that cannot some 2 us.
+template <int kD, bool kFp8, bool kBeside>
 __global__ void __launch_bounds__(kAttnThreads, kFp8 ? 4 : 3)
 decode_attn_kernel(const __grid_constant__ CUtensorMap tmap_kpool, const __grid_constant__ CUtensorMap tmap_vpool,
                    const __grid_constant__ CUtensorMap tmap_kring, const __grid_constant__ CUtensorMap tmap_vring,
@@ -206,9 +217,11 @@ decode_attn_kernel(const __grid_constant__ CUtensorMap tmap_kpool, const __grid_
     const CacheView &c = p.c;
     const int H = c.n_heads, B = c.n_seqs;
 
+    __shared__ int queries_s;               // kBeside: warps that are done with the queries in memory
     if (threadIdx.x == 0) {
         for (int i = 0; i < kAttnWarps * kAttnStages; ++i) mbar_init(bars + 8 * i, 1);
         *abort_flag = 0;
+        queries_s = 0;
         fence_mbar_init();
         prefetch_tensormap(&tmap_kpool);
         prefetch_tensormap(&tmap_vpool);
@@ -216,67 +229,154 @@ decode_attn_kernel(const __grid_constant__ CUtensorMap tmap_kpool, const __grid_
         prefetch_tensormap(&tmap_vring);
     }
     __syncthreads();
-    // started while the kernel ahead (the step that appended the newest rows) may still be running: nothing of the
-    // caller's or of the cache is read before it has completed
-    griddep_wait();
+    // Started while the kernel ahead may still be running: nothing of the caller's or of the cache is read before that has
+    // completed.  kBeside: that is the step which appends the newest rows, and nothing else that writes the cache is still
+    // running (the host knows, see attention_impl); every whole tile of rows that a list held before it is taken beside it.
+    // How long the lists were before the step, by which the CTAs of a launch share them out, all read in c.before: it does
+    // not change while this launch runs.  CTAs that find no room beside the step wait for it first.
+    bool beside = kBeside && static_cast<int>(blockIdx.x) < p.beside_ctas;
+    if (!beside) griddep_wait();
 
     int list, part, n_parts = p.n_parts;
-    int32_t n_total, n_prefix;
+    int32_t n_before = 0;                   // kBeside: prefix rows that nothing ahead of this launch still touches
+    int32_t n_prefix = 0, n_total = 0;      // rows and tokens now; beside the step not known yet
+    const int32_t *before = kBeside ? c.before : c.prefix_len;
     auto cache_list = [&](int i) {          // list i of the call among the cache's lists
         return (static_cast<int64_t>((i / H) % B) * c.n_layers + p.layer0 + i / (H * B)) * H + i % H;
     };
     if (n_parts > 0) {
         list = blockIdx.x / n_parts;
         part = blockIdx.x % n_parts;
-        n_total = __ldcg(c.n_tokens + cache_list(list));
-        n_prefix = __ldcg(c.prefix_len + cache_list(list));
+        if (kBeside) n_before = min(__ldcg(before + cache_list(list)), __ldcg(c.prefix_len + cache_list(list)));
+        if (!beside) {
+            n_total = __ldcg(c.n_tokens + cache_list(list));
+            n_prefix = __ldcg(c.prefix_len + cache_list(list));
+        }
     } else {
-        // over the stages, not in use yet: [list] tiles, then [list] (tokens, prefix rows)
+        // over the stages, not in use yet: [list] tiles, then [list] (prefix rows, tokens); kBeside: the window counts in full
         const int n_lists = p.n_layers_call * B * H;
         int32_t *lengths = reinterpret_cast<int32_t *>(smem);
         int2 *counts = reinterpret_cast<int2 *>(smem + 4 * 32 * kAttnListsPerLane);
         for (int i = threadIdx.x; i < n_lists; i += kAttnThreads) {
-            const int2 n = make_int2(__ldcg(c.n_tokens + cache_list(i)), __ldcg(c.prefix_len + cache_list(i)));
+            int2 n = make_int2(__ldcg(before + cache_list(i)), beside ? 0 : __ldcg(c.n_tokens + cache_list(i)));
+            if (kBeside) n.x = min(n.x, __ldcg(c.prefix_len + cache_list(i)));      // it never is less, nor may it be
             counts[i] = n;
-            lengths[i] = (n.y + kAttnTileRows - 1) / kAttnTileRows + (min(n.x, c.window) + kAttnTileRows - 1) / kAttnTileRows;
+            lengths[i] = (n.x + kAttnTileRows - 1) / kAttnTileRows + ((kBeside ? c.window : min(n.y, c.window)) + kAttnTileRows - 1) / kAttnTileRows;
         }
         __syncthreads();
-        n_parts = attn_unit(lengths, n_lists, gridDim.x, blockIdx.x, lane, list, part);
-        if (n_parts == 0) return;                                  // the whole CTA: more CTAs than parts
-        n_total = counts[list].x;
-        n_prefix = counts[list].y;
+        // One wave: beside the step, on the SMs that it leaves, if what that adds to the wave's time is less than the step's;
+        // else on all of them, behind it.
+        int n_units = gridDim.x;
+        if constexpr (kBeside) {
+            int sum = 0;
+            for (int i = lane; i < n_lists; i += 32) sum += lengths[i];
+            sum = __reduce_add_sync(0xffffffffu, sum);
+            if (n_lists <= p.beside_ctas && sum <= p.beside_tiles) {
+                n_units = p.beside_ctas;
+            } else if (beside) {
+                griddep_wait();
+                beside = false;
+                for (int i = threadIdx.x; i < n_lists; i += kAttnThreads) counts[i].y = __ldcg(c.n_tokens + cache_list(i));
+                __syncthreads();
+            }
+        }
+        n_parts = attn_unit(lengths, n_lists, n_units, blockIdx.x, lane, list, part);
+        if (n_parts == 0) {                                        // the whole CTA: more CTAs than parts
+            griddep_wait();
+            return;
+        }
+        n_before = n_prefix = counts[list].x;
+        n_total = counts[list].y;
+        if (kBeside && !beside) n_prefix = __ldcg(c.prefix_len + cache_list(list));
         fence_proxy_async_smem();                                  // the copies below write where these were read
         __syncthreads();
     }
-    const int h = list % H, b = (list / H) % B, l_rel = list / (H * B);
-    const int64_t li = cache_list(list);
 
-    const int32_t n_ring = c.window > 0 ? (n_total < c.window ? n_total : c.window) : 0;
+    // This CTA's tiles are its run [s_first, n_tiles) of the list's, the prefix's and then the window's.  kBeside: numbered s = 0, 1,
+    // ... n_tiles - 1, [t_first, t_first + n_early) of the prefix's whole tiles, which are there for good, and behind those every
+    // n_parts-th of the others (the end of the prefix, the window), known only when the kernel ahead has completed (learn_rest).
     const int tiles_per_page = c.page_tokens / kAttnTileRows;
-    const int n_pt = (n_prefix + kAttnTileRows - 1) / kAttnTileRows;
-    const int n_rt = (n_ring + kAttnTileRows - 1) / kAttnTileRows;
-    const int n_tiles_list = n_pt + n_rt;
-    // this CTA's run of the list's tiles
-    const int t_begin = static_cast<int>(static_cast<int64_t>(n_tiles_list) * part / n_parts);
-    const int n_tiles = static_cast<int>(static_cast<int64_t>(n_tiles_list) * (part + 1) / n_parts);
-    const int32_t *pages = c.page_table + li * c.max_pages;
+    const int32_t *pages = c.page_table + cache_list(list) * c.max_pages;
+    const int32_t ring_row0 = kBeside ? 0 : static_cast<int32_t>(cache_list(list) * c.window);
+    int t_first, n_tiles, n_early = 0;
+    int32_t n_ring = 0;
+    int n_pt = 0;
+    {
+        n_ring = c.window > 0 ? (n_total < c.window ? n_total : c.window) : 0;
+        n_pt = (n_prefix + kAttnTileRows - 1) / kAttnTileRows;
+        const int n_run = kBeside ? n_before / kAttnTileRows : n_pt + (n_ring + kAttnTileRows - 1) / kAttnTileRows;
+        t_first = static_cast<int>(static_cast<int64_t>(n_run) * part / n_parts);
+        n_tiles = static_cast<int>(static_cast<int64_t>(n_run) * (part + 1) / n_parts);
+        if (kBeside) n_early = n_tiles -= t_first;
+    }
+    const int s_first = kBeside ? 0 : t_first;
+    // kBeside, per warp, in shared memory for want of registers: what the main loop seldom needs
+    enum { kTail, kRing, kList, kPart, kParts, kFull, kKept };      // rows of the prefix's end and of the window; the rest as above
+    __shared__ volatile int32_t kept_s[kAttnWarps][kKept];
+    bool waited = !beside;
+    auto learn_rest = [&](int32_t tokens, int32_t rows) {          // whole warp, once
+        const int32_t tail = rows - kept_s[warp][kFull] * kAttnTileRows;
+        const int32_t ring = c.window > 0 ? (tokens < c.window ? tokens : c.window) : 0;
+        if (lane == 0) { kept_s[warp][kTail] = tail; kept_s[warp][kRing] = ring; }
+        __syncwarp();
+        const int n_rest = (tail + kAttnTileRows - 1) / kAttnTileRows + (ring + kAttnTileRows - 1) / kAttnTileRows;
+        const int mine = kept_s[warp][kPart], all = kept_s[warp][kParts];
+        n_tiles = n_early + (n_rest > mine ? (n_rest - mine + all - 1) / all : 0);
+        waited = true;
+    };
+    // tile s >= n_early: its first row in the prefix's end or in the window, rows left there; true in the window
+    auto rest_tile = [&](int s, int32_t &row, int32_t &left) -> bool {
+        const int32_t tail = kept_s[warp][kTail];
+        const int t = kept_s[warp][kPart] + (s - n_early) * kept_s[warp][kParts], tail_tiles = (tail + kAttnTileRows - 1) / kAttnTileRows;
+        const bool ring = t >= tail_tiles;
+        row = (ring ? t - tail_tiles : t) * kAttnTileRows;
+        left = (ring ? kept_s[warp][kRing] : tail) - row;
+        return ring;
+    };
+    if constexpr (kBeside) {
+        if (lane == 0) {
+            kept_s[warp][kList] = list;
+            kept_s[warp][kPart] = part;
+            kept_s[warp][kParts] = n_parts;
+            kept_s[warp][kFull] = n_before / kAttnTileRows;
+        }
+        __syncwarp();
+        if (!beside) learn_rest(n_total, n_prefix);
+    }
 
     const uint32_t my_stages = smem_base + warp * kAttnStages * kStageBytes;
     const uint32_t my_bars = bars + 8 * warp * kAttnStages;
     const uint64_t policy = l2_policy_evict_first();
 
-    // first row (in its tensor map) of tile t of this list; needs the page number for prefix tiles
-    auto tile_row = [&](int t) -> int32_t {
-        if (t < n_pt) {
-            const int32_t page = __ldcg(pages + t / tiles_per_page);
-            return page * c.page_tokens + (t % tiles_per_page) * kAttnTileRows;
-        }
-        return static_cast<int32_t>(li * c.window) + (t - n_pt) * kAttnTileRows;
+    // Tile s: its number among the prefix's tiles, or -1 - its first row in the rings; kBeside only
+    auto tile_at = [&](int s) -> int32_t {
+        if (s < n_early) return t_first + s;
+        int32_t row, left;
+        if (rest_tile(s, row, left)) return -1 - (static_cast<int32_t>(cache_list(kept_s[warp][kList]) * c.window) + row);
+        return kept_s[warp][kFull] + row / kAttnTileRows;
     };
-    auto issue = [&](int t, int32_t row, int stage) {
+    // the page that a prefix tile is in, and its first row (in its tensor map) from there; apart, so that the loads of several
+    // tiles go out together
+    auto page_of = [&](int32_t t) -> int32_t { return t >= 0 ? __ldcg(pages + t / tiles_per_page) : 0; };
+    auto row_of = [&](int32_t t, int32_t page) { return t >= 0 ? page * c.page_tokens + (t % tiles_per_page) * kAttnTileRows : t; };
+    // first row (in its tensor map) of tile s; needs the page number for prefix tiles.  kBeside: rows of the rings as -1 - row
+    auto tile_row = [&](int s) -> int32_t {
+        if constexpr (kBeside) {
+            const int32_t t = tile_at(s);
+            return row_of(t, page_of(t));
+        } else {
+            if (s < n_pt) {
+                const int32_t page = __ldcg(pages + s / tiles_per_page);
+                return page * c.page_tokens + (s % tiles_per_page) * kAttnTileRows;
+            }
+            return ring_row0 + (s - n_pt) * kAttnTileRows;
+        }
+    };
+    auto issue = [&](int s, int32_t row, int stage) {
         const uint32_t dst = my_stages + stage * kStageBytes;
         const uint32_t bar = my_bars + 8 * stage;
-        const bool prefix = t < n_pt;
+        const bool prefix = kBeside ? row >= 0 : s < n_pt;
+        if (kBeside && !prefix) row = -1 - row;
         mbar_arrive_expect_tx(bar, kStageBytes);
         if constexpr (kFp8) {
             // a tile of 8-bit rows is one contiguous piece of memory: coordinates (0, 0, tile)
@@ -291,82 +391,145 @@ decode_attn_kernel(const __grid_constant__ CUtensorMap tmap_kpool, const __grid_
         }
     };
 
-    // prologue: fill the stages, the pages of all of them looked up together; row_next belongs to the first tile not
-    // yet issued
-    int t_issue = t_begin + warp;
+    // Fills the stages, all free, from tile s_issue on, the pages of all of them looked up together; row_next belongs to the
+    // first tile not yet issued.
+    int s_issue = 0;
     int32_t row_next = 0;
-    {
+    auto fill = [&](int first_stage) {
         int32_t rows[kAttnStages + 1];
+        if constexpr (kBeside) {
+            int32_t t[kAttnStages + 1], page[kAttnStages + 1];
 #pragma unroll
-        for (int s = 0; s <= kAttnStages; ++s) rows[s] = t_issue + s * kAttnWarps < n_tiles ? tile_row(t_issue + s * kAttnWarps) : 0;
+            for (int i = 0; i <= kAttnStages; ++i) t[i] = s_issue + i * kAttnWarps < n_tiles ? tile_at(s_issue + i * kAttnWarps) : -1;
 #pragma unroll
-        for (int s = 0; s < kAttnStages; ++s)
-            if (t_issue < n_tiles) {
-                if (lane == 0) issue(t_issue, rows[s], s);
-                t_issue += kAttnWarps;
+            for (int i = 0; i <= kAttnStages; ++i) page[i] = page_of(t[i]);
+#pragma unroll
+            for (int i = 0; i <= kAttnStages; ++i) rows[i] = row_of(t[i], page[i]);
+        } else {
+#pragma unroll
+            for (int i = 0; i <= kAttnStages; ++i) rows[i] = s_issue + i * kAttnWarps < n_tiles ? tile_row(s_issue + i * kAttnWarps) : 0;
+        }
+#pragma unroll
+        for (int i = 0; i < kAttnStages; ++i)
+            if (s_issue < n_tiles) {
+                if (lane == 0) issue(s_issue, rows[i], (first_stage + i) % kAttnStages);
+                s_issue += kAttnWarps;
             }
         row_next = rows[kAttnStages];
-    }
+    };
 
     // the query rows of this KV head as A fragments: row g = lane / 4 (real for g < G), two packed
-    // elements at columns 16 ks + 2 (lane % 4) and the same + 8
+    // elements at columns 16 ks + 2 (lane % 4) and the same + 8.  8-bit rows: the summation index is renumbered, this lane's
+    // k-step ks covers columns c D/4 + 4 ks ..+3
     const int g = lane >> 2, qc = (lane & 3) * 2;
-    const int Hq = H * p.group;
-    uint32_t qa[kD / 16][2];
-    {
-        const uint16_t *qrow = p.q + ((static_cast<int64_t>(l_rel) * B + b) * Hq + h * p.group + g) * kD;
-#pragma unroll
-        for (int ks = 0; ks < kD / 16; ++ks) {
-            qa[ks][0] = qa[ks][1] = 0u;
-            if (g < p.group) {
-                if constexpr (kFp8) {      // summation index renumbered: this lane's k-step ks covers columns c D/4 + 4 ks ..+3
-                    qa[ks][0] = __ldg(reinterpret_cast<const uint32_t *>(qrow + (lane & 3) * (kD / 4) + ks * 4));
-                    qa[ks][1] = __ldg(reinterpret_cast<const uint32_t *>(qrow + (lane & 3) * (kD / 4) + ks * 4 + 2));
-                } else {
-                    qa[ks][0] = __ldg(reinterpret_cast<const uint32_t *>(qrow + ks * 16 + qc));
-                    qa[ks][1] = __ldg(reinterpret_cast<const uint32_t *>(qrow + ks * 16 + 8 + qc));
-                }
-            }
+    auto query_row = [&]() {                // of the list's first query head, in `q` and `out`
+        const int list_now = kBeside ? static_cast<int>(kept_s[warp][kList]) : list, l_rel = list_now / (H * B), b = (list_now / H) % B;
+        return (static_cast<int64_t>(l_rel) * B + b) * H * p.group + list_now % H * p.group;
+    };
+    auto load_query = [&](const uint16_t *qrow, int ks, uint32_t &lo, uint32_t &hi) {
+        lo = hi = 0u;
+        if (g < p.group) {
+            const uint32_t *at = reinterpret_cast<const uint32_t *>(kFp8 ? qrow + (lane & 3) * (kD / 4) + ks * 4 : qrow + ks * 16 + qc);
+            lo = kBeside ? __ldcg(at) : __ldg(at);                      // kBeside: read again later, past the L1
+            hi = kBeside ? __ldcg(at + (kFp8 ? 1 : 4)) : __ldg(at + (kFp8 ? 1 : 4));
         }
-    }
-
-    float logit_scale = p.scale_log2e;     // 8-bit rows: times the power of two taken out of this lane's query row
-    if constexpr (kFp8) {
+    };
+    // 8-bit rows: query rows in f16, divided by the power of two of their largest element, which is returned
+    auto query_to_f16 = [&](uint32_t (&q)[kD / 16][2]) -> float {
         float qmax = 0.0f;
 #pragma unroll
         for (int ks = 0; ks < kD / 16; ++ks)
-            qmax = fmaxf(fmaxf(qmax, fmaxf(fabsf(bf16_lo(qa[ks][0])), fabsf(bf16_hi(qa[ks][0])))),
-                         fmaxf(fabsf(bf16_lo(qa[ks][1])), fabsf(bf16_hi(qa[ks][1]))));
+            qmax = fmaxf(fmaxf(qmax, fmaxf(fabsf(bf16_lo(q[ks][0])), fabsf(bf16_hi(q[ks][0])))),
+                         fmaxf(fabsf(bf16_lo(q[ks][1])), fabsf(bf16_hi(q[ks][1]))));
         qmax = fmaxf(qmax, __shfl_xor_sync(0xffffffffu, qmax, 1));
         qmax = fmaxf(qmax, __shfl_xor_sync(0xffffffffu, qmax, 2));       // the four lanes of a row hold all its elements
         uint32_t e = __float_as_uint(qmax) >> 23;                        // biased exponent (qmax >= 0)
         e = e > 253u ? 253u : e;
         const float down = __uint_as_float((254u - e) << 23);            // 2^-(e - 127)
-        logit_scale *= __uint_as_float(e << 23);                         // 2^(e - 127); zero for a zero row
 #pragma unroll
         for (int ks = 0; ks < kD / 16; ++ks) {
-            qa[ks][0] = pack_f16x2(bf16_lo(qa[ks][0]) * down, bf16_hi(qa[ks][0]) * down);
-            qa[ks][1] = pack_f16x2(bf16_lo(qa[ks][1]) * down, bf16_hi(qa[ks][1]) * down);
+            q[ks][0] = pack_f16x2(bf16_lo(q[ks][0]) * down, bf16_hi(q[ks][0]) * down);
+            q[ks][1] = pack_f16x2(bf16_lo(q[ks][1]) * down, bf16_hi(q[ks][1]) * down);
         }
-    }
-
-    float o[kNTiles][4];
+        return __uint_as_float(e << 23);                                 // 2^(e - 127); zero for a zero row
+    };
+    uint32_t qa[kD / 16][2];
+    float logit_scale;                     // 8-bit rows: times the power of two taken out of this lane's query row
+    auto take_query = [&]() {
+        const uint16_t *qrow = p.q + (query_row() + g) * kD;
 #pragma unroll
-    for (int i = 0; i < kNTiles; ++i) o[i][0] = o[i][1] = o[i][2] = o[i][3] = 0.0f;
-    float m_run = -INFINITY, l_run = 0.0f;
+        for (int ks = 0; ks < kD / 16; ++ks) load_query(qrow, ks, qa[ks][0], qa[ks][1]);
+        logit_scale = p.scale_log2e;
+        if constexpr (kFp8) logit_scale *= query_to_f16(qa);
+    };
+    // Whether the queries are no longer what they were when they were read beside the kernel ahead (the caller only promises
+    // them in stream order): read again once it has completed.  Whole warp.
+    auto query_changed = [&]() -> bool {
+        const uint16_t *qrow = p.q + (query_row() + g) * kD;
+        uint32_t diff = 0u;
+        if constexpr (kFp8) {
+            uint32_t q[kD / 16][2];
+#pragma unroll
+            for (int ks = 0; ks < kD / 16; ++ks) load_query(qrow, ks, q[ks][0], q[ks][1]);
+            const float scale = p.scale_log2e * query_to_f16(q);
+            diff = __float_as_uint(scale) ^ __float_as_uint(logit_scale);
+#pragma unroll
+            for (int ks = 0; ks < kD / 16; ++ks) diff |= (q[ks][0] ^ qa[ks][0]) | (q[ks][1] ^ qa[ks][1]);
+        } else {
+#pragma unroll
+            for (int ks = 0; ks < kD / 16; ++ks) {
+                uint32_t lo, hi;
+                load_query(qrow, ks, lo, hi);
+                diff |= (lo ^ qa[ks][0]) | (hi ^ qa[ks][1]);
+            }
+        }
+        return __any_sync(0xffffffffu, diff != 0u);
+    };
+
+    // The launch behind may start when every CTA is here: everything ahead of this launch is complete and no query is read
+    // any more (what follows may reuse their memory); it still finds this launch running, reading the cache and storing `out`.
+    auto queries_taken = [&]() {            // whole warp, once
+        uint32_t seen = 0u;
+#pragma unroll
+        for (int ks = 0; ks < kD / 16; ++ks) seen |= qa[ks][0] | qa[ks][1];
+        seen = __reduce_or_sync(0xffffffffu, seen);                      // every lane's loads have returned
+        asm volatile("" ::"r"(seen) : "memory");
+        if (lane == 0 && atomicAdd(&queries_s, 1) == kAttnWarps - 1) griddep_launch_dependents();
+    };
+    float o[kNTiles][4];
+    float m_run = 0.0f, l_run = 0.0f;
     float vref = 0.0f;                     // 8-bit rows: the largest V scale met so far; o is in units of it
 
-    bool ok = true;
-    int stage = 0;
+    bool ok = true, again = true;          // again: from the first tile on
+    int s = 0, stage = 0;
     uint32_t parity = 0;
-    for (int t = t_begin + warp; t < n_tiles; t += kAttnWarps) {
+    for (;;) {
+    // no copies of this warp are in flight here
+    if (again) s = s_issue = s_first + warp;
+    fill(stage);
+    if (again) {
+        take_query();
+        if (kBeside && waited) queries_taken();
+#pragma unroll
+        for (int i = 0; i < kNTiles; ++i) o[i][0] = o[i][1] = o[i][2] = o[i][3] = 0.0f;
+        m_run = -INFINITY;
+        l_run = vref = 0.0f;
+        again = false;
+    }
+    for (; s < n_tiles; s += kAttnWarps) {
         if (!__all_sync(0xffffffffu, mbar_wait(my_bars + 8 * stage, parity, abort_flag))) {
             ok = false;
             break;
         }
         const uint32_t sK = my_stages + stage * kStageBytes;
         const uint32_t sV = sK + (kFp8 ? kTileBytes8 : kHalves * kAttnHalfBytes);
-        const int valid = t < n_pt ? n_prefix - t * kAttnTileRows : n_ring - (t - n_pt) * kAttnTileRows;   // >= 1
+        int32_t valid = kAttnTileRows;                    // rows of the tile, >= 1 (more than a tile's: all of them)
+        if constexpr (!kBeside) {
+            valid = s < n_pt ? n_prefix - s * kAttnTileRows : n_ring - (s - n_pt) * kAttnTileRows;
+        } else if (s >= n_early) {
+            int32_t row;
+            rest_tile(s, row, valid);
+        }
         if (valid < kAttnTileRows) {
             // zero the V rows past the end of the list (8-bit rows: codes and scale)
             if constexpr (kFp8) {
@@ -517,13 +680,22 @@ decode_attn_kernel(const __grid_constant__ CUtensorMap tmap_kpool, const __grid_
             }
         }
         __syncwarp();                                     // all lanes are done with this stage
-        if (t_issue < n_tiles) {
-            if (lane == 0) issue(t_issue, row_next, stage);
-            t_issue += kAttnWarps;
-            row_next = t_issue < n_tiles ? tile_row(t_issue) : 0;
+        if (s_issue < n_tiles) {
+            if (lane == 0) issue(s_issue, row_next, stage);
+            s_issue += kAttnWarps;
+            row_next = s_issue < n_tiles ? tile_row(s_issue) : 0;
         }
         if (++stage == kAttnStages) { stage = 0; parity ^= 1u; }
     }
+    if (!kBeside || !ok || waited) break;
+    // out of the tiles known beside the kernel ahead
+    griddep_wait();
+    const int64_t li = cache_list(kept_s[warp][kList]);
+    learn_rest(__ldcg(c.n_tokens + li), __ldcg(c.prefix_len + li));
+    again = query_changed();               // then all of them once more
+    if (!again) queries_taken();
+    }
+    if (!waited) griddep_wait();                          // only if a wait ran out
     if (!ok) {
         // a wait ran out: report it, give the copies already in flight a fixed time to land, merge nothing
         if (lane == 0) {
@@ -555,7 +727,12 @@ decode_attn_kernel(const __grid_constant__ CUtensorMap tmap_kpool, const __grid_
     }
     __syncthreads();
     const bool failed = *abort_flag != 0;
-    const int64_t out_row0 = (static_cast<int64_t>(l_rel) * B + b) * Hq + h * p.group;
+    const int64_t out_row0 = query_row();
+    if constexpr (kBeside) {
+        list = kept_s[warp][kList];
+        part = kept_s[warp][kPart];
+        n_parts = kept_s[warp][kParts];
+    }
     constexpr int kUnit = 16 + kAttnMaxGroup * kD;
     float *unit = n_parts > 1 ? p.part_scratch + static_cast<int64_t>(blockIdx.x) * kUnit : nullptr;
     // four elements of one query head per thread

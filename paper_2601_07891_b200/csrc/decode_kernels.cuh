@@ -34,6 +34,8 @@ struct CacheView {
     // 0 for a slot whose sequence has been released and that has not been given a new prompt: decode steps
     // leave its lists alone
     uint8_t *active;          // [n_seqs]
+    // prefix_len before the last one-launch step behind an attention, for the attention beside it (see decode_attn_kernel)
+    int32_t *before;          // [n_lists]
 };
 
 // One more page for a list: a released one if the stack has any, else the next never-used page of the

@@ -139,6 +139,19 @@ struct kvzap_ctx {
     // the same cache: those two order their cache accesses through the step counters, nothing else does.
     uint64_t op_seq = 0, fused_seq = 0;
     int fused_layout = -1;                          // ... in this layout of the few-token kernel
+    // ... for these layers, on this stream, with so many CTAs
+    int fused_layer0 = 0, fused_layer1 = 0, fused_ctas = 0;
+    // it started behind an attention: an attention behind it may run beside it, a step behind it is no link of a chain
+    bool fused_behind_attention = false;
+    cudaStream_t fused_stream = nullptr;
+    unsigned long long fused_capture = 0;
+    // the last attention call: its number, stream and output
+    uint64_t attn_seq = 0;
+    cudaStream_t attn_stream = nullptr;
+    unsigned long long attn_capture = 0;            // the capture it went to: what is directly ahead of a call in a graph is so
+                                                    // in every replay, across a capture's borders it may not be
+    const void *attn_out = nullptr;
+    size_t attn_out_bytes = 0;
     const kvzap_cache *fused_cache = nullptr;
     std::vector<kvzap_cache *> caches;              // caches created on this context (their step counters are
                                                     // cleared when a timeout has been polled)
@@ -201,6 +214,17 @@ static inline bool hazard(const kvzap_ctx *ctx, const void *p, size_t n, bool wr
     for (const auto &r : ctx->pending)
         if ((write || r.w) && a < r.p + r.n && r.p < a + n) return true;
     return false;
+}
+// The capture that the stream's work goes to: 0 for none, all ones if that cannot be told.
+static unsigned long long capture_of(cudaStream_t stream)
+{
+    cudaStreamCaptureStatus status = cudaStreamCaptureStatusNone;
+    unsigned long long id = 0;
+    if (cudaStreamGetCaptureInfo(stream, &status, &id) != cudaSuccess) {
+        cudaGetLastError();
+        return ~0ull;
+    }
+    return status == cudaStreamCaptureStatusNone ? 0 : id;
 }
 // everything enqueued so far is complete before whatever is enqueued next starts
 static inline void serial_point(kvzap_ctx *ctx) { ctx->pending.clear(); ctx->op_chain = 0; }
@@ -779,9 +803,31 @@ static kvzap_status launch_score(kvzap_ctx *ctx, int32_t layer, int32_t n_layers
         const bool overlap = fuse_ok && fuse_chain != nullptr && *fuse_chain == layout_i && !clash &&
                              p.n_tiles * n_ctas * 2 >= ctx->sm_count;
         const bool early = !ctx->profiling && ctx->weights_seq + 1 != ctx->op_seq;
-        p.wait_before_load = ctx->trusted && (!fuse_ok || overlap) ? 0 : 1;
+        // Directly behind an attention call, ahead of which everything is complete when this launch starts and which only reads
+        // the cache: scoring runs beside it, the stores of the cache update wait for it, and the next attention may start
+        // beside this step all the same -- it reads rows that neither of the two touches and stores nothing before this
+        // launch is complete.  Not for a step that takes more than a third of the SMs: an attention beside that waits longer
+        // for it, or finds less room, than it gains (12 layers x 64 sequences of 8-bit rows, 96 CTAs: 583 us one after the
+        // other, 615 us beside one another; 4 layers x 3 sequences of 35000 tokens, 64 CTAs: 71 and 88 us).
+        const char *o0 = static_cast<const char *>(ctx->attn_out);
+        auto attn_writes = [&](const void *q, size_t n) {
+            const char *q0 = static_cast<const char *>(q);
+            return q0 < o0 + ctx->attn_out_bytes && o0 < q0 + n;
+        };
+        const size_t x_bytes = static_cast<size_t>(n_layers) * n_tokens * c.d_model * (fp8 ? 1 : 2);
+        const size_t kv_bytes = static_cast<size_t>(n_layers) * n_tokens * c.n_kv_heads * c.head_dim * 2;
+        const bool behind_attention = fuse_ok && ctx->trusted && early && ctx->attn_seq + 1 == ctx->op_seq &&
+                                      ctx->attn_stream == stream && ctx->attn_capture == capture_of(stream) && ctx->attn_capture != ~0ull &&
+                                      p.n_tiles * n_ctas * 3 <= ctx->sm_count &&
+                                      !attn_writes(hidden, x_bytes) && !attn_writes(f.K_new, kv_bytes) && !attn_writes(f.V_new, kv_bytes);
+        f.behind_attention = behind_attention ? 1 : 0;
+        p.wait_before_load = ctx->trusted && (!fuse_ok || overlap || behind_attention) ? 0 : 1;
         p.late_trigger = (late_trigger || fuse_ok) && p.wait_before_load;
         ctx->last_score_late = p.late_trigger != 0;
+        if (fuse_ok) {
+            ctx->fused_ctas = p.n_tiles * n_ctas;
+            ctx->fused_behind_attention = behind_attention;
+        }
         ctx->last_score_early = early;
         {
             ProfScope prof(ctx, KVZAP_KERNEL_SCORE, stream);
@@ -2409,6 +2455,7 @@ kvzap_status kvzap_cache_create(kvzap_ctx *ctx, kvzap_cache **out, int32_t n_seq
     alloc(reinterpret_cast<void **>(&v.n_tokens), sizeof(int32_t) * n, true);
     alloc(reinterpret_cast<void **>(&v.prefix_len), sizeof(int32_t) * n, true);
     alloc(reinterpret_cast<void **>(&v.page_table), sizeof(int32_t) * n * max_pages_per_list, true);
+    alloc(reinterpret_cast<void **>(&v.before), sizeof(int32_t) * n, false);
     alloc(reinterpret_cast<void **>(&v.page_cursor), sizeof(int32_t), true);
     alloc(reinterpret_cast<void **>(&v.free_stack), sizeof(int32_t) * static_cast<size_t>(n_pages_pool > 0 ? n_pages_pool : 1), false);
     alloc(reinterpret_cast<void **>(&v.free_top), sizeof(int32_t), true);
@@ -2471,6 +2518,7 @@ kvzap_status kvzap_cache_destroy(kvzap_cache *cache)
     cudaFree(cache->v.n_tokens); cudaFree(cache->v.prefix_len); cudaFree(cache->v.page_table);
     cudaFree(cache->v.page_cursor); cudaFree(cache->scores); cudaFree(cache->done);
     cudaFree(cache->v.free_stack); cudaFree(cache->v.free_top); cudaFree(cache->v.active);
+    cudaFree(cache->v.before);
     cudaFree(cache->attn_scratch); cudaFree(cache->attn_arrive);
     delete cache;
     return KVZAP_OK;
@@ -2516,7 +2564,7 @@ static kvzap_status decode_step_impl(kvzap_ctx *ctx, kvzap_cache *cache, int32_t
     }
     int fused_layout = -1;
     // the call just before this one was a fused step on this cache: the two may overlap
-    const bool chain = ctx->fused_cache == cache && ctx->fused_seq + 1 == ctx->op_seq;
+    const bool chain = ctx->fused_cache == cache && ctx->fused_seq + 1 == ctx->op_seq && !ctx->fused_behind_attention;
     const int chain_layout = chain ? ctx->fused_layout : -1;
     kvzap_status st = KVZAP_OK;
     const int64_t step_tiles = (static_cast<int64_t>(cache->v.n_seqs) + kTileM - 1) / kTileM * n_layers;
@@ -2536,6 +2584,10 @@ static kvzap_status decode_step_impl(kvzap_ctx *ctx, kvzap_cache *cache, int32_t
         ctx->fused_cache = cache;
         ctx->fused_layout = fused_layout;
         ctx->fused_seq = ctx->op_seq;
+        ctx->fused_layer0 = layer_begin;
+        ctx->fused_layer1 = layer_end;
+        ctx->fused_stream = stream;
+        ctx->fused_capture = ctx->fused_behind_attention ? ctx->attn_capture : 0;
         return KVZAP_OK;
     }
     const int64_t n_groups = static_cast<int64_t>(n_layers) * cache->v.n_seqs * c.n_kv_heads;
@@ -2567,6 +2619,15 @@ kvzap_status kvzap_decode_step_fp8(kvzap_ctx *ctx, kvzap_cache *cache, int32_t l
                                    float tau, float *scores_out, void *stream_)
 {
     return decode_step_impl(ctx, cache, layer_begin, layer_end, hidden_e4m3, x_scale, K_new, V_new, tau, scores_out, stream_, true);
+}
+
+static decltype(&decode_attn_kernel<128, false, false>) attn_kernel(int d_attn, bool fp8, bool beside)
+{
+    if (d_attn == 128)
+        return fp8 ? (beside ? decode_attn_kernel<128, true, true> : decode_attn_kernel<128, true, false>)
+                   : (beside ? decode_attn_kernel<128, false, true> : decode_attn_kernel<128, false, false>);
+    return fp8 ? (beside ? decode_attn_kernel<64, true, true> : decode_attn_kernel<64, true, false>)
+               : (beside ? decode_attn_kernel<64, false, true> : decode_attn_kernel<64, false, false>);
 }
 
 static kvzap_status attention_impl(kvzap_ctx *ctx, kvzap_cache *cache, int32_t layer_begin, int32_t layer_end,
@@ -2617,13 +2678,9 @@ static kvzap_status attention_impl(kvzap_ctx *ctx, kvzap_cache *cache, int32_t l
                   make_tmap(ctx, &cache->tm_vring, vring, rr, c.head_dim, kAttnTileRows) == KVZAP_OK;
             if (maps_ok) {
                 const int smem = static_cast<int>(attn_smem_bytes(d_attn, fp8));
-                cudaError_t e;
-                if (fp8)
-                    e = d_attn == 128 ? cudaFuncSetAttribute(decode_attn_kernel<128, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem)
-                                      : cudaFuncSetAttribute(decode_attn_kernel<64, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
-                else
-                    e = d_attn == 128 ? cudaFuncSetAttribute(decode_attn_kernel<128, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem)
-                                      : cudaFuncSetAttribute(decode_attn_kernel<64, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+                cudaError_t e = cudaSuccess;
+                for (int beside = 0; beside < 2 && e == cudaSuccess; ++beside)
+                    e = cudaFuncSetAttribute(attn_kernel(d_attn, fp8, beside != 0), cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
                 if (e == cudaSuccess) cache->attn_state = fp8 ? 2 : 1;
             }
         }
@@ -2655,7 +2712,24 @@ static kvzap_status attention_impl(kvzap_ctx *ctx, kvzap_cache *cache, int32_t l
     // 4 parts 490 us, 1 part 355 us, of 4700 rows: 1 part 1678 us, 3 parts 1527 us (4 layers).  320 lists, by their
     // lengths: 898 us against 1115 us in 14 equal parts (8 layers).  The capacity stands for the lengths, which the host does
     // not know: 1024 lists of 300 rows take 32.8 us in a table for as many, 51.8 us in one for 32768.
-    const int64_t slots = static_cast<int64_t>(ctx->sm_count) * (fp8 && d_attn == 128 ? 4 : 3);
+    const int64_t per_sm = fp8 && d_attn == 128 ? 4 : 3;
+    const int64_t slots = static_cast<int64_t>(ctx->sm_count) * per_sm;
+    bool beside = false;
+    // Directly behind a step in one launch over these layers that itself came directly behind an attention: nothing else that
+    // writes the cache is still running, and the rows that the lists held before that step are read beside it.  Layer by
+    // layer, step and attention, us a layer: 8 sequences x 2176 rows a list 34.1 -> 24.2, 128 x 4736 rows 378 -> 357, 64 x 1664
+    // 8-bit rows 79.8 -> 78.6.
+    const unsigned long long capture = capture_of(stream);
+    if (ctx->trusted && !ctx->profiling && ctx->fused_capture == capture && ctx->fused_cache == cache && ctx->fused_seq + 1 == ctx->op_seq && ctx->fused_behind_attention &&
+        ctx->fused_stream == stream && ctx->fused_layer0 <= layer_begin && layer_end <= ctx->fused_layer1) {
+        beside = true;
+        const int64_t sms_left = ctx->sm_count - ctx->fused_ctas;
+        p.beside_ctas = static_cast<int32_t>(sms_left * per_sm);
+        // One wave on the SMs that the step leaves: what that adds, bytes / rate * taken / left, is to be less than the 14 us of
+        // a step, at 6.4 bytes a picosecond.  The host does not know the lists' lengths; the kernel does.
+        const int64_t tile_bytes = attn_stage_bytes(d_attn, fp8);
+        p.beside_tiles = static_cast<int32_t>(14 * int64_t{6400000} / tile_bytes * sms_left / ctx->fused_ctas);
+    }
     int64_t n_ctas = n_lists_call;
     p.n_parts = 1;
     if (n_lists_call < slots && n_lists_call <= 32 * kAttnListsPerLane) {
@@ -2671,15 +2745,19 @@ static kvzap_status attention_impl(kvzap_ctx *ctx, kvzap_cache *cache, int32_t l
     }
     p.part_scratch = cache->attn_scratch;
     p.part_arrive = cache->attn_arrive;
+    ctx->attn_seq = ctx->op_seq;
+    ctx->attn_stream = stream;
+    ctx->attn_capture = capture;
+    ctx->attn_out = O;
+    ctx->attn_out_bytes = static_cast<size_t>(p.n_layers_call) * v.n_seqs * n_q_heads * d_attn * 2;
     {
         ProfScope prof(ctx, KVZAP_KERNEL_ATTENTION, stream);
         cudaLaunchConfig_t cfg;
         cudaLaunchAttribute attrs[2];
         make_launch(&cfg, attrs, dim3(static_cast<unsigned>(n_ctas)), dim3(kAttnThreads), attn_smem_bytes(d_attn, fp8), stream,
                     !ctx->profiling, 1);
-        KVZAP_CUDA(ctx, cudaLaunchKernelEx(&cfg, fp8 ? (d_attn == 128 ? decode_attn_kernel<128, true> : decode_attn_kernel<64, true>)
-                                                     : (d_attn == 128 ? decode_attn_kernel<128, false> : decode_attn_kernel<64, false>),
-                                           cache->tm_kpool, cache->tm_vpool, cache->tm_kring, cache->tm_vring, p));
+        KVZAP_CUDA(ctx, cudaLaunchKernelEx(&cfg, attn_kernel(d_attn, fp8, beside), cache->tm_kpool, cache->tm_vpool, cache->tm_kring,
+                                           cache->tm_vring, p));
     }
     ctx->launches += 1;
     return KVZAP_OK;

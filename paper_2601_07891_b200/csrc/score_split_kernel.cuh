@@ -49,6 +49,10 @@ struct DecodeFuse {
     float tau;
     int32_t *done;                  // [n_layers * tiles_per_layer][n_split]
     int64_t wait_limit;             // cycles a cluster waits for the step before to be published
+    // 1: directly behind an attention over the cache, which may still be running and reads it.  The stores of the cache update
+    // wait for it, nothing before them does; and the next launch, an attention that runs beside this step, starts once the
+    // lists' present prefix lengths are in c.before.
+    int32_t behind_attention;
 };
 
 struct SplitSmemLayout {
@@ -142,7 +146,7 @@ score_split_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_cons
             fuse_step = atomicAdd(f.ticket + ((layer * p.tiles_per_layer + m_tile) * n_split + nh) * k_split + kh, 1);
         __syncthreads();
     }
-    if (!p.late_trigger) griddep_launch_dependents();
+    if (!p.late_trigger && !f.behind_attention) griddep_launch_dependents();
     const int own_n = ns / k_split;                      // accumulator columns this CTA finishes
     const int own_c0 = kh * own_n;                       // the first of them
     const int j_first = nh * ns + own_c0;                // = first hidden unit of this CTA
@@ -206,6 +210,22 @@ score_split_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_cons
     // ahead in the stream has completed (every thread waits: the loads below are issued by several warps)
     if (p.wait_before_load) griddep_wait();
     if (p.late_trigger) griddep_launch_dependents();     // whatever starts now finds all work ahead of this launch complete
+    if (f.behind_attention && warp >= 2) {
+        // the present length of this CTA's lists (those of the cache update below), in memory before the next launch starts
+        const CacheView &c = f.c;
+        const int etid = threadIdx.x - 64;
+        const int64_t seqs_left = static_cast<int64_t>(c.n_seqs) - static_cast<int64_t>(m_tile) * kTileM;
+        const int tile_seqs = seqs_left < kTileM ? static_cast<int>(seqs_left) : kTileM;
+        const int rows_per_cta = (tile_seqs + n_ctas - 1) / n_ctas;
+        const int b_loc = pos * rows_per_cta + etid / kMaxHeads, h = etid % kMaxHeads;
+        if (etid < rows_per_cta * kMaxHeads && b_loc < tile_seqs && h < c.n_heads) {
+            const int64_t li = ((static_cast<int64_t>(m_tile) * kTileM + b_loc) * c.n_layers + layer) * c.n_heads + h;
+            c.before[li] = __ldcg(c.prefix_len + li);
+            __threadfence();
+        }
+        named_barrier_sync(1, 256);
+        if (etid == 0) griddep_launch_dependents();
+    }
     if (warp == 0) {
         __syncwarp();
         if (elect_one())
@@ -320,16 +340,19 @@ score_split_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_cons
             const int tile_seqs = seqs_left < kTileM ? static_cast<int>(seqs_left) : kTileM;
             const int rows_per_cta = (tile_seqs + n_ctas - 1) / n_ctas;
             // one thread per list: which row leaves, where it goes, which slot the new token takes
+            int64_t li;
+            int32_t n = 0, idx = 0, page = -1;
             {
                 const int b_loc = pos * rows_per_cta + etid / kMaxHeads, h = etid % kMaxHeads;
                 const int64_t b = static_cast<int64_t>(m_tile) * kTileM + b_loc;
                 int64_t dst = -1, ring = -1;
+                li = -1;
                 if (go && etid < rows_per_cta * kMaxHeads && b_loc < tile_seqs && h < c.n_heads && c.active[b] != 0) {
-                    const int64_t li = (b * c.n_layers + layer) * c.n_heads + h;
+                    li = (b * c.n_layers + layer) * c.n_heads + h;
                     // two round trips to memory instead of four: both counters first, then the score of
                     // the slot's old token and the page the prefix ends in, whether or not it will be needed
-                    const int32_t n = __ldcg(c.n_tokens + li);
-                    const int32_t idx = __ldcg(c.prefix_len + li);
+                    n = __ldcg(c.n_tokens + li);
+                    idx = __ldcg(c.prefix_len + li);
                     const int slot = n % c.window;
                     ring = li * c.window + slot;
                     const int page_i = idx / c.page_tokens, in_page = idx % c.page_tokens;
@@ -338,26 +361,32 @@ score_split_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_cons
                     const int32_t page_old =
                         full && in_page != 0 && page_i < c.max_pages ? __ldcg(c.page_table + li * c.max_pages + page_i) : -1;
                     if (full && s_old >= f.tau) {
-                        int32_t page = -1;
                         if (page_i >= c.max_pages) {
                             atomicCAS(p.status, 0, 4 /* KVZAP_ERR_OOM_PAGES */);
                         } else if (in_page == 0) {
                             page = cache_take_page(c, p.status);
-                            if (page >= 0) c.page_table[li * c.max_pages + page_i] = page;
                         } else {
                             page = page_old;
                         }
-                        if (page >= 0) {
-                            dst = static_cast<int64_t>(page) * c.page_tokens + in_page;
-                            c.prefix_len[li] = idx + 1;
-                        }
+                        if (page >= 0) dst = static_cast<int64_t>(page) * c.page_tokens + in_page;
                     }
-                    c.n_tokens[li] = n + 1;
                 }
                 fuse_dst[etid] = dst;
                 fuse_ring[etid] = ring;
             }
             named_barrier_sync(1, 256);
+            bool counted = false;                            // every thread, once, before its first store to the cache
+            auto count = [&]() {
+                if (f.behind_attention) griddep_wait();
+                if (li >= 0) {
+                    if (page >= 0) {
+                        if (idx % c.page_tokens == 0) c.page_table[li * c.max_pages + idx / c.page_tokens] = page;
+                        c.prefix_len[li] = idx + 1;
+                    }
+                    c.n_tokens[li] = n + 1;
+                }
+                counted = true;
+            };
             // rows: 16 lanes per list, kLists lists at a time; a lane loads the (old row, new row) pairs of all
             // of them before it stores any of them, so that their round trips to memory overlap
             {
@@ -390,6 +419,7 @@ score_split_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_cons
                                 vn[i] = __ldg(f.V_new + src[i] + u);
                             }
                         }
+                        if (!counted) count();
 #pragma unroll
                         for (int i = 0; i < kLists; ++i) {
                             if (ring[i] >= 0 && dst[i] >= 0) {
@@ -404,6 +434,7 @@ score_split_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_cons
                     }
                 }
             }
+            if (!counted) count();
         }
         ok = mbar_wait(bar_tfull, 0, abort_flag);
         tc_fence_after_sync();
