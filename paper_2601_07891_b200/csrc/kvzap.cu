@@ -1318,14 +1318,14 @@ static kvzap_status launch_prune_onepass(kvzap_ctx *ctx, const float *scores, co
     p.scan_flag = ctx->op_scan_flag + set;
     p.epoch = ctx->op_epoch;
     p.wait_limit = ctx->wait_limit;
-    p.wait_first = tau_behind ? 2 : wait_first ? 1 : 0;
+    p.wait_first = wait_first ? 1 : 0;
     {
         ProfScope prof(ctx, KVZAP_KERNEL_COMPACT, stream);
         cudaLaunchConfig_t cfg;
         cudaLaunchAttribute attrs[2];
         make_launch(&cfg, attrs, dim3(static_cast<unsigned>(grid), static_cast<unsigned>(groups)), dim3(kOpThreads), kOpDynSmem,
                     stream, !ctx->profiling, 1);
-        KVZAP_CUDA(ctx, cudaLaunchKernelEx(&cfg, prune_onepass_kernel<kOpRows>, p));
+        KVZAP_CUDA(ctx, cudaLaunchKernelEx(&cfg, tau_behind ? prune_onepass_kernel<kOpRows, true> : prune_onepass_kernel<kOpRows, false>, p));
     }
     ctx->launches += 1;
     return KVZAP_OK;
@@ -1619,10 +1619,12 @@ kvzap_status kvzap_create(kvzap_ctx **out, const kvzap_config *cfg)
         // No shared-memory carve-out is asked for: with the largest one (which the compaction that runs beside
         // a scoring kernel needs) the L1 that is left holds too few lines in flight, and this kernel alone moved
         // rows at 2.4 TB/s instead of 4.9.
-        CREATE_CUDA(cudaFuncSetAttribute(prune_onepass_kernel<kOpRows>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+        CREATE_CUDA(cudaFuncSetAttribute(prune_onepass_kernel<kOpRows, false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                         static_cast<int>(kOpDynSmem)));
+        CREATE_CUDA(cudaFuncSetAttribute(prune_onepass_kernel<kOpRows, true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                          static_cast<int>(kOpDynSmem)));
         int per_sm = 0;
-        CREATE_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, prune_onepass_kernel<kOpRows>, kOpThreads, kOpDynSmem));
+        CREATE_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, prune_onepass_kernel<kOpRows, false>, kOpThreads, kOpDynSmem));
         if (per_sm < 1) per_sm = 1;
         // half of what fits: the next call's kernel then finds room beside this one
         ctx->op_capacity = per_sm * ctx->sm_count / 2;

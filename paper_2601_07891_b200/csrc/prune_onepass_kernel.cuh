@@ -81,8 +81,7 @@ struct PruneParams {
     int64_t clear_units;
     int32_t recount;           // 1: short dense input, one head per CTA: rows kept before the CTA's first token are counted
                                // from the scores, not learnt from the CTAs before it
-    int32_t wait_first;        // 1: wait for the work ahead in the stream before the first load; 2: before tau_list is read,
-                               // the launch ahead, which writes it, started only when everything ahead of it was complete
+    int32_t wait_first;        // 1: wait for the work ahead in the stream before the first load
 };
 
 // Spins until *flag == want (acquire); false when the cycle budget runs out.
@@ -173,7 +172,9 @@ __device__ __forceinline__ uint32_t keep_word(const PruneParams &p, const TokenS
 // one CTA that holds a sequence's window (all of whose rows are kept) has little more to move than the others.
 // Two CTAs per SM (128 registers each): three or four, with fewer rows in flight per thread, moved rows more slowly
 // in every case measured (4.4 against 5.6 TB/s at 128k tokens).
-template <int kRows>
+// kTauBehind: the launch ahead writes tau_list and started only when everything ahead of it was complete; the first scores are
+// read before the wait for it.  A kernel of its own: scores held over the wait cost the others 2 % (2 x 49260 tokens 69.3 -> 70.8 us).
+template <int kRows, bool kTauBehind>
 __global__ void __launch_bounds__(kOpThreads, 2)
 prune_onepass_kernel(const PruneParams p)
 {
@@ -184,7 +185,10 @@ prune_onepass_kernel(const PruneParams p)
     __shared__ int32_t run_s[kMaxHeads], base_s[kMaxHeads], p0_s[kMaxHeads];
     // kept (token, head) pairs of the blocks in work: byte offsets of the source row and of the destination row
     // (-1: nowhere) inside K / V and the outputs; room for a whole number of rounds of the move loop
-    extern __shared__ longlong2 ent_s[];
+    // Aligned, and with it the ring of rows behind the list: behind 5184 bytes of static shared memory every row lay across one
+    // 128-byte line of shared memory more (2 x 49260 tokens 71.3 -> 69.3 us, 3 x 500 tokens 8.7 -> 8.5 us; 16 bytes further on,
+    // where a 32-byte sector of a row did not fit one of shared memory either, 76.4 and 9.4 us).
+    extern __shared__ __align__(128) longlong2 ent_s[];
     __shared__ uint4 wsb_s[kOpPairs];                   // [block of the group in work][head of the group]
     __shared__ int32_t runb_s[kOpPairs + kMaxHeads];    // rows of that head kept before that block; last row: after all of them
     __shared__ int32_t off_s[kOpPairs + 1];
@@ -192,7 +196,7 @@ prune_onepass_kernel(const PruneParams p)
     __shared__ float tau_s[kMaxHeads];                  // thresholds of the sequence at the CTA's first token
 
     griddep_launch_dependents();
-    if (p.wait_first == 1) griddep_wait();
+    if (!kTauBehind && p.wait_first) griddep_wait();
 
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const int H = p.n_heads;
@@ -219,19 +223,15 @@ prune_onepass_kernel(const PruneParams p)
         b_hi = seq_of_token(p.cu_seqlens, p.n_seqs, t_last);
         s0 = p.cu_seqlens[b_lo];
     }
-    // the scores of the first words that this warp looks at, on their way during the wait for the thresholds
-    constexpr int kUnroll = 4;                                // words whose scores are in flight together
-    const int n_w = static_cast<int>(blk1 - blk0) * 4;        // 32-token words of this CTA
-    TokenScores ts[kUnroll];
-    auto load_words = [&](int w0) {
+    TokenScores early[kTauBehind ? 4 : 1];                // of the words that this warp looks at first
+    if constexpr (kTauBehind) {
 #pragma unroll
-        for (int u = 0; u < kUnroll; ++u) {
-            const int wl = w0 + u * (kOpThreads / 32);
-            if (wl < n_w) load_token(p, blk0 * 4 + wl, lane, multi, ts[u]);
+        for (int u = 0; u < 4; ++u) {
+            const int wl = warp + u * (kOpThreads / 32);
+            if (wl < static_cast<int>(blk1 - blk0) * 4) load_token(p, blk0 * 4 + wl, lane, multi, early[u]);
         }
-    };
-    load_words(warp);
-    if (p.wait_first == 2) griddep_wait();
+        griddep_wait();
+    }
     if (tid < kMaxHeads) tau_s[tid] = p.tau_list != nullptr && tid < H ? __ldcg(p.tau_list + b_lo * H + tid) : p.tau;
     const int j0 = static_cast<int>((s0 / kBlockTokens) / p.blocks_per_cta);      // the CTA (column) whose blocks hold s0
     __syncthreads();
@@ -239,8 +239,20 @@ prune_onepass_kernel(const PruneParams p)
     // ---------------------------------------------------------------- A: keep bits and counts of the CTA's blocks
     {
         int32_t my_cnt = 0;                                   // lane h: kept rows of head h in the words this warp made
+        const int n_w = static_cast<int>(blk1 - blk0) * 4;    // 32-token words of this CTA
+        constexpr int kUnroll = 4;                            // words whose scores are in flight together
         for (int w0 = warp; w0 < n_w; w0 += (kOpThreads / 32) * kUnroll) {
-            if (w0 != warp) load_words(w0);
+            TokenScores ts[kUnroll];
+            if (kTauBehind && w0 == warp) {
+#pragma unroll
+                for (int u = 0; u < kUnroll; ++u) ts[u] = early[kTauBehind ? u : 0];
+            } else {
+#pragma unroll
+                for (int u = 0; u < kUnroll; ++u) {
+                    const int wl = w0 + u * (kOpThreads / 32);
+                    if (wl < n_w) load_token(p, blk0 * 4 + wl, lane, multi, ts[u]);
+                }
+            }
 #pragma unroll
             for (int u = 0; u < kUnroll; ++u) {
                 const int wl = w0 + u * (kOpThreads / 32);
