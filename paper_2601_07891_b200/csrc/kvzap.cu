@@ -627,6 +627,14 @@ static const kvzap_ctx::SplitLayout *prompt_layout(const kvzap_ctx *ctx, int64_t
     return l ? l : i >= 0 ? &ctx->layouts[i] : nullptr;
 }
 
+static decltype(&score_split_kernel<false, false, false>) split_kernel(bool fp8, bool pair, bool fused)
+{
+    if (pair) return fp8 ? score_split_kernel<true, true, false> : score_split_kernel<false, true, false>;
+    if (fused) return fp8 ? score_split_kernel<true, false, true> : score_split_kernel<false, false, true>;
+    return fp8 ? score_split_kernel<true, false, false> : score_split_kernel<false, false, false>;
+}
+constexpr int kSplitKernels = 3;        // per input type: (pair, fused) = (0, 0), (1, 0), (0, 1)
+
 // Enqueues the few-token kernel over p.n_tiles tiles (of two blocks for a layout with CTA pairs).
 static cudaError_t launch_split(const kvzap_ctx::SplitLayout &l, int k, bool pair, bool fp8, const CUtensorMap &tmap_x, const ScoreParams &p,
                                 const DecodeFuse &f, bool early, cudaStream_t stream)
@@ -636,10 +644,7 @@ static cudaError_t launch_split(const kvzap_ctx::SplitLayout &l, int k, bool pai
     cudaLaunchAttribute attrs[2];
     make_launch(&cfg, attrs, dim3(static_cast<unsigned>(p.n_tiles * ctas * l.n * k)), dim3(kScoreThreads), l.smem, stream, early, ctas * k);
     const CUtensorMap &tmap_w = fp8 ? l.tmap_w8 : l.tmap_w;
-    if (pair) return fp8 ? cudaLaunchKernelEx(&cfg, score_split_kernel<true, true>, tmap_x, tmap_w, p, l.n, k, f)
-                         : cudaLaunchKernelEx(&cfg, score_split_kernel<false, true>, tmap_x, tmap_w, p, l.n, k, f);
-    return fp8 ? cudaLaunchKernelEx(&cfg, score_split_kernel<true, false>, tmap_x, tmap_w, p, l.n, k, f)
-               : cudaLaunchKernelEx(&cfg, score_split_kernel<false, false>, tmap_x, tmap_w, p, l.n, k, f);
+    return cudaLaunchKernelEx(&cfg, split_kernel(fp8, pair, f.enabled != 0), tmap_x, tmap_w, p, l.n, k, f);
 }
 
 // Blocks of a prompt that whole waves of CTA pairs leave over and that the few-token kernel takes instead, in a launch of its
@@ -1478,9 +1483,6 @@ kvzap_status kvzap_create(kvzap_ctx **out, const kvzap_config *cfg)
                                      static_cast<int>(cudaSharedmemCarveoutMaxShared)));
     CREATE_CUDA(cudaFuncSetAttribute(decode_update_kernel, cudaFuncAttributePreferredSharedMemoryCarveout,
                                      static_cast<int>(cudaSharedmemCarveoutMaxShared)));
-    if (c.hidden > 0)
-        CREATE_CUDA(cudaFuncSetAttribute(score_split_kernel<false, false>, cudaFuncAttributePreferredSharedMemoryCarveout,
-                                         static_cast<int>(cudaSharedmemCarveoutMaxShared)));
     if (c.hidden > 0) {
         CREATE_CUDA(cudaFuncSetAttribute(score_kernel<true, false>, cudaFuncAttributePreferredSharedMemoryCarveout,
                                          static_cast<int>(cudaSharedmemCarveoutMaxShared)));
@@ -1525,10 +1527,11 @@ kvzap_status kvzap_create(kvzap_ctx **out, const kvzap_config *cfg)
     if (c.hidden > 0) {
         ctx->split_smem_limit = budget + 1024 - 4608;       // the kernel has 4112 bytes of static shared memory
         // the limit is the function's, not the context's: the most that any layout of any context takes
-        CREATE_CUDA(cudaFuncSetAttribute(score_split_kernel<false, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, ctx->split_smem_limit));
-        CREATE_CUDA(cudaFuncSetAttribute(score_split_kernel<false, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, ctx->split_smem_limit));
-        CREATE_CUDA(cudaFuncSetAttribute(score_split_kernel<false, true>, cudaFuncAttributePreferredSharedMemoryCarveout,
-                                         static_cast<int>(cudaSharedmemCarveoutMaxShared)));
+        for (int i = 0; i < kSplitKernels; ++i) {
+            CREATE_CUDA(cudaFuncSetAttribute(split_kernel(false, i == 1, i == 2), cudaFuncAttributeMaxDynamicSharedMemorySize, ctx->split_smem_limit));
+            CREATE_CUDA(cudaFuncSetAttribute(split_kernel(false, i == 1, i == 2), cudaFuncAttributePreferredSharedMemoryCarveout,
+                                             static_cast<int>(cudaSharedmemCarveoutMaxShared)));
+        }
         // Few-token layouts.  The first takes the largest launches: four CTAs per tile, 2 x 2 (two slices of hidden
         // units, two parts of K) when a slice of hidden / 2 units fits one MMA and the K blocks divide evenly, else
         // four slices.  The others spread a tile over more CTAs, widest first; of two of the same width the one whose
@@ -1552,8 +1555,7 @@ kvzap_status kvzap_create(kvzap_ctx **out, const kvzap_config *cfg)
             cudaLaunchAttribute attrs[2];
             const int cluster = pair ? 2 * k : k;
             make_launch(&cfg, attrs, dim3(static_cast<unsigned>(n * cluster)), dim3(kScoreThreads), l.smem, nullptr, false, cluster);
-            return (pair ? cudaOccupancyMaxActiveClusters(&l.max_clusters, score_split_kernel<false, true>, &cfg)
-                         : cudaOccupancyMaxActiveClusters(&l.max_clusters, score_split_kernel<false, false>, &cfg)) == cudaSuccess &&
+            return cudaOccupancyMaxActiveClusters(&l.max_clusters, split_kernel(false, pair, !pair), &cfg) == cudaSuccess &&
                    (l.arrive != nullptr || cudaMalloc(&l.arrive, sizeof(uint32_t) * static_cast<size_t>(ctx->sm_count)) == cudaSuccess) &&
                    cudaMemset(l.arrive, 0, sizeof(uint32_t) * static_cast<size_t>(ctx->sm_count)) == cudaSuccess;
         };
@@ -1746,9 +1748,9 @@ kvzap_status kvzap_set_weights_fp8(kvzap_ctx *ctx, int32_t layer, const void *W1
                                static_cast<uint32_t>(c.hidden / l.n / (pair ? 2 : 1)), 0, true) == KVZAP_OK;
         }
         if (ctx->n_layouts > 0) {
-            for (auto kernel : {score_split_kernel<true, false>, score_split_kernel<true, true>}) {
-                KVZAP_CUDA(ctx, cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, ctx->split_smem_limit));
-                KVZAP_CUDA(ctx, cudaFuncSetAttribute(kernel, cudaFuncAttributePreferredSharedMemoryCarveout,
+            for (int i = 0; i < kSplitKernels; ++i) {
+                KVZAP_CUDA(ctx, cudaFuncSetAttribute(split_kernel(true, i == 1, i == 2), cudaFuncAttributeMaxDynamicSharedMemorySize, ctx->split_smem_limit));
+                KVZAP_CUDA(ctx, cudaFuncSetAttribute(split_kernel(true, i == 1, i == 2), cudaFuncAttributePreferredSharedMemoryCarveout,
                                                      static_cast<int>(cudaSharedmemCarveoutMaxShared)));
             }
         }

@@ -30,7 +30,7 @@
 
 namespace kvzap {
 
-// Decode step fused into the scoring launch (enabled != 0): while the MMAs run, the epilogue warps
+// Decode step fused into the scoring launch (kFused; enabled != 0): while the MMAs run, the epilogue warps
 // of a cluster do the cache update of the cluster's own lists -- 128 sequences x H heads of one layer,
 // an equal part per CTA -- exactly as decode_update_kernel does (the token that leaves the window is
 // judged by its buffered score, so nothing here needs the new scores); the cluster's first CTA puts
@@ -87,19 +87,20 @@ __host__ inline bool split_smem_fits(int ns, int n_stages, int k_split, int b_ro
 // A CTA ends up owning Ns / k_split hidden units.
 // kFp8: hidden states and W1 are E4M3 bytes (K blocks of 128 codes, tcgen05.mma kind::f8f6f4); the scales
 // x_scale[token] * w1_scale[hidden unit] multiply the summed pre-activation before the bias.
+// kFused: the decode step, a kernel of its own: the scoring of prompts and chunks carries none of its code.
 // kPair (prompts, not the fused step): two blocks of 128 tokens share every W1 tile.  A work tile is a pair of blocks, the
 // cluster has 2 * k_split CTAs, CTA 2 r + i holds block i's rows of K part r and half of the slice's W1 rows, and its first
 // one issues the MMAs of both (cta_group::2, as in score_kernel); everything behind the accumulators is per block, as without
 // pairs.  A CTA then loads (128 + Ns / 2) rows per K element instead of 128 + Ns, which is what bounds this kernel.
-template <bool kFp8, bool kPair>
+template <bool kFp8, bool kPair, bool kFused>
 __global__ void __maxnreg__(128)
 score_split_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_constant__ CUtensorMap tmap_w,
                    const ScoreParams p, const int n_split, const int k_split, const DecodeFuse f)
 {
     constexpr int kElems = kFp8 ? 2 * kBlockK : kBlockK;         // elements per 128-byte K block
     constexpr int kCtas = kPair ? 2 : 1;
-    __shared__ int64_t fuse_dst[256];       // fused decode step: page row of the evicted token (-1 = dropped)
-    __shared__ int64_t fuse_ring[256];      //                     ring row of the list's current slot (-1 = no list)
+    __shared__ int64_t fuse_dst[kFused ? 256 : 1];       // fused decode step: page row of the evicted token (-1 = dropped)
+    __shared__ int64_t fuse_ring[kFused ? 256 : 1];      //                     ring row of the list's current slot (-1 = no list)
     __shared__ int32_t fuse_step;           //                     number of the step this CTA works on (its ticket)
     extern __shared__ uint8_t smem_raw[];
     const uint32_t raw_addr = smem_u32(smem_raw);
@@ -139,14 +140,14 @@ score_split_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_cons
     const int m_tile = (tile - l_rel * p.tiles_per_layer) * kCtas + static_cast<int>(half) + p.block0;
     const int part_tile = tile * kCtas + static_cast<int>(half);        // among all blocks of the launch
     const int layer = p.layer0 + l_rel;
-    if (f.enabled) {
+    if constexpr (kFused) {
         // the step number, drawn before any thread of this CTA lets the next launch be placed: a CTA of that launch
         // starts only after every CTA of this one has passed the instruction below, hence after this draw
         if (threadIdx.x == 0)
             fuse_step = atomicAdd(f.ticket + ((layer * p.tiles_per_layer + m_tile) * n_split + nh) * k_split + kh, 1);
         __syncthreads();
     }
-    if (!p.late_trigger && !f.behind_attention) griddep_launch_dependents();
+    if (!p.late_trigger && !(kFused && f.behind_attention)) griddep_launch_dependents();
     const int own_n = ns / k_split;                      // accumulator columns this CTA finishes
     const int own_c0 = kh * own_n;                       // the first of them
     const int j_first = nh * ns + own_c0;                // = first hidden unit of this CTA
@@ -210,7 +211,7 @@ score_split_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_cons
     // ahead in the stream has completed (every thread waits: the loads below are issued by several warps)
     if (p.wait_before_load) griddep_wait();
     if (p.late_trigger) griddep_launch_dependents();     // whatever starts now finds all work ahead of this launch complete
-    if (f.behind_attention && warp >= 2) {
+    if (kFused && f.behind_attention && warp >= 2) {
         // the present length of this CTA's lists (those of the cache update below), in memory before the next launch starts
         const CacheView &c = f.c;
         const int etid = threadIdx.x - 64;
@@ -323,7 +324,7 @@ score_split_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_cons
         if constexpr (kFp8)
             for (int i = etid; i < own_n; i += 256) w1s[i] = __ldg(p.w1_scale + static_cast<int64_t>(layer) * p.n_hidden + j_first + i);
         named_barrier_sync(1, 256);
-        if (f.enabled) {
+        if constexpr (kFused) {
             // ---- the cache update of this CTA's lists, under the MMAs
             const CacheView &c = f.c;
             const int cid = layer * p.tiles_per_layer + m_tile;
@@ -581,7 +582,7 @@ score_split_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_cons
             named_barrier_sync(2, 128);
             if (*last_flag == 0) {
                 // not the last: this cluster's part of the cache update is complete, say so and leave
-                if (f.enabled && threadIdx.x == 64 && *abort_flag == 0) st_release_gpu(f.done + done_i, fuse_step + 1);
+                if (kFused && threadIdx.x == 64 && *abort_flag == 0) st_release_gpu(f.done + done_i, fuse_step + 1);
                 return;
             }
 #pragma unroll
@@ -597,7 +598,7 @@ score_split_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_cons
         for (int h = 0; h < kMaxHeads; ++h) s[h] += __ldg(p.b2 + layer * kMaxHeads + h);
         const int64_t t = static_cast<int64_t>(m_tile) * kTileM + row;
         const bool valid = t < p.n_tokens;
-        if (f.enabled) {
+        if constexpr (kFused) {
             // the new token's scores go into the slot it took (n_tokens was advanced by the list's CTA)
             const CacheView &c = f.c;
             if (valid && *abort_flag == 0 && c.active[t] != 0) {
