@@ -12,6 +12,7 @@
 #include <cstring>
 #include <new>
 #include <algorithm>
+#include <mutex>
 #include <vector>
 
 #include "attn_kernel.cuh"
@@ -215,6 +216,33 @@ static inline bool hazard(const kvzap_ctx *ctx, const void *p, size_t n, bool wr
         if ((write || r.w) && a < r.p + r.n && r.p < a + n) return true;
     return false;
 }
+// Clusters of a kernel that the device holds at once, -1 if that cannot be told.  The question takes the driver about 1 ms, and a
+// context asks some ten of them: answers, which are the device's and the kernel's alone, are kept for the contexts to come (all
+// threads; a bounded number).
+static int active_clusters(int device, const void *kernel, const cudaLaunchConfig_t &cfg)
+{
+    struct Known { int device; const void *kernel; unsigned cluster, threads; size_t smem; int n; };
+    static std::mutex mutex;
+    static std::vector<Known> known;
+    unsigned cluster = 1;
+    for (unsigned i = 0; i < cfg.numAttrs; ++i)
+        if (cfg.attrs[i].id == cudaLaunchAttributeClusterDimension) cluster = cfg.attrs[i].val.clusterDim.x;
+    std::lock_guard<std::mutex> lock(mutex);
+    for (const Known &k : known)
+        if (k.device == device && k.kernel == kernel && k.cluster == cluster && k.threads == cfg.blockDim.x && k.smem == cfg.dynamicSmemBytes)
+            return k.n;
+    int n = 0;
+    if (cudaOccupancyMaxActiveClusters(&n, kernel, &cfg) != cudaSuccess || n < 0) {
+        cudaGetLastError();
+        return -1;
+    }
+    try {
+        if (known.size() < 256) known.push_back({device, kernel, cluster, cfg.blockDim.x, cfg.dynamicSmemBytes, n});
+    } catch (...) {
+    }
+    return n;
+}
+
 // The capture that the stream's work goes to: 0 for none, all ones if that cannot be told.
 static unsigned long long capture_of(cudaStream_t stream)
 {
@@ -1463,11 +1491,9 @@ kvzap_status kvzap_create(kvzap_ctx **out, const kvzap_config *cfg)
         qattr[0].val.clusterDim.z = 1;
         qcfg.attrs = qattr;
         qcfg.numAttrs = 1;
-        int n_clusters = 0;
-        if (cudaOccupancyMaxActiveClusters(&n_clusters, score_kernel<true, true>, &qcfg) == cudaSuccess && n_clusters > 0)
+        const int n_clusters = active_clusters(c.device, reinterpret_cast<const void *>(&score_kernel<true, true, false>), qcfg);
+        if (n_clusters > 0)              // else pairs are unavailable: the one-CTA kernel serves every size
             ctx->pair_clusters = n_clusters < ctx->sm_count / 2 ? n_clusters : ctx->sm_count / 2;
-        else
-            cudaGetLastError();          // pairs unavailable: the one-CTA kernel serves every size
     } else {
         CREATE_CUDA(cudaFuncSetAttribute(score_kernel<false, false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                          static_cast<int>(ctx->sched[0].smem)));
@@ -1555,7 +1581,8 @@ kvzap_status kvzap_create(kvzap_ctx **out, const kvzap_config *cfg)
             cudaLaunchAttribute attrs[2];
             const int cluster = pair ? 2 * k : k;
             make_launch(&cfg, attrs, dim3(static_cast<unsigned>(n * cluster)), dim3(kScoreThreads), l.smem, nullptr, false, cluster);
-            return cudaOccupancyMaxActiveClusters(&l.max_clusters, split_kernel(false, pair, !pair), &cfg) == cudaSuccess &&
+            l.max_clusters = active_clusters(c.device, reinterpret_cast<const void *>(split_kernel(false, pair, !pair)), cfg);
+            return l.max_clusters >= 0 &&
                    (l.arrive != nullptr || cudaMalloc(&l.arrive, sizeof(uint32_t) * static_cast<size_t>(ctx->sm_count)) == cudaSuccess) &&
                    cudaMemset(l.arrive, 0, sizeof(uint32_t) * static_cast<size_t>(ctx->sm_count)) == cudaSuccess;
         };
@@ -1604,12 +1631,10 @@ kvzap_status kvzap_create(kvzap_ctx **out, const kvzap_config *cfg)
         cudaLaunchConfig_t cfg;
         cudaLaunchAttribute attrs[2];
         make_launch(&cfg, attrs, dim3(static_cast<unsigned>(cluster)), dim3(kSelectThreads), 0, nullptr, false, cluster);
-        int fit = 0;
-        if (cudaOccupancyMaxActiveClusters(&fit, select_cluster_kernel, &cfg) == cudaSuccess && fit >= c.n_kv_heads) {
+        if (active_clusters(c.device, reinterpret_cast<const void *>(select_cluster_kernel), cfg) >= c.n_kv_heads) {
             ctx->select_cluster = cluster;
             break;
         }
-        cudaGetLastError();
     }
     CREATE_CUDA(cudaMalloc(&ctx->select_arrive, sizeof(uint32_t) * static_cast<size_t>(c.max_seqs) * c.n_kv_heads));
     CREATE_CUDA(cudaMemset(ctx->select_arrive, 0, sizeof(uint32_t) * static_cast<size_t>(c.max_seqs) * c.n_kv_heads));
