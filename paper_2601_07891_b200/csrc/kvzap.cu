@@ -16,6 +16,7 @@
 #include <vector>
 
 #include "attn_kernel.cuh"
+#include "inflight.h"
 #include "decode_kernels.cuh"
 #include "prune_kernels.cuh"
 #include "prune_onepass_kernel.cuh"
@@ -167,14 +168,12 @@ struct kvzap_ctx {
     uint64_t *lin_counts = nullptr;      // [kOpRing][kLinMaxTiles][8]: tile counts of the scoring launch that also compacts
     uint64_t op_turn = 0;
     int32_t op_epoch = 0;
-    int op_chain = 0;                    // launches of that kernel in a row that did not wait for the work ahead
     uint64_t op_last_seq = 0;            // number (op_seq) of the last call that launched it
-    // Caller memory read or written by the launches of that kernel since the last one that waited for all
-    // work ahead of it: these launches may still be running.  Another one is started without such a wait
-    // only directly behind them and only if it conflicts with none of these ranges; the scoring kernels
+    // Caller memory of the launches of that kernel, and of the linear one that also compacts, which may still be running:
+    // another one is started without a wait only directly behind them, and if it conflicts with none of it; the scoring kernels
     // consult the list before they write a scores buffer early.
-    struct Range { const char *p; size_t n; bool w; };
-    std::vector<Range> pending;
+    kvzap::InFlight in_flight;
+    static_assert(kvzap::InFlight::kMaxChain + 2 <= kvzap::kOpRing, "launches that run beside one another use scratch sets of their own");
     char err[512] = "";
 };
 
@@ -200,22 +199,6 @@ static kvzap_status fail(kvzap_ctx *ctx, kvzap_status st, const char *fmt, ...)
 // Numbers a public call (see kvzap_ctx::op_seq).
 static inline void begin_op(kvzap_ctx *ctx) { ctx->op_seq += 1; }
 
-// ---- what the kernels in flight may still touch (see kvzap_ctx::pending)
-constexpr size_t kMaxPending = 96;
-static inline void note_range(kvzap_ctx *ctx, const void *p, size_t n, bool write)
-{
-    if (p != nullptr && n > 0) ctx->pending.push_back({static_cast<const char *>(p), n, write});
-}
-// true if [p, p + n) overlaps a pending range in a conflicting way (a write on either side)
-static inline bool hazard(const kvzap_ctx *ctx, const void *p, size_t n, bool write)
-{
-    if (p == nullptr || n == 0) return false;
-    if (ctx->pending.size() > kMaxPending) return true;
-    const char *a = static_cast<const char *>(p);
-    for (const auto &r : ctx->pending)
-        if ((write || r.w) && a < r.p + r.n && r.p < a + n) return true;
-    return false;
-}
 // Clusters of a kernel that the device holds at once, -1 if that cannot be told.  The question takes the driver about 1 ms, and a
 // context asks some ten of them: answers, which are the device's and the kernel's alone, are kept for the contexts to come (all
 // threads; a bounded number).
@@ -254,8 +237,6 @@ static unsigned long long capture_of(cudaStream_t stream)
     }
     return status == cudaStreamCaptureStatusNone ? 0 : id;
 }
-// everything enqueued so far is complete before whatever is enqueued next starts
-static inline void serial_point(kvzap_ctx *ctx) { ctx->pending.clear(); ctx->op_chain = 0; }
 
 // Clears the fused decode step's counters (device and host view) of every cache of the context.
 static void reset_step_counters(kvzap_ctx *ctx, cudaStream_t stream);
@@ -741,7 +722,7 @@ static kvzap_status launch_score(kvzap_ctx *ctx, int32_t layer, int32_t n_layers
     const int64_t blocks_per_layer = (n_tokens + kTileM - 1) / kTileM;
     // the scores buffer may still be in use by a kernel of an earlier call that has not completed
     const bool scores_busy = scores != nullptr &&
-                             hazard(ctx, scores, sizeof(float) * static_cast<size_t>(n_layers) * n_tokens * c.n_kv_heads, true);
+                             ctx->in_flight.busy(scores, sizeof(float) * static_cast<size_t>(n_layers) * n_tokens * c.n_kv_heads, true);
     // Few tiles (a decode step: one tile per layer): split every tile's hidden units (and K range) over
     // several CTAs, so that the launch fills the machine and every CTA reads only its own part of W1.
     // ... and with the K split left out (two CTAs per tile, each a slice of the hidden units over the whole K
@@ -929,28 +910,21 @@ static kvzap_status launch_score(kvzap_ctx *ctx, int32_t layer, int32_t n_layers
             ctx->op_turn += 1;
             ctx->op_epoch = ctx->op_epoch == 0x7fffffff ? 1 : ctx->op_epoch + 1;
             // the same rule as for the one-launch pruning kernel: rows and counts are written before the work
-            // ahead has completed only directly behind launches whose memory is on the pending list and does
-            // not conflict
-            bool wait_first = !ctx->trusted || ctx->profiling || ctx->op_last_seq + 1 != ctx->op_seq || ctx->op_chain >= kOpRing - 2;
-            if (!wait_first)
-                wait_first = hazard(ctx, hidden, static_cast<size_t>(n_tokens) * c.d_model * 2, false) ||
-                             hazard(ctx, compact->K, kv_bytes, false) || hazard(ctx, compact->V, kv_bytes, false);
+            // ahead has completed only directly behind launches whose memory is on the list and does not conflict.
             // Only what it writes is still in use (an output buffer of one of the last calls again): everything up to the
-            // loads of the rows goes ahead, its stores wait.  It stays a link of the chain: what follows may still meet the
-            // launches ahead of it.  4096 tokens, three contexts in turn, each with its own outputs: 15.4 -> 10.7 us per call.
-            const bool wait_stores = !wait_first && (clash || hazard(ctx, compact->K_out, kv_bytes, true) ||
-                                                     hazard(ctx, compact->V_out, kv_bytes, true) ||
-                                                     hazard(ctx, compact->lengths, sizeof(int32_t) * c.n_kv_heads, true));
-            if (wait_first) serial_point(ctx);
-            else ctx->op_chain += 1;
+            // loads of the rows goes ahead, its stores wait.  4096 tokens, three contexts in turn, each with its own outputs:
+            // 15.4 -> 10.7 us per call.
+            const InFlight::Use uses[] = {{hidden, static_cast<size_t>(n_tokens) * c.d_model * 2, false},
+                                          {compact->K, kv_bytes, false},
+                                          {compact->V, kv_bytes, false},
+                                          {scores, sbytes, true},
+                                          {compact->K_out, kv_bytes, true},
+                                          {compact->V_out, kv_bytes, true},
+                                          {compact->lengths, sizeof(int32_t) * c.n_kv_heads, true}};
+            if (ctx->in_flight.busy(hidden, uses[0].n, false)) p.wait_before_load = 1;
+            const InFlight::Order order = ctx->in_flight.next(
+                uses, 7, !ctx->trusted || ctx->profiling || ctx->op_last_seq + 1 != ctx->op_seq, true);
             ctx->op_last_seq = ctx->op_seq;
-            note_range(ctx, hidden, static_cast<size_t>(n_tokens) * c.d_model * 2, false);
-            note_range(ctx, scores, sbytes, true);
-            note_range(ctx, compact->K, kv_bytes, false);
-            note_range(ctx, compact->V, kv_bytes, false);
-            note_range(ctx, compact->K_out, kv_bytes, true);
-            note_range(ctx, compact->V_out, kv_bytes, true);
-            note_range(ctx, compact->lengths, sizeof(int32_t) * c.n_kv_heads, true);
             fc.enabled = 1;
             fc.row_bytes = c.head_dim * 2;
             fc.K = static_cast<const char *>(compact->K);
@@ -964,8 +938,8 @@ static kvzap_status launch_score(kvzap_ctx *ctx, int32_t layer, int32_t n_layers
             fc.epoch = ctx->op_epoch;
             fc.n_stages = kLinStagesCompact;
             fc.wait_limit = ctx->wait_limit;
-            p.wait_before_write = wait_first ? 1 : wait_stores ? 2 : 0;
-            p.late_trigger = wait_first && ctx->trusted;     // what starts behind finds all work ahead of this launch complete
+            p.wait_before_write = order.wait;
+            p.late_trigger = order.late && ctx->trusted;
             p.maskbits = nullptr;
             smem = lin_smem_bytes(kLinStagesCompact);
             if (compacted) *compacted = true;
@@ -1134,7 +1108,7 @@ static kvzap_status launch_score_fp8(kvzap_ctx *ctx, int32_t layer, const void *
     p.tile_counter_reset = ctx->tile_counters + (ctx->score_turn + 2) % kMaskRing;
     ctx->score_turn += 1;
     const size_t scores_bytes = scores ? sizeof(float) * static_cast<size_t>(n_tokens) * c.n_kv_heads : 0;
-    bool scores_clash = scores != nullptr && hazard(ctx, scores, scores_bytes, true);
+    bool scores_clash = scores != nullptr && ctx->in_flight.busy(scores, scores_bytes, true);
     if (scores && ctx->last_scores) {
         const char *a0 = reinterpret_cast<const char *>(scores), *b0 = static_cast<const char *>(ctx->last_scores);
         scores_clash = scores_clash || (a0 < b0 + ctx->last_scores_bytes && b0 < a0 + scores_bytes);
@@ -1259,32 +1233,24 @@ static kvzap_status launch_prune_onepass(kvzap_ctx *ctx, const float *scores, co
     const size_t out_bytes = page_tokens > 0 ? static_cast<size_t>(n_pages_pool) * page_tokens * c.head_dim * 2 : kv_bytes;
     const size_t sc_bytes = sizeof(float) * static_cast<size_t>(n_tokens) * c.n_kv_heads;
     // Started before the work ahead of it has completed only on a context that trusts its producers,
-    // directly behind another launch of this kernel (whose memory is on the pending list, and whose scratch
-    // set is a different one for kOpRing - 2 launches in a row), and when it conflicts with none of them.
-    bool wait_first = !ctx->trusted || ctx->profiling || tau_list != nullptr || scores_just_made ||
-                      ctx->op_last_seq + 1 != ctx->op_seq || ctx->op_chain >= kOpRing - 2;
-    if (!wait_first)
-        wait_first = hazard(ctx, scores, sc_bytes, false) || hazard(ctx, K, kv_bytes, false) || hazard(ctx, V, kv_bytes, false) ||
-                     hazard(ctx, cu_seqlens, sizeof(int32_t) * (n_seqs + 1), false) ||
-                     hazard(ctx, K_out, out_bytes, true) || hazard(ctx, V_out, out_bytes, true) ||
-                     hazard(ctx, lengths, sizeof(int32_t) * n_lists, true) ||
-                     hazard(ctx, page_table, sizeof(int32_t) * n_lists * max_pages, true) ||
-                     hazard(ctx, n_pages_used, sizeof(int32_t), true) ||
-                     hazard(ctx, slot_out, sizeof(int32_t) * static_cast<size_t>(n_tokens) * c.n_kv_heads, true);
-    if (wait_first) serial_point(ctx);
-    else ctx->op_chain += 1;
+    // directly behind another launch of this kernel (whose memory is on the list, and whose scratch set is another), and when
+    // it conflicts with none on the list.  The cut values are the library's own or the caller's: they are read until this
+    // launch is complete, like its other inputs.
+    const InFlight::Use uses[] = {{scores, sc_bytes, false},
+                                  {K, kv_bytes, false},
+                                  {V, kv_bytes, false},
+                                  {cu_seqlens, sizeof(int32_t) * (n_seqs + 1), false},
+                                  {tau_list, sizeof(float) * n_lists, false},
+                                  {K_out, out_bytes, true},
+                                  {V_out, out_bytes, true},
+                                  {lengths, sizeof(int32_t) * n_lists, true},
+                                  {page_table, page_tokens > 0 ? sizeof(int32_t) * n_lists * max_pages : 0, true},
+                                  {n_pages_used, page_tokens > 0 ? sizeof(int32_t) : 0, true},
+                                  {slot_out, sizeof(int32_t) * static_cast<size_t>(n_tokens) * c.n_kv_heads, true}};
+    const InFlight::Order order = ctx->in_flight.next(
+        uses, 11, !ctx->trusted || ctx->profiling || tau_list != nullptr || scores_just_made || ctx->op_last_seq + 1 != ctx->op_seq, false);
+    const bool wait_first = order.wait != InFlight::kNone;
     ctx->op_last_seq = ctx->op_seq;
-    note_range(ctx, scores, sc_bytes, false);
-    note_range(ctx, K, kv_bytes, false);
-    note_range(ctx, V, kv_bytes, false);
-    note_range(ctx, K_out, out_bytes, true);
-    note_range(ctx, V_out, out_bytes, true);
-    note_range(ctx, lengths, sizeof(int32_t) * n_lists, true);
-    note_range(ctx, slot_out, sizeof(int32_t) * static_cast<size_t>(n_tokens) * c.n_kv_heads, true);
-    if (page_tokens > 0) {
-        note_range(ctx, page_table, sizeof(int32_t) * n_lists * max_pages, true);
-        note_range(ctx, n_pages_used, sizeof(int32_t), true);
-    }
     // A launch that waits for the work ahead takes every slot of the device (32k tokens, a quarter kept: 40 -> 31 us); one
     // that may run beside the launch ahead (and the one behind it beside this one) half of them, and so does the paged
     // output, whose CTAs all wait for one another: two such launches on two streams still fit side by side.  Half of them
@@ -1352,6 +1318,7 @@ static kvzap_status launch_prune_onepass(kvzap_ctx *ctx, const float *scores, co
     p.epoch = ctx->op_epoch;
     p.wait_limit = ctx->wait_limit;
     p.wait_first = wait_first ? 1 : 0;
+    p.late_trigger = order.late && ctx->trusted ? 1 : 0;
     {
         ProfScope prof(ctx, KVZAP_KERNEL_COMPACT, stream);
         cudaLaunchConfig_t cfg;
@@ -1743,7 +1710,6 @@ kvzap_status kvzap_set_weights_fp8(kvzap_ctx *ctx, int32_t layer, const void *W1
     NvtxRange nvtx_range("kvzap_set_weights_fp8");
     if (!ctx) return KVZAP_ERR_INVALID_ARG;
     begin_op(ctx);
-    serial_point(ctx);
     cudaStream_t stream = static_cast<cudaStream_t>(stream_);
     const kvzap_config &c = ctx->cfg;
     if (layer < 0 || layer >= c.n_layers) return fail(ctx, KVZAP_ERR_INVALID_ARG, "layer %d out of range", layer);
@@ -3058,7 +3024,6 @@ kvzap_status kvzap_prefill_layers_host(kvzap_ctx *ctx, int32_t layer_begin, int3
     NvtxRange nvtx_range("kvzap_prefill_layers_host");
     if (!ctx) return KVZAP_ERR_INVALID_ARG;
     begin_op(ctx);
-    serial_point(ctx);
     cudaStream_t stream = static_cast<cudaStream_t>(stream_);
     const kvzap_config &c = ctx->cfg;
     if (layer_begin < 0 || layer_end > c.n_layers || layer_begin >= layer_end)
