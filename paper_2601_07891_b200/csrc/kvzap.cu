@@ -913,7 +913,12 @@ static kvzap_status launch_score(kvzap_ctx *ctx, int32_t layer, int32_t n_layers
             // ahead has completed only directly behind launches whose memory is on the list and does not conflict.
             // Only what it writes is still in use (an output buffer of one of the last calls again): everything up to the
             // loads of the rows goes ahead, its stores wait.  4096 tokens, three contexts in turn, each with its own outputs:
-            // 15.4 -> 10.7 us per call.
+            // 15.4 -> 10.7 us per call.  With four sets of outputs or more on one context it is faster that one call of a
+            // round waits altogether, up to 4096 tokens (us a call, every call's stores waiting against one call of a round:
+            // 1000 tokens, 5 sets 7.9 and 5.7, 4096 tokens, 4 / 5 / 8 sets 10.3 / 10.6 / 10.4 and 10.1 / 9.0 / 9.8); with more
+            // the next launch finds little room beside this one and loses more than the stores (4736 tokens 5 sets 11.6 and
+            // 12.1, 8 sets 11.6 and 10.7; 6500 tokens 4 sets 13.6 and 15.9; 8192 tokens 5 sets 16.0 and 17.4).  Three sets:
+            // 4096 tokens 10.6 and 11.1, 300 tokens 8.2 and 7.2.
             const InFlight::Use uses[] = {{hidden, static_cast<size_t>(n_tokens) * c.d_model * 2, false},
                                           {compact->K, kv_bytes, false},
                                           {compact->V, kv_bytes, false},
@@ -923,7 +928,8 @@ static kvzap_status launch_score(kvzap_ctx *ctx, int32_t layer, int32_t n_layers
                                           {compact->lengths, sizeof(int32_t) * c.n_kv_heads, true}};
             if (ctx->in_flight.busy(hidden, uses[0].n, false)) p.wait_before_load = 1;
             const InFlight::Order order = ctx->in_flight.next(
-                uses, 7, !ctx->trusted || ctx->profiling || ctx->op_last_seq + 1 != ctx->op_seq, true);
+                uses, 7, !ctx->trusted || ctx->profiling || ctx->op_last_seq + 1 != ctx->op_seq,
+                p.n_tiles * kLinSplit * 8 <= ctx->sm_count * 7 ? 3 : InFlight::kMaxChain + 1);
             ctx->op_last_seq = ctx->op_seq;
             fc.enabled = 1;
             fc.row_bytes = c.head_dim * 2;
@@ -1248,7 +1254,7 @@ static kvzap_status launch_prune_onepass(kvzap_ctx *ctx, const float *scores, co
                                   {n_pages_used, page_tokens > 0 ? sizeof(int32_t) : 0, true},
                                   {slot_out, sizeof(int32_t) * static_cast<size_t>(n_tokens) * c.n_kv_heads, true}};
     const InFlight::Order order = ctx->in_flight.next(
-        uses, 11, !ctx->trusted || ctx->profiling || tau_list != nullptr || scores_just_made || ctx->op_last_seq + 1 != ctx->op_seq, false);
+        uses, 11, !ctx->trusted || ctx->profiling || tau_list != nullptr || scores_just_made || ctx->op_last_seq + 1 != ctx->op_seq, 0);
     const bool wait_first = order.wait != InFlight::kNone;
     ctx->op_last_seq = ctx->op_seq;
     // A launch that waits for the work ahead takes every slot of the device (32k tokens, a quarter kept: 40 -> 31 us); one

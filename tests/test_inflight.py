@@ -33,7 +33,7 @@ def lib():
 
 
 def _orders(lib, launches):
-    """[(wait, late)] of launches ([(address, bytes, write)], wait_all, stores_may_wait) in a row."""
+    """[(wait, late)] of launches ([(address, bytes, write)], wait_all, stores_wait) in a row."""
     f, out = lib.inflight_new(), []
     for uses, wait_all, stores in launches:
         flat = [x for u in uses for x in u]
@@ -65,7 +65,7 @@ def _unordered(launches, orders):
 
 
 def _random(seed, n=400):
-    """Prune-like (all or nothing), linear-like (stores may wait) and fixed-budget-like (wait in any case) launches over a few
+    """Prune-like (all or nothing), linear-like (stores may wait by themselves) and fixed-budget-like (wait in any case) launches over a few
     buffers, outputs of earlier ones among the inputs."""
     rng = random.Random(seed)
     buffers = [(4096 * (i + 1), 4096) for i in range(rng.choice([3, 6, 12, 40]))]
@@ -77,7 +77,7 @@ def _random(seed, n=400):
             a, size = rng.choice(buffers)
             off = rng.choice([0, 0, 0, size // 2])
             uses.append((a + off, rng.choice([16, size - off]), 1 if k < 2 else int(rng.random() < 0.3)))
-        out.append((uses, int(kind == "budget" or rng.random() < 0.05), int(kind == "linear")))
+        out.append((uses, int(kind == "budget" or rng.random() < 0.05), rng.choice([3, 15]) if kind == "linear" else 0))
     return out
 
 
@@ -96,6 +96,17 @@ def test_a_waiting_launch_that_lets_the_next_one_go_early_is_not_enough(lib):
     orders = _orders(lib, launches)
     assert not _unordered(launches, orders)[0]
     assert _unordered(launches, [(w, 0) for w, _ in orders])[0] == [(1, 3)]
+
+
+@pytest.mark.parametrize("sets,stores_wait,waits", [(1, 3, 99), (3, 3, 85), (4, 3, 24), (5, 3, 19), (8, 3, 12), (13, 3, 7), (5, 15, 71),
+                                                    (5, 0, 19)])
+def test_outputs_in_rotation(lib, sets, stores_wait, waits):
+    """Launches of 100 that wait for anything, where outputs come round after `sets` launches.  Those whose stores wait by
+    themselves do so from the first repetition to the end of a chain of 15; one of the others in each round of outputs."""
+    launches = [([(1 << 20, 64, 0), (4096 * (i % sets + 1), 64, 1)], 0, stores_wait) for i in range(100)]
+    orders = _orders(lib, launches)
+    assert not _unordered(launches, orders)[0]
+    assert sum(w != NONE for w, _ in orders) == waits
 
 
 @pytest.mark.parametrize("uses", [1, 12])
