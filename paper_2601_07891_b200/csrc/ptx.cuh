@@ -353,8 +353,10 @@ __device__ __forceinline__ void mbar_arrive_cluster(uint32_t cluster_addr)
     asm volatile("mbarrier.arrive.release.cluster.shared::cluster.b64 _, [%0];" ::"r"(cluster_addr) : "memory");
 }
 // All threads of all CTAs of the cluster.  Every thread reaches it: the kernels' own waits are bounded.
+// The aligned form wants the whole warp at the instruction together, which it need not be behind a branch on the lane.
 __device__ __forceinline__ void cluster_sync_all()
 {
+    __syncwarp();
     asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");
 }
 // Tiled loads issued by either CTA of a pair; the mbarrier (cluster address) may be the other CTA's.
