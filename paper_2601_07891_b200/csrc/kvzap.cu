@@ -1337,6 +1337,29 @@ static kvzap_status launch_prune_onepass(kvzap_ctx *ctx, const float *scores, co
     return KVZAP_OK;
 }
 
+// CTAs per (sequence, head) of a selection in one launch (select_cluster_kernel); 0 where three launches are the better form.
+// Some 2048 candidates of an average sequence to a CTA, and fewer where all lists still fit in one wave.  The host does not
+// know the lengths: where nearly all tokens are one sequence's, a few CTAs count them, at some 1.7 us a thousand, which three
+// launches spread over the device -- but those take longer the more lists there are.  So a CTA's share of all tokens is bounded,
+// the bound growing with the sequences, for up to twice the CTAs.  One against three launches, the whole call, us: 30000 + 20 x 20
+// tokens 48 and 48 (bound 10176), 100000 + 9 x 20 86 and 87, 30000 + 70 x 20 67 and 63, 45000 + 90 x 20 88 and 89, 60 x 546 50
+// and 57; beyond the bound 50000 + 30 x 20 86 and 66, 300000 + 7 x 3000 200 and 180, 100000 + 50 x 20 226 and 126 (but 64 x 2048
+// 91 and 113).  From some 200 sequences on one launch always wins: 200000 + 199 x 20 489 and 519, 200 x 1000 144 and 172.
+static int select_ctas(const kvzap_ctx *ctx, int64_t n_tokens, int32_t n_seqs)
+{
+    if (ctx->select_cluster == 0 || n_tokens > kSelectClusterTokens * n_seqs || n_seqs > 65535) return 0;
+    int cluster = 1;
+    const int64_t lists = static_cast<int64_t>(ctx->cfg.n_kv_heads) * n_seqs;
+    while (cluster < ctx->select_cluster &&
+           (static_cast<int64_t>(cluster) * kSelectKept * kSelectThreads * n_seqs < n_tokens ||
+            (2 * cluster * lists <= 4 * static_cast<int64_t>(ctx->sm_count) && static_cast<int64_t>(cluster) * 2 * 8192 <= n_tokens)))
+        cluster *= 2;
+    if (n_seqs == 1 || n_seqs >= 192) return cluster;
+    const int64_t share = std::max<int64_t>(9216, 6144 + 192 * static_cast<int64_t>(n_seqs));
+    if (n_tokens > share * cluster && cluster < ctx->select_cluster) cluster *= 2;
+    return n_tokens > share * cluster ? 0 : cluster;
+}
+
 static kvzap_status check_prune_args(kvzap_ctx *ctx, const void *K, const void *V, const void *K_out,
                                      const void *V_out, const int32_t *lengths, int32_t w)
 {
@@ -1902,15 +1925,8 @@ kvzap_status kvzap_prune_prefill_topk(kvzap_ctx *ctx, const void *K, const void 
     st = check_prune_args(ctx, K, V, K_out, V_out, lengths, w);
     if (st != KVZAP_OK) return st;
     if (!scores) return fail(ctx, KVZAP_ERR_INVALID_ARG, "scores is NULL");
-    if (!per_layer && ctx->select_cluster > 0 && n_tokens <= kSelectClusterTokens * n_seqs && n_seqs <= 65535) {
-        // One launch: CTAs of some 2048 candidates of an average sequence, at most as many as a cluster may have; and more
-        // than that, for batches with one sequence far longer than the others, where all of them still fit in one wave.
-        int cluster = 1;
-        const int64_t lists = static_cast<int64_t>(c.n_kv_heads) * n_seqs;
-        while (cluster < ctx->select_cluster &&
-               (static_cast<int64_t>(cluster) * kSelectKept * kSelectThreads * n_seqs < n_tokens ||
-                (2 * cluster * lists <= 4 * static_cast<int64_t>(ctx->sm_count) && static_cast<int64_t>(cluster) * 2 * 8192 <= n_tokens)))
-            cluster *= 2;
+    const int cluster = per_layer ? 0 : select_ctas(ctx, n_tokens, n_seqs);
+    if (cluster > 0) {
         cudaLaunchConfig_t cfg;
         cudaLaunchAttribute attrs[2];
         make_launch(&cfg, attrs, dim3(static_cast<unsigned>(cluster), static_cast<unsigned>(c.n_kv_heads), static_cast<unsigned>(n_seqs)),

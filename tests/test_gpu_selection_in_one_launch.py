@@ -18,3 +18,15 @@ def test_cut_values(lens, kind, ratio):
     for window in (0, 128):
         check(ctx, lens, window, kind, ratio, False)
     ctx.close()
+
+
+@pytest.mark.parametrize("lens,launches", [
+    ([16000] + [20] * 2, 2), ([546] * 60, 2), ([200] * 200, 2), ([30000] + [20] * 20, 2), ([100000] + [20] * 9, 2),   # one
+    ([50000] + [20] * 30, 4), ([100000] + [20] * 50, 4), ([120000] + [20] * 2, 2), ([300000] + [20] * 2, 4)])       # or three
+def test_one_long_sequence_among_short_ones(lens, launches):
+    """A few CTAs would count nearly all tokens of such a batch: three launches take it instead."""
+    ctx = binding.Kvzap(256, 0, H, D, 1, max_tokens=sum(lens), max_seqs=len(lens))
+    before = ctx.launch_count()
+    check(ctx, lens, 128, "normal", 0.25, False)
+    assert ctx.launch_count() - before == 2 * launches       # the check calls twice
+    ctx.close()
