@@ -619,6 +619,9 @@ kvzap_status kvzap_cache_debug_skew_steps(kvzap_cache *cache, int32_t delta);
  * created (for launch accounting in benchmarks). */
 int64_t kvzap_launch_count(const kvzap_ctx *ctx);
 
+/* Of those, the attention launches that were let run beside the decode step ahead of them (0 for NULL). */
+int64_t kvzap_beside_count(const kvzap_ctx *ctx);
+
 #ifdef __cplusplus
 }
 #endif

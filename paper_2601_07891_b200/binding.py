@@ -90,6 +90,7 @@ SIGNATURES = {
     "kvzap_get_profile": (_i32, [_vp, _i32, ctypes.POINTER(ctypes.c_double), ctypes.POINTER(_i64)]),
     "kvzap_poll_status": (_i32, [_vp, _vp]),
     "kvzap_launch_count": (_i64, [_vp]),
+    "kvzap_beside_count": (_i64, [_vp]),
 }
 
 
@@ -568,6 +569,10 @@ def kvzap_poll_status(handle, stream=None) -> int:
 
 def kvzap_launch_count(handle) -> int:
     return int(load().kvzap_launch_count(handle))
+
+
+def kvzap_beside_count(handle) -> int:
+    return int(load().kvzap_beside_count(handle))
 
 
 class Kvzap:

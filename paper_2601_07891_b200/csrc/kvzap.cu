@@ -111,7 +111,7 @@ struct kvzap_ctx {
     int32_t *list_base = nullptr;    // [max_seqs * H] appending to lists: rows each list held before
     int32_t *status_dev = nullptr;
     int32_t *status_host = nullptr;  // pinned
-    int64_t launches = 0;
+    int64_t launches = 0, beside = 0;
     // tensor maps of recently used hidden-state buffers (encoding one costs about as much as a launch)
     struct TmapEntry { const void *base; int64_t rows; int32_t slabs; CUtensorMap map; };
     std::vector<TmapEntry> tmap_cache;
@@ -1690,6 +1690,8 @@ const char *kvzap_last_error(const kvzap_ctx *ctx) { return ctx ? ctx->err : g_c
 
 int64_t kvzap_launch_count(const kvzap_ctx *ctx) { return ctx ? ctx->launches : 0; }
 
+int64_t kvzap_beside_count(const kvzap_ctx *ctx) { return ctx ? ctx->beside : 0; }
+
 kvzap_status kvzap_set_weights(kvzap_ctx *ctx, int32_t layer, const void *W1, const float *b1, const void *W2,
                                const float *b2, void *stream_)
 {
@@ -2777,6 +2779,7 @@ static kvzap_status attention_impl(kvzap_ctx *ctx, kvzap_cache *cache, int32_t l
                                            cache->tm_vring, p));
     }
     ctx->launches += 1;
+    ctx->beside += beside ? 1 : 0;
     return KVZAP_OK;
 }
 

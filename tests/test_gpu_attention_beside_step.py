@@ -75,17 +75,25 @@ def _close(got, want):
     return bool((d <= 2e-2 + 2.0 ** -8 * want.float().abs()).all()) and bool(torch.isfinite(got.float()).all())
 
 
-@pytest.mark.parametrize("D,G,B,L,group,w,longest,fp8", [
-    (128, 4, 3, 3, 1, 16, 70, False),         # short lists, every tile remainder, layer by layer
-    (128, 4, 8, 2, 1, 128, 3000, False),      # parts by length
-    (128, 8, 70, 2, 1, 32, 200, False),       # more lists than CTAs of a wave
-    (64, 4, 5, 4, 2, 48, 500, False),         # rows of 64 elements, two layers a call
-    (128, 1, 130, 2, 1, 16, 90, False),       # two tiles of sequences per layer
-    (128, 4, 4, 3, 1, 16, 900, True),         # 8-bit rows
-    (64, 8, 9, 3, 3, 16, 60, True),
+# A step of hidden 512 takes 32 CTAs per layer and 128 sequences, one of hidden 128 eight: up to six tiles leave room beside it.
+@pytest.mark.parametrize("D,G,B,L,group,w,longest,fp8,hidden,beside", [
+    (128, 4, 3, 3, 1, 16, 70, False, 512, True),         # short lists, every tile remainder, layer by layer
+    (128, 4, 8, 2, 1, 128, 3000, False, 512, True),      # parts by length
+    (128, 4, 8, 2, 1, 16, 26000, False, 512, True),      # so long that all CTAs wait for the step
+    (128, 8, 70, 2, 1, 32, 200, False, 512, True),       # more lists than CTAs of a wave
+    (128, 2, 64, 2, 1, 32, 2700, False, 512, True),      # ... in two parts each
+    (64, 4, 5, 4, 2, 48, 500, False, 128, True),         # rows of 64 elements, two layers a call
+    (64, 4, 5, 3, 1, 48, 500, False, 512, True),
+    (64, 2, 60, 2, 1, 16, 90, False, 128, True),
+    (128, 1, 130, 2, 1, 16, 90, False, 128, True),       # two tiles of sequences per layer
+    (128, 4, 4, 3, 1, 16, 900, True, 512, True),         # 8-bit rows
+    (128, 4, 70, 2, 1, 16, 300, True, 128, True),        # ... of as many lists as find room beside the step
+    (64, 8, 9, 3, 3, 16, 60, True, 128, True),
+    (64, 8, 9, 3, 1, 16, 60, True, 512, True),
+    (128, 4, 8, 3, 2, 16, 60, False, 512, False),        # steps on too many SMs
 ])
-def test_outputs_are_those_of_a_context_that_waits(binding, D, G, B, L, group, w, longest, fp8):
-    d_model, hidden, steps = 1024, 512, w + 40
+def test_outputs_are_those_of_a_context_that_waits(binding, D, G, B, L, group, w, longest, fp8, hidden, beside):
+    d_model, steps = 1024, w + 40
     rng = np.random.default_rng(D + B)
     prefix = rng.integers(0, longest, size=B * L * H)
     prefix[:6] = [0, 1, 15, 16, 17, longest]
@@ -100,9 +108,10 @@ def test_outputs_are_those_of_a_context_that_waits(binding, D, G, B, L, group, w
             scale = scale.view(L, B)
         K, V = (sides[0]._rows((L, B, H), D, 200 + 2 * k + i) for i in (0, 1))
         inputs.append((X.view(L, B, d_model), scale, K.view(L, B, H, row), V.view(L, B, H, row)))
-    Q = synth.hidden_states(L * B * H * G, D, seed=7, device="cuda").view(L, B, H * G, D)
+    Q7 = [synth.hidden_states(L * B * H * G, D, seed=7 + k, device="cuda").view(L, B, H * G, D) for k in range(7)]
     for side, out in zip(sides, outs):
         for k in range(steps):
+            Q = Q7[k % 7]
             X, scale, K, V = inputs[k % 7]
             O = torch.full((L, B, H * G, D), 7.0, dtype=torch.bfloat16, device="cuda")
             scores = torch.zeros(L, B, H, dtype=torch.float32, device="cuda")
@@ -113,6 +122,10 @@ def test_outputs_are_those_of_a_context_that_waits(binding, D, G, B, L, group, w
             out.append((O, scores))
         torch.cuda.synchronize()
         assert side.ctx.poll_status() == 0
+    # all attentions but the first, whose step has none ahead of it; a last call of fewer layers has steps small enough
+    calls = [e - l for _ in range(steps) for l in range(0, L, group) for e in [min(L, l + group)]]
+    assert binding.kvzap_beside_count(sides[1].ctx.handle) == 0
+    assert binding.kvzap_beside_count(sides[0].ctx.handle) == sum(beside or n < group for n in calls[1:])
     n = [torch.empty(B, L, H, dtype=torch.int32, device="cuda") for _ in sides]
     for side, ln in zip(sides, n):
         binding.kvzap_cache_lengths(side.ctx.handle, side.cache, ln)
@@ -124,10 +137,10 @@ def test_outputs_are_those_of_a_context_that_waits(binding, D, G, B, L, group, w
         side.close()
 
 
-@pytest.mark.parametrize("fp8", [False, True])
-def test_queries_written_between_step_and_attention(binding, producer, fp8):  # noqa: F811
+@pytest.mark.parametrize("D,fp8", [(128, False), (128, True), (64, False), (64, True)])
+def test_queries_written_between_step_and_attention(binding, producer, D, fp8):  # noqa: F811
     """The kernel between the two signals before it stores the queries: they are read again once it has completed."""
-    D, G, B, L, w, d_model, hidden = 128, 4, 6, 2, 16, 1024, 512
+    G, B, L, w, d_model, hidden = 4, 6, 2, 16, 1024, 128
     prefix = np.random.default_rng(3).integers(0, 700, size=B * L * H)
     sides = [_Side(binding, t, d_model, hidden, D, L, B, w, prefix, 4, fp8) for t in (True, False)]
     row = sides[0].pools[0].shape[-1]
@@ -142,8 +155,9 @@ def test_queries_written_between_step_and_attention(binding, producer, fp8):  # 
         got = []
         for side in sides:
             Q, O = old.clone(), torch.full_like(old, 7.0)
-            scores = torch.zeros(L, B, H, dtype=torch.float32, device="cuda")
+            scores, O0 = torch.zeros(L, B, H, dtype=torch.float32, device="cuda"), torch.empty_like(O)
             torch.cuda.synchronize()
+            side.attend(0, L, old, O0)                           # for the step to start behind
             side.step(0, L, X.view(L, B, d_model), scale, K, V, -0.1, scores)
             producer(new, Q)
             side.attend(0, L, Q, O)
@@ -151,6 +165,7 @@ def test_queries_written_between_step_and_attention(binding, producer, fp8):  # 
             assert side.ctx.poll_status() == 0
             got.append(O)
         assert _close(got[0], got[1]), k
+    assert binding.kvzap_beside_count(sides[0].ctx.handle) == 6
     for side in sides:
         side.close()
 
