@@ -154,6 +154,7 @@ struct kvzap_ctx {
                                                     // in every replay, across a capture's borders it may not be
     const void *attn_out = nullptr;
     size_t attn_out_bytes = 0;
+    int attn_per_sm = 0;                            // CTAs of it that an SM takes
     const kvzap_cache *fused_cache = nullptr;
     std::vector<kvzap_cache *> caches;              // caches created on this context (their step counters are
                                                     // cleared when a timeout has been polled)
@@ -695,6 +696,16 @@ static kvzap_status launch_score_rest(kvzap_ctx *ctx, ScoreParams p, const CUten
     return KVZAP_OK;
 }
 
+// Whether an attention over so many lists, per_sm of its CTAs to an SM, is let run beside a step of so many CTAs.  More lists than
+// CTAs find room beside it, and still one wave: all of them wait for the step, and what is left to gain is the next step's start.
+// Rows of 8 bits (four CTAs): not worth the slower kernel.  Six layers of step and attention, us, beside / not, calls in a row and
+// with other work ahead of every step: 64 sequences x 1540 8-bit rows 475 / 480 and 525 / 505, 60 x 500 273 / 272 and 322 / 294;
+// 50 x 1024 bf16 rows 391 / 410 and 448 / 433.
+static bool beside_pays(const kvzap_ctx *ctx, int64_t lists, int per_sm, int step_ctas)
+{
+    return per_sm < 4 || lists <= static_cast<int64_t>(ctx->sm_count - step_ctas) * per_sm || lists >= static_cast<int64_t>(ctx->sm_count) * per_sm;
+}
+
 // Launches the scoring kernel over layers [layer, layer + n_layers); hidden is [n_layers][n_tokens][d_model],
 // scores [n_layers][n_tokens][H]; maskbits != nullptr fuses the threshold/window test.
 static kvzap_status launch_score(kvzap_ctx *ctx, int32_t layer, int32_t n_layers, const void *hidden, int64_t n_tokens,
@@ -833,6 +844,7 @@ static kvzap_status launch_score(kvzap_ctx *ctx, int32_t layer, int32_t n_layers
         const bool behind_attention = fuse_ok && ctx->trusted && early && ctx->attn_seq + 1 == ctx->op_seq &&
                                       ctx->attn_stream == stream && ctx->attn_capture == capture_of(stream) && ctx->attn_capture != ~0ull &&
                                       p.n_tiles * n_ctas * 3 <= ctx->sm_count &&
+                                      beside_pays(ctx, n_tokens * n_layers * c.n_kv_heads, ctx->attn_per_sm, p.n_tiles * n_ctas) &&
                                       !attn_writes(hidden, x_bytes) && !attn_writes(f.K_new, kv_bytes) && !attn_writes(f.V_new, kv_bytes);
         f.behind_attention = behind_attention ? 1 : 0;
         p.wait_before_load = ctx->trusted && (!fuse_ok || overlap || behind_attention) ? 0 : 1;
@@ -2731,7 +2743,7 @@ static kvzap_status attention_impl(kvzap_ctx *ctx, kvzap_cache *cache, int32_t l
     // 4 parts 490 us, 1 part 355 us, of 4700 rows: 1 part 1678 us, 3 parts 1527 us (4 layers).  320 lists, by their
     // lengths: 898 us against 1115 us in 14 equal parts (8 layers).  The capacity stands for the lengths, which the host does
     // not know: 1024 lists of 300 rows take 32.8 us in a table for as many, 51.8 us in one for 32768.
-    const int64_t per_sm = fp8 && d_attn == 128 ? 4 : 3;
+    const int per_sm = fp8 && d_attn == 128 ? 4 : 3;
     const int64_t slots = static_cast<int64_t>(ctx->sm_count) * per_sm;
     bool beside = false;
     // Directly behind a step in one launch over these layers that itself came directly behind an attention: nothing else that
@@ -2740,7 +2752,8 @@ static kvzap_status attention_impl(kvzap_ctx *ctx, kvzap_cache *cache, int32_t l
     // 8-bit rows 79.8 -> 78.6.
     const unsigned long long capture = capture_of(stream);
     if (ctx->trusted && !ctx->profiling && ctx->fused_capture == capture && ctx->fused_cache == cache && ctx->fused_seq + 1 == ctx->op_seq && ctx->fused_behind_attention &&
-        ctx->fused_stream == stream && ctx->fused_layer0 <= layer_begin && layer_end <= ctx->fused_layer1) {
+        ctx->fused_stream == stream && ctx->fused_layer0 <= layer_begin && layer_end <= ctx->fused_layer1 &&
+        beside_pays(ctx, n_lists_call, per_sm, ctx->fused_ctas)) {
         beside = true;
         const int64_t sms_left = ctx->sm_count - ctx->fused_ctas;
         p.beside_ctas = static_cast<int32_t>(sms_left * per_sm);
@@ -2768,6 +2781,7 @@ static kvzap_status attention_impl(kvzap_ctx *ctx, kvzap_cache *cache, int32_t l
     ctx->attn_stream = stream;
     ctx->attn_capture = capture;
     ctx->attn_out = O;
+    ctx->attn_per_sm = per_sm;
     ctx->attn_out_bytes = static_cast<size_t>(p.n_layers_call) * v.n_seqs * n_q_heads * d_attn * 2;
     {
         ProfScope prof(ctx, KVZAP_KERNEL_ATTENTION, stream);

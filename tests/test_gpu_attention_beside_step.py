@@ -88,6 +88,8 @@ def _close(got, want):
     (128, 1, 130, 2, 1, 16, 90, False, 128, True),       # two tiles of sequences per layer
     (128, 4, 4, 3, 1, 16, 900, True, 512, True),         # 8-bit rows
     (128, 4, 70, 2, 1, 16, 300, True, 128, True),        # ... of as many lists as find room beside the step
+    (128, 4, 60, 2, 1, 16, 100, True, 512, False),       # ... and of more
+    (128, 4, 50, 2, 1, 16, 100, False, 512, True),
     (64, 8, 9, 3, 3, 16, 60, True, 128, True),
     (64, 8, 9, 3, 1, 16, 60, True, 512, True),
     (128, 4, 8, 3, 2, 16, 60, False, 512, False),        # steps on too many SMs
