@@ -854,7 +854,7 @@ static kvzap_status launch_score(kvzap_ctx *ctx, int32_t layer, int32_t n_layers
             ctx->fused_ctas = p.n_tiles * n_ctas;
             ctx->fused_behind_attention = behind_attention;
         }
-        ctx->last_score_early = early;
+        ctx->last_score_early = early && !p.late_trigger;
         {
             ProfScope prof(ctx, KVZAP_KERNEL_SCORE, stream);
             KVZAP_CUDA(ctx, launch_split(layout, split_k, pairs != nullptr, fp8, tmap_x, p, f, early, stream));
@@ -1076,7 +1076,7 @@ static kvzap_status launch_score_fp8(kvzap_ctx *ctx, int32_t layer, const void *
     bool pairs;
     if (!ctx->trusted && prompt_layout(ctx, blocks_per_layer, true, false, &pairs) != nullptr)
         return launch_score(ctx, layer, 1, hidden8, n_tokens, scores, maskbits, cu_seqlens, n_seqs, tau, w, stream, 1, nullptr, nullptr,
-                            nullptr, nullptr, nullptr, true, x_scale);
+                            nullptr, nullptr, nullptr, true, x_scale, update_behind);
     const bool pair = c.hidden > 0 && ctx->pair_clusters > 0 && blocks_per_layer >= 2;
     const kvzap_ctx::Schedule &sc = ctx->sched[pair ? 1 : 0];
     const int64_t rest = pair && !update_behind ? rest_blocks(ctx, blocks_per_layer, true) : 0;
