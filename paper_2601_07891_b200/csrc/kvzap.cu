@@ -2777,12 +2777,6 @@ static kvzap_status attention_impl(kvzap_ctx *ctx, kvzap_cache *cache, int32_t l
     }
     p.part_scratch = cache->attn_scratch;
     p.part_arrive = cache->attn_arrive;
-    ctx->attn_seq = ctx->op_seq;
-    ctx->attn_stream = stream;
-    ctx->attn_capture = capture;
-    ctx->attn_out = O;
-    ctx->attn_per_sm = per_sm;
-    ctx->attn_out_bytes = static_cast<size_t>(p.n_layers_call) * v.n_seqs * n_q_heads * d_attn * 2;
     {
         ProfScope prof(ctx, KVZAP_KERNEL_ATTENTION, stream);
         cudaLaunchConfig_t cfg;
@@ -2794,6 +2788,13 @@ static kvzap_status attention_impl(kvzap_ctx *ctx, kvzap_cache *cache, int32_t l
     }
     ctx->launches += 1;
     ctx->beside += beside ? 1 : 0;
+    // only now: a step may start beside this attention only if it is there
+    ctx->attn_seq = ctx->op_seq;
+    ctx->attn_stream = stream;
+    ctx->attn_capture = capture;
+    ctx->attn_out = O;
+    ctx->attn_per_sm = per_sm;
+    ctx->attn_out_bytes = static_cast<size_t>(p.n_layers_call) * v.n_seqs * n_q_heads * d_attn * 2;
     return KVZAP_OK;
 }
 
