@@ -1335,8 +1335,7 @@ static kvzap_status launch_prune_onepass(kvzap_ctx *ctx, const float *scores, co
     p.scan_flag = ctx->op_scan_flag + set;
     p.epoch = ctx->op_epoch;
     p.wait_limit = ctx->wait_limit;
-    p.wait_first = wait_first ? 1 : 0;
-    p.late_trigger = order.late && ctx->trusted ? 1 : 0;
+    p.wait_first = !wait_first ? 0 : order.late && ctx->trusted ? 2 : 1;
     {
         ProfScope prof(ctx, KVZAP_KERNEL_COMPACT, stream);
         cudaLaunchConfig_t cfg;

@@ -81,8 +81,8 @@ struct PruneParams {
     int64_t clear_units;
     int32_t recount;           // 1: short dense input, one head per CTA: rows kept before the CTA's first token are counted
                                // from the scores, not learnt from the CTAs before it
-    int32_t wait_first;        // 1: wait for the work ahead in the stream before the first load
-    int32_t late_trigger;      // 1: the next launch may start once that wait is over (else at once)
+    int32_t wait_first;        // 1: wait for the work ahead in the stream before the first load; 2: and the next launch may
+                               // start once that wait is over (else at once)
 };
 
 // Spins until *flag == want (acquire); false when the cycle budget runs out.
@@ -197,11 +197,13 @@ prune_onepass_kernel(const PruneParams p)
     __shared__ float tau_s[kMaxHeads];                  // thresholds of the sequence at the CTA's first token
 
     // On a context that trusts its producers the next launch may wait for nothing: behind a launch that does, it starts only
-    // when everything ahead of that one is complete, of which the host then keeps no list.
-    if (!p.late_trigger) griddep_launch_dependents();
-    if (!kTauBehind && p.wait_first) {
-        griddep_wait();
-        if (p.late_trigger) griddep_launch_dependents();
+    // when everything ahead of that one is complete, of which the host then keeps no list.  (kTauBehind: it does on any.)
+    if constexpr (!kTauBehind) {
+        if (p.wait_first < 2) griddep_launch_dependents();
+        if (p.wait_first > 0) {
+            griddep_wait();
+            if (p.wait_first == 2) griddep_launch_dependents();
+        }
     }
 
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
@@ -237,7 +239,7 @@ prune_onepass_kernel(const PruneParams p)
             if (wl < static_cast<int>(blk1 - blk0) * 4) load_token(p, blk0 * 4 + wl, lane, multi, early[u]);
         }
         griddep_wait();
-        if (p.late_trigger) griddep_launch_dependents();
+        griddep_launch_dependents();
     }
     if (tid < kMaxHeads) tau_s[tid] = p.tau_list != nullptr && tid < H ? __ldcg(p.tau_list + b_lo * H + tid) : p.tau;
     const int j0 = static_cast<int>((s0 / kBlockTokens) / p.blocks_per_cta);      // the CTA (column) whose blocks hold s0
