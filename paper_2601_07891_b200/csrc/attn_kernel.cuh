@@ -426,6 +426,8 @@ decode_attn_kernel(const __grid_constant__ CUtensorMap tmap_kpool, const __grid_
         const int list_now = kBeside ? static_cast<int>(kept_s[warp][kList]) : list, l_rel = list_now / (H * B), b = (list_now / H) % B;
         return (static_cast<int64_t>(l_rel) * B + b) * H * p.group + list_now % H * p.group;
     };
+    // kBeside has no registers to keep it in
+    const int64_t row0 = kBeside ? 0 : query_row();
     auto load_query = [&](const uint16_t *qrow, int ks, uint32_t &lo, uint32_t &hi) {
         lo = hi = 0u;
         if (g < p.group) {
@@ -456,7 +458,7 @@ decode_attn_kernel(const __grid_constant__ CUtensorMap tmap_kpool, const __grid_
     uint32_t qa[kD / 16][2];
     float logit_scale;                     // 8-bit rows: times the power of two taken out of this lane's query row
     auto take_query = [&]() {
-        const uint16_t *qrow = p.q + (query_row() + g) * kD;
+        const uint16_t *qrow = p.q + ((kBeside ? query_row() : row0) + g) * kD;
 #pragma unroll
         for (int ks = 0; ks < kD / 16; ++ks) load_query(qrow, ks, qa[ks][0], qa[ks][1]);
         logit_scale = p.scale_log2e;
@@ -727,7 +729,7 @@ decode_attn_kernel(const __grid_constant__ CUtensorMap tmap_kpool, const __grid_
     }
     __syncthreads();
     const bool failed = *abort_flag != 0;
-    const int64_t out_row0 = query_row();
+    const int64_t out_row0 = kBeside ? query_row() : row0;
     if constexpr (kBeside) {
         list = kept_s[warp][kList];
         part = kept_s[warp][kPart];
