@@ -39,6 +39,13 @@
  *     that does not itself signal early.  (2) Passing the same scores buffer
  *     to two consecutive calls is allowed in either mode; the library then
  *     launches the second call's scoring kernel without overlap of its stores.
+ *     (3) An output of a call does not lie in memory that the previous call on that stream reads, or that
+ *     calls of another context on that stream use, unless an ordinary kernel or copy is enqueued between: an
+ *     allocator that hands freed memory out again in stream order could do that.  The pruning calls and
+ *     linear prompts of up to 8192 tokens see to it themselves among the calls of their own context.
+ *     Decoding layer by layer in this mode: enqueue kvzap_decode_attention directly behind kvzap_decode_step of
+ *     the same layers, where the queries are there by then.  The attention then runs beside the step; with a
+ *     kernel of the caller between the two (which is safe) it cannot, and takes a few microseconds longer.
  *   - Stream capture (CUDA graphs): kvzap_decode_step(_fp8) and kvzap_decode_attention(_fp8) may be captured
  *     and replayed.  The other calls rotate scratch sets and counters on the host from call to call and must
  *     be enqueued, not captured.

@@ -26,7 +26,7 @@
 // (kBeside): the step behind an attention scores beside it and only its stores to the cache wait, and the attention behind
 // that step reads all rows that the lists held before it while it runs; what the step changes (the prefix's last tile, the
 // window) is read when it has completed, and so are the queries, once more -- if they are not what they were, the CTA starts
-// again.  36 layers x 8 sequences x 2176 rows 1238 -> 836 us, 4 layers x 128 sequences x 4736 rows 1596 -> 1524 us.
+// again.  36 layers x 8 sequences x 2176 rows 1235 -> 855 to 900 us, 4 layers x 128 sequences x 4736 rows 1600 -> 1500 to 1545 us.
 //
 // Math per tile, on the warp-level tensor-core path (the work is HBM-bound; 16-row MMAs are enough):
 //   S[16 x 16]  = Q[16 x D] K^T      m16n8k16, Q rows 0..G-1 real, the rest zero
@@ -188,8 +188,8 @@ __device__ __forceinline__ void attn_store(uint16_t *out, const float4 &num, flo
     *reinterpret_cast<uint2 *>(out) = v;
 }
 
-// kBeside: the launch may run beside the step ahead of it (p.after_step); a kernel of its own, since what that takes (the rest
-// of a list learnt late, queries read twice) costs a launch that cannot some 2 us.
+// kBeside: the launch may run beside the step ahead of it; a kernel of its own, since what that takes (the rest of a list learnt
+// late, queries read twice, more code) costs a launch 2 to 5 us where nothing runs beside it: behind other work of the caller.
 template <int kD, bool kFp8, bool kBeside>
 __global__ void __launch_bounds__(kAttnThreads, kFp8 ? 4 : 3)
 decode_attn_kernel(const __grid_constant__ CUtensorMap tmap_kpool, const __grid_constant__ CUtensorMap tmap_vpool,

@@ -22,7 +22,7 @@ namespace kvzap {
 constexpr int kLinSplit = 4;
 constexpr int kLinStages = 8;             // pipeline stages; kLinStagesCompact when the compaction runs in the same launch
 constexpr int kLinStagesCompact = 2;      // (four CTAs then fit an SM: the launches of the next calls run beside this one;
-                                          //  measured per call at 4096 tokens: 8.8 us with 2 stages, 9.9 with 3, 9.6 with 5)
+                                          //  measured per call at 4096 tokens: 8.8 us with 2 stages (9.0 today), 9.9 with 3, 9.6 with 5)
 constexpr int kLinThreads = 192;          // producer warp, MMA warp, four epilogue warps
 constexpr int kLinMaxTiles = 64;          // tiles of a launch that also compacts (its clusters wait for one another)
 constexpr uint32_t kLinBTileBytes = 16 * kBlockK * 2;                 // 16 weight rows (H <= 8, padded) of one K block

@@ -234,14 +234,14 @@ select_pass_kernel(const float *__restrict__ scores, int64_t n_tokens, int n_hea
 // the CTA that owns them (2048 / gridDim.x each, in distributed shared memory), and after one cluster barrier every CTA
 // reads all bins and takes the digit itself: no global memory, no launch and no grid-wide meeting between the passes.  The
 // pruning behind it reads its first scores before it waits for the cut values.  32k tokens x 8 heads, a quarter kept, the
-// whole call: 38.8 us with three launches, 36.0 us with this one, 35.8 us with the early scores (4 x 8192 tokens 43.1 and
-// 42.1 us); a first pass on new inputs 74 -> 65 us.  (Bins owned in turn, so that neighbouring ones, which most keys share, spread over the CTAs: 65 us, a thread's
+// whole call: 38.8 us with three launches, 36.5 us with this one, 35.8 us with the early scores as well (4 x 8192 tokens 43.1 and
+// 39 us); a first pass on new inputs 74 -> 65 us.  (Bins owned in turn, so that neighbouring ones, which most keys share, spread over the CTAs: 65 us, a thread's
 // eight bins then come from eight CTAs.)
 constexpr int kSelectKept = 8;
 constexpr int kSelectMaxCluster = 16;
 // Tokens of an average sequence up to which it is taken.  The whole call, us: one sequence of 300 tokens 23.4 -> 17.8, 16000
-// tokens 29.9 -> 26.0, 32768 tokens 38.3 -> 36.5, but 65536 tokens 55.9 -> 57.4, 131072 tokens 87.5 -> 91.8 (16 CTAs a head are
-// too few for the counting); 4 x 32768 tokens 99 -> 88, 7 x 4681 tokens 49.2 -> 42.7, 60 x 546 tokens 63 -> 45.5.
+// tokens 29.9 -> 26.0, 32768 tokens 38.3 -> 35.8, but 65536 tokens 55.9 -> 57.4, 131072 tokens 87.5 -> 91.8 (16 CTAs a head are
+// too few for the counting); 4 x 32768 tokens 99 -> 88, 7 x 4681 tokens 49.2 -> 42.7.  Batches have a bound of their own as well (select_ctas).
 constexpr int64_t kSelectClusterTokens = 40960;
 
 __global__ void __launch_bounds__(kSelectThreads)

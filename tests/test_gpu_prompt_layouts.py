@@ -1,6 +1,5 @@
 """Prompts of every number of 128-token blocks at which the MLP scoring changes its launches: single CTAs or CTA pairs per
-block, odd numbers of blocks, whole waves of CTA pairs with the blocks they leave over in a launch of their own, and the
-compaction of the first waves beside the scoring of the last.
+block, odd numbers of blocks, and whole waves of CTA pairs with the blocks they leave over in a launch of their own.
 
 Scores against a product in 64 bits.  Products of bf16 or E4M3 values are exact in fp32; a pre-activation sums 1024 of them,
 2^-24 * sqrt(1024) of about one each at worst of a few standard deviations: 1e-5; the second layer sums up to 640 such times
