@@ -637,24 +637,30 @@ static const kvzap_ctx::SplitLayout *prompt_layout(const kvzap_ctx *ctx, int64_t
     return l ? l : i >= 0 ? &ctx->layouts[i] : nullptr;
 }
 
-static decltype(&score_split_kernel<false, false, false>) split_kernel(bool fp8, bool pair, bool fused)
+static decltype(&score_split_kernel<false, false, kNoStep>) split_kernel(bool fp8, bool pair, SplitStep step)
 {
-    if (pair) return fp8 ? score_split_kernel<true, true, false> : score_split_kernel<false, true, false>;
-    if (fused) return fp8 ? score_split_kernel<true, false, true> : score_split_kernel<false, false, true>;
-    return fp8 ? score_split_kernel<true, false, false> : score_split_kernel<false, false, false>;
+    if (pair) return fp8 ? score_split_kernel<true, true, kNoStep> : score_split_kernel<false, true, kNoStep>;
+    if (step == kStep) return fp8 ? score_split_kernel<true, false, kStep> : score_split_kernel<false, false, kStep>;
+    if (step == kStepBehindAttention)
+        return fp8 ? score_split_kernel<true, false, kStepBehindAttention> : score_split_kernel<false, false, kStepBehindAttention>;
+    return fp8 ? score_split_kernel<true, false, kNoStep> : score_split_kernel<false, false, kNoStep>;
 }
-constexpr int kSplitKernels = 3;        // per input type: (pair, fused) = (0, 0), (1, 0), (0, 1)
+constexpr int kSplitKernels = 4;        // per input type, numbered: by step without pairs, then pairs
+static decltype(&score_split_kernel<false, false, kNoStep>) split_kernel(bool fp8, int i)
+{
+    return split_kernel(fp8, i == 3, i < 3 ? static_cast<SplitStep>(i) : kNoStep);
+}
 
 // Enqueues the few-token kernel over p.n_tiles tiles (of two blocks for a layout with CTA pairs).
 static cudaError_t launch_split(const kvzap_ctx::SplitLayout &l, int k, bool pair, bool fp8, const CUtensorMap &tmap_x, const ScoreParams &p,
-                                const DecodeFuse &f, bool early, cudaStream_t stream)
+                                const DecodeFuse &f, bool early, cudaStream_t stream, bool behind_attention = false)
 {
     const int ctas = pair ? 2 : 1;
     cudaLaunchConfig_t cfg;
     cudaLaunchAttribute attrs[2];
     make_launch(&cfg, attrs, dim3(static_cast<unsigned>(p.n_tiles * ctas * l.n * k)), dim3(kScoreThreads), l.smem, stream, early, ctas * k);
     const CUtensorMap &tmap_w = fp8 ? l.tmap_w8 : l.tmap_w;
-    return cudaLaunchKernelEx(&cfg, split_kernel(fp8, pair, f.enabled != 0), tmap_x, tmap_w, p, l.n, k, f);
+    return cudaLaunchKernelEx(&cfg, split_kernel(fp8, pair, behind_attention ? kStepBehindAttention : f.enabled != 0 ? kStep : kNoStep), tmap_x, tmap_w, p, l.n, k, f);
 }
 
 // Blocks of a prompt that whole waves of CTA pairs leave over and that the few-token kernel takes instead, in a launch of its
@@ -846,7 +852,6 @@ static kvzap_status launch_score(kvzap_ctx *ctx, int32_t layer, int32_t n_layers
                                       p.n_tiles * n_ctas * 3 <= ctx->sm_count &&
                                       beside_pays(ctx, n_tokens * n_layers * c.n_kv_heads, ctx->attn_per_sm, p.n_tiles * n_ctas) &&
                                       !attn_writes(hidden, x_bytes) && !attn_writes(f.K_new, kv_bytes) && !attn_writes(f.V_new, kv_bytes);
-        f.behind_attention = behind_attention ? 1 : 0;
         p.wait_before_load = ctx->trusted && (!fuse_ok || overlap || behind_attention) ? 0 : 1;
         p.late_trigger = (late_trigger || fuse_ok) && p.wait_before_load;
         ctx->last_score_late = p.late_trigger != 0;
@@ -857,7 +862,7 @@ static kvzap_status launch_score(kvzap_ctx *ctx, int32_t layer, int32_t n_layers
         ctx->last_score_early = early && !p.late_trigger;
         {
             ProfScope prof(ctx, KVZAP_KERNEL_SCORE, stream);
-            KVZAP_CUDA(ctx, launch_split(layout, split_k, pairs != nullptr, fp8, tmap_x, p, f, early, stream));
+            KVZAP_CUDA(ctx, launch_split(layout, split_k, pairs != nullptr, fp8, tmap_x, p, f, early, stream, behind_attention));
         }
         ctx->launches += 1;
         return KVZAP_OK;
@@ -1561,8 +1566,8 @@ kvzap_status kvzap_create(kvzap_ctx **out, const kvzap_config *cfg)
         ctx->split_smem_limit = budget + 1024 - 4608;       // the kernel has 4112 bytes of static shared memory
         // the limit is the function's, not the context's: the most that any layout of any context takes
         for (int i = 0; i < kSplitKernels; ++i) {
-            CREATE_CUDA(cudaFuncSetAttribute(split_kernel(false, i == 1, i == 2), cudaFuncAttributeMaxDynamicSharedMemorySize, ctx->split_smem_limit));
-            CREATE_CUDA(cudaFuncSetAttribute(split_kernel(false, i == 1, i == 2), cudaFuncAttributePreferredSharedMemoryCarveout,
+            CREATE_CUDA(cudaFuncSetAttribute(split_kernel(false, i), cudaFuncAttributeMaxDynamicSharedMemorySize, ctx->split_smem_limit));
+            CREATE_CUDA(cudaFuncSetAttribute(split_kernel(false, i), cudaFuncAttributePreferredSharedMemoryCarveout,
                                              static_cast<int>(cudaSharedmemCarveoutMaxShared)));
         }
         // Few-token layouts.  The first takes the largest launches: four CTAs per tile, 2 x 2 (two slices of hidden
@@ -1588,7 +1593,7 @@ kvzap_status kvzap_create(kvzap_ctx **out, const kvzap_config *cfg)
             cudaLaunchAttribute attrs[2];
             const int cluster = pair ? 2 * k : k;
             make_launch(&cfg, attrs, dim3(static_cast<unsigned>(n * cluster)), dim3(kScoreThreads), l.smem, nullptr, false, cluster);
-            l.max_clusters = active_clusters(c.device, reinterpret_cast<const void *>(split_kernel(false, pair, !pair)), cfg);
+            l.max_clusters = active_clusters(c.device, reinterpret_cast<const void *>(split_kernel(false, pair, pair ? kNoStep : kStep)), cfg);
             return l.max_clusters >= 0 &&
                    (l.arrive != nullptr || cudaMalloc(&l.arrive, sizeof(uint32_t) * static_cast<size_t>(ctx->sm_count)) == cudaSuccess) &&
                    cudaMemset(l.arrive, 0, sizeof(uint32_t) * static_cast<size_t>(ctx->sm_count)) == cudaSuccess;
@@ -1782,8 +1787,8 @@ kvzap_status kvzap_set_weights_fp8(kvzap_ctx *ctx, int32_t layer, const void *W1
         }
         if (ctx->n_layouts > 0) {
             for (int i = 0; i < kSplitKernels; ++i) {
-                KVZAP_CUDA(ctx, cudaFuncSetAttribute(split_kernel(true, i == 1, i == 2), cudaFuncAttributeMaxDynamicSharedMemorySize, ctx->split_smem_limit));
-                KVZAP_CUDA(ctx, cudaFuncSetAttribute(split_kernel(true, i == 1, i == 2), cudaFuncAttributePreferredSharedMemoryCarveout,
+                KVZAP_CUDA(ctx, cudaFuncSetAttribute(split_kernel(true, i), cudaFuncAttributeMaxDynamicSharedMemorySize, ctx->split_smem_limit));
+                KVZAP_CUDA(ctx, cudaFuncSetAttribute(split_kernel(true, i), cudaFuncAttributePreferredSharedMemoryCarveout,
                                                      static_cast<int>(cudaSharedmemCarveoutMaxShared)));
             }
         }

@@ -30,7 +30,7 @@
 
 namespace kvzap {
 
-// Decode step fused into the scoring launch (kFused; enabled != 0): while the MMAs run, the epilogue warps
+// Decode step fused into the scoring launch (enabled != 0): while the MMAs run, the epilogue warps
 // of a cluster do the cache update of the cluster's own lists -- 128 sequences x H heads of one layer,
 // an equal part per CTA -- exactly as decode_update_kernel does (the token that leaves the window is
 // judged by its buffered score, so nothing here needs the new scores); the cluster's first CTA puts
@@ -49,10 +49,6 @@ struct DecodeFuse {
     float tau;
     int32_t *done;                  // [n_layers * tiles_per_layer][n_split]
     int64_t wait_limit;             // cycles a cluster waits for the step before to be published
-    // 1: directly behind an attention over the cache, which may still be running and reads it.  The stores of the cache update
-    // wait for it, nothing before them does; and the next launch, an attention that runs beside this step, starts once the
-    // lists' present prefix lengths are in c.before.
-    int32_t behind_attention;
 };
 
 struct SplitSmemLayout {
@@ -87,18 +83,24 @@ __host__ inline bool split_smem_fits(int ns, int n_stages, int k_split, int b_ro
 // A CTA ends up owning Ns / k_split hidden units.
 // kFp8: hidden states and W1 are E4M3 bytes (K blocks of 128 codes, tcgen05.mma kind::f8f6f4); the scales
 // x_scale[token] * w1_scale[hidden unit] multiply the summed pre-activation before the bias.
-// kFused: the decode step, a kernel of its own: the scoring of prompts and chunks carries none of its code.
+// kStepKind: none; or the decode step, a kernel of its own, so that the scoring of prompts and chunks carries none of its code;
+// or the step directly behind an attention over the cache, which may still be running and reads it: the stores of the cache
+// update wait for it, nothing before them does, and the next launch, an attention that runs beside this step, starts once the
+// lists' present prefix lengths are in c.before.  That too is a kernel of its own: asked for at run time it cost the other
+// steps 1 to 2 % (2 layers x 4 sequences 12.97 -> 12.70 us, 12 x 2 18.0 -> 17.8).
 // kPair (prompts, not the fused step): two blocks of 128 tokens share every W1 tile.  A work tile is a pair of blocks, the
 // cluster has 2 * k_split CTAs, CTA 2 r + i holds block i's rows of K part r and half of the slice's W1 rows, and its first
 // one issues the MMAs of both (cta_group::2, as in score_kernel); everything behind the accumulators is per block, as without
 // pairs.  A CTA then loads (128 + Ns / 2) rows per K element instead of 128 + Ns, which is what bounds this kernel.
-template <bool kFp8, bool kPair, bool kFused>
+enum SplitStep { kNoStep, kStep, kStepBehindAttention };
+template <bool kFp8, bool kPair, SplitStep kStepKind>
 __global__ void __maxnreg__(128)
 score_split_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_constant__ CUtensorMap tmap_w,
                    const ScoreParams p, const int n_split, const int k_split, const DecodeFuse f)
 {
     constexpr int kElems = kFp8 ? 2 * kBlockK : kBlockK;         // elements per 128-byte K block
     constexpr int kCtas = kPair ? 2 : 1;
+    constexpr bool kFused = kStepKind != kNoStep, kBehind = kStepKind == kStepBehindAttention;
     __shared__ int64_t fuse_dst[kFused ? 256 : 1];       // fused decode step: page row of the evicted token (-1 = dropped)
     __shared__ int64_t fuse_ring[kFused ? 256 : 1];      //                     ring row of the list's current slot (-1 = no list)
     __shared__ int32_t fuse_step;           //                     number of the step this CTA works on (its ticket)
@@ -147,7 +149,7 @@ score_split_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_cons
             fuse_step = atomicAdd(f.ticket + ((layer * p.tiles_per_layer + m_tile) * n_split + nh) * k_split + kh, 1);
         __syncthreads();
     }
-    if (!p.late_trigger && !(kFused && f.behind_attention)) griddep_launch_dependents();
+    if (!p.late_trigger && !kBehind) griddep_launch_dependents();
     const int own_n = ns / k_split;                      // accumulator columns this CTA finishes
     const int own_c0 = kh * own_n;                       // the first of them
     const int j_first = nh * ns + own_c0;                // = first hidden unit of this CTA
@@ -211,7 +213,7 @@ score_split_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_cons
     // ahead in the stream has completed (every thread waits: the loads below are issued by several warps)
     if (p.wait_before_load) griddep_wait();
     if (p.late_trigger) griddep_launch_dependents();     // whatever starts now finds all work ahead of this launch complete
-    if (kFused && f.behind_attention && warp >= 2) {
+    if (kBehind && warp >= 2) {
         // the present length of this CTA's lists (those of the cache update below), in memory before the next launch starts
         const CacheView &c = f.c;
         const int etid = threadIdx.x - 64;
@@ -378,7 +380,7 @@ score_split_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_cons
             named_barrier_sync(1, 256);
             bool counted = false;                            // every thread, once, before its first store to the cache
             auto count = [&]() {
-                if (f.behind_attention) griddep_wait();
+                if (kBehind) griddep_wait();
                 if (li >= 0) {
                     if (page >= 0) {
                         if (idx % c.page_tokens == 0) c.page_table[li * c.max_pages + idx / c.page_tokens] = page;
