@@ -41,6 +41,9 @@ constexpr int kMaskRing = 4;
 
 }  // namespace kvzap
 
+// Arrival counters of the few-token kernel: one per tile, then kFewWarps per tile for steps of few tokens.
+namespace kvzap { constexpr size_t kSplitArrive = 1 + kFewWarps; }
+
 struct kvzap_ctx {
     kvzap_config cfg;
     int sm_count = 0;
@@ -64,7 +67,7 @@ struct kvzap_ctx {
         CUtensorMap tmap_w;
         CUtensorMap tmap_w8;             // the 8-bit copy of the weights, same slices (set by kvzap_set_weights_fp8)
         bool ok8 = false;
-        uint32_t *arrive = nullptr;      // [sm_count] slices of a tile that have arrived, zero between launches
+        uint32_t *arrive = nullptr;      // [kSplitArrive * sm_count] slices of a tile that have arrived, zero between launches
     };
     static constexpr int kMaxLayouts = 4, kMaxPairLayouts = 6;
     SplitLayout layouts[kMaxLayouts];
@@ -113,7 +116,7 @@ struct kvzap_ctx {
     int32_t *status_host = nullptr;  // pinned
     int64_t launches = 0, beside = 0;
     // tensor maps of recently used hidden-state buffers (encoding one costs about as much as a launch)
-    struct TmapEntry { const void *base; int64_t rows; int32_t slabs; CUtensorMap map; };
+    struct TmapEntry { const void *base; int64_t rows; int32_t slabs, box; CUtensorMap map; };
     std::vector<TmapEntry> tmap_cache;
     size_t tmap_next = 0;
     // optional per-kernel timing (kvzap_set_profiling)
@@ -487,16 +490,16 @@ static kvzap_status check_common(kvzap_ctx *ctx, int64_t n_tokens, int32_t n_seq
 
 static bool aligned16(const void *p) { return (reinterpret_cast<uintptr_t>(p) & 15u) == 0; }
 
-// Tensor map of hidden states [slabs][rows][d_model] (box 128 x 64), from a small cache keyed by the
+// Tensor map of hidden states [slabs][rows][d_model] (box: box rows x 64), from a small cache keyed by the
 // buffer's address and shape.
-static kvzap_status hidden_tmap(kvzap_ctx *ctx, CUtensorMap *out, const void *base, int64_t rows, int32_t slabs)
+static kvzap_status hidden_tmap(kvzap_ctx *ctx, CUtensorMap *out, const void *base, int64_t rows, int32_t slabs, int32_t box = kTileM)
 {
     for (const auto &e : ctx->tmap_cache)
-        if (e.base == base && e.rows == rows && e.slabs == slabs) { *out = e.map; return KVZAP_OK; }
+        if (e.base == base && e.rows == rows && e.slabs == slabs && e.box == box) { *out = e.map; return KVZAP_OK; }
     kvzap_ctx::TmapEntry e;
-    e.base = base; e.rows = rows; e.slabs = slabs;
+    e.base = base; e.rows = rows; e.slabs = slabs; e.box = box;
     kvzap_status st = make_tmap(ctx, &e.map, base, static_cast<uint64_t>(rows), static_cast<uint64_t>(ctx->cfg.d_model),
-                                kTileM, static_cast<uint64_t>(slabs));
+                                static_cast<uint32_t>(box), static_cast<uint64_t>(slabs));
     if (st != KVZAP_OK) return st;
     constexpr size_t kEntries = 128;
     if (ctx->tmap_cache.size() < kEntries) ctx->tmap_cache.push_back(e);
@@ -637,18 +640,24 @@ static const kvzap_ctx::SplitLayout *prompt_layout(const kvzap_ctx *ctx, int64_t
     return l ? l : i >= 0 ? &ctx->layouts[i] : nullptr;
 }
 
-static decltype(&score_split_kernel<false, false, kNoStep>) split_kernel(bool fp8, bool pair, SplitStep step)
+using SplitKernel = decltype(&score_split_kernel<false, false, kNoStep, false>);
+template <bool kFp8>
+static SplitKernel split_kernel_of(bool pair, SplitStep step, bool few)
 {
-    if (pair) return fp8 ? score_split_kernel<true, true, kNoStep> : score_split_kernel<false, true, kNoStep>;
-    if (step == kStep) return fp8 ? score_split_kernel<true, false, kStep> : score_split_kernel<false, false, kStep>;
+    if (pair) return score_split_kernel<kFp8, true, kNoStep, false>;
+    if (step == kStep) return few ? score_split_kernel<kFp8, false, kStep, true> : score_split_kernel<kFp8, false, kStep, false>;
     if (step == kStepBehindAttention)
-        return fp8 ? score_split_kernel<true, false, kStepBehindAttention> : score_split_kernel<false, false, kStepBehindAttention>;
-    return fp8 ? score_split_kernel<true, false, kNoStep> : score_split_kernel<false, false, kNoStep>;
+        return few ? score_split_kernel<kFp8, false, kStepBehindAttention, true> : score_split_kernel<kFp8, false, kStepBehindAttention, false>;
+    return score_split_kernel<kFp8, false, kNoStep, false>;
 }
-constexpr int kSplitKernels = 4;        // per input type, numbered: by step without pairs, then pairs
-static decltype(&score_split_kernel<false, false, kNoStep>) split_kernel(bool fp8, int i)
+static SplitKernel split_kernel(bool fp8, bool pair, SplitStep step, bool few = false)
 {
-    return split_kernel(fp8, i == 3, i < 3 ? static_cast<SplitStep>(i) : kNoStep);
+    return fp8 ? split_kernel_of<true>(pair, step, few) : split_kernel_of<false>(pair, step, few);
+}
+constexpr int kSplitKernels = 6;        // per input type, numbered: by step without pairs, pairs, the two steps of few tokens
+static SplitKernel split_kernel(bool fp8, int i)
+{
+    return i < 4 ? split_kernel(fp8, i == 3, i < 3 ? static_cast<SplitStep>(i) : kNoStep) : split_kernel(fp8, false, i == 4 ? kStep : kStepBehindAttention, true);
 }
 
 // Enqueues the few-token kernel over p.n_tiles tiles (of two blocks for a layout with CTA pairs).
@@ -656,11 +665,13 @@ static cudaError_t launch_split(const kvzap_ctx::SplitLayout &l, int k, bool pai
                                 const DecodeFuse &f, bool early, cudaStream_t stream, bool behind_attention = false)
 {
     const int ctas = pair ? 2 : 1;
+    const bool few = p.x_rows > 0;
+    const uint32_t smem = few ? split_smem_layout(p.chunk_n, p.n_stages, k, p.chunk_n, p.x_rows).total + 1024 : l.smem;
     cudaLaunchConfig_t cfg;
     cudaLaunchAttribute attrs[2];
-    make_launch(&cfg, attrs, dim3(static_cast<unsigned>(p.n_tiles * ctas * l.n * k)), dim3(kScoreThreads), l.smem, stream, early, ctas * k);
+    make_launch(&cfg, attrs, dim3(static_cast<unsigned>(p.n_tiles * ctas * l.n * k)), dim3(kScoreThreads), smem, stream, early, ctas * k);
     const CUtensorMap &tmap_w = fp8 ? l.tmap_w8 : l.tmap_w;
-    return cudaLaunchKernelEx(&cfg, split_kernel(fp8, pair, behind_attention ? kStepBehindAttention : f.enabled != 0 ? kStep : kNoStep), tmap_x, tmap_w, p, l.n, k, f);
+    return cudaLaunchKernelEx(&cfg, split_kernel(fp8, pair, behind_attention ? kStepBehindAttention : f.enabled != 0 ? kStep : kNoStep, few), tmap_x, tmap_w, p, l.n, k, f);
 }
 
 // Blocks of a prompt that whole waves of CTA pairs leave over and that the few-token kernel takes instead, in a launch of its
@@ -758,13 +769,27 @@ static kvzap_status launch_score(kvzap_ctx *ctx, int32_t layer, int32_t n_layers
     if (layout_i >= 0 || slices_only || pairs != nullptr) {
         const kvzap_ctx::SplitLayout &layout = pairs ? *pairs : ctx->layouts[slices_only ? 0 : layout_i];
         const int split_n = layout.n, split_k = slices_only && !pairs ? 1 : layout.k;
-        CUtensorMap tmap_x;
-        kvzap_status st = fp8 ? make_tmap8(ctx, &tmap_x, hidden, static_cast<uint64_t>(n_tokens), static_cast<uint64_t>(c.d_model),
-                                           kTileM, static_cast<uint64_t>(n_layers), false)
-                              : hidden_tmap(ctx, &tmap_x, hidden, n_tokens, n_layers);
-        if (st != KVZAP_OK) return st;
+        const bool fuse_ok = fuse != nullptr && !ctx->profiling && !slices_only;
         ScoreParams p;
         memset(&p, 0, sizeof p);
+        p.n_stages = layout.stages;
+        if (fuse_ok && n_tokens <= kFewTokens) {
+            // a step of few tokens (kFew): stages of few rows of X, as many as there are K blocks or room for
+            const int ns = c.hidden / split_n, x_rows = static_cast<int>((n_tokens + 7) / 8 * 8);
+            int stages = c.d_model / (fp8 ? 2 * kBlockK : kBlockK) / split_k;
+            if (stages > kMaxStages) stages = kMaxStages;
+            while (stages > 1 && !split_smem_fits(ns, stages, split_k, ns, ctx->split_smem_limit - 1024, x_rows)) --stages;
+            if (split_smem_fits(ns, stages, split_k, ns, ctx->split_smem_limit - 1024, x_rows)) {
+                p.x_rows = x_rows;
+                p.n_stages = stages;
+            }
+        }
+        const int32_t box = p.x_rows > 0 ? p.x_rows : kTileM;
+        CUtensorMap tmap_x;
+        kvzap_status st = fp8 ? make_tmap8(ctx, &tmap_x, hidden, static_cast<uint64_t>(n_tokens), static_cast<uint64_t>(c.d_model),
+                                           static_cast<uint32_t>(box), static_cast<uint64_t>(n_layers), false)
+                              : hidden_tmap(ctx, &tmap_x, hidden, n_tokens, n_layers, box);
+        if (st != KVZAP_OK) return st;
         p.x_scale = x_scale;
         p.w1_scale = ctx->w1_scale_all;
         p.n_tokens = n_tokens;
@@ -777,7 +802,6 @@ static kvzap_status launch_score(kvzap_ctx *ctx, int32_t layer, int32_t n_layers
         p.d_model = c.d_model;
         p.group_w = p.chunk_n = c.hidden / split_n;
         p.n_groups = p.n_chunks = 1;
-        p.n_stages = layout.stages;
         p.acc_bufs = 1;
         p.tmem_cols = layout.tmem_cols;
         p.n_hidden = c.hidden;
@@ -795,7 +819,7 @@ static kvzap_status launch_score(kvzap_ctx *ctx, int32_t layer, int32_t n_layers
         p.tau = tau;
         p.status = ctx->status_dev;
         p.split_part = ctx->split_part;
-        p.split_arrive = layout.arrive;
+        p.split_arrive = layout.arrive + (p.x_rows > 0 ? ctx->sm_count : 0);
         // Early start (consecutive decode steps): this kernel reads only hidden states and weights; the one
         // thing it may not do is write a scores buffer that the kernels of the previous call still read.
         const size_t sbytes = scores ? sizeof(float) * static_cast<size_t>(n_layers) * n_tokens * c.n_kv_heads : 0;
@@ -809,7 +833,6 @@ static kvzap_status launch_score(kvzap_ctx *ctx, int32_t layer, int32_t n_layers
         const int n_ctas = split_n * split_k;
         DecodeFuse f;
         memset(&f, 0, sizeof f);
-        const bool fuse_ok = fuse != nullptr && !ctx->profiling && !slices_only;
         if (fuse_ok) {
             f = *fuse;
             f.enabled = 1;
@@ -1595,8 +1618,8 @@ kvzap_status kvzap_create(kvzap_ctx **out, const kvzap_config *cfg)
             make_launch(&cfg, attrs, dim3(static_cast<unsigned>(n * cluster)), dim3(kScoreThreads), l.smem, nullptr, false, cluster);
             l.max_clusters = active_clusters(c.device, reinterpret_cast<const void *>(split_kernel(false, pair, pair ? kNoStep : kStep)), cfg);
             return l.max_clusters >= 0 &&
-                   (l.arrive != nullptr || cudaMalloc(&l.arrive, sizeof(uint32_t) * static_cast<size_t>(ctx->sm_count)) == cudaSuccess) &&
-                   cudaMemset(l.arrive, 0, sizeof(uint32_t) * static_cast<size_t>(ctx->sm_count)) == cudaSuccess;
+                   (l.arrive != nullptr || cudaMalloc(&l.arrive, sizeof(uint32_t) * kSplitArrive * static_cast<size_t>(ctx->sm_count)) == cudaSuccess) &&
+                   cudaMemset(l.arrive, 0, sizeof(uint32_t) * kSplitArrive * static_cast<size_t>(ctx->sm_count)) == cudaSuccess;
         };
         for (const auto &sh : shapes) {
             const int n = sh[0], k = sh[1], i = ctx->n_layouts;
@@ -2089,9 +2112,9 @@ kvzap_status kvzap_poll_status(kvzap_ctx *ctx, void *stream_)
     // a scoring kernel that gave up may have left its work-tile counter in an unknown state
     cudaMemsetAsync(ctx->tile_counters, 0, sizeof(int32_t) * kMaskRing, stream);
     for (int i = 0; i < ctx->n_layouts; ++i)
-        cudaMemsetAsync(ctx->layouts[i].arrive, 0, sizeof(uint32_t) * static_cast<size_t>(ctx->sm_count), stream);
+        cudaMemsetAsync(ctx->layouts[i].arrive, 0, sizeof(uint32_t) * kSplitArrive * static_cast<size_t>(ctx->sm_count), stream);
     for (int i = 0; i < ctx->n_pair_layouts; ++i)
-        cudaMemsetAsync(ctx->pair_layouts[i].arrive, 0, sizeof(uint32_t) * static_cast<size_t>(ctx->sm_count), stream);
+        cudaMemsetAsync(ctx->pair_layouts[i].arrive, 0, sizeof(uint32_t) * kSplitArrive * static_cast<size_t>(ctx->sm_count), stream);
     if (v == KVZAP_ERR_TIMEOUT) {
         reset_step_counters(ctx, stream);
         // a one-launch pruning call that gave up may have left its list-length sums and arrival count behind

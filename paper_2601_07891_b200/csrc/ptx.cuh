@@ -317,6 +317,14 @@ __device__ __forceinline__ bool arrive_last(uint32_t *counter, uint32_t n)
     return atomicInc(counter, n - 1u) == n - 1u;
 }
 
+// The same as release and acquire: what the threads before it in its warp or CTA have stored is seen by whoever is last.
+__device__ __forceinline__ bool arrive_last_acq_rel(uint32_t *counter, uint32_t n)
+{
+    uint32_t before;
+    asm volatile("atom.acq_rel.gpu.global.inc.u32 %0, [%1], %2;" : "=r"(before) : "l"(counter), "r"(n - 1u) : "memory");
+    return before == n - 1u;
+}
+
 // ---------------------------------------------------------------- programmatic dependent launch
 // A kernel launched with the programmatic-stream-serialization attribute may start once every CTA
 // of the kernel before it in the stream has executed griddep_launch_dependents() (or exited);
@@ -358,6 +366,16 @@ __device__ __forceinline__ void cluster_sync_all()
 {
     __syncwarp();
     asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");
+}
+// Its two halves; the whole warp is at each of them together.
+__device__ __forceinline__ void cluster_arrive()
+{
+    asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
+}
+__device__ __forceinline__ void cluster_wait()
+{
+    __syncwarp();
+    asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
 }
 // Tiled loads issued by either CTA of a pair; the mbarrier (cluster address) may be the other CTA's.
 __device__ __forceinline__ void tma_load_3d_pair(uint32_t smem_dst, const CUtensorMap *map, uint32_t bar_cluster,

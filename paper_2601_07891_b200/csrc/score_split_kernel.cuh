@@ -52,30 +52,44 @@ struct DecodeFuse {
 };
 
 struct SplitSmemLayout {
-    uint32_t stage_bytes, stages_end, w2s, b1s, w1s, part, xpart, bars, total;
+    uint32_t a_bytes, stage_bytes, stages_end, w2s, b1s, w1s, part, recv, xpart, bars, total;
 };
 // The parts received from the other CTAs of the cluster ([k_split - 1][own / 4][128 rows] float4) lie over the
 // stages, idle by then, and behind them the sums that the cluster's CTAs leave with its first one ([k_split][128][8]).
-// b_rows: rows of W1 that a CTA stages, ns or, for CTA pairs, half of them.
-__host__ __device__ inline SplitSmemLayout split_smem_layout(int ns, int n_stages, int k_split, int b_rows)
+// b_rows: rows of W1 that a CTA stages, ns or, for CTA pairs, half of them.  x_rows (kFew; else 0): a stage holds only so many
+// rows of X, and what the CTAs send one another ([k_split][x_rows][own + 4] and [k_split][x_rows][8]) has a place of its own.
+// The MMAs read 128 rows all the same: those behind the staged ones are whatever lies there, within the block (see total), and
+// so are their results.
+__host__ __device__ inline SplitSmemLayout split_smem_layout(int ns, int n_stages, int k_split, int b_rows, int x_rows = 0)
 {
     SplitSmemLayout L;
-    L.stage_bytes = kATileBytes + static_cast<uint32_t>(b_rows) * kBlockK * 2;
+    const uint32_t own = static_cast<uint32_t>(ns / k_split), k = static_cast<uint32_t>(k_split);
+    L.a_bytes = x_rows > 0 ? static_cast<uint32_t>(x_rows) * 128u : kATileBytes;
+    L.stage_bytes = L.a_bytes + static_cast<uint32_t>(b_rows) * kBlockK * 2;
     L.stages_end = L.stage_bytes * n_stages;
     L.w2s = L.stages_end;
     L.b1s = L.w2s + static_cast<uint32_t>(ns) * kMaxHeads * 4;
     L.w1s = L.b1s + static_cast<uint32_t>(ns) * 4;            // first-layer row scales (8-bit inputs)
     L.part = L.w1s + static_cast<uint32_t>(ns) * 4;
-    L.xpart = static_cast<uint32_t>(ns / k_split * (k_split - 1)) * kTileM * 4;
-    L.bars = L.part + kTileM * kMaxHeads * 4;
+    if (x_rows > 0) {
+        L.recv = L.part;
+        L.xpart = L.recv + k * static_cast<uint32_t>(x_rows) * (own + 4) * 4;
+        L.bars = L.xpart + k * static_cast<uint32_t>(x_rows) * kMaxHeads * 4;
+    } else {
+        L.recv = 0;
+        L.xpart = own * (k - 1) * kTileM * 4;
+        L.bars = L.part + kTileM * kMaxHeads * 4;
+    }
     L.total = L.bars + 256;
+    const uint32_t last_read = L.stages_end - L.stage_bytes + kATileBytes;
+    if (L.total < last_read) L.total = last_read;
     return L;
 }
-__host__ inline bool split_smem_fits(int ns, int n_stages, int k_split, int b_rows, int budget)
+__host__ inline bool split_smem_fits(int ns, int n_stages, int k_split, int b_rows, int budget, int x_rows = 0)
 {
-    const SplitSmemLayout L = split_smem_layout(ns, n_stages, k_split, b_rows);
+    const SplitSmemLayout L = split_smem_layout(ns, n_stages, k_split, b_rows, x_rows);
     return static_cast<int>(L.total) <= budget &&
-           L.xpart + static_cast<uint32_t>(k_split) * kTileM * kMaxHeads * 4 <= L.stages_end;
+           (x_rows > 0 || L.xpart + static_cast<uint32_t>(k_split) * kTileM * kMaxHeads * 4 <= L.stages_end);
 }
 
 // p.group_w = p.chunk_n = Ns (the MMA's N); p.n_chunks = 1; p.acc_bufs = 1; p.n_tiles = 128-token tiles
@@ -92,8 +106,18 @@ __host__ inline bool split_smem_fits(int ns, int n_stages, int k_split, int b_ro
 // cluster has 2 * k_split CTAs, CTA 2 r + i holds block i's rows of K part r and half of the slice's W1 rows, and its first
 // one issues the MMAs of both (cta_group::2, as in score_kernel); everything behind the accumulators is per block, as without
 // pairs.  A CTA then loads (128 + Ns / 2) rows per K element instead of 128 + Ns, which is what bounds this kernel.
+// kFew (steps of up to kFewTokens tokens a layer): what bounds such a step is a chain of round trips and barriers, and code that is
+// fetched to be run once.  A stage holds x_rows rows of X instead of 128, so that in the layouts of few layers all of a CTA's loads
+// are out at once; the receive buffers lie beside the stages (no barrier before the exchange); GELU and second layer are shared out
+// over all epilogue warps, a pair of hidden units of one token per thread, where one warp had 16 units of all tokens; and
+// the last slice to arrive is found per warp, which then needs one round trip for partial sums, bias and ring slots.
+// 4096 -> 512 -> 8, one layer a call, calls in a row, us: 1 sequence 11.7 -> 7.7, 8 12.4 -> 8.4, 16 12.7 -> 8.6, 32 13.2 -> 9.3; 8-bit, 8
+// sequences 12.6 -> 8.5; 36 layers a call, 8 sequences 33.3 -> 29.3, 32 38.2 -> 35.3.  32 tokens are one lane quarter of the accumulator; more
+// would need the exchange's other quarters, and their X fills the stages again.
 enum SplitStep { kNoStep, kStep, kStepBehindAttention };
-template <bool kFp8, bool kPair, SplitStep kStepKind>
+constexpr int kFewTokens = 32;
+constexpr int kFewWarps = 8;            // arrival counters of a tile: one per four tokens
+template <bool kFp8, bool kPair, SplitStep kStepKind, bool kFew>
 __global__ void __maxnreg__(128)
 score_split_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_constant__ CUtensorMap tmap_w,
                    const ScoreParams p, const int n_split, const int k_split, const DecodeFuse f)
@@ -111,7 +135,8 @@ score_split_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_cons
     const uint32_t smem_base = raw_addr + pad;
     const int ns = p.chunk_n;
     const int n_ctas = n_split * k_split;
-    const SplitSmemLayout L = split_smem_layout(ns, p.n_stages, k_split, ns / kCtas);
+    static_assert(!kFew || (kFused && !kPair), "few tokens: decode steps only");
+    const SplitSmemLayout L = split_smem_layout(ns, p.n_stages, k_split, ns / kCtas, kFew ? p.x_rows : 0);
 
     ulonglong2 *w2p = reinterpret_cast<ulonglong2 *>(smem + L.w2s);
     float *w2f = reinterpret_cast<float *>(smem + L.w2s);
@@ -119,6 +144,7 @@ score_split_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_cons
     float *w1s = reinterpret_cast<float *>(smem + L.w1s);
     float *part = reinterpret_cast<float *>(smem + L.part);
     float *xpart = reinterpret_cast<float *>(smem + L.xpart);
+    float *recv_few = reinterpret_cast<float *>(smem + L.recv);           // kFew: [k_split][x_rows][own + 4]
     const uint32_t bars = smem_base + L.bars;
     const uint32_t bar_full = bars;                      // [kMaxStages] TMA -> MMA
     const uint32_t bar_empty = bars + 8 * kMaxStages;    // [kMaxStages] MMA -> TMA
@@ -150,6 +176,7 @@ score_split_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_cons
         __syncthreads();
     }
     if (!p.late_trigger && !kBehind) griddep_launch_dependents();
+    if constexpr (kFew) cluster_arrive();                // waited for before the first store to another CTA: it runs by then
     const int own_n = ns / k_split;                      // accumulator columns this CTA finishes
     const int own_c0 = kh * own_n;                       // the first of them
     const int j_first = nh * ns + own_c0;                // = first hidden unit of this CTA
@@ -184,10 +211,10 @@ score_split_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_cons
     auto load_w = [&](uint32_t st, uint32_t sa, int kb) {
         if constexpr (kPair) {
             if (half == 0) mbar_arrive_expect_tx(bar_full + 8 * st, 2u * L.stage_bytes);
-            tma_load_3d_pair(sa + kATileBytes, &tmap_w, full0 + 8 * st, 0, w_row, kb_first + kb, pol_w);
+            tma_load_3d_pair(sa + L.a_bytes, &tmap_w, full0 + 8 * st, 0, w_row, kb_first + kb, pol_w);
         } else {
             mbar_arrive_expect_tx(bar_full + 8 * st, L.stage_bytes);
-            tma_load_3d(sa + kATileBytes, &tmap_w, bar_full + 8 * st, 0, w_row, kb_first + kb, pol_w);
+            tma_load_3d(sa + L.a_bytes, &tmap_w, bar_full + 8 * st, 0, w_row, kb_first + kb, pol_w);
         }
     };
     auto load_x = [&](uint32_t st, uint32_t sa, int kb) {
@@ -284,7 +311,7 @@ score_split_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_cons
             }
             tc_fence_after_sync();
             if (elected) {
-                issue_k_block<kPair, 1, kFp8>(tmem_base, a_lo, a_lo + (kATileBytes >> 4), desc_hi, 0, 0, idesc, kb == 0);
+                issue_k_block<kPair, 1, kFp8>(tmem_base, a_lo, a_lo + (L.a_bytes >> 4), desc_hi, 0, 0, idesc, kb == 0);
                 if constexpr (kPair) umma_commit_pair(bar_empty + 8 * st, both);
                 else umma_commit(bar_empty + 8 * st);
             }
@@ -313,22 +340,14 @@ score_split_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_cons
     const int row = q * 32 + lane;
     const uint32_t t_row = tmem_base + (static_cast<uint32_t>(q * 32) << 16);
     bool ok = true;
-    if (epi) {
-        // this CTA's slice of b1 and W2 (pairs of hidden units, see mlp_columns)
-        const int etid = threadIdx.x - 64;
-        const float *w2g = p.w2t + (static_cast<int64_t>(layer) * p.n_hidden + j_first) * kMaxHeads;
-        const float *b1g = p.b1 + static_cast<int64_t>(layer) * p.n_hidden + j_first;
-        for (int i = etid; i < own_n * kMaxHeads; i += 256) {
-            const int j = i >> 3, h = i & 7;
-            w2f[(((j >> 1) * kMaxHeads + h) << 1) + (j & 1)] = __ldg(w2g + i);
-        }
-        for (int i = etid; i < own_n; i += 256) b1s[i] = __ldg(b1g + i);
-        if constexpr (kFp8)
-            for (int i = etid; i < own_n; i += 256) w1s[i] = __ldg(p.w1_scale + static_cast<int64_t>(layer) * p.n_hidden + j_first + i);
-        named_barrier_sync(1, 256);
+    // ---- the cache update of this CTA's lists: what moves where, then the rows
+    int64_t li = -1;
+    int32_t n_list = 0, prefix = 0, page = -1;
+    int rows_per_cta = 0;
+    auto update_plan = [&]() {
         if constexpr (kFused) {
-            // ---- the cache update of this CTA's lists, under the MMAs
             const CacheView &c = f.c;
+            const int etid = threadIdx.x - 64;
             const int cid = layer * p.tiles_per_layer + m_tile;
             if (etid < n_split) {
                 const long long t0 = clock64();
@@ -341,15 +360,13 @@ score_split_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_cons
             const bool go = *abort_flag == 0;
             const int64_t seqs_left = static_cast<int64_t>(c.n_seqs) - static_cast<int64_t>(m_tile) * kTileM;
             const int tile_seqs = seqs_left < kTileM ? static_cast<int>(seqs_left) : kTileM;
-            const int rows_per_cta = (tile_seqs + n_ctas - 1) / n_ctas;
+            rows_per_cta = (tile_seqs + n_ctas - 1) / n_ctas;
             // one thread per list: which row leaves, where it goes, which slot the new token takes
-            int64_t li;
-            int32_t n = 0, idx = 0, page = -1;
             {
                 const int b_loc = pos * rows_per_cta + etid / kMaxHeads, h = etid % kMaxHeads;
                 const int64_t b = static_cast<int64_t>(m_tile) * kTileM + b_loc;
                 int64_t dst = -1, ring = -1;
-                li = -1;
+                int32_t n = 0, idx = 0;
                 if (go && etid < rows_per_cta * kMaxHeads && b_loc < tile_seqs && h < c.n_heads && c.active[b] != 0) {
                     li = (b * c.n_layers + layer) * c.n_heads + h;
                     // two round trips to memory instead of four: both counters first, then the score of
@@ -374,19 +391,27 @@ score_split_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_cons
                         if (page >= 0) dst = static_cast<int64_t>(page) * c.page_tokens + in_page;
                     }
                 }
+                n_list = n;
+                prefix = idx;
                 fuse_dst[etid] = dst;
                 fuse_ring[etid] = ring;
             }
             named_barrier_sync(1, 256);
+        }
+    };
+    auto update_rows = [&]() {
+        if constexpr (kFused) {
+            const CacheView &c = f.c;
+            const int etid = threadIdx.x - 64;
             bool counted = false;                            // every thread, once, before its first store to the cache
             auto count = [&]() {
                 if (kBehind) griddep_wait();
                 if (li >= 0) {
                     if (page >= 0) {
-                        if (idx % c.page_tokens == 0) c.page_table[li * c.max_pages + idx / c.page_tokens] = page;
-                        c.prefix_len[li] = idx + 1;
+                        if (prefix % c.page_tokens == 0) c.page_table[li * c.max_pages + prefix / c.page_tokens] = page;
+                        c.prefix_len[li] = prefix + 1;
                     }
-                    c.n_tokens[li] = n + 1;
+                    c.n_tokens[li] = n_list + 1;
                 }
                 counted = true;
             };
@@ -439,107 +464,200 @@ score_split_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_cons
             }
             if (!counted) count();
         }
+    };
+    if (epi) {
+        // this CTA's slice of b1 and W2 (pairs of hidden units, see mlp_columns)
+        const int etid = threadIdx.x - 64;
+        const float *w2g = p.w2t + (static_cast<int64_t>(layer) * p.n_hidden + j_first) * kMaxHeads;
+        const float *b1g = p.b1 + static_cast<int64_t>(layer) * p.n_hidden + j_first;
+        for (int i = etid; i < own_n * kMaxHeads; i += 256) {
+            const int j = i >> 3, h = i & 7;
+            w2f[kFew ? i : (((j >> 1) * kMaxHeads + h) << 1) + (j & 1)] = __ldg(w2g + i);
+        }
+        for (int i = etid; i < own_n; i += 256) b1s[i] = __ldg(b1g + i);
+        if constexpr (kFp8)
+            for (int i = etid; i < own_n; i += 256) w1s[i] = __ldg(p.w1_scale + static_cast<int64_t>(layer) * p.n_hidden + j_first + i);
+        named_barrier_sync(1, 256);
+        // under the MMAs; the rows of a step behind an attention, for which they wait, when all else of this CTA is done (kFew)
+        update_plan();
+        if constexpr (!(kFew && kBehind)) update_rows();
         ok = mbar_wait(bar_tfull, 0, abort_flag);
         tc_fence_after_sync();
     }
     const int n16 = own_n >> 4;             // 16-column chunks this CTA owns (and as many it sends to each of the others)
-    // lanes of a warp whose 32 tokens all lie past the input take no part in the exchange and the second layer
-    const bool rows_live = ok && static_cast<int64_t>(row0) + q * 32 < p.n_tokens;
-    float4 *recv = reinterpret_cast<float4 *>(smem);          // [k_split - 1][own_n / 4][128 rows] float4, over the idle stages
-    if (k_split > 1) {
-        // every CTA's MMAs are complete once all have passed this barrier: the stages may be overwritten
-        tc_fence_before_sync();
-        cluster_sync_all();
-        if (epi && rows_live) {
-            for (int i = hsel; i < (k_split - 1) * n16; i += 2) {
+    if constexpr (kFew) {
+        // all tokens lie in the first lane quarter: its two warps send every CTA of the cluster, this one too, its columns
+        const int x_rows = p.x_rows, pitch = own_n + 4;
+        cluster_wait();
+        if (epi && q == 0 && ok) {
+            for (int i = hsel; i < k_split * n16; i += 2) {
                 const uint32_t c = static_cast<uint32_t>(i % n16);
-                const uint32_t to = (rank + 1u + static_cast<uint32_t>(i / n16)) % static_cast<uint32_t>(k_split);
-                const uint32_t slot = rank < to ? rank : rank - 1u;         // the receiver's parts in rank order, itself left out
-                const uint32_t dst0 = map_to_cta(smem_base, to * kCtas + half) + (slot * (static_cast<uint32_t>(own_n) >> 2) + c * 4) * kTileM * 16;
+                const uint32_t to = (rank + static_cast<uint32_t>(i / n16)) % static_cast<uint32_t>(k_split);
                 uint32_t r[16];
                 tmem_ld_x16(t_row + to * own_n + c * 16, r);
                 tmem_wait_ld();
                 reg_fence16(r);
+                const uint32_t dst = map_to_cta(smem_base + L.recv + ((rank * x_rows + lane) * pitch + c * 16) * 4, to);
+                if (lane < x_rows) {
 #pragma unroll
-                for (int j = 0; j < 4; ++j)
-                    st_shared_cluster_v4(dst0 + (static_cast<uint32_t>(j) * kTileM + row) * 16,
-                                         __uint_as_float(r[4 * j]), __uint_as_float(r[4 * j + 1]),
-                                         __uint_as_float(r[4 * j + 2]), __uint_as_float(r[4 * j + 3]));
-            }
-        }
-        cluster_sync_all();                                     // the others' parts have arrived
-    }
-    // adds what the other CTAs of the cluster sent for 16-column chunk c of this CTA's columns
-    auto add_received = [&](uint32_t (&r)[16], int c) {
-        for (int part_i = 0; part_i < k_split - 1; ++part_i) {
-#pragma unroll
-            for (int i = 0; i < 4; ++i) {
-                const float4 o = recv[(part_i * (own_n >> 2) + c * 4 + i) * kTileM + row];
-                r[4 * i] = __float_as_uint(__uint_as_float(r[4 * i]) + o.x);
-                r[4 * i + 1] = __float_as_uint(__uint_as_float(r[4 * i + 1]) + o.y);
-                r[4 * i + 2] = __float_as_uint(__uint_as_float(r[4 * i + 2]) + o.z);
-                r[4 * i + 3] = __float_as_uint(__uint_as_float(r[4 * i + 3]) + o.w);
-            }
-        }
-    };
-    if (epi) {
-        uint64_t acc[kMaxHeads];
-#pragma unroll
-        for (int h = 0; h < kMaxHeads; ++h) acc[h] = 0ull;
-        if (rows_live) {
-            // the first warp of a lane quarter takes the 16-column chunks 0, 2, 4, ..., the second the odd ones
-            uint32_t ra[16], rb[16];
-            uint64_t sx2 = 0ull;                                   // 8-bit inputs: this row's token scale, twice
-            if constexpr (kFp8) {
-                float sx = 1.0f;
-                if (p.x_scale != nullptr && row0 + row < p.n_tokens)
-                    sx = __ldg(p.x_scale + static_cast<int64_t>(l_rel) * p.n_tokens + row0 + row);
-                sx2 = f2_pack(sx, sx);
-            }
-            int c = hsel;
-            if (c < n16) tmem_ld_x16(t_row + own_c0 + c * 16, ra);
-            while (c < n16) {
-                tmem_wait_ld();
-                reg_fence16(ra);
-                if (c + 2 < n16) tmem_ld_x16(t_row + own_c0 + (c + 2) * 16, rb);
-                add_received(ra, c);
-                if constexpr (kFp8) mlp_columns_scaled<16>(ra, c * 16, b1s, w1s, sx2, w2p, acc);
-                else mlp_columns<16>(ra, c * 16, b1s, w2p, acc);
-                c += 2;
-                if (c < n16) {
-                    tmem_wait_ld();
-                    reg_fence16(rb);
-                    if (c + 2 < n16) tmem_ld_x16(t_row + own_c0 + (c + 2) * 16, ra);
-                    add_received(rb, c);
-                    if constexpr (kFp8) mlp_columns_scaled<16>(rb, c * 16, b1s, w1s, sx2, w2p, acc);
-                    else mlp_columns<16>(rb, c * 16, b1s, w2p, acc);
-                    c += 2;
+                    for (int j = 0; j < 4; ++j)
+                        st_shared_cluster_v4(dst + 16 * j, __uint_as_float(r[4 * j]), __uint_as_float(r[4 * j + 1]),
+                                             __uint_as_float(r[4 * j + 2]), __uint_as_float(r[4 * j + 3]));
                 }
             }
         }
-        float s[kMaxHeads];
+        tc_fence_before_sync();
+        cluster_sync_all();                                     // every part has arrived
+        const int token = (warp - 2) * 4 + (lane >> 3), pair = lane & 7;
+        if (epi && (warp - 2) * 4 < x_rows) {
+            float acc[kMaxHeads];
 #pragma unroll
-        for (int h = 0; h < kMaxHeads; ++h) {
-            float lo, hi;
-            f2_unpack(acc[h], lo, hi);
-            s[h] = lo + hi;
+            for (int h = 0; h < kMaxHeads; ++h) acc[h] = 0.0f;
+            float sx = 1.0f;
+            if constexpr (kFp8)
+                if (p.x_scale != nullptr && token < p.n_tokens) sx = __ldg(p.x_scale + static_cast<int64_t>(l_rel) * p.n_tokens + token);
+#pragma unroll 1
+            for (int j = 2 * pair; j < own_n; j += 16) {
+                float z0 = 0.0f, z1 = 0.0f;                     // the parts in rank order
+#pragma unroll 4
+                for (int part_i = 0; part_i < k_split; ++part_i) {
+                    const float2 o = *reinterpret_cast<const float2 *>(recv_few + (part_i * x_rows + token) * pitch + j);
+                    z0 += o.x;
+                    z1 += o.y;
+                }
+                const float2 b = *reinterpret_cast<const float2 *>(b1s + j);
+                if constexpr (kFp8) {
+                    const float2 sw = *reinterpret_cast<const float2 *>(w1s + j);
+                    z0 = fmaf(z0, sw.x * sx, b.x);
+                    z1 = fmaf(z1, sw.y * sx, b.y);
+                } else {
+                    z0 += b.x;
+                    z1 += b.y;
+                }
+                float g0, g1;
+                f2_unpack(gelu_pair(f2_pack(z0, z1)), g0, g1);
+                const float4 *w = reinterpret_cast<const float4 *>(w2f + j * kMaxHeads);
+#pragma unroll
+                for (int i = 0; i < 2; ++i) {
+                    const float4 wa = w[i], wb = w[2 + i];
+                    acc[4 * i] = fmaf(g1, wb.x, fmaf(g0, wa.x, acc[4 * i]));
+                    acc[4 * i + 1] = fmaf(g1, wb.y, fmaf(g0, wa.y, acc[4 * i + 1]));
+                    acc[4 * i + 2] = fmaf(g1, wb.z, fmaf(g0, wa.z, acc[4 * i + 2]));
+                    acc[4 * i + 3] = fmaf(g1, wb.w, fmaf(g0, wa.w, acc[4 * i + 3]));
+                }
+            }
+            // the sums over a token's eight lanes; lane h of them ends up with head h
+#pragma unroll
+            for (int half_n = 4; half_n > 0; half_n >>= 1) {
+                const bool up = pair & half_n;
+#pragma unroll
+                for (int i = 0; i < half_n; ++i) {
+                    const float got = __shfl_xor_sync(0xffffffffu, up ? acc[i] : acc[half_n + i], half_n);
+                    acc[i] = (up ? acc[half_n + i] : acc[i]) + got;
+                }
+            }
+            st_shared_cluster_u32(map_to_cta(smem_base + L.xpart + ((rank * x_rows + token) * kMaxHeads + pair) * 4, 0), __float_as_uint(acc[0]));
         }
-        if (hsel == 1) {
-            float4 *dst = reinterpret_cast<float4 *>(part + row * kMaxHeads);
-            dst[0] = make_float4(s[0], s[1], s[2], s[3]);
-            dst[1] = make_float4(s[4], s[5], s[6], s[7]);
-            __syncwarp();
-            if (lane == 0) mbar_arrive(bar_pfull);
-        } else {
-            mbar_wait(bar_pfull, 0, abort_flag);
-            const float4 *src = reinterpret_cast<const float4 *>(part + row * kMaxHeads);
-            const float4 pa = src[0], pb = src[1];
-            s[0] += pa.x; s[1] += pa.y; s[2] += pa.z; s[3] += pa.w;
-            s[4] += pb.x; s[5] += pb.y; s[6] += pb.z; s[7] += pb.w;
-            // hand this CTA's partial sums to its cluster's first CTA: xpart[rank][row][8]
-            const uint32_t dst = map_to_cta(smem_base + L.xpart + (rank * kTileM + row) * kMaxHeads * 4, half);
-            st_shared_cluster_v4(dst, s[0], s[1], s[2], s[3]);
-            st_shared_cluster_v4(dst + 16, s[4], s[5], s[6], s[7]);
+        if (epi && kBehind) update_rows();
+    } else {
+        // lanes of a warp whose 32 tokens all lie past the input take no part in the exchange and the second layer
+        const bool rows_live = ok && static_cast<int64_t>(row0) + q * 32 < p.n_tokens;
+        float4 *recv = reinterpret_cast<float4 *>(smem);          // [k_split - 1][own_n / 4][128 rows] float4, over the idle stages
+        if (k_split > 1) {
+            // every CTA's MMAs are complete once all have passed this barrier: the stages may be overwritten
+            tc_fence_before_sync();
+            cluster_sync_all();
+            if (epi && rows_live) {
+                for (int i = hsel; i < (k_split - 1) * n16; i += 2) {
+                    const uint32_t c = static_cast<uint32_t>(i % n16);
+                    const uint32_t to = (rank + 1u + static_cast<uint32_t>(i / n16)) % static_cast<uint32_t>(k_split);
+                    const uint32_t slot = rank < to ? rank : rank - 1u;         // the receiver's parts in rank order, itself left out
+                    const uint32_t dst0 = map_to_cta(smem_base, to * kCtas + half) + (slot * (static_cast<uint32_t>(own_n) >> 2) + c * 4) * kTileM * 16;
+                    uint32_t r[16];
+                    tmem_ld_x16(t_row + to * own_n + c * 16, r);
+                    tmem_wait_ld();
+                    reg_fence16(r);
+#pragma unroll
+                    for (int j = 0; j < 4; ++j)
+                        st_shared_cluster_v4(dst0 + (static_cast<uint32_t>(j) * kTileM + row) * 16,
+                                             __uint_as_float(r[4 * j]), __uint_as_float(r[4 * j + 1]),
+                                             __uint_as_float(r[4 * j + 2]), __uint_as_float(r[4 * j + 3]));
+                }
+            }
+            cluster_sync_all();                                     // the others' parts have arrived
+        }
+        // adds what the other CTAs of the cluster sent for 16-column chunk c of this CTA's columns
+        auto add_received = [&](uint32_t (&r)[16], int c) {
+            for (int part_i = 0; part_i < k_split - 1; ++part_i) {
+#pragma unroll
+                for (int i = 0; i < 4; ++i) {
+                    const float4 o = recv[(part_i * (own_n >> 2) + c * 4 + i) * kTileM + row];
+                    r[4 * i] = __float_as_uint(__uint_as_float(r[4 * i]) + o.x);
+                    r[4 * i + 1] = __float_as_uint(__uint_as_float(r[4 * i + 1]) + o.y);
+                    r[4 * i + 2] = __float_as_uint(__uint_as_float(r[4 * i + 2]) + o.z);
+                    r[4 * i + 3] = __float_as_uint(__uint_as_float(r[4 * i + 3]) + o.w);
+                }
+            }
+        };
+        if (epi) {
+            uint64_t acc[kMaxHeads];
+#pragma unroll
+            for (int h = 0; h < kMaxHeads; ++h) acc[h] = 0ull;
+            if (rows_live) {
+                // the first warp of a lane quarter takes the 16-column chunks 0, 2, 4, ..., the second the odd ones
+                uint32_t ra[16], rb[16];
+                uint64_t sx2 = 0ull;                                   // 8-bit inputs: this row's token scale, twice
+                if constexpr (kFp8) {
+                    float sx = 1.0f;
+                    if (p.x_scale != nullptr && row0 + row < p.n_tokens)
+                        sx = __ldg(p.x_scale + static_cast<int64_t>(l_rel) * p.n_tokens + row0 + row);
+                    sx2 = f2_pack(sx, sx);
+                }
+                int c = hsel;
+                if (c < n16) tmem_ld_x16(t_row + own_c0 + c * 16, ra);
+                while (c < n16) {
+                    tmem_wait_ld();
+                    reg_fence16(ra);
+                    if (c + 2 < n16) tmem_ld_x16(t_row + own_c0 + (c + 2) * 16, rb);
+                    add_received(ra, c);
+                    if constexpr (kFp8) mlp_columns_scaled<16>(ra, c * 16, b1s, w1s, sx2, w2p, acc);
+                    else mlp_columns<16>(ra, c * 16, b1s, w2p, acc);
+                    c += 2;
+                    if (c < n16) {
+                        tmem_wait_ld();
+                        reg_fence16(rb);
+                        if (c + 2 < n16) tmem_ld_x16(t_row + own_c0 + (c + 2) * 16, ra);
+                        add_received(rb, c);
+                        if constexpr (kFp8) mlp_columns_scaled<16>(rb, c * 16, b1s, w1s, sx2, w2p, acc);
+                        else mlp_columns<16>(rb, c * 16, b1s, w2p, acc);
+                        c += 2;
+                    }
+                }
+            }
+            float s[kMaxHeads];
+#pragma unroll
+            for (int h = 0; h < kMaxHeads; ++h) {
+                float lo, hi;
+                f2_unpack(acc[h], lo, hi);
+                s[h] = lo + hi;
+            }
+            if (hsel == 1) {
+                float4 *dst = reinterpret_cast<float4 *>(part + row * kMaxHeads);
+                dst[0] = make_float4(s[0], s[1], s[2], s[3]);
+                dst[1] = make_float4(s[4], s[5], s[6], s[7]);
+                __syncwarp();
+                if (lane == 0) mbar_arrive(bar_pfull);
+            } else {
+                mbar_wait(bar_pfull, 0, abort_flag);
+                const float4 *src = reinterpret_cast<const float4 *>(part + row * kMaxHeads);
+                const float4 pa = src[0], pb = src[1];
+                s[0] += pa.x; s[1] += pa.y; s[2] += pa.z; s[3] += pa.w;
+                s[4] += pb.x; s[5] += pb.y; s[6] += pb.z; s[7] += pb.w;
+                // hand this CTA's partial sums to its cluster's first CTA: xpart[rank][row][8]
+                const uint32_t dst = map_to_cta(smem_base + L.xpart + (rank * kTileM + row) * kMaxHeads * 4, half);
+                st_shared_cluster_v4(dst, s[0], s[1], s[2], s[3]);
+                st_shared_cluster_v4(dst + 16, s[4], s[5], s[6], s[7]);
+            }
         }
     }
 
@@ -556,6 +674,45 @@ score_split_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_cons
     // If this launch was allowed to start before the kernel ahead of it had finished (consecutive decode
     // steps), it still completes after it: every thread waits here.
     griddep_wait();
+    if constexpr (kFew) {
+        // ---------------------------------------------------------- first CTA of the cluster: the slice's sums, a (token, head) per thread
+        if (rank != 0 || warp < 2) return;
+        const int w8 = warp - 2, token = w8 * 4 + (lane >> 3), head = lane & 7;
+        const int done_i = layer * n_split + nh;
+        if (w8 * 4 < p.x_rows) {
+            float sum = 0.0f;
+            for (int r = 0; r < k_split; ++r) sum += xpart[(r * p.x_rows + token) * kMaxHeads + head];
+            bool last = true;
+            const float *parts = p.split_part + static_cast<int64_t>(part_tile) * n_split * kTileM * kMaxHeads + token * kMaxHeads + head;
+            if (n_split > 1) {
+                // whichever slice brings a warp's tokens in last finishes them
+                __stcg(const_cast<float *>(parts) + static_cast<int64_t>(nh) * kTileM * kMaxHeads, sum);
+                __syncwarp();
+                int l = 0;
+                if (lane == 0) l = arrive_last_acq_rel(p.split_arrive + part_tile * kFewWarps + w8, static_cast<uint32_t>(n_split));
+                last = __shfl_sync(0xffffffffu, l, 0) != 0;
+            }
+            const CacheView &c = f.c;
+            if (last && token < p.n_tokens && head < c.n_heads) {
+                // all slices have arrived, so every CTA of the tile has counted its lists: one round trip for all of it
+                const int64_t list = (static_cast<int64_t>(token) * c.n_layers + layer) * c.n_heads + head;
+                const int32_t n = __ldcg(c.n_tokens + list);
+                const bool live = c.active[token] != 0;
+                float v = __ldg(p.b2 + layer * kMaxHeads + head);
+                if (n_split > 1) {
+                    sum = 0.0f;                                 // in slice order, whoever was last
+#pragma unroll 4
+                    for (int r = 0; r < n_split; ++r) sum += __ldcg(parts + static_cast<int64_t>(r) * kTileM * kMaxHeads);
+                }
+                v += sum;
+                if (*abort_flag == 0 && live) c.score_ring[list * c.window + (n - 1) % c.window] = v;
+                if (p.scores != nullptr) p.scores[(static_cast<int64_t>(l_rel) * p.n_tokens + token) * p.n_heads + head] = v;
+            }
+        }
+        named_barrier_sync(1, 256);
+        if (threadIdx.x == 64 && *abort_flag == 0) st_release_gpu(f.done + done_i, fuse_step + 1);
+        return;
+    }
     if (rank != 0 || warp < 2 || warp >= 6 || m_tile >= p.blocks_per_layer) return;
 
     // ------------------------------------------------------------ first CTA of the cluster: the slice's sums
