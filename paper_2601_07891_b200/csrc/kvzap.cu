@@ -41,8 +41,8 @@ constexpr int kMaskRing = 4;
 
 }  // namespace kvzap
 
-// Arrival counters of the few-token kernel: one per tile, then kFewWarps per tile for steps of few tokens.
-namespace kvzap { constexpr size_t kSplitArrive = 1 + kFewWarps; }
+// Arrival counters of the few-token kernel: kTileWarps per tile, then kFewWarps per tile for steps of few tokens.
+namespace kvzap { constexpr size_t kSplitArrive = kTileWarps + kFewWarps; }
 
 struct kvzap_ctx {
     kvzap_config cfg;
@@ -819,7 +819,7 @@ static kvzap_status launch_score(kvzap_ctx *ctx, int32_t layer, int32_t n_layers
         p.tau = tau;
         p.status = ctx->status_dev;
         p.split_part = ctx->split_part;
-        p.split_arrive = layout.arrive + (p.x_rows > 0 ? ctx->sm_count : 0);
+        p.split_arrive = layout.arrive + (p.x_rows > 0 ? kTileWarps * ctx->sm_count : 0);
         // Early start (consecutive decode steps): this kernel reads only hidden states and weights; the one
         // thing it may not do is write a scores buffer that the kernels of the previous call still read.
         const size_t sbytes = scores ? sizeof(float) * static_cast<size_t>(n_layers) * n_tokens * c.n_kv_heads : 0;
