@@ -104,6 +104,7 @@ struct kvzap_ctx {
     float *plan_scores = nullptr;        // kvzap_prefill_plan without scores_out: [max_tokens][H] (allocated on first use)
     int64_t *batch_map = nullptr;        // chunks into a cache: first list of each sequence of the call [max_seqs]
     uint32_t *chunk_arrive = nullptr;    //                      lists that are done, zero between launches
+    int32_t *chunk_taken = nullptr;      //                      [2] page cursor and stack height behind the window side
     float *split_part = nullptr;         // few-token kernel: [tile][slice][128][8] partial scores, tiles * slices <= sm_count
     uint64_t score_turn = 0;
     bool last_score_early = false;       // the launch behind the last scoring launch may start while work ahead of that one runs
@@ -449,6 +450,7 @@ static void free_all(kvzap_ctx *ctx)
     cudaFree(ctx->split_part);
     cudaFree(ctx->plan_scores);
     cudaFree(ctx->batch_map);
+    cudaFree(ctx->chunk_taken);
     cudaFree(ctx->chunk_arrive);
     cudaFree(ctx->select_hist);
     cudaFree(ctx->select_tau);
@@ -1231,6 +1233,50 @@ static cudaError_t launch_compact_kernel(const CompactShape &s, cudaStream_t str
     return cudaLaunchKernelEx(&cfg, compact_dense_kernel<kDenseThreads, false>, args...);
 }
 
+// The compaction of a short input that runs beside nothing (compact_short_kernel): two CTAs to a block's rows or more where the
+// device holds them at once.
+static kvzap_status launch_compact_short(kvzap_ctx *ctx, ShortCompact a, cudaStream_t stream)
+{
+    a.page_shift = -1;
+    for (int i = 0; i < 31; ++i)
+        if (a.page_tokens == 1 << i) a.page_shift = i;
+    unsigned nz = 1;
+    while (nz < 4 && 2 * nz * a.n_blocks * a.n_heads <= 4 * ctx->sm_count) nz *= 2;
+    ProfScope prof(ctx, KVZAP_KERNEL_COMPACT, stream);
+    cudaLaunchConfig_t cfg;
+    cudaLaunchAttribute attrs[2];
+    make_launch(&cfg, attrs, dim3(static_cast<unsigned>(a.n_blocks) + 1, static_cast<unsigned>(a.n_heads), nz), dim3(kDenseThreadsShort), 0, stream,
+                !ctx->profiling, 1);
+    KVZAP_CUDA(ctx, cudaLaunchKernelEx(&cfg, a.list_base != nullptr ? compact_short_kernel<kShortAppend>
+                                             : a.page_tokens > 0    ? compact_short_kernel<kShortPaged>
+                                                                    : compact_short_kernel<kShortDense>, a));
+    ctx->launches += 1;
+    return KVZAP_OK;
+}
+static ShortCompact short_args(const kvzap_ctx *ctx, const uint32_t *mask, const void *K, const void *V, const int32_t *cu_seqlens,
+                               int32_t n_seqs, int64_t n_tokens, void *K_out, void *V_out, int32_t *lengths, bool tok_major)
+{
+    const kvzap_config &c = ctx->cfg;
+    ShortCompact a;
+    memset(&a, 0, sizeof a);
+    a.K = static_cast<const uint4 *>(K);
+    a.V = static_cast<const uint4 *>(V);
+    a.K_out = static_cast<uint4 *>(K_out);
+    a.V_out = static_cast<uint4 *>(V_out);
+    a.maskbits = mask;
+    a.cu_seqlens = cu_seqlens;
+    a.lengths = lengths;
+    a.n_tokens = n_tokens;
+    a.in_stride_h = tok_major ? int64_t{1} : n_tokens;
+    a.in_stride_t = tok_major ? static_cast<int64_t>(c.n_kv_heads) : int64_t{1};
+    a.n_blocks = static_cast<int32_t>((n_tokens + kBlockTokens - 1) / kBlockTokens);
+    a.n_words = 4 * a.n_blocks;
+    a.n_seqs = n_seqs;
+    a.n_heads = c.n_kv_heads;
+    a.row_units = c.head_dim / 8;
+    return a;
+}
+
 // Dense-ragged compaction over the mask words in `mask` (one kernel, no scan pass).
 static kvzap_status launch_compaction(kvzap_ctx *ctx, const uint32_t *mask, const void *K, const void *V,
                                       const int32_t *cu_seqlens, int32_t n_seqs, int64_t n_tokens, void *K_out,
@@ -1239,6 +1285,10 @@ static kvzap_status launch_compaction(kvzap_ctx *ctx, const uint32_t *mask, cons
     const kvzap_config &c = ctx->cfg;
     const int64_t n_blocks = (n_tokens + kBlockTokens - 1) / kBlockTokens;
     const int64_t n_words = n_blocks * 4;
+    // as long as the device holds two CTAs per block: beyond, nothing is left of what the shorter chain gains without pages to find
+    // (4096 -> 8, 2 sequences, 6000 tokens 109.0 us with the other kernel, 110.3 with this; MLP 8100 tokens 169.5 and 170.9)
+    if (!ctx->trusted && short_input(n_words, c.n_kv_heads, n_seqs) && 2 * n_blocks * c.n_kv_heads <= 4 * ctx->sm_count)
+        return launch_compact_short(ctx, short_args(ctx, mask, K, V, cu_seqlens, n_seqs, n_tokens, K_out, V_out, lengths, tok_major), stream);
     const CompactShape shape = compact_shape(ctx, n_blocks, false, false);
     {
         ProfScope prof(ctx, KVZAP_KERNEL_COMPACT, stream);
@@ -1647,6 +1697,7 @@ kvzap_status kvzap_create(kvzap_ctx **out, const kvzap_config *cfg)
     CREATE_CUDA(cudaMalloc(&ctx->list_page0, sizeof(int32_t) * static_cast<int64_t>(c.max_seqs) * c.n_kv_heads));
     CREATE_CUDA(cudaMalloc(&ctx->list_base, sizeof(int32_t) * static_cast<int64_t>(c.max_seqs) * c.n_kv_heads));
     CREATE_CUDA(cudaMalloc(&ctx->batch_map, sizeof(int64_t) * static_cast<size_t>(c.max_seqs)));
+    CREATE_CUDA(cudaMalloc(&ctx->chunk_taken, 2 * sizeof(int32_t)));
     CREATE_CUDA(cudaMalloc(&ctx->chunk_arrive, sizeof(uint32_t)));
     CREATE_CUDA(cudaMemset(ctx->chunk_arrive, 0, sizeof(uint32_t)));
     CREATE_CUDA(cudaMalloc(&ctx->tile_counters, sizeof(int32_t) * kMaskRing));
@@ -2312,6 +2363,17 @@ static kvzap_status launch_compaction_paged(kvzap_ctx *ctx, const uint32_t *mask
     const kvzap_config &c = ctx->cfg;
     const int64_t n_blocks = (n_tokens + kBlockTokens - 1) / kBlockTokens;
     const int64_t n_words = n_blocks * 4;
+    if (!ctx->trusted && !append && page_cursor == nullptr && short_input(n_words, c.n_kv_heads, n_seqs)) {
+        ShortCompact a = short_args(ctx, mask, K, V, cu_seqlens, n_seqs, n_tokens, K_pool, V_pool, lengths, tok_major);
+        a.page_tokens = page_tokens;
+        a.first_page = first_page;
+        a.max_pages = max_pages;
+        a.n_pages_pool = n_pages_pool;
+        a.page_table = page_table;
+        a.n_pages_used = n_pages_used;
+        a.status = ctx->status_dev;
+        return launch_compact_short(ctx, a, stream);
+    }
     PageAssign assign;
     memset(&assign, 0, sizeof assign);
     if (!append && page_cursor == nullptr && n_words * c.n_kv_heads <= kAssignWords &&
@@ -2940,6 +3002,7 @@ static kvzap_status append_chunk(kvzap_ctx *ctx, kvzap_cache *cache, int32_t lay
     const int64_t n_words = (n_tokens + kBlockTokens - 1) / kBlockTokens * 4;
     // directly behind a scoring launch that lets it start when all work ahead of that launch has completed
     const bool beside = ctx->last_score_late && by_value.n > 0;
+    const bool short_chunk = v.window > 0 && short_input(n_words, v.n_heads, n_seqs);
     if (v.window > 0) {
         cudaLaunchConfig_t cfg;
         cudaLaunchAttribute attrs[2];
@@ -2948,12 +3011,31 @@ static kvzap_status append_chunk(kvzap_ctx *ctx, kvzap_cache *cache, int32_t lay
         KVZAP_CUDA(ctx, cudaLaunchKernelEx(&cfg, chunk_ring_kernel, v, by_value, static_cast<int>(layer), ctx->batch_map, scores,
                                            static_cast<const uint4 *>(K), static_cast<const uint4 *>(V), n_tokens, tau, cu_seqlens, mask,
                                            n_words, ctx->list_base, ctx->list_page0, ctx->chunk_arrive, ctx->status_dev,
-                                           beside ? 1 : 0));
+                                           beside ? 1 : 0, short_chunk ? 0 : 1, ctx->chunk_taken));
     } else {
         tokens_add_kernel<<<static_cast<unsigned>(n_seqs), 32, 0, stream>>>(v, by_value, layer, ctx->batch_map, n_tokens, cu_seqlens);
         KVZAP_CUDA(ctx, cudaGetLastError());
     }
     ctx->launches += 1;
+    if (short_chunk) {
+        ShortCompact a = short_args(ctx, mask, K, V, cu_seqlens, n_seqs, n_tokens, v.k_pool, v.v_pool, v.prefix_len, false);
+        a.page_tokens = v.page_tokens;
+        a.max_pages = v.max_pages;
+        a.n_pages_pool = v.n_pages_pool;
+        a.page_table = v.page_table;
+        a.status = ctx->status_dev;
+        a.list_base = ctx->list_base;
+        a.list_map = ctx->batch_map;
+        a.page_cursor = v.page_cursor;
+        a.free_stack = v.free_stack;
+        a.free_top = v.free_top;
+        a.taken = ctx->chunk_taken;
+        a.scores = scores;
+        a.score_ring = v.score_ring;
+        a.n_tokens_list = v.n_tokens;
+        a.window = v.window;
+        return launch_compact_short(ctx, a, stream);
+    }
     return launch_compaction_paged(ctx, mask, K, V, cu_seqlens, n_seqs, n_tokens, v.k_pool, v.v_pool, v.n_pages_pool,
                                    v.page_tokens, 0, v.page_table, v.max_pages, v.prefix_len, nullptr, stream, v.page_cursor,
                                    false, true, v.free_stack, v.free_top, ctx->batch_map, v.window > 0);

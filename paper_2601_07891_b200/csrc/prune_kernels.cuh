@@ -503,7 +503,8 @@ __device__ __forceinline__ int popc_below(uint32_t w0, uint32_t w1, uint32_t w2,
 
 // Paged output of a short input: every CTA counts all lists from the mask words and works out all first pages itself,
 // instead of a launch of one CTA ahead of the compaction (777 tokens: 8.6 -> 5.5 us from the end of the scoring launch to
-// the end of the compaction).  The counting is H * n_words words per CTA, hence the limits: at 8192 tokens x 8 heads it
+// the end of the compaction).  On contexts that trust their producers, where the compaction runs beside the next scoring; elsewhere
+// compact_short_kernel.  The counting is H * n_words words per CTA, hence the limits: at 8192 tokens x 8 heads it
 // takes the 256 threads 8 loads each.
 struct PageAssign {
     int32_t enabled;
@@ -740,6 +741,301 @@ compact_dense_kernel(const uint4 *__restrict__ K, const uint4 *__restrict__ V, u
         base_cur = base_next_s;
         __syncthreads();
     }
+}
+
+// ---------------------------------------------------------------------------
+// The compaction of a short input (mask words and lists as for assign_pages_locally) that runs beside nothing: behind the scoring of
+// a default context, or of a chunk.  There the launch is a chain of round trips, and this kernel has as few as there are: mask words,
+// sequence offsets, old lengths and the page cursor together; then the rows' loads, for which a CTA needs only its own block's
+// words, go out before the lists are counted and pages found; then the stores.  Grid (blocks + 1, H, z): z CTAs share the rows
+// of a block, and the last x does the bookkeeping of a head's lists (lengths, tables, for a chunk also the ring's scores), which no
+// row waits for.  An append finds the pages of new rows itself, from the cursor and the stack as the launch ahead left them (`taken`).
+// Scoring and this, us a call of several layers: 8 x 777 tokens into pages 146.6 -> 136.4, 4 x 5 x 300 93.3 -> 82.1, 4 x 3000 118.6 -> 110.6, dense
+// 4 x 777 67.5 -> 63.5; 5120 -> 640 -> 8, 4 x 2000 dense 90.3 -> 86.0.  Chunks, whose launch ahead had spent 7 us on counting and a one-CTA page
+// assignment behind the scoring: four prompts in two chunks of 500 tokens, 4 layers, 274.3 -> 224.3, eight of 64 in three 304.9 -> 268.7.
+// Two rows in flight per lane group and four CTAs to a block rather than four rows and two CTAs (3000 tokens 110.5 and 117.4).
+struct ShortCompact {
+    const uint4 *K, *V;
+    uint4 *K_out, *V_out;
+    const uint32_t *maskbits;         // [H][n_words]
+    const int32_t *cu_seqlens;
+    int32_t *lengths;                 // [n_lists]; append: of all lists of the cache
+    int64_t n_tokens, in_stride_h, in_stride_t;
+    int32_t n_words, n_blocks, n_seqs, n_heads, row_units;
+    int32_t page_tokens;              // 0: dense-ragged output
+    int32_t page_shift;               // its logarithm, or -1: a division takes some 150 cycles of a chain
+    int32_t first_page, max_pages;
+    int64_t n_pages_pool;
+    int32_t *page_table, *n_pages_used, *status;
+    // append (list_base != nullptr)
+    const int32_t *list_base;         // [n_lists] rows that a list holds now
+    const int64_t *list_map;          // [n_seqs] list of head 0 of each sequence
+    int32_t *page_cursor;
+    const int32_t *free_stack;
+    int32_t *free_top;
+    const int32_t *taken;             // page cursor and height of the stack, as copied by the launch ahead
+    // the ring's scores: those of the last min(length, window) tokens of each sequence
+    const float *scores;
+    float *score_ring;
+    const int32_t *n_tokens_list;     // tokens of each list, these included
+    int32_t window;
+};
+constexpr int kShortRows = 2;         // rows of K and of V in flight per lane group
+__host__ inline bool short_input(int64_t n_words, int n_heads, int64_t n_seqs)
+{
+    return n_words * n_heads <= kAssignWords && n_seqs * n_heads <= kAssignLists;
+}
+
+// seq_of_token over offsets in shared memory
+__device__ __forceinline__ int seq_of_shared(const int32_t *cu, int n_seqs, int32_t t)
+{
+    int lo = 0, hi = n_seqs;
+    while (hi - lo > 1) {
+        const int mid = (lo + hi) >> 1;
+        if (cu[mid] <= t) lo = mid; else hi = mid;
+    }
+    return lo;
+}
+
+enum ShortKind { kShortDense, kShortPaged, kShortAppend };
+template <ShortKind kKind>
+__global__ void __launch_bounds__(kDenseThreadsShort, 4)
+compact_short_kernel(const ShortCompact a)
+{
+    constexpr int kThreads = kDenseThreadsShort, kWarps = kThreads / 32;
+    constexpr bool kPages = kKind != kShortDense, kAppend = kKind == kShortAppend;
+    __shared__ uint32_t s_words[kAssignWords];        // dense: of this CTA's head, else of all heads
+    __shared__ int32_t s_cu[kAssignLists + 1], s_len[kAssignLists], s_base[kPages ? kAssignLists : 1], s_page0[kPages ? kAssignLists : 1];
+    __shared__ int64_t s_list[kPages ? kAssignLists : 1];      // [n_seqs] this head's lists among those of the table
+    __shared__ int32_t s_last[kAppend ? kAssignLists : 1];     // [n_seqs] ... the pages that they end in now
+    __shared__ int32_t src_tok[kBlockTokens];
+    __shared__ int64_t dst_row[kBlockTokens];
+    __shared__ int32_t running_s, before_s, cursor_s, free_s, stack_s;
+    const int h = blockIdx.y, H = a.n_heads, z = blockIdx.z, nz = gridDim.z;
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    const int blk = blockIdx.x;
+    const bool books = blk == a.n_blocks;
+    griddep_launch_dependents();
+    griddep_wait();
+    if (books && z != 0) return;
+
+    const int n_lists = a.n_seqs * H, n_words = a.n_words;
+    const bool multi = a.cu_seqlens != nullptr && a.n_seqs > 1;
+    {
+        // all loads before the first store: one round trip
+        constexpr int kWordsEach = kAssignWords / kThreads;
+        const int total = kPages ? n_words * H : n_words;
+        const uint32_t *words = a.maskbits + (kPages ? 0 : static_cast<int64_t>(h) * n_words);
+        uint32_t w[kWordsEach];
+#pragma unroll
+        for (int k = 0; k < kWordsEach; ++k) w[k] = tid + k * kThreads < total ? __ldcg(words + tid + k * kThreads) : 0u;
+        int32_t start = 0, end = static_cast<int32_t>(a.n_tokens), base = 0, cursor = a.first_page, top = 0;
+        int64_t list0 = static_cast<int64_t>(tid) * H;
+        if (multi && tid < a.n_seqs) start = __ldg(a.cu_seqlens + tid);
+        if (multi && tid == 0) end = __ldg(a.cu_seqlens + a.n_seqs);
+        if constexpr (kAppend) {
+            if (tid < n_lists) base = __ldcg(a.list_base + tid);
+            if (tid < a.n_seqs) list0 = __ldcg(a.list_map + tid);
+            if (tid == 0) {
+                cursor = __ldcg(a.taken);
+                top = __ldcg(a.taken + 1);
+            }
+        }
+#pragma unroll
+        for (int k = 0; k < kWordsEach; ++k)
+            if (tid + k * kThreads < total) s_words[tid + k * kThreads] = w[k];
+        if (tid < a.n_seqs) s_cu[tid] = start;
+        if (tid == 0) s_cu[a.n_seqs] = end;
+        if constexpr (kPages) {
+            if (tid < n_lists) s_base[tid] = base;
+            if (tid < a.n_seqs) s_list[tid] = list0 + h;
+            if (tid == 0) { cursor_s = cursor; free_s = top > 0 ? top : 0; }
+        }
+    }
+    __syncthreads();
+    const uint32_t *mine = s_words + (kPages ? h * n_words : 0);
+    auto whole_pages = [&](int32_t rows) -> int32_t { return a.page_shift >= 0 ? rows >> a.page_shift : rows / a.page_tokens; };
+    auto pages_of = [&](int32_t rows) -> int32_t { return whole_pages(rows + a.page_tokens - 1); };
+    auto seq_at = [&](int64_t t) -> int { return multi ? seq_of_shared(s_cu, a.n_seqs, static_cast<int32_t>(t)) : 0; };
+    // set bits of head words `w` for tokens [lo, hi), by a whole warp
+    auto count = [&](const uint32_t *w, int32_t lo, int32_t hi) -> int32_t {
+        int32_t n = 0;
+        for (int i = lo / 32 + lane; i * 32 < hi; i += 32) {
+            uint32_t v = w[i];
+            if (i * 32 < lo) v &= ~0u << (lo - i * 32);
+            if (i * 32 + 32 > hi) v &= (1u << (hi - i * 32)) - 1u;
+            n += __popc(v);
+        }
+        return __reduce_add_sync(0xffffffffu, n);
+    };
+
+    // the rows of this block: which they are needs nothing but its words, so their loads go out first
+    const int group = tid >> 4, gl = tid & 15;
+    constexpr int kGroups = kThreads / 16;
+    const int blk_start = blk * kBlockTokens, first = group + z * kGroups, step = nz * kGroups;
+    uint32_t w0 = 0, w1 = 0, w2 = 0, w3 = 0;
+    int cnt = 0, rank = 0;
+    bool keep = false;
+    uint4 kv[kShortRows], vv[kShortRows];
+    const int64_t head_row0 = static_cast<int64_t>(h) * a.in_stride_h + blk_start * a.in_stride_t;
+    auto load_rows = [&](int i0, int u0) {
+#pragma unroll
+        for (int j = 0; j < kShortRows; ++j) {
+            const int i = i0 + j * step;
+            if (i < cnt && u0 < a.row_units) {
+                const int64_t src = (head_row0 + src_tok[i] * a.in_stride_t) * a.row_units + u0;
+                kv[j] = __ldg(a.K + src);
+                vv[j] = __ldg(a.V + src);
+            }
+        }
+    };
+    if (!books) {
+        w0 = mine[blk * 4]; w1 = mine[blk * 4 + 1]; w2 = mine[blk * 4 + 2]; w3 = mine[blk * 4 + 3];
+        cnt = __popc(w0) + __popc(w1) + __popc(w2) + __popc(w3);
+        if (tid < kBlockTokens) {
+            rank = popc_below(w0, w1, w2, w3, tid);
+            const uint32_t w = tid < 32 ? w0 : tid < 64 ? w1 : tid < 96 ? w2 : w3;
+            keep = (w >> (tid & 31)) & 1u;
+            if (keep) src_tok[rank] = tid;
+        }
+        __syncthreads();
+        load_rows(first, gl);
+        if (warp == kWarps - 1) {
+            // kept rows before the block, and before the start of the sequence in progress there
+            const int32_t s0 = s_cu[seq_at(blk_start)];
+            const int32_t before = count(mine, 0, s0 < blk_start ? s0 : blk_start), rest = s0 < blk_start ? count(mine, s0, blk_start) : 0;
+            if (lane == 0) { before_s = before; running_s = before + rest; }
+        }
+    }
+    if constexpr (kAppend) {
+        if (tid < a.n_seqs) {
+            const int32_t have = pages_of(s_base[tid * H + h]);
+            s_last[tid] = have > 0 ? __ldcg(a.page_table + s_list[tid] * a.max_pages + have - 1) : 0;
+        }
+    }
+    // kept rows of every list (dense: of this head's, and only for the bookkeeping), by as many threads per list as there are
+    if (kPages || books) {
+        const int lists = kPages ? n_lists : a.n_seqs;
+        int each = 32;
+        while (each * lists > kThreads) each >>= 1;
+        const int i = tid / each, sub = tid & (each - 1);
+        int32_t n = 0;
+        if (i < lists) {
+            const int b = kPages ? i / H : i;
+            const uint32_t *w = s_words + (kPages ? (i - b * H) * n_words : 0);
+            const int32_t lo = s_cu[b], hi = s_cu[b + 1];
+            for (int j = lo / 32 + sub; j * 32 < hi; j += each) {
+                uint32_t v = w[j];
+                if (j * 32 < lo) v &= ~0u << (lo - j * 32);
+                if (j * 32 + 32 > hi) v &= (1u << (hi - j * 32)) - 1u;
+                n += __popc(v);
+            }
+        }
+        for (int o = each >> 1; o > 0; o >>= 1) n += __shfl_xor_sync(0xffffffffu, n, o);
+        if (i < lists && sub == 0) s_len[i] = n;
+    }
+    __syncthreads();
+    if constexpr (kPages) {
+        if (warp == 0) {
+            // pages in list order: those that a list needs beside the ones it has; all or nothing
+            int32_t carry = 0;
+            bool fail = false;
+            for (int base = 0; base < n_lists; base += 32) {
+                const int idx = base + lane;
+                int32_t need = 0;
+                if (idx < n_lists) {
+                    const int32_t pages = pages_of(s_base[idx] + s_len[idx]);
+                    fail = fail || pages > a.max_pages;
+                    need = pages - pages_of(s_base[idx]);
+                }
+                int32_t incl = need;
+#pragma unroll
+                for (int o = 1; o < 32; o <<= 1) {
+                    const int32_t y = __shfl_up_sync(0xffffffffu, incl, o);
+                    if (lane >= o) incl += y;
+                }
+                if (idx < n_lists) s_page0[idx] = carry + incl - need;       // ordinal of its first new page
+                carry += __shfl_sync(0xffffffffu, incl, 31);
+            }
+            const int32_t from_stack = carry < free_s ? carry : free_s;
+            // an append that needs no page but released ones fits wherever the cursor stands
+            const bool fits = static_cast<int64_t>(cursor_s) + (carry - from_stack) <= a.n_pages_pool || (kAppend && carry == from_stack);
+            fail = __any_sync(0xffffffffu, fail) || !fits;
+            const bool first_cta = books && h == 0;
+            if (fail) {
+                for (int idx = lane; idx < n_lists; idx += 32) s_page0[idx] = -1;
+                if (first_cta && lane == 0) atomicCAS(a.status, 0, 4 /* KVZAP_ERR_OOM_PAGES */);
+            }
+            if (lane == 0) {
+                stack_s = from_stack;
+                if (first_cta && a.n_pages_used != nullptr) *a.n_pages_used = fail ? 0 : carry;
+            }
+            if (kAppend && first_cta && lane == 0 && !fail) {
+                *a.page_cursor = cursor_s + carry - from_stack;
+                if (from_stack > 0) *a.free_top = free_s - from_stack;
+            }
+        }
+        __syncthreads();
+    }
+    auto page_at = [&](int32_t ordinal) -> int32_t {
+        if (kAppend && ordinal < stack_s) return __ldcg(a.free_stack + free_s - 1 - ordinal);
+        return cursor_s + ordinal - (kAppend ? stack_s : 0);
+    };
+
+    if (books) {
+        for (int b = warp; b < a.n_seqs; b += kWarps) {
+            const int64_t li = kPages ? s_list[b] : static_cast<int64_t>(b) * H + h;
+            const int32_t kept = s_len[kPages ? b * H + h : b];
+            if constexpr (kPages) {
+                const int idx = b * H + h;
+                const int32_t p0 = s_page0[idx], have = pages_of(s_base[idx]);
+                const int32_t need = p0 < 0 ? 0 : pages_of(s_base[idx] + kept) - have;
+                for (int32_t i = lane; i < need; i += 32) a.page_table[li * a.max_pages + have + i] = page_at(p0 + i);
+                // an append that found no room leaves its lists as they were; a paged call says how long they would be
+                if (lane == 0) a.lengths[li] = kAppend ? s_base[idx] + (p0 < 0 ? 0 : kept) : kept;
+            } else {
+                if (lane == 0) a.lengths[li] = kept;
+            }
+            if constexpr (kAppend) {
+                const int32_t m = s_cu[b + 1] - s_cu[b], n_win = m < a.window ? m : a.window;
+                const int32_t n_now = __ldcg(a.n_tokens_list + li);
+                for (int32_t i = lane; i < n_win; i += 32)
+                    a.score_ring[li * a.window + (n_now - n_win + i) % a.window] =
+                        __ldcg(a.scores + (static_cast<int64_t>(s_cu[b + 1]) - n_win + i) * H + h);
+            }
+        }
+        return;
+    }
+    if (keep) {
+        const int64_t t = blk_start + tid;
+        const int b = seq_at(t);
+        const int32_t s = s_cu[b];
+        // its rank in its list: kept rows before it less those before the start of its sequence
+        const int32_t n = running_s + rank - (s >= blk_start ? running_s + popc_below(w0, w1, w2, w3, s - blk_start) : before_s);
+        if constexpr (kPages) {
+            const int idx = b * H + h;
+            const int32_t p0 = s_page0[idx], nn = s_base[idx] + n, pi = whole_pages(nn), have = pages_of(s_base[idx]);
+            int64_t page = -1;
+            if (p0 >= 0) page = kAppend && pi < have ? s_last[b] : page_at(p0 + pi - have);
+            dst_row[rank] = p0 < 0 ? -1 : page * a.page_tokens + (nn - pi * a.page_tokens);
+        } else {
+            dst_row[rank] = static_cast<int64_t>(h) * a.n_tokens + s + n;
+        }
+    }
+    __syncthreads();
+    for (int i0 = first; i0 < cnt; i0 += kShortRows * step)
+        for (int u0 = gl; u0 < a.row_units; u0 += 16) {
+            if (i0 != first || u0 != gl) load_rows(i0, u0);
+#pragma unroll
+            for (int j = 0; j < kShortRows; ++j) {
+                const int i = i0 + j * step;
+                if (i < cnt && dst_row[i] >= 0) {
+                    const int64_t d = dst_row[i] * a.row_units + u0;
+                    a.K_out[d] = kv[j];
+                    a.V_out[d] = vv[j];
+                }
+            }
+        }
 }
 
 }  // namespace kvzap
