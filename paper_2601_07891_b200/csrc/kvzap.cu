@@ -1235,7 +1235,7 @@ static cudaError_t launch_compact_kernel(const CompactShape &s, cudaStream_t str
 
 // The compaction of a short input that runs beside nothing (compact_short_kernel): two CTAs to a block's rows or more where the
 // device holds them at once.
-static kvzap_status launch_compact_short(kvzap_ctx *ctx, ShortCompact a, cudaStream_t stream)
+static kvzap_status launch_compact_short(kvzap_ctx *ctx, ShortCompact a, cudaStream_t stream, ShortSource from = kFromWords)
 {
     a.page_shift = -1;
     for (int i = 0; i < 31; ++i)
@@ -1247,9 +1247,12 @@ static kvzap_status launch_compact_short(kvzap_ctx *ctx, ShortCompact a, cudaStr
     cudaLaunchAttribute attrs[2];
     make_launch(&cfg, attrs, dim3(static_cast<unsigned>(a.n_blocks) + 1, static_cast<unsigned>(a.n_heads), nz), dim3(kDenseThreadsShort), 0, stream,
                 !ctx->profiling, 1);
-    KVZAP_CUDA(ctx, cudaLaunchKernelEx(&cfg, a.list_base != nullptr ? compact_short_kernel<kShortAppend>
-                                             : a.page_tokens > 0    ? compact_short_kernel<kShortPaged>
-                                                                    : compact_short_kernel<kShortDense>, a));
+    const bool paged = a.page_tokens > 0;
+    KVZAP_CUDA(ctx, cudaLaunchKernelEx(&cfg, a.list_base != nullptr   ? compact_short_kernel<kShortAppend, kFromWords>
+                                             : from == kFromScores    ? (paged ? compact_short_kernel<kShortPaged, kFromScores>
+                                                                               : compact_short_kernel<kShortDense, kFromScores>)
+                                             : paged                  ? compact_short_kernel<kShortPaged, kFromWords>
+                                                                      : compact_short_kernel<kShortDense, kFromWords>, a));
     ctx->launches += 1;
     return KVZAP_OK;
 }
@@ -1347,6 +1350,25 @@ static kvzap_status launch_prune_onepass(kvzap_ctx *ctx, const float *scores, co
         uses, 11, !ctx->trusted || ctx->profiling || tau_list != nullptr || scores_just_made || ctx->op_last_seq + 1 != ctx->op_seq, 0);
     const bool wait_first = order.wait != InFlight::kNone;
     ctx->op_last_seq = ctx->op_seq;
+    if (slot_out == nullptr && n_blocks <= (page_tokens > 0 ? kShortScoreBlocksPaged : kShortScoreBlocks) &&
+        short_input(4 * n_blocks, c.n_kv_heads, n_seqs) && !tau_behind && (page_tokens == 0 || tau_list == nullptr)) {
+        ShortCompact a = short_args(ctx, nullptr, K, V, cu_seqlens, n_seqs, n_tokens, K_out, V_out, lengths, false);
+        a.page_tokens = page_tokens;
+        a.first_page = first_page;
+        a.max_pages = max_pages;
+        a.n_pages_pool = n_pages_pool;
+        a.page_table = page_table;
+        a.n_pages_used = n_pages_used;
+        a.status = ctx->status_dev;
+        a.scores = scores;
+        a.window = w;
+        a.tau = tau;
+        a.tau_list = tau_list;
+        a.wait_first = !wait_first ? 0 : order.late && ctx->trusted ? 2 : 1;
+        a.clear = reinterpret_cast<uint4 *>(clear);
+        a.clear_units = clear_words / 4;
+        return launch_compact_short(ctx, a, stream, kFromScores);
+    }
     // A launch that waits for the work ahead takes every slot of the device (32k tokens, a quarter kept: 40 -> 31 us); one
     // that may run beside the launch ahead (and the one behind it beside this one) half of them, and so does the paged
     // output, whose CTAs all wait for one another: two such launches on two streams still fit side by side.  Half of them

@@ -779,6 +779,13 @@ struct ShortCompact {
     float *score_ring;
     const int32_t *n_tokens_list;     // tokens of each list, these included
     int32_t window;
+    // keep bits from given scores (kFromScores): threshold, or one per list, and the order with the launches around this one
+    // as in PruneParams; `scores` as above
+    float tau;
+    const float *tau_list;
+    int32_t wait_first;
+    uint4 *clear;
+    int64_t clear_units;
 };
 constexpr int kShortRows = 2;         // rows of K and of V in flight per lane group
 __host__ inline bool short_input(int64_t n_words, int n_heads, int64_t n_seqs)
@@ -798,7 +805,15 @@ __device__ __forceinline__ int seq_of_shared(const int32_t *cu, int n_seqs, int3
 }
 
 enum ShortKind { kShortDense, kShortPaged, kShortAppend };
-template <ShortKind kKind>
+// Where the keep bits come from: mask words, or given scores (the pruning calls).  Then every CTA makes the words that it needs
+// itself: dense, those of its head up to its block; paged, all of them, a token of all heads per load.
+// In place of prune_onepass_kernel, whose CTAs look sequences up in memory one after the other, and whose paged form meets at an arrival
+// counter, a page assignment and a flag; us a call: 3 x 500 tokens 8.6 -> 5.8, 800 7.4 -> 4.1, 2200 10.3 -> 5.2, 4000 10.2 -> 7.3, 8000 13.1 -> 11.7,
+// 4 x 1250 15.5 -> 12.6; paged 300 12.1 -> 5.0, 2 x 450 14.9 -> 8.8, 1500 13.4 -> 11.0 (2500 equal, 4000 in three 16.8 -> 22.4: every CTA reads all
+// scores there, so 16 blocks at most).
+enum ShortSource { kFromWords, kFromScores };
+constexpr int kShortScoreBlocks = 64, kShortScoreBlocksPaged = 16;
+template <ShortKind kKind, ShortSource kFrom>
 __global__ void __launch_bounds__(kDenseThreadsShort, 4)
 compact_short_kernel(const ShortCompact a)
 {
@@ -808,6 +823,7 @@ compact_short_kernel(const ShortCompact a)
     __shared__ int32_t s_cu[kAssignLists + 1], s_len[kAssignLists], s_base[kPages ? kAssignLists : 1], s_page0[kPages ? kAssignLists : 1];
     __shared__ int64_t s_list[kPages ? kAssignLists : 1];      // [n_seqs] this head's lists among those of the table
     __shared__ int32_t s_last[kAppend ? kAssignLists : 1];     // [n_seqs] ... the pages that they end in now
+    __shared__ float s_tau[kFrom == kFromScores && !kPages ? kAssignLists : 1];
     __shared__ int32_t src_tok[kBlockTokens];
     __shared__ int64_t dst_row[kBlockTokens];
     __shared__ int32_t running_s, before_s, cursor_s, free_s, stack_s;
@@ -815,8 +831,16 @@ compact_short_kernel(const ShortCompact a)
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const int blk = blockIdx.x;
     const bool books = blk == a.n_blocks;
-    griddep_launch_dependents();
-    griddep_wait();
+    if constexpr (kFrom == kFromWords) {
+        griddep_launch_dependents();
+        griddep_wait();
+    } else {
+        if (a.wait_first < 2) griddep_launch_dependents();
+        if (a.wait_first > 0) {
+            griddep_wait();
+            if (a.wait_first == 2) griddep_launch_dependents();
+        }
+    }
     if (books && z != 0) return;
 
     const int n_lists = a.n_seqs * H, n_words = a.n_words;
@@ -827,8 +851,35 @@ compact_short_kernel(const ShortCompact a)
         const int total = kPages ? n_words * H : n_words;
         const uint32_t *words = a.maskbits + (kPages ? 0 : static_cast<int64_t>(h) * n_words);
         uint32_t w[kWordsEach];
+        constexpr int kScoresEach = kPages ? 4 : 8;               // tokens per thread whose scores are loaded together
+        constexpr int kHeadsEach = kPages ? kMaxHeads : 1;
+        float sc[kFrom == kFromWords ? 1 : kScoresEach][kHeadsEach];
+        // tokens whose scores this CTA needs
+        const int32_t n_scores = kPages || books || (blk + 1) * kBlockTokens > a.n_tokens ? static_cast<int32_t>(a.n_tokens) : (blk + 1) * kBlockTokens;
+        if constexpr (kFrom == kFromWords) {
 #pragma unroll
-        for (int k = 0; k < kWordsEach; ++k) w[k] = tid + k * kThreads < total ? __ldcg(words + tid + k * kThreads) : 0u;
+            for (int k = 0; k < kWordsEach; ++k) w[k] = tid + k * kThreads < total ? __ldcg(words + tid + k * kThreads) : 0u;
+        }
+        auto load_scores = [&](int32_t t0) {
+#pragma unroll
+            for (int k = 0; k < kScoresEach; ++k) {
+                const int32_t t = t0 + tid + k * kThreads;
+                const float *src = a.scores + static_cast<int64_t>(t) * H;
+                if constexpr (kPages) {
+                    if (H == kMaxHeads && t < n_scores) {
+                        const float4 x = __ldcg(reinterpret_cast<const float4 *>(src)), y = __ldcg(reinterpret_cast<const float4 *>(src) + 1);
+                        sc[k][0] = x.x; sc[k][1] = x.y; sc[k][2] = x.z; sc[k][3] = x.w;
+                        sc[k][4] = y.x; sc[k][5] = y.y; sc[k][6] = y.z; sc[k][7] = y.w;
+                    } else {
+#pragma unroll
+                        for (int i = 0; i < kHeadsEach; ++i) sc[k][i] = i < H && t < n_scores ? __ldcg(src + i) : 0.0f;
+                    }
+                } else {
+                    sc[k][0] = t < n_scores ? __ldcg(src + h) : 0.0f;
+                }
+            }
+        };
+        if constexpr (kFrom == kFromScores) load_scores(0);
         int32_t start = 0, end = static_cast<int32_t>(a.n_tokens), base = 0, cursor = a.first_page, top = 0;
         int64_t list0 = static_cast<int64_t>(tid) * H;
         if (multi && tid < a.n_seqs) start = __ldg(a.cu_seqlens + tid);
@@ -841,15 +892,45 @@ compact_short_kernel(const ShortCompact a)
                 top = __ldcg(a.taken + 1);
             }
         }
+        if constexpr (kFrom == kFromWords) {
 #pragma unroll
-        for (int k = 0; k < kWordsEach; ++k)
-            if (tid + k * kThreads < total) s_words[tid + k * kThreads] = w[k];
+            for (int k = 0; k < kWordsEach; ++k)
+                if (tid + k * kThreads < total) s_words[tid + k * kThreads] = w[k];
+        }
+        float tau = a.tau;
+        if constexpr (kFrom == kFromScores && !kPages)
+            if (a.tau_list != nullptr && tid < a.n_seqs) tau = __ldcg(a.tau_list + tid * H + h);
+        if constexpr (kFrom == kFromScores && !kPages)
+            if (tid < a.n_seqs) s_tau[tid] = tau;
         if (tid < a.n_seqs) s_cu[tid] = start;
         if (tid == 0) s_cu[a.n_seqs] = end;
         if constexpr (kPages) {
             if (tid < n_lists) s_base[tid] = base;
             if (tid < a.n_seqs) s_list[tid] = list0 + h;
             if (tid == 0) { cursor_s = cursor; free_s = top > 0 ? top : 0; }
+        }
+        if constexpr (kFrom == kFromScores) {
+            __syncthreads();
+            for (int32_t t0 = 0;;) {
+#pragma unroll
+                for (int k = 0; k < kScoresEach; ++k) {
+                    const int32_t t = t0 + tid + k * kThreads, word = t / 32;
+                    if (word * 32 >= n_scores) break;               // the whole warp: no token of it is wanted
+                    const int b = multi ? seq_of_shared(s_cu, a.n_seqs, t) : 0;
+                    const bool valid = t < n_scores, in_window = t >= s_cu[b + 1] - a.window;
+#pragma unroll
+                    for (int i = 0; i < kHeadsEach; ++i) {
+                        const uint32_t bits = __ballot_sync(0xffffffffu, valid && (in_window || sc[k][i] >= (kPages ? a.tau : s_tau[b])));
+                        if (lane == 0 && (!kPages || i < H)) s_words[(kPages ? i * n_words : 0) + word] = bits;
+                    }
+                }
+                t0 += kScoresEach * kThreads;
+                if (t0 >= n_scores) break;
+                load_scores(t0);
+            }
+            // the words of a last block that are all past the end
+            for (int i = (n_scores + 31) / 32 + tid; i < (n_scores + kBlockTokens - 1) / kBlockTokens * 4; i += kThreads)
+                for (int j = 0; j < (kPages ? H : 1); ++j) s_words[j * n_words + i] = 0u;
         }
     }
     __syncthreads();
@@ -982,6 +1063,17 @@ compact_short_kernel(const ShortCompact a)
         return cursor_s + ordinal - (kAppend ? stack_s : 0);
     };
 
+    // given scores: this launch completes after the one ahead of it, whose scratch it clears
+    auto finish = [&]() {
+        if constexpr (kFrom == kFromScores) {
+            griddep_wait();
+            if (a.clear != nullptr) {
+                const int64_t n_ctas = (static_cast<int64_t>(a.n_blocks) * nz + 1) * H;
+                const int64_t cta = books ? n_ctas - H + h : (static_cast<int64_t>(blk) * nz + z) * H + h;
+                for (int64_t i = cta * kThreads + tid; i < a.clear_units; i += n_ctas * kThreads) a.clear[i] = make_uint4(0u, 0u, 0u, 0u);
+            }
+        }
+    };
     if (books) {
         for (int b = warp; b < a.n_seqs; b += kWarps) {
             const int64_t li = kPages ? s_list[b] : static_cast<int64_t>(b) * H + h;
@@ -1004,6 +1096,7 @@ compact_short_kernel(const ShortCompact a)
                         __ldcg(a.scores + (static_cast<int64_t>(s_cu[b + 1]) - n_win + i) * H + h);
             }
         }
+        finish();
         return;
     }
     if (keep) {
@@ -1036,6 +1129,7 @@ compact_short_kernel(const ShortCompact a)
                 }
             }
         }
+    finish();
 }
 
 }  // namespace kvzap

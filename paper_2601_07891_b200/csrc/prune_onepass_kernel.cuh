@@ -1,7 +1,7 @@
 // Algorithm 1 after the scoring step in ONE launch: threshold and window test, per-(sequence, head)
 // counts and prefix sums, ordered K/V gather (dense-ragged or paged).  This is the kernel behind
 // kvzap_prune_prefill, kvzap_prune_prefill_paged and kvzap_prune_prefill_topk, where the scores are
-// given and no scoring kernel runs beside the compaction.
+// given and no scoring kernel runs beside the compaction.  (Short inputs: compact_short_kernel.)
 //
 // A CTA owns a run of consecutive 128-token blocks and a group of heads (all eight, or four, two, one: see the
 // kernel), so a score is read by at most eight CTAs (out of L2 after the first).

@@ -1,6 +1,6 @@
-"""The compaction of short inputs on contexts that do not trust their producers, at the edges of what it takes (2048 mask words over all
-heads, 256 lists) and just beyond: prompts against the pruning of given scores, which is another kernel, chunks against the selection
-by score of their whole streams."""
+"""The kernel for short inputs, at the edges of what it takes (2048 mask words over all heads, 256 lists; 64 or, paged, 16 blocks of given
+scores) and just beyond: prompts of contexts that do not trust their producers and the pruning of given scores against the oracle,
+chunks against the selection by score of their whole streams."""
 import numpy as np
 import pytest
 import torch
@@ -13,8 +13,8 @@ pytestmark = pytest.mark.gpu
 TAU, W = 0.05, 16
 
 
-def _case(T, B, H, D, seed):
-    ctx = binding.Kvzap(128, 64, H, D, 1, max_tokens=T, max_seqs=B)
+def _case(T, B, H, D, seed, trusted=False):
+    ctx = binding.Kvzap(128, 64, H, D, 1, max_tokens=T, max_seqs=B, trusted_producers=trusted)
     ctx.set_weights(0, *synth.mlp_weights(128, 64, H, seed, "cuda", 0.1))
     rng = np.random.default_rng(seed)
     ends = np.sort(rng.integers(0, T + 1, B - 1))           # empty sequences among them
@@ -22,34 +22,39 @@ def _case(T, B, H, D, seed):
     return ctx, synth.hidden_states(T, 128, seed, "cuda"), cu
 
 
-@pytest.mark.parametrize("T,B,H,D", [(1, 1, 8, 64), (129, 3, 8, 128), (8192, 1, 8, 64), (8192, 32, 8, 40), (8193, 1, 8, 64), (2000, 33, 8, 64),
-                                     (65536, 5, 1, 64), (5000, 255, 1, 64), (4000, 7, 3, 512), (3001, 2, 5, 72)])
-@pytest.mark.parametrize("tok_major", [False, True])
-def test_prompts(T, B, H, D, tok_major):
-    ctx, X, cu = _case(T, B, H, D, T + B)
+@pytest.mark.parametrize("T,B,H,D", [(1, 1, 8, 64), (129, 3, 8, 128), (300, 1, 8, 64), (2048, 2, 8, 64), (2049, 7, 8, 64), (8192, 1, 8, 64),
+                                     (8192, 32, 8, 40), (8193, 1, 8, 64), (2000, 33, 8, 64), (65536, 5, 1, 64), (5000, 255, 1, 64),
+                                     (4000, 7, 3, 512), (3001, 2, 5, 72)])
+@pytest.mark.parametrize("how", ["head major", "token major", "given scores", "given scores, trusted"])
+def test_prompts(oracle, T, B, H, D, how):
+    ctx, X, cu = _case(T, B, H, D, T + B, "trusted" in how)
     K, V = synth.keys_values(H, T, D, 3, "cuda")
+    tok_major = how == "token major"
     Ki, Vi = (x.transpose(0, 1).contiguous() if tok_major else x for x in (K, V))
-    P = 16
+    P, first = 16, 2
     pages, max_pages = H * (T // P + B + 1), T // P + 2
-    outs = []
-    for fused in (True, False):
-        s = torch.zeros(T, H, device="cuda") if fused else outs[0][0]
-        Ko, Vo = parity.poison_like(K), parity.poison_like(V)
-        n = torch.full((B, H), -1, dtype=torch.int32, device="cuda")
-        Kp, Vp = (torch.full((pages, P, D), 3.0, dtype=torch.bfloat16, device="cuda") for _ in range(2))
-        table, np_, used = torch.full((B * H, max_pages), -1, dtype=torch.int32, device="cuda"), n.clone(), n.new_zeros(1)
-        if fused:
-            (binding.kvzap_prefill_write if tok_major else binding.kvzap_prefill_fused)(ctx.handle, 0, X, Ki, Vi, cu, B, TAU, W, Ko, Vo, n, s)
-            (binding.kvzap_prefill_write_paged if tok_major else binding.kvzap_prefill_fused_paged)(
-                ctx.handle, 0, X, Ki, Vi, cu, B, TAU, W, Kp, Vp, P, 2, table, np_, used, s)
-        else:
-            binding.kvzap_prune_prefill(ctx.handle, K, V, s, cu, B, TAU, W, Ko, Vo, n)
-            binding.kvzap_prune_prefill_paged(ctx.handle, K, V, s, cu, B, TAU, W, Kp, Vp, P, 2, table, np_, used)
-        torch.cuda.synchronize()
-        assert ctx.poll_status() == 0
-        outs.append([s, n, Ko.view(torch.int16), Vo.view(torch.int16), np_, table, used, Kp.view(torch.int16), Vp.view(torch.int16)])
-    for a, b in zip(*outs):
-        assert torch.equal(a, b)
+    s = torch.randn(T, H, generator=torch.Generator(device="cuda").manual_seed(T), device="cuda")
+    Ko, Vo = parity.poison_like(K), parity.poison_like(V)
+    n = torch.full((B, H), -1, dtype=torch.int32, device="cuda")
+    Kp, Vp = (torch.full((pages, P, D), -5.0, dtype=torch.bfloat16, device="cuda") for _ in range(2))
+    table, n_paged, used = torch.full((B * H, max_pages), -1, dtype=torch.int32, device="cuda"), n.clone(), torch.zeros(1, dtype=torch.int32, device="cuda")
+    h = ctx.handle
+    if how.startswith("given"):
+        binding.kvzap_prune_prefill(h, K, V, s, cu, B, TAU, W, Ko, Vo, n)
+        binding.kvzap_prune_prefill_paged(h, K, V, s, cu, B, TAU, W, Kp, Vp, P, first, table, n_paged, used)
+    else:
+        (binding.kvzap_prefill_write if tok_major else binding.kvzap_prefill_fused)(h, 0, X, Ki, Vi, cu, B, TAU, W, Ko, Vo, n, s)
+        (binding.kvzap_prefill_write_paged if tok_major else binding.kvzap_prefill_fused_paged)(
+            h, 0, X, Ki, Vi, cu, B, TAU, W, Kp, Vp, P, first, table, n_paged, used, s)
+    torch.cuda.synchronize()
+    assert ctx.poll_status() == 0
+    cu_np = cu.cpu().numpy() if cu is not None else None
+    keep, _ = parity.check_compaction(oracle, K, V, s.cpu().numpy(), TAU, W, cu_np, Ko, Vo, n)
+    fill = int(synth.bits(torch.tensor([-5.0], dtype=torch.bfloat16))[0])
+    want = oracle.compact_paged(synth.bits(K), synth.bits(V), keep, P, pages, max_pages, cu_seqlens=cu_np, first_page=first, fill=fill)
+    for got, ref in zip((synth.bits(Kp), synth.bits(Vp), table.cpu().numpy(), n_paged.cpu().numpy()), want[:4]):
+        np.testing.assert_array_equal(got, ref)
+    assert int(used) == want[4]
     ctx.close()
 
 
