@@ -15,6 +15,8 @@
 // a few long sequences), each list is cut into n_parts equal runs of tiles, one CTA each; the parts
 // leave their triples in global memory and the part that arrives last (a counter per list) merges
 // them in part order, so the result does not depend on which one that was.
+// Of a call of many lists the last ones have more parts than the others: the device takes CTAs in order, and a long list among the
+// last would be worked on when all others are done.
 // With fewer lists than resident CTAs (a small batch, layer by layer) there is one wave, and it lasts as
 // long as its longest part: equal parts of lists whose lengths spread over 1 : 7 (contexts of one batch x
 // what each head keeps) leave most of it idle.  There the CTAs share the lists out themselves (attn_unit):
@@ -89,6 +91,9 @@ struct AttnParams {
     int32_t n_parts;            // CTAs per list (1 = the CTA writes the output itself); 0 = by length, see attn_unit
     float *part_scratch;        // [CTA] { m[8], l[8], O[8][D] }: the parts of a list are consecutive CTAs
     uint32_t *part_arrive;      // [list] parts that have stored their triple; back to 0 after the launch
+    // n_parts > 0: the lists from head_lists on have tail_parts CTAs each, or as many as leave a CTA kAttnTailTiles tiles
+    int32_t head_lists, tail_parts;
+    int32_t unit0, list0;       // CTA and list of part_scratch[0] and part_arrive[0]
     int32_t beside_ctas;        // kBeside: CTAs [0, beside_ctas) run beside the step, as many as find room
     int32_t beside_tiles;       // n_parts == 0: with more tiles than this in all lists all CTAs wait for the step
 };
@@ -100,6 +105,7 @@ struct AttnParams {
 // into, 0 if there is no such unit; `list` and `part` say which.
 constexpr int kAttnListsPerLane = 20;       // n <= 32 * this
 constexpr float kAttnMinPart = 16.0f;       // tiles
+constexpr int kAttnTailTiles = 40;          // a part of the lists at the end of a launch of many, at least
 __device__ __forceinline__ int attn_unit(const int32_t *lengths, int n, int n_units, int unit, int lane, int &list, int &part)
 {
     // lane l owns lists [l * per, (l + 1) * per), in registers
@@ -250,12 +256,23 @@ decode_attn_kernel(const __grid_constant__ CUtensorMap tmap_kpool, const __grid_
         return (static_cast<int64_t>((i / H) % B) * c.n_layers + p.layer0 + i / (H * B)) * H + i % H;
     };
     if (n_parts > 0) {
-        list = blockIdx.x / n_parts;
-        part = blockIdx.x % n_parts;
+        const int head_ctas = p.head_lists * n_parts, at = static_cast<int>(blockIdx.x) - head_ctas;
+        const bool tail = at >= 0;
+        if (tail) n_parts = p.tail_parts;
+        list = tail ? p.head_lists + at / n_parts : static_cast<int>(blockIdx.x) / n_parts;
+        part = tail ? at % n_parts : static_cast<int>(blockIdx.x) % n_parts;
         if (kBeside) n_before = min(__ldcg(before + cache_list(list)), __ldcg(c.prefix_len + cache_list(list)));
         if (!beside) {
             n_total = __ldcg(c.n_tokens + cache_list(list));
             n_prefix = __ldcg(c.prefix_len + cache_list(list));
+        }
+        if (tail) {
+            const int tiles = ((kBeside ? n_before : n_prefix) + min(kBeside ? c.window : n_total, c.window)) / kAttnTileRows;
+            n_parts = min(n_parts, max(1, tiles / kAttnTailTiles));
+            if (part >= n_parts) {                                 // the whole CTA
+                if (beside) griddep_wait();
+                return;
+            }
         }
     } else {
         // over the stages, not in use yet: [list] tiles, then [list] (prefix rows, tokens); kBeside: the window counts in full
@@ -757,7 +774,7 @@ decode_attn_kernel(const __grid_constant__ CUtensorMap tmap_kpool, const __grid_
         n_parts = kept_s[warp][kParts];
     }
     constexpr int kUnit = 16 + kAttnMaxGroup * kD;
-    float *unit = n_parts > 1 ? p.part_scratch + static_cast<int64_t>(blockIdx.x) * kUnit : nullptr;
+    float *unit = n_parts > 1 ? p.part_scratch + static_cast<int64_t>(static_cast<int>(blockIdx.x) - p.unit0) * kUnit : nullptr;
     // four elements of one query head per thread
     for (int idx = threadIdx.x; idx < p.group * (kD / 4); idx += kAttnThreads) {
         const int gq = idx / (kD / 4), d = idx % (kD / 4) * 4;
@@ -791,10 +808,10 @@ decode_attn_kernel(const __grid_constant__ CUtensorMap tmap_kpool, const __grid_
     // ---- several CTAs per list: the one that arrives last merges all parts, in part order
     __shared__ int last_s;
     __syncthreads();
-    if (threadIdx.x == 0) last_s = arrive_last_acq_rel(p.part_arrive + list, static_cast<uint32_t>(n_parts));
+    if (threadIdx.x == 0) last_s = arrive_last_acq_rel(p.part_arrive + (list - p.list0), static_cast<uint32_t>(n_parts));
     __syncthreads();
     if (!last_s) return;
-    const float *units = p.part_scratch + static_cast<int64_t>(blockIdx.x - part) * kUnit;
+    const float *units = p.part_scratch + static_cast<int64_t>(static_cast<int>(blockIdx.x) - part - p.unit0) * kUnit;
     constexpr int kBatch = 8;               // parts whose values are loaded together: one round trip to memory
     for (int idx = threadIdx.x; idx < p.group * (kD / 4); idx += kAttnThreads) {
         const int gq = idx / (kD / 4), d = idx % (kD / 4) * 4;
