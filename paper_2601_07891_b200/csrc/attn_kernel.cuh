@@ -29,9 +29,8 @@
 // that step reads all rows that the lists held before it while it runs; what the step changes (the prefix's last tile, the
 // window) is read when it has completed, and so are the queries, once more -- if they are not what they were, the CTA starts
 // again.  36 layers x 8 sequences x 2176 rows 1235 -> 855 to 900 us, 4 layers x 128 sequences x 4736 rows 1600 -> 1500 to 1545 us.
-// A warp waits for the step, and lets the next one start, when the last tile that it knows is about to be issued and two more
-// are in flight (behind all of them the copies ran dry, and the chain step - wait - next step was the longer by the time of two
-// tiles), the new lengths and the second look at the queries share a round trip, and the parts of a list are counted in by one
+// A warp waits for the step, and lets the next one start, while tiles are in flight (behind all of them the copies ran dry, and the
+// chain step - wait - next step was the longer by the time of two tiles; when it does: kWaitBase), the new lengths and the second look at the queries share a round trip, and the parts of a list are counted in by one
 // release instead of two fences: 36 layers x 8 sequences x 2176 rows 808 -> 740 us, 12 x 4 201 -> 193, 12 x 8 8-bit 279 -> 265, 12 x 32 8-bit
 // 419 -> 392 (with the steps of score_split_kernel's kFew on both sides).
 //
@@ -105,6 +104,15 @@ struct AttnParams {
 // into, 0 if there is no such unit; `list` and `part` say which.
 constexpr int kAttnListsPerLane = 20;       // n <= 32 * this
 constexpr float kAttnMinPart = 16.0f;       // tiles
+// Beside a step, in one wave: cycles from a CTA's start to its wait for that step, with it the start of the next one, as a base and by
+// its tiles of 128 elements.  The step is over by then, and the next one, its launch and the next attention's first CTAs (on the SMs
+// that the steps use) are there when this launch ends; earlier the wait would be one, later the memory idles between the two.  Us, 12
+// layers, waiting at the last known tile / at this time / a quarter of the tiles' share earlier / later: 16 sequences x 2176 rows 402 /
+// 359 / 361 / 356, 32 x 2176 765 / 636 / 643 / 639, 12 x 1628 263 / 247 / 248 / 248, 4 x 7628 346 / 322 / 326 / 320; 8-bit 32 x 1152 402 / 357 / 363 /
+// 365, 16 x 2176 349 / 317 / 314 / 328, 30 x 2378 619 / 533 / 551 / 540, 8 x 2176 260 / 263 / 263 / 261; 36 layers, 8 x 2176 730 / 698 / 698 / 702.
+// (When half of the tiles are issued, whatever the clock: 361, 640, 248, 323; 366, 321, 542, 257; 693.)  Not with several waves: 512 lists
+// of 1128 rows 263 / 271.
+constexpr int kWaitBase = 12000, kWaitTile = 270, kWaitTile8 = 400;
 constexpr int kAttnTailTiles = 40;          // a part of the lists at the end of a launch of many, at least
 __device__ __forceinline__ int attn_unit(const int32_t *lengths, int n, int n_units, int unit, int lane, int &list, int &part)
 {
@@ -227,6 +235,7 @@ decode_attn_kernel(const __grid_constant__ CUtensorMap tmap_kpool, const __grid_
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const CacheView &c = p.c;
     const int H = c.n_heads, B = c.n_seqs;
+    const clock_t started = kBeside ? clock() : 0;
 
     __shared__ int queries_s;               // kBeside: warps that are done with the queries in memory
     if (threadIdx.x == 0) {
@@ -550,9 +559,11 @@ decode_attn_kernel(const __grid_constant__ CUtensorMap tmap_kpool, const __grid_
         again = false;
     }
     for (; s < n_tiles; s += kAttnWarps) {
-        if (kBeside && !waited && s_issue < n_tiles && s_issue + kAttnWarps >= n_tiles) {
-            // the last of the tiles known beside the kernel ahead is about to be issued: what comes next is learnt while those
-            // in flight are worked on
+        if (kBeside && !waited && s_issue < n_tiles &&
+            (s_issue + kAttnWarps >= n_tiles ||
+             (p.n_parts == 0 && clock() - started > kWaitBase + (kFp8 ? kWaitTile8 : kWaitTile) * kD / 128 * n_early))) {
+            // time for the next step to start (see kWaitBase), or the last of the tiles known beside the kernel ahead is about to
+            // be issued: what comes next is learnt while those in flight are worked on
             wait_for_rest();
             if (again) {                                  // no copy may be in flight then
                 for (int d = s; ok && d < s_issue; d += kAttnWarps) {
