@@ -520,7 +520,7 @@ score_split_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_cons
             if constexpr (kFp8)
                 if (p.x_scale != nullptr && token < p.n_tokens) sx = __ldg(p.x_scale + static_cast<int64_t>(l_rel) * p.n_tokens + token);
 #pragma unroll 1
-            for (int j = 2 * pair; j < own_n; j += 16) {
+            for (int j = 2 * pair; ok && j < own_n; j += 16) {
                 float z0 = 0.0f, z1 = 0.0f;                     // the parts in rank order
 #pragma unroll 4
                 for (int part_i = 0; part_i < k_split; ++part_i) {
