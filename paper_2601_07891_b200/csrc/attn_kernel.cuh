@@ -93,6 +93,7 @@ struct AttnParams {
     // n_parts > 0: the lists from head_lists on have tail_parts CTAs each, or as many as leave a CTA kAttnTailTiles tiles
     int32_t head_lists, tail_parts;
     int32_t unit0, list0;       // CTA and list of part_scratch[0] and part_arrive[0]
+    int32_t tiles_shift;        // logarithm of the tiles per page, or -1
     int32_t beside_ctas;        // kBeside: CTAs [0, beside_ctas) run beside the step, as many as find room
     int32_t beside_tiles;       // n_parts == 0: with more tiles than this in all lists all CTAs wait for the step
 };
@@ -342,7 +343,11 @@ decode_attn_kernel(const __grid_constant__ CUtensorMap tmap_kpool, const __grid_
     }
     const int s_first = kBeside ? 0 : t_first;
     // kBeside, per warp, in shared memory for want of registers: what the main loop seldom needs
-    enum { kTail, kRing, kList, kPart, kParts, kFull, kKept };      // rows of the prefix's end and of the window; the rest as above
+    // rows of the prefix's end and of the window; the list among the cache's; the rest as above.  What can be looked up here is not
+    // worked out again: code that is run once is waited for (ncu: of a warp's cycles per instruction here 3.9 went by for want of
+    // the next instruction, 1.8 for memory).  With page numbers by a shift where that can be, us: 36 layers x 8 sequences x 2176 rows 705 -> 693,
+    // 12 x 32 x 1152 8-bit rows 356 -> 339, x 30 x 2378 531 -> 497; 12 layers in one call x 64 x 1664 507 -> 495
+    enum { kTail, kRing, kCacheList, kList, kPart, kParts, kFull, kKept };
     __shared__ volatile int32_t kept_s[kAttnWarps][kKept];
     bool waited = !beside;
     auto learn_rest = [&](int32_t tokens, int32_t rows) {          // whole warp, once
@@ -367,6 +372,7 @@ decode_attn_kernel(const __grid_constant__ CUtensorMap tmap_kpool, const __grid_
     if constexpr (kBeside) {
         if (lane == 0) {
             kept_s[warp][kList] = list;
+            kept_s[warp][kCacheList] = static_cast<int32_t>(cache_list(list));
             kept_s[warp][kPart] = part;
             kept_s[warp][kParts] = n_parts;
             kept_s[warp][kFull] = n_before / kAttnTileRows;
@@ -383,13 +389,16 @@ decode_attn_kernel(const __grid_constant__ CUtensorMap tmap_kpool, const __grid_
     auto tile_at = [&](int s) -> int32_t {
         if (s < n_early) return t_first + s;
         int32_t row, left;
-        if (rest_tile(s, row, left)) return -1 - (static_cast<int32_t>(cache_list(kept_s[warp][kList]) * c.window) + row);
+        if (rest_tile(s, row, left)) return -1 - (kept_s[warp][kCacheList] * c.window + row);
         return kept_s[warp][kFull] + row / kAttnTileRows;
     };
     // the page that a prefix tile is in, and its first row (in its tensor map) from there; apart, so that the loads of several
     // tiles go out together
-    auto page_of = [&](int32_t t) -> int32_t { return t >= 0 ? __ldcg(pages + t / tiles_per_page) : 0; };
-    auto row_of = [&](int32_t t, int32_t page) { return t >= 0 ? page * c.page_tokens + (t % tiles_per_page) * kAttnTileRows : t; };
+    auto page_index = [&](int32_t t) -> int32_t { return p.tiles_shift >= 0 ? t >> p.tiles_shift : t / tiles_per_page; };
+    auto page_of = [&](int32_t t) -> int32_t { return t >= 0 ? __ldcg(pages + page_index(t)) : 0; };
+    auto row_of = [&](int32_t t, int32_t page) {
+        return t >= 0 ? page * c.page_tokens + (t - page_index(t) * tiles_per_page) * kAttnTileRows : t;
+    };
     // first row (in its tensor map) of tile s; needs the page number for prefix tiles.  kBeside: rows of the rings as -1 - row
     auto tile_row = [&](int s) -> int32_t {
         if constexpr (kBeside) {
@@ -397,8 +406,8 @@ decode_attn_kernel(const __grid_constant__ CUtensorMap tmap_kpool, const __grid_
             return row_of(t, page_of(t));
         } else {
             if (s < n_pt) {
-                const int32_t page = __ldcg(pages + s / tiles_per_page);
-                return page * c.page_tokens + (s % tiles_per_page) * kAttnTileRows;
+                const int32_t pi = page_index(s), page = __ldcg(pages + pi);
+                return page * c.page_tokens + (s - pi * tiles_per_page) * kAttnTileRows;
             }
             return ring_row0 + (s - n_pt) * kAttnTileRows;
         }
@@ -454,8 +463,7 @@ decode_attn_kernel(const __grid_constant__ CUtensorMap tmap_kpool, const __grid_
     // k-step ks covers columns c D/4 + 4 ks ..+3
     const int g = lane >> 2, qc = (lane & 3) * 2;
     auto query_row = [&]() {                // of the list's first query head, in `q` and `out`
-        const int list_now = kBeside ? static_cast<int>(kept_s[warp][kList]) : list, l_rel = list_now / (H * B), b = (list_now / H) % B;
-        return (static_cast<int64_t>(l_rel) * B + b) * H * p.group + list_now % H * p.group;
+        return static_cast<int64_t>(kBeside ? static_cast<int>(kept_s[warp][kList]) : list) * p.group;
     };
     // kBeside has no registers to keep it in
     const int64_t row0 = kBeside ? 0 : query_row();
@@ -538,7 +546,7 @@ decode_attn_kernel(const __grid_constant__ CUtensorMap tmap_kpool, const __grid_
     uint32_t parity = 0;
     auto wait_for_rest = [&]() {            // whole warp: the end of the kernel ahead, and what it has left to be read
         griddep_wait();
-        const int64_t li = cache_list(kept_s[warp][kList]);
+        const int32_t li = kept_s[warp][kCacheList];
         const int32_t tokens = __ldcg(c.n_tokens + li), rows = __ldcg(c.prefix_len + li);      // on their way beside the queries
         again = query_changed();           // then all of them once more
         if (!again) queries_taken();

@@ -2901,6 +2901,9 @@ static kvzap_status attention_impl(kvzap_ctx *ctx, kvzap_cache *cache, int32_t l
             p.list0 = p.head_lists;
         }
     }
+    p.tiles_shift = -1;
+    for (int i = 0; i < 31; ++i)
+        if (v.page_tokens / kAttnTileRows == 1 << i) p.tiles_shift = i;
     p.part_scratch = cache->attn_scratch;
     p.part_arrive = cache->attn_arrive;
     {
