@@ -437,7 +437,7 @@ compact_kernel(const uint4 *__restrict__ K, const uint4 *__restrict__ V, uint4 *
             int64_t dst;
             if constexpr (kPaged) {
                 const int32_t p0 = list_page0[b * n_heads + h];
-                dst = p0 < 0 ? -1 : (static_cast<int64_t>(p0) + n / page_tokens) * page_tokens + n % page_tokens;
+                dst = p0 < 0 ? -1 : static_cast<int64_t>(p0) * page_tokens + n;                 // pages in a row
             } else {
                 dst = static_cast<int64_t>(h) * n_tokens + seq_start + n;
             }
@@ -688,15 +688,16 @@ compact_dense_kernel(const uint4 *__restrict__ K, const uint4 *__restrict__ V, u
                     if (paged) {
                         const int32_t p0 = assign.enabled ? s_page0[b * n_heads + h] : __ldcg(list_page0 + b * n_heads + h);
                         if (list_base == nullptr) {
-                            dst_row[r] = p0 < 0 ? -1 : (static_cast<int64_t>(p0) + n / page_tokens) * page_tokens + n % page_tokens;
+                            dst_row[r] = p0 < 0 ? -1 : static_cast<int64_t>(p0) * page_tokens + n;      // pages in a row
                         } else {
-                            const int64_t nn = __ldcg(list_base + b * n_heads + h) + n;
+                            const uint32_t nn = static_cast<uint32_t>(__ldcg(list_base + b * n_heads + h) + static_cast<int32_t>(n));
+                            const uint32_t pi = nn / static_cast<uint32_t>(page_tokens);
                             if (p0 < 0) {
                                 dst_row[r] = -1;
                             } else {
                                 const int64_t trow = list_map != nullptr ? __ldcg(list_map + b) + h : static_cast<int64_t>(b * n_heads + h);
-                                const int64_t page = __ldcg(page_table + trow * max_pages + nn / page_tokens);
-                                dst_row[r] = page * page_tokens + nn % page_tokens;
+                                const int64_t page = __ldcg(page_table + trow * max_pages + pi);
+                                dst_row[r] = page * page_tokens + (nn - pi * static_cast<uint32_t>(page_tokens));
                             }
                         }
                     } else {

@@ -208,7 +208,7 @@ prune_onepass_kernel(const PruneParams p)
 
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const int H = p.n_heads;
-    const int HG = p.heads_per_cta;
+    const int HG = p.heads_per_cta, hg_shift = __ffs(HG) - 1;          // 8, 4, 2 or 1
     const int c = static_cast<int>(blockIdx.x), g = static_cast<int>(blockIdx.y);
     const int h0 = g * HG;
     auto own = [&](int h) -> bool { return h >= h0 && h < h0 + HG && h < H; };
@@ -217,7 +217,7 @@ prune_onepass_kernel(const PruneParams p)
     const bool multi = p.cu_seqlens != nullptr && p.n_seqs > 1;
     const bool paged = p.page_tokens > 0;
     const uint64_t tag = static_cast<uint64_t>(static_cast<uint32_t>(p.epoch)) << 32;
-    const int smem_blocks = kOpSmemWords / HG;            // blocks whose words stay in shared memory
+    const int smem_blocks = kOpSmemWords >> hg_shift;            // blocks whose words stay in shared memory
 
     if (tid < kMaxHeads) { cnt_s[tid] = 0; part_s[tid] = 0; }
     if (tid == 0) flag_s = 0;
@@ -242,7 +242,7 @@ prune_onepass_kernel(const PruneParams p)
         griddep_launch_dependents();
     }
     if (tid < kMaxHeads) tau_s[tid] = p.tau_list != nullptr && tid < H ? __ldcg(p.tau_list + b_lo * H + tid) : p.tau;
-    const int j0 = static_cast<int>((s0 / kBlockTokens) / p.blocks_per_cta);      // the CTA (column) whose blocks hold s0
+    const int j0 = static_cast<int>(s0 / kBlockTokens) / p.blocks_per_cta;      // the CTA (column) whose blocks hold s0
     __syncthreads();
 
     // ---------------------------------------------------------------- A: keep bits and counts of the CTA's blocks
@@ -446,7 +446,7 @@ prune_onepass_kernel(const PruneParams p)
     const int group = tid >> 4, gl = tid & 15;
     constexpr int kGroups = kOpThreads / 16;
     constexpr int kStep = kGroups * kRows;
-    const int sb_blocks = kOpPairs / HG;
+    const int sb_blocks = kOpPairs >> hg_shift;
     const int64_t row_bytes = static_cast<int64_t>(p.row_units) * 16;
     const char *Kb = reinterpret_cast<const char *>(p.K), *Vb = reinterpret_cast<const char *>(p.V);
     char *Ko = reinterpret_cast<char *>(p.K_out), *Vo = reinterpret_cast<char *>(p.V_out);
@@ -454,7 +454,7 @@ prune_onepass_kernel(const PruneParams p)
         const int nb = static_cast<int>(blk1 - sb0 < sb_blocks ? blk1 - sb0 : sb_blocks);
         const int64_t sb_start = sb0 * kBlockTokens;
         if (tid < 32) {                                         // one warp; lanes beyond the pairs count nothing
-            const int bl = tid / HG, hh = tid % HG, h = h0 + hh;
+            const int bl = tid >> hg_shift, hh = tid & (HG - 1), h = h0 + hh;
             uint4 w = make_uint4(0u, 0u, 0u, 0u);
             if (tid < kOpPairs && bl < nb && h < H)
                 w = sb0 - blk0 + bl < smem_blocks
@@ -494,7 +494,7 @@ prune_onepass_kernel(const PruneParams p)
         int bl_seq = -1, b = 0;
         int64_t s = 0, e = p.n_tokens;
         for (int pi = half; pi < kOpPairs; pi += 2) {
-            const int bl = pi / HG, hh = pi % HG, h = h0 + hh;
+            const int bl = pi >> hg_shift, hh = pi & (HG - 1), h = h0 + hh;
             if (bl >= nb || h >= H) continue;
             const int64_t t = sb_start + bl * kBlockTokens + tok;
             if (t >= p.n_tokens) continue;
