@@ -244,6 +244,42 @@ score_linear_split_kernel(const __grid_constant__ CUtensorMap tmap_x, const __gr
                             __popc(wt_s[threadIdx.x][3]);
             st_relaxed_gpu_u64(fc.tile_counts + tile * kMaxHeads + threadIdx.x, tag | static_cast<uint32_t>(cnt));
         }
+        // this CTA's quarter of the tile: tokens 32 * rank .. + 31, all heads; its kept rows listed by (head, token)
+        const int64_t t_q0 = static_cast<int64_t>(m_tile) * kTileM + rank * 32;
+        int n_rows = 0;
+        for (int h = 0; h < p.n_heads; ++h) n_rows += __popc(wt_s[h][rank]);
+        for (int pi = threadIdx.x; pi < p.n_heads * 32; pi += kLinThreads) {
+            const int h = pi >> 5, tk = pi & 31;
+            const uint32_t w = wt_s[h][rank];
+            if ((w >> tk) & 1u) {
+                int idx = __popc(w & ((1u << tk) - 1u));
+                for (int hh = 0; hh < h; ++hh) idx += __popc(wt_s[hh][rank]);
+                ent_src_s[idx] = (h * fc.in_stride_h + (t_q0 + tk) * fc.in_stride_t) * fc.row_bytes;
+            }
+        }
+        __syncthreads();
+        // rows travel global -> the idle pipeline stages (and the partial sums behind them, summed up by now) -> global; as
+        // many per round as they hold: 96 rows of 256 bytes, where a quarter of a tile keeps 85 on average
+        const int cap = static_cast<int>(bars_off / (2u * fc.row_bytes));
+        // as asynchronous 16-byte copies into shared memory (they pass by the L1 and the registers, so the rows of
+        // a round are all in flight at once), 16 lanes per row, then ordinary loads from there and stores
+        const int group = threadIdx.x >> 4, gl = threadIdx.x & 15;
+        auto load_rows = [&](int c0) {
+            const int n_chunk = n_rows - c0 < cap ? n_rows - c0 : cap;
+            for (int i = group; i < n_chunk; i += kLinThreads / 16) {
+                const uint32_t slot = smem_base + static_cast<uint32_t>(i) * 2u * fc.row_bytes;
+                const int64_t src = ent_src_s[c0 + i];
+                for (uint32_t u = gl * 16u; u < static_cast<uint32_t>(fc.row_bytes); u += 256u) {
+                    asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(slot + u), "l"(fc.K + src + u) : "memory");
+                    asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(slot + fc.row_bytes + u), "l"(fc.V + src + u) : "memory");
+                }
+            }
+            asm volatile("cp.async.commit_group;" ::: "memory");
+        };
+        // Which rows they are is known now, where they go only when the tiles before have said how many they keep: the first
+        // round's loads go out ahead of that (us a layer, calls in a row: 300 tokens 6.3 -> 6.0, 8100 16.1 -> 15.7; default contexts 4000 25.6 ->
+        // 24.5, 8000 30.1 -> 28.6)
+        load_rows(0);
         // rows kept before this tile: the counts of the tiles before it (every CTA of the cluster adds them up itself)
         {
             int32_t acc[kMaxHeads];
@@ -286,23 +322,20 @@ score_linear_split_kernel(const __grid_constant__ CUtensorMap tmap_x, const __gr
         }
         if (*abort_flag == 2) {                             // a tile before this one never published: nothing is moved
             if (threadIdx.x == 0) atomicCAS(p.status, 0, 5 /* KVZAP_ERR_TIMEOUT */);
+            asm volatile("cp.async.wait_group 0;" ::: "memory");
             griddep_wait();
             return;
         }
-        // this CTA's quarter of the tile: tokens 32 * rank .. + 31, all heads; its kept rows listed by (head, token)
-        const int64_t t_q0 = static_cast<int64_t>(m_tile) * kTileM + rank * 32;
-        int n_rows = 0;
-        for (int h = 0; h < p.n_heads; ++h) n_rows += __popc(wt_s[h][rank]);
+        // where those rows go
         for (int pi = threadIdx.x; pi < p.n_heads * 32; pi += kLinThreads) {
             const int h = pi >> 5, tk = pi & 31;
             const uint32_t w = wt_s[h][rank];
             if ((w >> tk) & 1u) {
-                int idx = __popc(w & ((1u << tk) - 1u)), before = 0;
+                const int at = __popc(w & ((1u << tk) - 1u));
+                int idx = at, before = 0;
                 for (int hh = 0; hh < h; ++hh) idx += __popc(wt_s[hh][rank]);
                 for (uint32_t qq = 0; qq < rank; ++qq) before += __popc(wt_s[h][qq]);
-                const int64_t n = run_s[h] + before + __popc(w & ((1u << tk) - 1u));          // rank inside head h's list
-                ent_src_s[idx] = (h * fc.in_stride_h + (t_q0 + tk) * fc.in_stride_t) * fc.row_bytes;
-                ent_dst_s[idx] = (static_cast<int64_t>(h) * p.n_tokens + n) * fc.row_bytes;
+                ent_dst_s[idx] = (static_cast<int64_t>(h) * p.n_tokens + run_s[h] + before + at) * fc.row_bytes;      // rank inside head h's list
             }
         }
         __syncthreads();
@@ -325,23 +358,9 @@ score_linear_split_kernel(const __grid_constant__ CUtensorMap tmap_x, const __gr
                 fc.lengths[h] = run_s[h] + __popc(wt_s[h][0]) + __popc(wt_s[h][1]) + __popc(wt_s[h][2]) + __popc(wt_s[h][3]);
             }
         };
-        // rows travel global -> the idle pipeline stages (and the partial sums behind them, summed up by now) -> global; as
-        // many per round as they hold: 96 rows of 256 bytes, where a quarter of a tile keeps 85 on average
-        const int cap = static_cast<int>(bars_off / (2u * fc.row_bytes));
-        // as asynchronous 16-byte copies into shared memory (they pass by the L1 and the registers, so the rows of
-        // a round are all in flight at once), 16 lanes per row, then ordinary loads from there and stores
-        const int group = threadIdx.x >> 4, gl = threadIdx.x & 15;
         for (int c0 = 0; c0 == 0 || c0 < n_rows; c0 += cap) {
             const int n_chunk = n_rows - c0 < cap ? n_rows - c0 : cap;
-            for (int i = group; i < n_chunk; i += kLinThreads / 16) {
-                const uint32_t slot = smem_base + static_cast<uint32_t>(i) * 2u * fc.row_bytes;
-                const int64_t src = ent_src_s[c0 + i];
-                for (uint32_t u = gl * 16u; u < static_cast<uint32_t>(fc.row_bytes); u += 256u) {
-                    asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(slot + u), "l"(fc.K + src + u) : "memory");
-                    asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(slot + fc.row_bytes + u), "l"(fc.V + src + u) : "memory");
-                }
-            }
-            asm volatile("cp.async.commit_group;" ::: "memory");
+            if (c0 > 0) load_rows(c0);
             if (c0 == 0) {
                 // the first round's rows are on their way; outputs may be in use by the work ahead up to here
                 if (p.wait_before_write == 2) griddep_wait();
