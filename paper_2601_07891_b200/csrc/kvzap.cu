@@ -895,8 +895,11 @@ static kvzap_status launch_score(kvzap_ctx *ctx, int32_t layer, int32_t n_layers
     // KVzap-Linear on few tiles (a short prompt, or a decode step): four CTAs share a tile, each a quarter
     // of the K range.  The kernel writes only after it has waited for the kernel ahead, so it may always
     // be placed early.
-    // (with the compaction in the same launch the CTAs are small enough for several per SM: up to kLinMaxTiles tiles)
-    const bool lin_one_launch = compact != nullptr && n_layers == 1 && n_seqs == 1 && maskbits != nullptr && window_keep == 1 &&
+    // (with the compaction in the same launch the CTAs are small enough for several per SM: up to kLinMaxTiles tiles.  Only on
+    // contexts that trust their producers, whose calls run beside one another: a call that waits for the one before is as long as its
+    // own chain, of two pipeline stages a CTA, look-back and rows, and longer than two launches'.  Default contexts, us a layer, one
+    // launch / two: 300 tokens 20.2 / 9.6, 1000 22.0 / 10.3, 2000 22.4 / 10.6, 4000 24.5 / 14.6, 6500 27.0 / 26.2, 8000 28.6 / 27.1.)
+    const bool lin_one_launch = compact != nullptr && ctx->trusted && n_layers == 1 && n_seqs == 1 && maskbits != nullptr && window_keep == 1 &&
                                 blocks_per_layer <= kLinMaxTiles && c.head_dim * 2 <= 2048;
     if (c.hidden == 0 && ctx->lin_split_ok &&
         (blocks_per_layer * n_layers * kLinSplit <= ctx->sm_count ||
