@@ -901,8 +901,13 @@ static kvzap_status launch_score(kvzap_ctx *ctx, int32_t layer, int32_t n_layers
     // launch / two: 300 tokens 20.2 / 9.6, 1000 22.0 / 10.3, 2000 22.4 / 10.6, 4000 24.5 / 14.6, 6500 27.0 / 26.2, 8000 28.6 / 27.1.)
     const bool lin_one_launch = compact != nullptr && ctx->trusted && n_layers == 1 && n_seqs == 1 && maskbits != nullptr && window_keep == 1 &&
                                 blocks_per_layer <= kLinMaxTiles && c.head_dim * 2 <= 2048;
+    // A prompt that runs beside nothing takes it with up to two CTAs of fewer stages per SM as well, as long as a quarter of the SMs
+    // have one only: default contexts, us a layer, one CTA per tile / this: 5000 tokens 25.6 / 18.7, 6500 26.1 / 21.5, 8000 27.0 / 24.2, 9400
+    // (296 CTAs) 28.8 / 31.3; with three per SM 10000 tokens 30.1 / 29.3, 14000 37.7 / 40.9.
+    const int64_t lin_ctas = blocks_per_layer * n_layers * kLinSplit;
+    const int lin_per_sm = !ctx->trusted && n_layers == 1 && lin_ctas > ctx->sm_count && 4 * lin_ctas <= 7 * ctx->sm_count ? 2 : 1;
     if (c.hidden == 0 && ctx->lin_split_ok &&
-        (blocks_per_layer * n_layers * kLinSplit <= ctx->sm_count ||
+        (lin_ctas <= lin_per_sm * ctx->sm_count ||
          (lin_one_launch && blocks_per_layer * kLinSplit <= 2 * static_cast<int64_t>(ctx->sm_count)))) {
         CUtensorMap tmap_x;
         kvzap_status st = hidden_tmap(ctx, &tmap_x, hidden, n_tokens, n_layers);
@@ -948,7 +953,8 @@ static kvzap_status launch_score(kvzap_ctx *ctx, int32_t layer, int32_t n_layers
         // Scoring and compaction in one launch: one layer, one sequence, the window kept, few enough tiles.
         LinCompact fc;
         memset(&fc, 0, sizeof fc);
-        uint32_t smem = kLinSmemBytes;
+        fc.n_stages = lin_per_sm == 1 ? kLinStages : kLinStagesTwo;
+        uint32_t smem = lin_smem_bytes(fc.n_stages);
         if (lin_one_launch) {
             const size_t kv_bytes = static_cast<size_t>(c.n_kv_heads) * n_tokens * c.head_dim * 2;
             const int set = static_cast<int>(ctx->op_turn % kOpRing);

@@ -21,6 +21,7 @@ namespace kvzap {
 
 constexpr int kLinSplit = 4;
 constexpr int kLinStages = 8;             // pipeline stages; kLinStagesCompact when the compaction runs in the same launch
+constexpr int kLinStagesTwo = 5;          // two CTAs per SM
 constexpr int kLinStagesCompact = 2;      // (four CTAs then fit an SM: the launches of the next calls run beside this one;
                                           //  measured per call at 4096 tokens: 8.8 us with 2 stages (9.0 today), 9.9 with 3, 9.6 with 5)
 constexpr int kLinThreads = 192;          // producer warp, MMA warp, four epilogue warps
@@ -47,7 +48,7 @@ struct LinCompact {
     int32_t *lengths;            // [H]
     uint64_t *tile_counts;       // [n_tiles][8]: (call number << 32) | rows of head h kept in the tile
     int32_t epoch;               // the call's number, never 0
-    int32_t n_stages;
+    int32_t n_stages;            // of the pipeline, with or without the compaction: 2 .. kLinStages
     int64_t wait_limit;
 };
 
@@ -61,7 +62,7 @@ score_linear_split_kernel(const __grid_constant__ CUtensorMap tmap_x, const __gr
     __shared__ int32_t run_s[kMaxHeads];                //             rows of head h kept before the tile
     __shared__ int32_t red_s[kLinThreads / 32][kMaxHeads];
     __shared__ int64_t ent_src_s[kMaxHeads * 32], ent_dst_s[kMaxHeads * 32];     // kept rows of this CTA's quarter (byte offsets)
-    const int n_st = fc.enabled ? fc.n_stages : kLinStages;
+    const int n_st = fc.n_stages;
     extern __shared__ uint8_t lin_smem_raw[];
     const uint32_t raw_addr = smem_u32(lin_smem_raw);
     const uint32_t pad = (1024u - (raw_addr & 1023u)) & 1023u;
