@@ -15,8 +15,9 @@
 // a few long sequences), each list is cut into n_parts equal runs of tiles, one CTA each; the parts
 // leave their triples in global memory and the part that arrives last (a counter per list) merges
 // them in part order, so the result does not depend on which one that was.
-// Of a call of many lists the last ones have more parts than the others: the device takes CTAs in order, and a long list among the
-// last would be worked on when all others are done.
+// Of a call of many lists the last ones may have more parts than the others: the device takes CTAs in order, and a long list among the
+// last would be worked on when all others are done.  The CTAs that this takes are the last of the launch: of a list that turns out
+// short they have nothing to do, and pass through slots that the others have left.
 // With fewer lists than resident CTAs (a small batch, layer by layer) there is one wave, and it lasts as
 // long as its longest part: equal parts of lists whose lengths spread over 1 : 7 (contexts of one batch x
 // what each head keeps) leave most of it idle.  There the CTAs share the lists out themselves (attn_unit):
@@ -88,11 +89,12 @@ struct AttnParams {
     uint16_t *out;              // same shape
     int32_t *status;
     int32_t n_parts;            // CTAs per list (1 = the CTA writes the output itself); 0 = by length, see attn_unit
-    float *part_scratch;        // [CTA] { m[8], l[8], O[8][D] }: the parts of a list are consecutive CTAs
-    uint32_t *part_arrive;      // [list] parts that have stored their triple; back to 0 after the launch
-    // n_parts > 0: the lists from head_lists on have tail_parts CTAs each, or as many as leave a CTA kAttnTailTiles tiles
-    int32_t head_lists, tail_parts;
-    int32_t unit0, list0;       // CTA and list of part_scratch[0] and part_arrive[0]
+    float *part_scratch;        // [unit] { m[8], l[8], O[8][D] }: the parts of a list are consecutive units; n_parts == 0: unit = CTA
+    uint32_t *part_arrive;      // [list - list0] parts that have stored their triple; back to 0 after the launch
+    // n_parts > 0: CTAs [0, extra0) are the parts of all lists; behind them the lists from head_lists on have tail_parts - n_parts
+    // more each, of which as many take part as leave a part kAttnTailTiles tiles
+    int32_t extra0, head_lists, tail_parts;
+    int32_t tail_unit0, list0;  // unit of the first part of list head_lists; first list with several parts
     int32_t tiles_shift;        // logarithm of the tiles per page, or -1
     int32_t beside_ctas;        // kBeside: CTAs [0, beside_ctas) run beside the step, as many as find room
     int32_t beside_tiles;       // n_parts == 0: with more tiles than this in all lists all CTAs wait for the step
@@ -266,19 +268,23 @@ decode_attn_kernel(const __grid_constant__ CUtensorMap tmap_kpool, const __grid_
         return (static_cast<int64_t>((i / H) % B) * c.n_layers + p.layer0 + i / (H * B)) * H + i % H;
     };
     if (n_parts > 0) {
-        const int head_ctas = p.head_lists * n_parts, at = static_cast<int>(blockIdx.x) - head_ctas;
-        const bool tail = at >= 0;
-        if (tail) n_parts = p.tail_parts;
-        list = tail ? p.head_lists + at / n_parts : static_cast<int>(blockIdx.x) / n_parts;
-        part = tail ? at % n_parts : static_cast<int>(blockIdx.x) % n_parts;
+        const int extra = static_cast<int>(blockIdx.x) - p.extra0;
+        if (extra < 0) {
+            list = static_cast<int>(blockIdx.x) / n_parts;
+            part = static_cast<int>(blockIdx.x) - list * n_parts;
+        } else {
+            const int each = p.tail_parts - n_parts;
+            list = p.head_lists + extra / each;
+            part = n_parts + extra % each;
+        }
         if (kBeside) n_before = min(__ldcg(before + cache_list(list)), __ldcg(c.prefix_len + cache_list(list)));
         if (!beside) {
             n_total = __ldcg(c.n_tokens + cache_list(list));
             n_prefix = __ldcg(c.prefix_len + cache_list(list));
         }
-        if (tail) {
+        if (list >= p.head_lists) {
             const int tiles = ((kBeside ? n_before : n_prefix) + min(kBeside ? c.window : n_total, c.window)) / kAttnTileRows;
-            n_parts = min(n_parts, max(1, tiles / kAttnTailTiles));
+            n_parts = max(n_parts, min(p.tail_parts, tiles / kAttnTailTiles));
             if (part >= n_parts) {                                 // the whole CTA
                 if (beside) griddep_wait();
                 return;
@@ -793,7 +799,10 @@ decode_attn_kernel(const __grid_constant__ CUtensorMap tmap_kpool, const __grid_
         n_parts = kept_s[warp][kParts];
     }
     constexpr int kUnit = 16 + kAttnMaxGroup * kD;
-    float *unit = n_parts > 1 ? p.part_scratch + static_cast<int64_t>(static_cast<int>(blockIdx.x) - p.unit0) * kUnit : nullptr;
+    // the list's first unit
+    const int unit0 = p.n_parts == 0 ? static_cast<int>(blockIdx.x) - part
+                      : list >= p.head_lists ? p.tail_unit0 + (list - p.head_lists) * p.tail_parts : list * p.n_parts;
+    float *unit = n_parts > 1 ? p.part_scratch + static_cast<int64_t>(unit0 + part) * kUnit : nullptr;
     // four elements of one query head per thread
     for (int idx = threadIdx.x; idx < p.group * (kD / 4); idx += kAttnThreads) {
         const int gq = idx / (kD / 4), d = idx % (kD / 4) * 4;
@@ -830,7 +839,7 @@ decode_attn_kernel(const __grid_constant__ CUtensorMap tmap_kpool, const __grid_
     if (threadIdx.x == 0) last_s = arrive_last_acq_rel(p.part_arrive + (list - p.list0), static_cast<uint32_t>(n_parts));
     __syncthreads();
     if (!last_s) return;
-    const float *units = p.part_scratch + static_cast<int64_t>(static_cast<int>(blockIdx.x) - part - p.unit0) * kUnit;
+    const float *units = p.part_scratch + static_cast<int64_t>(unit0) * kUnit;
     constexpr int kBatch = 8;               // parts whose values are loaded together: one round trip to memory
     for (int idx = threadIdx.x; idx < p.group * (kD / 4); idx += kAttnThreads) {
         const int gq = idx / (kD / 4), d = idx % (kD / 4) * 4;

@@ -2895,20 +2895,21 @@ static kvzap_status attention_impl(kvzap_ctx *ctx, kvzap_cache *cache, int32_t l
         if (parts > 1) p.n_parts = static_cast<int32_t>(parts);
         // The lists that the device takes up last are cut finer: their CTAs end when few others are left to share the memory
         // with.  One wave of them, into parts of no less than 900 rows of the longest list, as far as the scratch goes (of a list that
-        // turns out short the kernel makes fewer).  Us: 4 layers x 128 sequences x 4736 rows layer by layer 1523 -> 1500, 12 layers in one call
-        // x 20 sequences x 2130 rows 341 -> 323, x 64 x 1664 8-bit rows 537 -> 530, 36 x 32 x 1150 858 -> 850; with parts of 1200 rows 1499, 323, 533, 850; with
-        // four parts whatever the lists' room, 12 x 100 x 880 8-bit rows 482 -> 487, 4 x 60 x 750 103.5 -> 106.
+        // turns out short the kernel makes fewer, but no fewer than of the others).  The CTAs for it come last: among the others those
+        // of short lists, which leave at once, cost 2 to 3 us a launch.  Us, lists cut alike / the last ones finer: 4 layers x 128
+        // sequences x 4736 rows layer by layer 1537 / 1489, 12 layers in one call x 20 sequences x 2130 rows 342 / 320, x 64 x 1664 8-bit
+        // rows 542 / 521, 36 x 32 x 1150 856 / 845; a call in tables for 32768 rows a list, 480 lists of some 600 rows 52.4 / 49.0, 2048 of 100
+        // 31.9 / 32.3.  With four parts whatever the lists' room, 12 x 100 x 880 8-bit rows 482 / 487, 4 x 60 x 750 103.5 / 106.
         int64_t tail = std::min<int64_t>(slots / p.n_parts, n_lists_call / 2);
         p.tail_parts = static_cast<int32_t>(std::min<int64_t>(p.n_parts == 1 ? 4 : 2 * p.n_parts, longest / 900));
         if (p.tail_parts <= p.n_parts) tail = 0;
         const int64_t units = p.n_parts == 1 ? tail * p.tail_parts : (n_lists_call - tail) * p.n_parts + tail * p.tail_parts;
         if (units > cache->attn_units) tail = 0;            // (scratch)
         p.head_lists = static_cast<int32_t>(n_lists_call - tail);
-        n_ctas = p.head_lists * static_cast<int64_t>(p.n_parts) + tail * p.tail_parts;
-        if (p.n_parts == 1) {
-            p.unit0 = p.head_lists;
-            p.list0 = p.head_lists;
-        }
+        p.extra0 = static_cast<int32_t>(n_lists_call * p.n_parts);
+        n_ctas = p.extra0 + (tail > 0 ? tail * (p.tail_parts - p.n_parts) : 0);
+        p.tail_unit0 = p.n_parts == 1 ? 0 : p.head_lists * p.n_parts;
+        p.list0 = p.n_parts == 1 ? p.head_lists : 0;
     }
     p.tiles_shift = -1;
     for (int i = 0; i < 31; ++i)

@@ -11,22 +11,24 @@ pytestmark = pytest.mark.gpu
 H, P = 8, 16
 
 
-@pytest.mark.parametrize("B,L,D,G,fp8,longest", [
-    (80, 1, 128, 4, False, 2000),       # one part a list, then two
-    (75, 1, 128, 4, True, 2800),        # 8-bit rows: 600 lists of which half are cut
-    (60, 2, 64, 2, False, 3700),        # 960 lists in three parts, then four
-    (77, 1, 128, 8, False, 1700),       # no list long enough for a second part
-    (230, 1, 64, 1, True, 1900),        # 1840 lists
+@pytest.mark.parametrize("B,L,D,G,fp8,longest,room", [
+    (80, 1, 128, 4, False, 2000, 2000),     # one part a list, then two
+    (75, 1, 128, 4, True, 2800, 2800),      # 8-bit rows: 600 lists of which half are cut
+    (60, 2, 64, 2, False, 3700, 3700),      # 960 lists in three parts, then four
+    (77, 1, 128, 8, False, 1700, 1700),     # no list long enough for a second part
+    (230, 1, 64, 1, True, 1900, 1900),      # 1840 lists
+    (60, 1, 128, 4, False, 700, 32768),     # short lists where there is room for long ones: seven parts each, none more
+    (61, 1, 64, 4, True, 12000, 32768),     # ... and some long ones
 ])
-def test_many_lists(B, L, D, G, fp8, longest):
+def test_many_lists(B, L, D, G, fp8, longest, room):
     rng = np.random.default_rng(B)
     prefix = rng.integers(0, longest, size=B * L * H)
-    edges = [0, 1, 15, 16, 17, 639, 640, 641, 1279, 1280, 1281, longest]
+    edges = [n for n in (0, 1, 15, 16, 17, 639, 640, 641, 1279, 1280, 1281, longest) if n <= longest]
     prefix[:len(edges)] = edges
     prefix[-2 * len(edges)::2] = edges
     pages = (prefix + P - 1) // P
     first = np.concatenate([[0], np.cumsum(pages)[:-1]])
-    max_pages = longest // P + 1
+    max_pages = room // P + 1
     row = (D + synth.E4M3_ROW_TRAILER) // 2 if fp8 else D
     g = torch.Generator(device="cuda").manual_seed(B)
     raw = [torch.empty(int(pages.sum()) * P, D, device="cuda").normal_(generator=g).to(torch.bfloat16) for _ in range(2)]
