@@ -1254,7 +1254,7 @@ static kvzap_status launch_compact_short(kvzap_ctx *ctx, ShortCompact a, cudaStr
     ProfScope prof(ctx, KVZAP_KERNEL_COMPACT, stream);
     cudaLaunchConfig_t cfg;
     cudaLaunchAttribute attrs[2];
-    make_launch(&cfg, attrs, dim3(static_cast<unsigned>(a.n_blocks) + 1, static_cast<unsigned>(a.n_heads), nz), dim3(kDenseThreadsShort), 0, stream,
+    make_launch(&cfg, attrs, dim3(static_cast<unsigned>(a.n_blocks + a.n_books), static_cast<unsigned>(a.n_heads), nz), dim3(kDenseThreadsShort), 0, stream,
                 !ctx->profiling, 1);
     const bool paged = a.page_tokens > 0;
     KVZAP_CUDA(ctx, cudaLaunchKernelEx(&cfg, a.list_base != nullptr   ? compact_short_kernel<kShortAppend, kFromWords>
@@ -1286,6 +1286,7 @@ static ShortCompact short_args(const kvzap_ctx *ctx, const uint32_t *mask, const
     a.n_seqs = n_seqs;
     a.n_heads = c.n_kv_heads;
     a.row_units = c.head_dim / 8;
+    a.n_books = 1;
     return a;
 }
 
@@ -3074,6 +3075,7 @@ static kvzap_status append_chunk(kvzap_ctx *ctx, kvzap_cache *cache, int32_t lay
         a.n_pages_pool = v.n_pages_pool;
         a.page_table = v.page_table;
         a.status = ctx->status_dev;
+        a.n_books = (n_seqs + kDenseThreadsShort / 32 - 1) / (kDenseThreadsShort / 32);
         a.list_base = ctx->list_base;
         a.list_map = ctx->batch_map;
         a.page_cursor = v.page_cursor;

@@ -748,9 +748,10 @@ compact_dense_kernel(const uint4 *__restrict__ K, const uint4 *__restrict__ V, u
 // The compaction of a short input (mask words and lists as for assign_pages_locally) that runs beside nothing: behind the scoring of
 // a default context, or of a chunk.  There the launch is a chain of round trips, and this kernel has as few as there are: mask words,
 // sequence offsets, old lengths and the page cursor together; then the rows' loads, for which a CTA needs only its own block's
-// words, go out before the lists are counted and pages found; then the stores.  Grid (blocks + 1, H, z): z CTAs share the rows
-// of a block, and the last x does the bookkeeping of a head's lists (lengths, tables, for a chunk also the ring's scores), which no
-// row waits for.  An append finds the pages of new rows itself, from the cursor and the stack as the launch ahead left them (`taken`).
+// words, go out before the lists are counted and pages found; then the stores.  Grid (blocks + n_books, H, z): z CTAs share the rows
+// of a block, and the last x do the bookkeeping of a head's lists (lengths, tables, for a chunk also the ring's scores), which no
+// row waits for.  A chunk has one of them to as many sequences as a CTA has warps: with one for all, 256 sequences of 200 tokens, one head,
+// took 181 us in two chunks, 130 with the launches that this one replaces, now 101.  An append finds the pages of new rows itself, from the cursor and the stack as the launch ahead left them (`taken`).
 // Scoring and this, us a call of several layers: 8 x 777 tokens into pages 146.6 -> 136.4, 4 x 5 x 300 93.3 -> 82.1, 4 x 3000 118.6 -> 110.6, dense
 // 4 x 777 67.5 -> 63.5; 5120 -> 640 -> 8, 4 x 2000 dense 90.3 -> 86.0.  Chunks, whose launch ahead had spent 7 us on counting and a one-CTA page
 // assignment behind the scoring: four prompts in two chunks of 500 tokens, 4 layers, 274.3 -> 224.3, eight of 64 in three 304.9 -> 268.7.
@@ -763,6 +764,7 @@ struct ShortCompact {
     int32_t *lengths;                 // [n_lists]; append: of all lists of the cache
     int64_t n_tokens, in_stride_h, in_stride_t;
     int32_t n_words, n_blocks, n_seqs, n_heads, row_units;
+    int32_t n_books;                  // bookkeeping CTAs per head
     int32_t page_tokens;              // 0: dense-ragged output
     int32_t page_shift;               // its logarithm, or -1: a division takes some 150 cycles of a chain
     int32_t first_page, max_pages;
@@ -831,7 +833,7 @@ compact_short_kernel(const ShortCompact a)
     const int h = blockIdx.y, H = a.n_heads, z = blockIdx.z, nz = gridDim.z;
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const int blk = blockIdx.x;
-    const bool books = blk == a.n_blocks;
+    const bool books = blk >= a.n_blocks;
     if constexpr (kFrom == kFromWords) {
         griddep_launch_dependents();
         griddep_wait();
@@ -1043,7 +1045,7 @@ compact_short_kernel(const ShortCompact a)
             // an append that needs no page but released ones fits wherever the cursor stands
             const bool fits = static_cast<int64_t>(cursor_s) + (carry - from_stack) <= a.n_pages_pool || (kAppend && carry == from_stack);
             fail = __any_sync(0xffffffffu, fail) || !fits;
-            const bool first_cta = books && h == 0;
+            const bool first_cta = blk == a.n_blocks && h == 0;
             if (fail) {
                 for (int idx = lane; idx < n_lists; idx += 32) s_page0[idx] = -1;
                 if (first_cta && lane == 0) atomicCAS(a.status, 0, 4 /* KVZAP_ERR_OOM_PAGES */);
@@ -1076,7 +1078,7 @@ compact_short_kernel(const ShortCompact a)
         }
     };
     if (books) {
-        for (int b = warp; b < a.n_seqs; b += kWarps) {
+        for (int b = (blk - a.n_blocks) * kWarps + warp; b < a.n_seqs; b += a.n_books * kWarps) {
             const int64_t li = kPages ? s_list[b] : static_cast<int64_t>(b) * H + h;
             const int32_t kept = s_len[kPages ? b * H + h : b];
             if constexpr (kPages) {
@@ -1092,9 +1094,20 @@ compact_short_kernel(const ShortCompact a)
             if constexpr (kAppend) {
                 const int32_t m = s_cu[b + 1] - s_cu[b], n_win = m < a.window ? m : a.window;
                 const int32_t n_now = __ldcg(a.n_tokens_list + li);
-                for (int32_t i = lane; i < n_win; i += 32)
-                    a.score_ring[li * a.window + (n_now - n_win + i) % a.window] =
-                        __ldcg(a.scores + (static_cast<int64_t>(s_cu[b + 1]) - n_win + i) * H + h);
+                constexpr int kEach = 4;                          // scores per lane on their way together
+                for (int32_t i0 = lane; i0 < n_win; i0 += 32 * kEach) {
+                    float sc[kEach];
+#pragma unroll
+                    for (int k = 0; k < kEach; ++k) {
+                        const int32_t i = i0 + 32 * k;
+                        sc[k] = i < n_win ? __ldcg(a.scores + (static_cast<int64_t>(s_cu[b + 1]) - n_win + i) * H + h) : 0.0f;
+                    }
+#pragma unroll
+                    for (int k = 0; k < kEach; ++k) {
+                        const int32_t i = i0 + 32 * k;
+                        if (i < n_win) a.score_ring[li * a.window + (n_now - n_win + i) % a.window] = sc[k];
+                    }
+                }
             }
         }
         finish();

@@ -58,9 +58,11 @@ def test_prompts(oracle, T, B, H, D, how):
     ctx.close()
 
 
-@pytest.mark.parametrize("T,B,H,D", [(500, 4, 8, 128), (8192, 3, 8, 64), (8300, 3, 8, 64), (3000, 32, 8, 64), (3000, 33, 8, 64), (40, 6, 2, 40)])
-def test_chunks(T, B, H, D):
-    P, C = 16, 3
+# the last three: pages whose size is no power of two, and more sequences than a bookkeeping CTA has warps
+@pytest.mark.parametrize("T,B,H,D,P", [(500, 4, 8, 128, 16), (8192, 3, 8, 64, 16), (8300, 3, 8, 64, 16), (3000, 32, 8, 64, 16), (3000, 33, 8, 64, 16),
+                                       (40, 6, 2, 40, 16), (700, 3, 8, 64, 24), (2100, 100, 2, 40, 7), (5000, 255, 1, 64, 5)])
+def test_chunks(T, B, H, D, P):
+    C = 3
     ctx, _, _ = _case(T, B, H, D, T + B)
     max_pages = C * T // P + 2
     pool = [torch.zeros(B * H * (C * T // P // B + 4) + C * T * H // P, P, D, dtype=torch.bfloat16, device="cuda") for _ in range(2)]
