@@ -1319,6 +1319,22 @@ static kvzap_status launch_compaction(kvzap_ctx *ctx, const uint32_t *mask, cons
     return KVZAP_OK;
 }
 
+// Whether the pruning of given scores takes compact_short_kernel, whose CTAs wait for no other but read the scores of the tokens before
+// them (paged: all scores) and look for every token's sequence.  Up to how many blocks that is the shorter chain depends on the
+// sequences; prune_onepass_kernel / it, us a call: 1 x 7000 tokens, 8 heads 12.7 / 11.1, 8192 11.9 / 13.2; 2 x 3000 15.4 / 12.6, 2 x 3500, 2 heads
+// 10.4 / 10.5; 8 x 625 15.7 / 14.0, 8 x 750, 2 heads 10.7 / 11.7; 30 x 133 16.9 / 14.8, 30 x 200 18.9 / 20.3; pages 30 x 50 18.5 / 15.8, 16 x 128 16.0 / 16.2.
+// Calls that run beside one another on a context that trusts its producers are not a matter of the chain: dense, it gains where 8
+// heads fill the device (2 x 1500 7.0 / 5.2, 4 x 1250 8.6 / 8.1; 4 x 250 3.8 / 4.0, 8 x 750 9.7 / 10.3; 4 heads, 8 x 375 4.9 / 5.6), paged, as long as
+// the scores are few (8 heads, 8 x 125 6.2 / 5.2, 1500 5.3 / 7.4; 4 heads, 8 x 187 6.2 / 5.1, 8 x 256 6.3 / 7.1).
+static bool short_prune(const kvzap_ctx *ctx, int64_t n_blocks, int64_t n_seqs, bool paged)
+{
+    const int H = ctx->cfg.n_kv_heads;
+    if (!short_input(4 * n_blocks, H, n_seqs)) return false;
+    if (ctx->trusted) return paged ? n_blocks <= std::min(16, 4 + 32 / H) : H > 4 && n_blocks >= 12 && n_blocks <= 32;
+    if (paged) return n_blocks <= (n_seqs <= 8 ? 16 : 12);
+    return n_blocks <= (n_seqs == 1 ? 56 : n_seqs == 2 ? 48 : n_seqs <= 8 ? 40 : 32);
+}
+
 // Threshold / window mask, counts, prefix sums and the ordered gather in one launch (prune_onepass_kernel),
 // dense-ragged (page_tokens == 0) or paged.  tau_list != nullptr: a threshold per list, written by the
 // kernel ahead in the stream.
@@ -1360,8 +1376,7 @@ static kvzap_status launch_prune_onepass(kvzap_ctx *ctx, const float *scores, co
         uses, 11, !ctx->trusted || ctx->profiling || tau_list != nullptr || scores_just_made || ctx->op_last_seq + 1 != ctx->op_seq, 0);
     const bool wait_first = order.wait != InFlight::kNone;
     ctx->op_last_seq = ctx->op_seq;
-    if (slot_out == nullptr && n_blocks <= (page_tokens > 0 ? kShortScoreBlocksPaged : kShortScoreBlocks) &&
-        short_input(4 * n_blocks, c.n_kv_heads, n_seqs) && !tau_behind && (page_tokens == 0 || tau_list == nullptr)) {
+    if (slot_out == nullptr && short_prune(ctx, n_blocks, n_seqs, page_tokens > 0) && !tau_behind && (page_tokens == 0 || tau_list == nullptr)) {
         ShortCompact a = short_args(ctx, nullptr, K, V, cu_seqlens, n_seqs, n_tokens, K_out, V_out, lengths, false);
         a.page_tokens = page_tokens;
         a.first_page = first_page;

@@ -811,11 +811,9 @@ enum ShortKind { kShortDense, kShortPaged, kShortAppend };
 // Where the keep bits come from: mask words, or given scores (the pruning calls).  Then every CTA makes the words that it needs
 // itself: dense, those of its head up to its block; paged, all of them, a token of all heads per load.
 // In place of prune_onepass_kernel, whose CTAs look sequences up in memory one after the other, and whose paged form meets at an arrival
-// counter, a page assignment and a flag; us a call: 3 x 500 tokens 8.6 -> 5.8, 800 7.4 -> 4.1, 2200 10.3 -> 5.2, 4000 10.2 -> 7.3, 8000 13.1 -> 11.7,
-// 4 x 1250 15.5 -> 12.6; paged 300 12.1 -> 5.0, 2 x 450 14.9 -> 8.8, 1500 13.4 -> 11.0 (2500 equal, 4000 in three 16.8 -> 22.4: every CTA reads all
-// scores there, so 16 blocks at most).
+// counter, a page assignment and a flag; us a call: 3 x 500 tokens 8.6 -> 5.8, 800 7.4 -> 4.1, 2200 10.3 -> 5.2, 4000 10.2 -> 7.3; paged 300 12.1 -> 5.0,
+// 2 x 450 14.9 -> 8.8, 1500 13.4 -> 11.0.  Up to which sizes: short_prune.
 enum ShortSource { kFromWords, kFromScores };
-constexpr int kShortScoreBlocks = 64, kShortScoreBlocksPaged = 16;
 template <ShortKind kKind, ShortSource kFrom>
 __global__ void __launch_bounds__(kDenseThreadsShort, 4)
 compact_short_kernel(const ShortCompact a)

@@ -1,5 +1,5 @@
-"""The kernel for short inputs, at the edges of what it takes (2048 mask words over all heads, 256 lists; 64 or, paged, 16 blocks of given
-scores) and just beyond: prompts of contexts that do not trust their producers and the pruning of given scores against the oracle,
+"""The kernel for short inputs, at the edges of what it takes (2048 mask words over all heads, 256 lists; of given scores 32 to 56 blocks by
+the sequences, paged 12 or 16) and just beyond: prompts of contexts that do not trust their producers and the pruning of given scores against the oracle,
 chunks against the selection by score of their whole streams."""
 import numpy as np
 import pytest
@@ -24,7 +24,8 @@ def _case(T, B, H, D, seed, trusted=False):
 
 @pytest.mark.parametrize("T,B,H,D", [(1, 1, 8, 64), (129, 3, 8, 128), (300, 1, 8, 64), (2048, 2, 8, 64), (2049, 7, 8, 64), (8192, 1, 8, 64),
                                      (8192, 32, 8, 40), (8193, 1, 8, 64), (2000, 33, 8, 64), (65536, 5, 1, 64), (5000, 255, 1, 64),
-                                     (4000, 7, 3, 512), (3001, 2, 5, 72)])
+                                     (4000, 7, 3, 512), (3001, 2, 5, 72), (7168, 1, 8, 64), (7169, 1, 8, 64), (6144, 2, 4, 64), (5121, 8, 8, 64),
+                                     (4096, 9, 8, 64), (1536, 9, 8, 64), (1537, 9, 8, 64), (1024, 4, 8, 64), (1025, 4, 8, 64)])
 @pytest.mark.parametrize("how", ["head major", "token major", "given scores", "given scores, trusted"])
 def test_prompts(oracle, T, B, H, D, how):
     ctx, X, cu = _case(T, B, H, D, T + B, "trusted" in how)
