@@ -836,7 +836,7 @@ decode_attn_kernel(const __grid_constant__ CUtensorMap tmap_kpool, const __grid_
     // ---- several CTAs per list: the one that arrives last merges all parts, in part order
     __shared__ int last_s;
     __syncthreads();
-    if (threadIdx.x == 0) last_s = arrive_last_acq_rel(p.part_arrive + (list - p.list0), static_cast<uint32_t>(n_parts));
+    if (threadIdx.x == 0) last_s = arrive_last(p.part_arrive + (list - p.list0), static_cast<uint32_t>(n_parts));
     __syncthreads();
     if (!last_s) return;
     const float *units = p.part_scratch + static_cast<int64_t>(unit0) * kUnit;

@@ -185,7 +185,7 @@ chunk_ring_kernel(const CacheView c, const __grid_constant__ ChunkSeqs seqs, int
         list_base[b * H + h] = static_cast<int32_t>(len_s);
         c.n_tokens[li] = static_cast<int32_t>(n_old + m);
         if (h == 0 && m > 0) c.active[li / (static_cast<int64_t>(c.n_layers) * H)] = 1;     // the slot holds a sequence again
-        if (arrive_last_acq_rel(arrive, gridDim.x * gridDim.y)) {
+        if (arrive_last(arrive, gridDim.x * gridDim.y)) {
             taken[0] = __ldcg(c.page_cursor);
             taken[1] = c.free_top != nullptr ? __ldcg(c.free_top) : 0;
         }

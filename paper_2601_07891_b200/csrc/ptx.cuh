@@ -323,18 +323,23 @@ __device__ __forceinline__ void st_release_gpu(int32_t *p, int32_t v)
 
 // Counts one of n arrivals in: true for the last one, and the counter is back at zero with it.  (A count that runs on over
 // all launches and is taken modulo n goes wrong for good when it wraps, unless n is a power of two: 2^32 arrivals of five
-// per launch are some hours of decoding.)
+// per launch are some hours of decoding.)  A release and an acquire of this thread: others' stores before it are taken along, and others
+// see what the last one sees, if a barrier of theirs (of the warp, the CTA) is on either side.
 __device__ __forceinline__ bool arrive_last(uint32_t *counter, uint32_t n)
-{
-    return atomicInc(counter, n - 1u) == n - 1u;
-}
-
-// The same as release and acquire: what the threads before it in its warp or CTA have stored is seen by whoever is last.
-__device__ __forceinline__ bool arrive_last_acq_rel(uint32_t *counter, uint32_t n)
 {
     uint32_t before;
     asm volatile("atom.acq_rel.gpu.global.inc.u32 %0, [%1], %2;" : "=r"(before) : "l"(counter), "r"(n - 1u) : "memory");
     return before == n - 1u;
+}
+// A whole warp's arrival: every lane of the last one sees what the lanes of all stored before theirs.
+__device__ __forceinline__ bool arrive_last_warp(uint32_t *counter, uint32_t n)
+{
+    __syncwarp();
+    int last = 0;
+    if ((threadIdx.x & 31) == 0) last = arrive_last(counter, n);
+    last = __shfl_sync(0xffffffffu, last, 0);
+    __syncwarp();                           // a shuffle orders no memory
+    return last != 0;
 }
 
 // ---------------------------------------------------------------- programmatic dependent launch

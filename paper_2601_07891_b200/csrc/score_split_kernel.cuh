@@ -681,10 +681,7 @@ score_split_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_cons
             if (n_split > 1) {
                 // whichever slice brings a warp's tokens in last finishes them
                 __stcg(const_cast<float *>(parts) + static_cast<int64_t>(nh) * kTileM * kMaxHeads, sum);
-                __syncwarp();
-                int l = 0;
-                if (lane == 0) l = arrive_last_acq_rel(p.split_arrive + part_tile * kFewWarps + w8, static_cast<uint32_t>(n_split));
-                last = __shfl_sync(0xffffffffu, l, 0) != 0;
+                last = arrive_last_warp(p.split_arrive + part_tile * kFewWarps + w8, static_cast<uint32_t>(n_split));
             }
             const CacheView &c = f.c;
             if (last && token < p.n_tokens && head < c.n_heads) {
@@ -729,10 +726,7 @@ score_split_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_cons
             // the slices meet in global memory; of each quarter of the rows, whoever brings it in last finishes it
             __stcg(parts + static_cast<int64_t>(nh) * kSlice, make_float4(s[0], s[1], s[2], s[3]));
             __stcg(parts + static_cast<int64_t>(nh) * kSlice + 1, make_float4(s[4], s[5], s[6], s[7]));
-            __syncwarp();
-            int l = 0;
-            if (lane == 0) l = arrive_last_acq_rel(p.split_arrive + part_tile * kTileWarps + q, static_cast<uint32_t>(n_split));
-            last = __shfl_sync(0xffffffffu, l, 0) != 0;
+            last = arrive_last_warp(p.split_arrive + part_tile * kTileWarps + q, static_cast<uint32_t>(n_split));
         }
         // the new token's scores go into the slot it took: n_tokens was advanced by the list's CTA, and those of the tile have all
         // arrived.  All loads before the first use of one: one round trip

@@ -95,15 +95,20 @@ def test_decode_steps_that_change_layout(oracle, B, L, trusted):
     ctx.close()
 
 
-@pytest.mark.parametrize("n", [2, 4, 5, 8])
-def test_arrivals_of_the_slices_do_not_add_up_over_launches(n):
-    """Every n-th arrival is the last of its launch and leaves the counter at zero, so that no number of launches wraps it."""
+@pytest.fixture(scope="module")
+def arrivals():
     lib = os.path.join(HERE, "_build", "libarrivals.so")
     os.makedirs(os.path.dirname(lib), exist_ok=True)
     subprocess.run([shutil.which("nvcc") or "/usr/local/cuda/bin/nvcc", "-gencode", "arch=compute_100a,code=sm_100a", "-O2",
                     "-std=c++17", "-shared", "-Xcompiler", "-fPIC", "-o", lib, os.path.join(HERE, "helpers", "arrivals.cu")],
                    check=True)
-    launch = ctypes.CDLL(lib).launch_arrivals
+    return ctypes.CDLL(lib)
+
+
+@pytest.mark.parametrize("n", [2, 4, 5, 8])
+def test_arrivals_of_the_slices_do_not_add_up_over_launches(arrivals, n):
+    """Every n-th arrival is the last of its launch and leaves the counter at zero, so that no number of launches wraps it."""
+    launch = arrivals.launch_arrivals
     launch.argtypes = [ctypes.c_void_p, ctypes.c_uint, ctypes.c_int] + 3 * [ctypes.c_void_p]
     rounds = 7
     counter = torch.zeros(1, dtype=torch.int32, device="cuda")
@@ -113,6 +118,22 @@ def test_arrivals_of_the_slices_do_not_add_up_over_launches(n):
         torch.cuda.synchronize()
         assert last.tolist() == ([0] * (n - 1) + [1]) * rounds
         assert after.tolist() == (list(range(1, n)) + [0]) * rounds
+
+
+@pytest.mark.parametrize("n", [1, 2, 5, 8, 148])
+def test_every_lane_of_the_last_warp_sees_what_all_lanes_stored(arrivals, n):
+    launch = arrivals.launch_warp_arrivals
+    launch.argtypes = [ctypes.c_void_p, ctypes.c_uint, ctypes.c_void_p, ctypes.c_int] + 3 * [ctypes.c_void_p]
+    counter, lasts = (torch.zeros(1, dtype=torch.int32, device="cuda") for _ in range(2))
+    parts, sums = torch.full((n * 32,), -1, dtype=torch.int32, device="cuda"), torch.zeros(50, 32, dtype=torch.int32, device="cuda")
+    for i in range(50):
+        assert launch(counter.data_ptr(), n, parts.data_ptr(), 1000 * i, sums[i].data_ptr(), lasts.data_ptr(),
+                      torch.cuda.current_stream().cuda_stream) == 0
+    torch.cuda.synchronize()
+    assert int(lasts) == 50 * 32 and int(counter) == 0       # all lanes of one warp a launch
+    lane = (torch.arange(32) * 5 + 7) % 32
+    for i in range(50):
+        assert torch.equal(sums[i].cpu().long(), n * (1000 * i + lane) + 32 * n * (n - 1) // 2)
 
 
 @pytest.mark.parametrize("hidden", [256, 512, 640, 1024])
