@@ -114,7 +114,8 @@ constexpr float kAttnMinPart = 16.0f;       // tiles
 // 359 / 361 / 356, 32 x 2176 765 / 636 / 643 / 639, 12 x 1628 263 / 247 / 248 / 248, 4 x 7628 346 / 322 / 326 / 320; 8-bit 32 x 1152 402 / 357 / 363 /
 // 365, 16 x 2176 349 / 317 / 314 / 328, 30 x 2378 619 / 533 / 551 / 540, 8 x 2176 260 / 263 / 263 / 261; 36 layers, 8 x 2176 730 / 698 / 698 / 702.
 // (When half of the tiles are issued, whatever the clock: 361, 640, 248, 323; 366, 321, 542, 257; 693.)  Not with several waves: 512 lists
-// of 1128 rows 263 / 271.
+// of 1128 rows 263 / 271.  Cycles of the SM's clock, at the 1.75 to 1.97 GHz that it has in such calls, which wait for memory: slower, and the wait comes later, at
+// the latest with the last known tile.
 constexpr int kWaitBase = 12000, kWaitTile = 270, kWaitTile8 = 400;
 constexpr int kAttnTailTiles = 40;          // a part of the lists at the end of a launch of many, at least
 __device__ __forceinline__ int attn_unit(const int32_t *lengths, int n, int n_units, int unit, int lane, int &list, int &part)
@@ -238,7 +239,7 @@ decode_attn_kernel(const __grid_constant__ CUtensorMap tmap_kpool, const __grid_
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const CacheView &c = p.c;
     const int H = c.n_heads, B = c.n_seqs;
-    const clock_t started = kBeside ? clock() : 0;
+    const uint32_t started = kBeside ? static_cast<uint32_t>(clock()) : 0u;       // differences are right across its wrap
 
     __shared__ int queries_s;               // kBeside: warps that are done with the queries in memory
     if (threadIdx.x == 0) {
@@ -575,7 +576,7 @@ decode_attn_kernel(const __grid_constant__ CUtensorMap tmap_kpool, const __grid_
     for (; s < n_tiles; s += kAttnWarps) {
         if (kBeside && !waited && s_issue < n_tiles &&
             (s_issue + kAttnWarps >= n_tiles ||
-             (p.n_parts == 0 && clock() - started > kWaitBase + (kFp8 ? kWaitTile8 : kWaitTile) * kD / 128 * n_early))) {
+             (p.n_parts == 0 && static_cast<uint32_t>(clock()) - started > static_cast<uint32_t>(kWaitBase + (kFp8 ? kWaitTile8 : kWaitTile) * kD / 128 * n_early)))) {
             // time for the next step to start (see kWaitBase), or the last of the tiles known beside the kernel ahead is about to
             // be issued: what comes next is learnt while those in flight are worked on
             wait_for_rest();
