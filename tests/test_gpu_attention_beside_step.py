@@ -29,7 +29,7 @@ def binding():
 class _Side:
     """One context and cache with imported prefixes; the same for both sides but for the trust in the producers."""
 
-    def __init__(self, binding, trusted, d_model, hidden, D, L, B, w, prefix, grow, fp8):
+    def __init__(self, binding, trusted, d_model, hidden, D, L, B, w, prefix, grow, fp8, P=P):
         self.b, self.fp8 = binding, fp8
         row = (D + synth.E4M3_ROW_TRAILER) // 2 if fp8 else D
         self.ctx = binding.Kvzap(d_model, hidden, H, row, L, max_tokens=max(B, 128), trusted_producers=trusted)
@@ -93,13 +93,19 @@ def _close(got, want):
     (64, 8, 9, 3, 3, 16, 60, True, 128, True),
     (64, 8, 9, 3, 1, 16, 60, True, 512, True),
     (128, 4, 8, 3, 2, 16, 60, False, 512, False),        # steps on too many SMs
+    (128, 4, 70, 2, 1, 32, 1900, False, 512, True),      # more lists than CTAs of a wave, whole, the last ones in two parts
+    (128, 4, 80, 2, 1, 16, 1900, True, 128, True),       # ... of 8-bit rows
+    (64, 2, 60, 2, 1, 16, 2900, False, 128, True),       # ... the last ones in three
 ])
-def test_outputs_are_those_of_a_context_that_waits(binding, D, G, B, L, group, w, longest, fp8, hidden, beside):
+@pytest.mark.parametrize("page", [P, 48])
+def test_outputs_are_those_of_a_context_that_waits(binding, D, G, B, L, group, w, longest, fp8, hidden, beside, page):
     d_model, steps = 1024, w + 40
+    if page != P and longest > 3000:
+        pytest.skip("pages of another size: the shorter lists reach the same")
     rng = np.random.default_rng(D + B)
     prefix = rng.integers(0, longest, size=B * L * H)
     prefix[:6] = [0, 1, 15, 16, 17, longest]
-    sides = [_Side(binding, t, d_model, hidden, D, L, B, w, prefix, steps // P + 2, fp8) for t in (True, False)]
+    sides = [_Side(binding, t, d_model, hidden, D, L, B, w, prefix, steps // P + 2, fp8, page) for t in (True, False)]
     outs = [[], []]
     row = sides[0].pools[0].shape[-1]
     inputs = []
@@ -139,11 +145,15 @@ def test_outputs_are_those_of_a_context_that_waits(binding, D, G, B, L, group, w
         side.close()
 
 
+# A warp has two tiles in flight (of 8-bit rows three), a CTA four warps.  Up to 700 rows a list, in parts of 16 tiles or more: warps whose tiles
+# are all in flight, which wait behind them, and warps with one or two more, which learn of new queries when the last is about to be
+# issued.  From 9000 rows: some 35 tiles a warp, and the wait comes at its time, in the middle of them.
+@pytest.mark.parametrize("shortest,longest", [(0, 700), (9000, 9400)])
 @pytest.mark.parametrize("D,fp8", [(128, False), (128, True), (64, False), (64, True)])
-def test_queries_written_between_step_and_attention(binding, producer, D, fp8):  # noqa: F811
+def test_queries_written_between_step_and_attention(binding, producer, D, fp8, shortest, longest):  # noqa: F811
     """The kernel between the two signals before it stores the queries: they are read again once it has completed."""
     G, B, L, w, d_model, hidden = 4, 6, 2, 16, 1024, 128
-    prefix = np.random.default_rng(3).integers(0, 700, size=B * L * H)
+    prefix = np.random.default_rng(3).integers(shortest, longest, size=B * L * H)
     sides = [_Side(binding, t, d_model, hidden, D, L, B, w, prefix, 4, fp8) for t in (True, False)]
     row = sides[0].pools[0].shape[-1]
     for k in range(6):

@@ -8,19 +8,21 @@ from paper_2601_07891_b200 import binding, synth
 
 pytestmark = pytest.mark.gpu
 
-H, P = 8, 16
+H = 8
 
 
-@pytest.mark.parametrize("B,L,D,G,fp8,longest,room", [
-    (80, 1, 128, 4, False, 2000, 2000),     # one part a list, then two
-    (75, 1, 128, 4, True, 2800, 2800),      # 8-bit rows: 600 lists of which half are cut
-    (60, 2, 64, 2, False, 3700, 3700),      # 960 lists in three parts, then four
-    (77, 1, 128, 8, False, 1700, 1700),     # no list long enough for a second part
-    (230, 1, 64, 1, True, 1900, 1900),      # 1840 lists
-    (60, 1, 128, 4, False, 700, 32768),     # short lists where there is room for long ones: seven parts each, none more
-    (61, 1, 64, 4, True, 12000, 32768),     # ... and some long ones
+@pytest.mark.parametrize("B,L,D,G,fp8,longest,room,P", [
+    (80, 1, 128, 4, False, 2000, 2000, 16),     # one part a list, then two
+    (75, 1, 128, 4, True, 2800, 2800, 16),      # 8-bit rows: 600 lists of which half are cut
+    (60, 2, 64, 2, False, 3700, 3700, 16),      # 960 lists in three parts, then four
+    (77, 1, 128, 8, False, 1700, 1700, 16),     # no list long enough for a second part
+    (230, 1, 64, 1, True, 1900, 1900, 16),      # 1840 lists
+    (60, 1, 128, 4, False, 700, 32768, 16),     # short lists where there is room for long ones: seven parts each, none more
+    (61, 1, 64, 4, True, 12000, 32768, 16),     # ... and some long ones
+    (80, 1, 128, 4, False, 2000, 2016, 48),     # pages of three tiles
+    (9, 2, 128, 4, True, 2500, 2500, 80),       # ... of five, the lists shared out by their lengths
 ])
-def test_many_lists(B, L, D, G, fp8, longest, room):
+def test_many_lists(B, L, D, G, fp8, longest, room, P):
     rng = np.random.default_rng(B)
     prefix = rng.integers(0, longest, size=B * L * H)
     edges = [n for n in (0, 1, 15, 16, 17, 639, 640, 641, 1279, 1280, 1281, longest) if n <= longest]

@@ -8,16 +8,28 @@ from tests import test_gpu_step_order as order
 
 pytestmark = pytest.mark.gpu
 
-H = order.H
 
-
-# d_model 512, 8 heads.  hidden 512: up to 8 CTAs along K and 4 slices; 128: one slice; 48: slices of 16, no cluster; 640: five slices
+# d_model 512, 8 heads.  Slices x CTAs along K: hidden 512 4 x 8, of many layers a call 2 x 2; 128 4 x 2; 64 2 x 2; 640 5 x 8; 1024 8 x 8; the
+# last two of many layers a call 4 x 1, without a cluster
 @pytest.mark.parametrize("B,L,hidden,group,trusted,fp8", [
     (1, 2, 512, 1, True, False), (4, 3, 512, 1, False, False), (5, 2, 512, 2, True, True), (8, 12, 512, 12, True, False),
     (9, 2, 512, 1, True, False), (16, 2, 640, 1, True, False), (17, 2, 512, 1, True, True), (24, 3, 128, 1, False, False),
     (25, 36, 512, 36, True, False), (31, 2, 1024, 1, True, False), (32, 2, 512, 1, True, False), (32, 30, 512, 30, True, True),
-    (33, 2, 512, 1, True, False), (33, 2, 512, 2, True, True), (7, 2, 64, 1, True, False)])
+    (33, 2, 512, 1, True, False), (33, 2, 512, 2, True, True), (7, 2, 64, 1, True, False),
+    (8, 36, 640, 36, True, False), (32, 30, 1024, 30, True, False), (5, 30, 1024, 30, False, True)])
 def test_steps_of_few_sequences(B, L, hidden, group, trusted, fp8):
+    _steps(B, L, hidden, group, trusted, fp8)
+
+
+@pytest.mark.parametrize("heads", [1, 2, 5, 7])
+@pytest.mark.parametrize("B,L,hidden,group,trusted,fp8", [(9, 2, 512, 1, True, False), (32, 12, 512, 12, False, False), (3, 2, 512, 1, True, True)])
+def test_fewer_heads(monkeypatch, heads, B, L, hidden, group, trusted, fp8):
+    monkeypatch.setattr(order, "H", heads)
+    _steps(B, L, hidden, group, trusted, fp8)
+
+
+def _steps(B, L, hidden, group, trusted, fp8):
+    H = order.H
     n = order.W + 24
     s = order._Server(hidden, B, L, trusted, n + 2, fp8)
     for _ in range(n):
