@@ -979,7 +979,7 @@ static kvzap_status launch_score(kvzap_ctx *ctx, int32_t layer, int32_t n_layers
                                           {compact->lengths, sizeof(int32_t) * c.n_kv_heads, true}};
             if (ctx->in_flight.busy(hidden, uses[0].n, false)) p.wait_before_load = 1;
             const InFlight::Order order = ctx->in_flight.next(
-                uses, 7, !ctx->trusted || ctx->profiling || ctx->op_last_seq + 1 != ctx->op_seq,
+                uses, 7, ctx->profiling || ctx->op_last_seq + 1 != ctx->op_seq,
                 p.n_tiles * kLinSplit * 8 <= ctx->sm_count * 7 ? 3 : InFlight::kMaxChain + 1);
             ctx->op_last_seq = ctx->op_seq;
             fc.enabled = 1;
@@ -996,7 +996,7 @@ static kvzap_status launch_score(kvzap_ctx *ctx, int32_t layer, int32_t n_layers
             fc.n_stages = kLinStagesCompact;
             fc.wait_limit = ctx->wait_limit;
             p.wait_before_write = order.wait;
-            p.late_trigger = order.late && ctx->trusted;
+            p.late_trigger = order.late;
             p.maskbits = nullptr;
             smem = lin_smem_bytes(kLinStagesCompact);
             if (compacted) *compacted = true;
@@ -2423,8 +2423,7 @@ static kvzap_status launch_compaction_paged(kvzap_ctx *ctx, const uint32_t *mask
     }
     PageAssign assign;
     memset(&assign, 0, sizeof assign);
-    if (!append && page_cursor == nullptr && n_words * c.n_kv_heads <= kAssignWords &&
-        static_cast<int64_t>(n_seqs) * c.n_kv_heads <= kAssignLists) {
+    if (ctx->trusted && !append && page_cursor == nullptr && short_input(n_words, c.n_kv_heads, n_seqs)) {
         assign.enabled = 1;
         assign.first_page = first_page;
         assign.max_pages = max_pages;

@@ -588,7 +588,7 @@ assign_pages_locally(const PageAssign &a, const uint32_t *__restrict__ maskbits,
 // l runs beside the scoring of layer l + 1 at full width; at 72 registers only one fits and the layer
 // period of the fused path grows by ~10 us.
 // kAlone: the launch that runs beside nothing (a context that does not trust its producers: the scoring behind it waits
-// for it); see launch_compaction.  gridDim.z CTAs share the kept rows of a block.
+// for it); see launch_compaction.  It assigns no pages: the inputs short enough for that take compact_short_kernel.  gridDim.z CTAs share the kept rows of a block.
 template <int kThreads, bool kAlone>
 __global__ void __launch_bounds__(kThreads, 1024 / kThreads)
 compact_dense_kernel(const uint4 *__restrict__ K, const uint4 *__restrict__ V, uint4 *__restrict__ K_out,
@@ -611,7 +611,7 @@ compact_dense_kernel(const uint4 *__restrict__ K, const uint4 *__restrict__ V, u
     __shared__ int64_t dst_row[kBlockTokens];
     __shared__ int32_t red[2][kThreads / 32];
     __shared__ int32_t base_next_s;
-    __shared__ int32_t s_page0[kAssignLists];
+    __shared__ int32_t s_page0[kAlone ? 1 : kAssignLists];
     const int h = blockIdx.y;
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const int64_t blk0 = static_cast<int64_t>(blockIdx.x) * blocks_per_cta;
@@ -628,8 +628,9 @@ compact_dense_kernel(const uint4 *__restrict__ K, const uint4 *__restrict__ V, u
     if (blockIdx.x == 0 && z == 0 && cu_seqlens != nullptr && !paged)   // empty sequences have no last token to write for them
         for (int b = tid; b < n_seqs; b += kThreads)
             if (cu_seqlens[b + 1] == cu_seqlens[b]) lengths[b * n_heads + h] = 0;
-    if (assign.enabled)
-        assign_pages_locally<kThreads>(assign, maskbits, n_words, cu_seqlens, n_seqs, n_tokens, n_heads, page_tokens, lengths, s_page0);
+    const bool assigned = !kAlone && assign.enabled;
+    if constexpr (!kAlone)
+        if (assigned) assign_pages_locally<kThreads>(assign, maskbits, n_words, cu_seqlens, n_seqs, n_tokens, n_heads, page_tokens, lengths, s_page0);
     if (blk0 >= n_blocks) return;
 
     // rows kept before this CTA's first token, and before the start of the sequence in progress there
@@ -686,7 +687,7 @@ compact_dense_kernel(const uint4 *__restrict__ K, const uint4 *__restrict__ V, u
                     src_tok[r] = tid;
                     const int64_t n = running + r - base;                  // rank inside list (b,h)
                     if (paged) {
-                        const int32_t p0 = assign.enabled ? s_page0[b * n_heads + h] : __ldcg(list_page0 + b * n_heads + h);
+                        const int32_t p0 = assigned ? s_page0[b * n_heads + h] : __ldcg(list_page0 + b * n_heads + h);
                         if (list_base == nullptr) {
                             dst_row[r] = p0 < 0 ? -1 : static_cast<int64_t>(p0) * page_tokens + n;      // pages in a row
                         } else {

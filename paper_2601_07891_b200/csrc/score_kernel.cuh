@@ -87,7 +87,7 @@ struct ScoreParams {
     const float *w1_scale;        // stacked over all layers [L][w_rows], one scale per first-layer output row
     // few-token kernel only: the clusters of one tile combine their partial scores through global memory
     float *split_part;            // [n_tiles][n_split][128][8]
-    uint32_t *split_arrive;       // [n_tiles] slices that have arrived, zero between launches
+    uint32_t *split_arrive;       // [n_tiles][kTileWarps] (kFew: [kFewWarps]) slices that have arrived, zero between launches
     int32_t x_rows;               // few-token kernel, kFew: rows of X that a CTA stages, n_tokens in whole eights
     int32_t block0;               // first 128-token block of the launch (the blocks that whole waves leave over)
 };

@@ -278,8 +278,7 @@ score_linear_split_kernel(const __grid_constant__ CUtensorMap tmap_x, const __gr
             asm volatile("cp.async.commit_group;" ::: "memory");
         };
         // Which rows they are is known now, where they go only when the tiles before have said how many they keep: the first
-        // round's loads go out ahead of that (us a layer, calls in a row: 300 tokens 6.3 -> 6.0, 8100 16.1 -> 15.7; default contexts 4000 25.6 ->
-        // 24.5, 8000 30.1 -> 28.6)
+        // round's loads go out ahead of that (us a layer, calls in a row: 300 tokens 6.3 -> 6.0, 8100 16.1 -> 15.7)
         load_rows(0);
         // rows kept before this tile: the counts of the tiles before it (every CTA of the cluster adds them up itself)
         {

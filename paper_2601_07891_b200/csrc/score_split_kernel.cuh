@@ -25,7 +25,7 @@
 // ahead in the stream.
 //
 // Warp roles as in score_kernel: warp 0 TMA producer, warp 1 MMA issuer / TMEM owner, warps 2..9
-// epilogue (TMEM lane quarter = warp % 4; the two warps of a quarter take alternate 16-column chunks).
+// epilogue (TMEM lane quarter = warp % 4; the two warps of a quarter take eight columns in turn; kFew: see below).
 #pragma once
 
 #include "decode_kernels.cuh"
