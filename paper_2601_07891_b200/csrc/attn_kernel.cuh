@@ -33,7 +33,8 @@
 // A warp waits for the step, and lets the next one start, while tiles are in flight (behind all of them the copies ran dry, and the
 // chain step - wait - next step was the longer by the time of two tiles; when it does: kWaitBase), the new lengths and the second look at the queries share a round trip, and the parts of a list are counted in by one
 // release instead of two fences: 36 layers x 8 sequences x 2176 rows 808 -> 740 us, 12 x 4 201 -> 193, 12 x 8 8-bit 279 -> 265, 12 x 32 8-bit
-// 419 -> 392 (with the steps of score_split_kernel's kFew on both sides).
+// 419 -> 392 (with the steps of score_split_kernel's kFew on both sides).  (Each pair here and below is of one GPU; from one GPU to another the
+// same code differs by up to a tenth, most over 8-bit rows.)
 //
 // Math per tile, on the warp-level tensor-core path (the work is HBM-bound; 16-row MMAs are enough):
 //   S[16 x 16]  = Q[16 x D] K^T      m16n8k16, Q rows 0..G-1 real, the rest zero
