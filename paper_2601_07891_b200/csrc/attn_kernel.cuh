@@ -286,7 +286,8 @@ decode_attn_kernel(const __grid_constant__ CUtensorMap tmap_kpool, const __grid_
         }
         if (list >= p.head_lists) {
             const int tiles = ((kBeside ? n_before : n_prefix) + min(kBeside ? c.window : n_total, c.window)) / kAttnTileRows;
-            n_parts = max(n_parts, min(p.tail_parts, tiles / kAttnTailTiles));
+            // as many as the other lists have, or more; a list that is over in 16 tiles has one
+            n_parts = tiles < 16 ? 1 : max(n_parts, min(p.tail_parts, tiles / kAttnTailTiles));
             if (part >= n_parts) {                                 // the whole CTA
                 if (beside) griddep_wait();
                 return;

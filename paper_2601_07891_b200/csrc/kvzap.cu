@@ -2910,8 +2910,9 @@ static kvzap_status attention_impl(kvzap_ctx *ctx, kvzap_cache *cache, int32_t l
         if (parts > 1) p.n_parts = static_cast<int32_t>(parts);
         // The lists that the device takes up last are cut finer: their CTAs end when few others are left to share the memory
         // with.  One wave of them, into parts of no less than 900 rows of the longest list, as far as the scratch goes (of a list that
-        // turns out short the kernel makes fewer, but no fewer than of the others).  The CTAs for it come last: among the others those
-        // of short lists, which leave at once, cost 2 to 3 us a launch.  Us, lists cut alike / the last ones finer: 4 layers x 128
+        // turns out short the kernel makes fewer, but no fewer than of the others, down to 16 tiles: 480 lists of 100 rows 20.0 us as the
+        // others, 17.6 in one part).  The CTAs for it come last: among the others those of short lists, which leave at
+        // once, cost 2 to 3 us a launch.  Us, lists cut alike / the last ones finer: 4 layers x 128
         // sequences x 4736 rows layer by layer 1537 / 1489, 12 layers in one call x 20 sequences x 2130 rows 342 / 320, x 64 x 1664 8-bit
         // rows 542 / 521, 36 x 32 x 1150 856 / 845; a call in tables for 32768 rows a list, 480 lists of some 600 rows 52.4 / 49.0, 2048 of 100
         // 31.9 / 32.3.  With four parts whatever the lists' room, 12 x 100 x 880 8-bit rows 482 / 487, 4 x 60 x 750 103.5 / 106.
